@@ -1,0 +1,85 @@
+// Integer (fixed-point) evaluation of the exponential.
+//
+// Why: an FP64 warp instruction occupies this part's FP64 pipe for 16 cycles
+// per SM (2 lanes a clock), a 32 x 32 -> 64 multiply-add (IMAD.WIDE) about
+// 1.1 and a plain integer instruction 0.3 to 0.5 (measured, cycles per warp
+// instruction per SM).  A Horner step in 64-bit fixed point (three
+// IMAD.WIDE) therefore costs a quarter of an FP64 FMA, and its 60 or more
+// significant bits leave the final rounding to binary64 as the only error
+// that matters (below 0.54 ulp in all).  Against the same method in nine FP64
+// operations: 53-species source terms, 1 Mi states, 35.8 -> 22.3 ms; CSR
+// Jacobian, 256 ki states, 22.8 -> 19.9 ms; VJP, 64 ki states, 10.3 -> 8.8 ms.
+//
+// Method: table-driven reduction after P. T. P. Tang, "Table-driven
+// implementation of the exponential function in IEEE floating-point
+// arithmetic", ACM TOMS 15 (1989), in base 2:
+//   2^(n + j/256 + f) = 2^n T_j (1 + f c1 + f^2 c2 + .. + f^5 c5),
+//   0 <= f < 2^-8, c_k = (ln 2)^k / k! (Taylor; truncation below 2^-60),
+// with T_j = 2^(j/256) and the polynomial in unsigned fixed point.
+#pragma once
+
+#include <cstdint>
+
+#include <cuda_runtime.h>
+
+namespace pj {
+
+// high 64 bits of a b, short of the exact value by at most 1 (the low
+// partial product is left out)
+__host__ __device__ __forceinline__ uint64_t mulhi_approx(uint64_t a, uint64_t b) {
+  const uint32_t a0 = (uint32_t)a, a1 = (uint32_t)(a >> 32), b0 = (uint32_t)b, b1 = (uint32_t)(b >> 32);
+  const uint64_t u = (uint64_t)a0 * b1;
+  const uint64_t v = (uint64_t)a1 * b0 + (uint32_t)u;
+  return (uint64_t)a1 * b1 + (u >> 32) + (v >> 32);
+}
+
+__host__ __device__ __forceinline__ uint32_t mulhi32(uint32_t a, uint32_t b) {
+  return (uint32_t)(((uint64_t)a * b) >> 32);
+}
+
+// bits of the double 2^(n + frac 2^-64), -1022 <= n <= 1022, rounded to
+// nearest; tab[j] = round(2^63 2^(j/256)).  Error before the rounding below
+// 2^-59 relative.
+__host__ __device__ __forceinline__ uint64_t exp2_fixed(int n, uint64_t frac, const uint64_t* tab) {
+  const uint64_t T = tab[(uint32_t)(frac >> 56)];
+  const uint64_t F = frac << 8;                                  // f 2^72
+  const uint32_t F1 = (uint32_t)(F >> 32);                       // f 2^40
+  uint32_t q = 0x5762u;                                          // c5 2^24
+  q = 0x00276557u + (mulhi32(F1, q) >> 4);                        // c4 2^28 (q 2^32 -> 2^28)
+  q = 0xe35846b8u + mulhi32(F1, q);                              // c3 2^36
+  const uint32_t h = mulhi32(F1, q);                             // (c3 f + ..) 2^44
+  const uint64_t s = 0x0f5fdeffc162c754ull + ((uint64_t)h << 18);  // c2 2^62
+  const uint64_t P = 0xb17217f7d1cf79acull + (mulhi_approx(F, s) >> 6);  // c1 2^64
+  const uint64_t v = mulhi_approx(F, P);                         // (2^f - 1) 2^72
+  const uint64_t M = T + (mulhi_approx(T, v) >> 8);              // 2^63 2^(j/256 + f)
+  return (((M >> 10) + 1u) >> 1) + ((uint64_t)(int64_t)(n + 1022) << 52);
+}
+
+// bits of exp(x) for the double with bits b, |x| < 704: |x| and |x| log2(e)
+// in 86 fractional bits (exact for |x| >= 2^-34), the sign applied to the
+// fixed-point value.
+__host__ __device__ __forceinline__ uint64_t exp_fixed_bits(uint64_t b, const uint64_t* tab) {
+  const uint32_t hi = (uint32_t)(b >> 32);
+  const int sh = 1032 - (int)((hi >> 20) & 0x7ffu);              // >= 0
+  const int shc = sh > 63 ? 63 : sh;                             // |x| < 2^-54 (zero, subnormal): exp(x) rounds to 1
+  const uint64_t m = (b << 11) | 0x8000000000000000ull;          // significand 2^63
+  const uint64_t X = sh > 63 ? 0 : m >> shc;                     // |x| 2^54 ...
+  const uint32_t r = (uint32_t)(((m << 1) << (63 - shc)) >> 32);   // ... and the 32 bits below
+  // |x| (log2(e) - 1) from the constant's first 96 bits
+  const uint32_t x0 = (uint32_t)X, x1 = (uint32_t)(X >> 32);
+  const uint64_t u = (uint64_t)x0 * 0x71547652u;
+  const uint64_t v = (uint64_t)x1 * 0xb82fe177u + (uint32_t)u;
+  const uint64_t w = (uint64_t)r + (uint32_t)v + mulhi32(x1, 0x7d0ffda0u) + mulhi32(x0, 0xb82fe177u) + mulhi32(r, 0x71547652u);
+  uint64_t Y = X + ((uint64_t)x1 * 0x71547652u + (u >> 32) + (v >> 32) + (w >> 32));
+  uint32_t y = (uint32_t)w;
+  int n = 0;
+  if ((int32_t)hi < 0) {
+    n = (Y | y) != 0 ? -1024 : 0;
+    y = 0u - y;
+    Y = ~Y + (y == 0u);
+  }
+  n += (int)(Y >> 54);
+  return exp2_fixed(n, (Y << 10) | (y >> 22), tab);
+}
+
+}  // namespace pj

@@ -68,7 +68,7 @@ __global__ void __launch_bounds__(128) k_source_terms(DevMech m, int64_t n, cons
 }
 
 // pj_exp next to the library exp, for verification (pj_diag_exp).
-__global__ void k_diag_exp(const double* __restrict__ tab, int64_t n, const double* __restrict__ x,
+__global__ void k_diag_exp(const uint64_t* __restrict__ tab, int64_t n, const double* __restrict__ x,
                            double* __restrict__ y_ours, double* __restrict__ y_lib) {
   load_exp_table(tab);
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {

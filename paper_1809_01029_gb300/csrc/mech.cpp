@@ -508,14 +508,14 @@ int mech_build(pj_mech* m) {
   const size_t o_pcsc = align256(o_pcsr + (size_t)N * N * sizeof(int32_t));
   const size_t o_perm = align256(o_pcsc + (size_t)N * N * sizeof(int32_t));
   const size_t o_etab = align256(o_perm + (size_t)nr * sizeof(int32_t));
-  const size_t o_tab = align256(o_etab + 256 * sizeof(double));
+  const size_t o_tab = align256(o_etab + 256 * sizeof(uint64_t));
   const size_t o_tcsr = align256(o_tab + tab.size() * sizeof(double));
   const size_t o_tcsc = align256(o_tcsr + tgt_csr.size() * sizeof(int32_t));
   const size_t o_dbg = align256(o_tcsc + tgt_csc.size() * sizeof(int32_t));
   const size_t total = align256(o_dbg + sizeof(uint32_t));
-  // 2^(j/256) in extended precision, rounded once to double
-  double etab[256];
-  for (int j = 0; j < 256; j++) etab[j] = (double)std::exp2((long double)j / 256.0L);
+  // 2^63 2^(j/256) from extended precision
+  uint64_t etab[256];
+  for (int j = 0; j < 256; j++) etab[j] = (uint64_t)std::floor(std::exp2((long double)j / 256.0L) * 0x1p63L + 0.5L);
 
   std::vector<char> blob(total, 0);
   auto put = [&](size_t off, const void* src, size_t bytes) { if (bytes) std::memcpy(blob.data() + off, src, bytes); };
@@ -568,7 +568,7 @@ int mech_build(pj_mech* m) {
   dm.pos_csr = reinterpret_cast<const int32_t*>(b + o_pcsr);
   dm.pos_csc = reinterpret_cast<const int32_t*>(b + o_pcsc);
   dm.perm = reinterpret_cast<const int32_t*>(b + o_perm);
-  dm.exp_tab = reinterpret_cast<const double*>(b + o_etab);
+  dm.exp_tab = reinterpret_cast<const uint64_t*>(b + o_etab);
   dm.tab = reinterpret_cast<const double*>(b + o_tab);
   dm.tgt_csr = reinterpret_cast<const int32_t*>(b + o_tcsr);
   dm.tgt_csc = reinterpret_cast<const int32_t*>(b + o_tcsc);

@@ -84,7 +84,7 @@ struct DevMech {
   const int32_t* tgt_csr;         // per reaction, the value indices its sparse contributions
   const int32_t* tgt_csc;         //   go to, in the order the Jacobian kernels make them
   const int32_t* perm;            // [nr] kernel order -> original reaction index
-  const double* exp_tab;          // [256] 2^(j/256), correctly rounded (pj_exp)
+  const uint64_t* exp_tab;        // [256] 2^63 2^(j/256), rounded (pj_exp)
   const double* tab;              // P-log entries (ln P, ln A, beta, theta) and Chebyshev
                                   // blocks (cT1, cT0, cP1, cP0, ln10 * a_tp row-major)
   int32_t has_pdep;               // some reaction depends on P (P-log, Chebyshev)
