@@ -1,4 +1,5 @@
-// Integer (fixed-point) evaluation of the exponential.
+// Integer (fixed-point) evaluation of exponentials, logarithms and the
+// exponents of rate constants.
 //
 // Why: an FP64 warp instruction occupies this part's FP64 pipe for 16 cycles
 // per SM (2 lanes a clock), a 32 x 32 -> 64 multiply-add (IMAD.WIDE) about
@@ -80,6 +81,67 @@ __host__ __device__ __forceinline__ uint64_t exp_fixed_bits(uint64_t b, const ui
   }
   n += (int)(Y >> 54);
   return exp2_fixed(n, (Y << 10) | (y >> 22), tab);
+}
+
+// One entry of the logarithm's table: r = ceil(2^15 / (1 + j/256)),
+// t = round(2^62 log2(2^15 / r)).
+struct LogEntry {
+  uint64_t t;
+  uint64_t r;
+};
+
+// log2 of the positive normal double with bits b as e + f 2^-62, e the
+// exponent of b (returned in e), 0 <= f <= 2^62.  With m the significand and
+// r from the table, z = m r 2^-15 - 1 lies in [0, 1.02 2^-8] and is exact in
+// 64 bits (m r - 2^67 modulo 2^64); log2(m) = t + log2(1 + z) by the series
+// z (k1 - z (k2 - ..)), k_i = 1 / (i ln 2), six terms.  Absolute error below
+// 2^-54.
+__host__ __device__ __forceinline__ uint64_t log2_fixed(uint64_t b, int& e, const LogEntry* __restrict__ tab) {
+  const uint32_t hi = (uint32_t)(b >> 32);
+  e = (int)(hi >> 20) - 1023;
+  const LogEntry t = tab[(hi >> 12) & 255u];
+  const uint64_t m = (b & 0x000fffffffffffffull) | 0x0010000000000000ull;
+  const uint64_t F = (m * (uint32_t)t.r) << 4;                   // z 2^71
+  const uint32_t F1 = (uint32_t)(F >> 32), z32 = F1 >> 7;        // z 2^39, z 2^32
+  uint32_t q = 0x49ddb144u - mulhi32(z32, 0x3d8e13b8u);          // (k5 - z k6) 2^32
+  q = 0x5c551d95u - mulhi32(z32, q);                             // k4
+  q = 0x7b1c2771u - mulhi32(z32, q);                             // k3
+  const uint64_t s = 0x5c551d94ae0bf85eull - (((uint64_t)F1 * q) >> 8);  // (k2 - ..) 2^63
+  const uint64_t P = 0x5c551d94ae0bf85eull - (mulhi_approx(F, s) >> 8);  // (k1 - ..) 2^62
+  return t.t + (mulhi_approx(F, P) >> 7);
+}
+
+// c b 2^-64 for a signed constant c and an unsigned b, short by at most 2
+__host__ __device__ __forceinline__ int64_t mulhi_su(int64_t c, uint64_t b) {
+  return (int64_t)(mulhi_approx((uint64_t)c, b) - (c < 0 ? b : 0));
+}
+
+__host__ __device__ __forceinline__ int clz64(uint64_t x) {
+#ifdef __CUDA_ARCH__
+  return __clzll((long long)x);
+#else
+  return x ? __builtin_clzll(x) : 64;
+#endif
+}
+
+// bits of the double x 2^-s (rounded to nearest, ties up), |x| 2^-s within
+// the normal range or 0; integer instructions where the hardware conversion
+// would take an FP64-pipe slot
+__host__ __device__ __forceinline__ uint64_t fixed_to_double(int64_t x, int s) {
+  const uint64_t a = x < 0 ? 0 - (uint64_t)x : (uint64_t)x;
+  const int lz = clz64(a);
+  const uint64_t m = a << (lz & 63);
+  const uint64_t r = (((m >> 10) + 1u) >> 1) + ((uint64_t)(1085 - lz - s) << 52);
+  return a == 0 ? 0 : r | ((uint64_t)x & 0x8000000000000000ull);
+}
+
+// log2 of an Arrhenius rate constant, 2^51: A, beta and theta as packed in a
+// reaction's record (fA holds 3/4 of a unit per product, their mean truncation),
+// L = log2(T) 2^59, IT = 2^70 / T.  128 <= T < 65536 keeps both unsigned and
+// below 2^63.
+__host__ __device__ __forceinline__ int64_t arrhenius_fixed(int64_t fA, int64_t fB, int64_t fT, uint64_t L,
+                                                            uint64_t IT) {
+  return fA + mulhi_su(fB, L) + mulhi_su(fT, IT);
 }
 
 }  // namespace pj

@@ -63,11 +63,10 @@ __global__ void __launch_bounds__(128) k_eval_y(DevMech m, int64_t n, const doub
     for (int k = 0; k < ns; k++) {
       double cp, h, sr;
       nasa_eval(nasa_block(m, k, T), T, invT, lnT, cp, h, sr);
-      A.at(aG, k) = h - sr;
+      A.at(aG, k) = fixed_gibbs(m, h - sr, st.fx.fast);
       den = fma(A.at(aC, k), MODE == PJ_CONP ? cp : cp - 1.0, den);
     }
     den *= RU;
-    const double logPRT = m.log_pstd_over_r - lnT;
     double w_bath = 0.0;
     // Plain reactions (the first m.nr_plain in kernel order) run through a
     // body compiled without the special cases (chemically activated, explicit
@@ -77,23 +76,18 @@ __global__ void __launch_bounds__(128) k_eval_y(DevMech m, int64_t n, const doub
       const Rxn* __restrict__ r = m.rxn + i;
       const int kind = __ldg(&r->kind);
       const int nre = __ldg(&r->nreac), npr = __ldg(&r->nprod), rev = __ldg(&r->rev);
-      double lnkinf, u0, u1, u2;
-      const double lnkf = ln_kf<false, GEN>(m, r, kind, lnT, invT, st.lnP, lnkinf, u0, u1, u2);
-      double kf, kr;
-      rate_constants<GEN>(m, A, aG, r, rev, nre, npr, lnkf, logPRT, lnT, invT, kf, kr);
+      const RateK k = rate_constants<GEN>(m, A, aG, r, kind, rev, nre, npr, st.fx, T, lnT, invT, st.lnP);
       double dmy[PJ_MAX_SP];
-      const double Rf = side_rate<false>(A, aC, r, 0, __ldg(&r->shape[0]), nre, kf, dmy);
-      const double Rr = rev ? side_rate<false>(A, aC, r, PJ_MAX_SP, __ldg(&r->shape[1]), npr, kr, dmy) : 0.0;
+      const double Rf = side_rate<false>(A, aC, r, 0, __ldg(&r->shape[0]), nre, k.kf, dmy);
+      const double Rr = rev ? side_rate<false>(A, aC, r, PJ_MAX_SP, __ldg(&r->shape[1]), npr, k.kr, dmy) : 0.0;
       double c = 1.0;
       if (has_third_body(kind)) {
         const double M = third_body(m, A, aC, r, st.Ctot);
         if (kind == PJ_THIRD_BODY) {
           c = M;
         } else {
-          const double lnk0 = fma(__ldg(&r->beta0), lnT, __ldg(&r->lnA0)) - __ldg(&r->theta0) * invT;
-          const double Pr = pj_exp(lnk0 - lnkinf) * M;
-          double d1, d2;
-          const double F = falloff_F<false>(r, kind, T, invT, lnT, Pr, d1, d2);
+          double F, d1, d2;
+          const double Pr = falloff_Pr_F<false>(m, r, kind, st.fx, T, invT, lnT, k, M, F, d1, d2);
           c = ((GEN && __ldg(&r->chem)) ? 1.0 : Pr) / (1.0 + Pr) * F;
         }
       }
@@ -166,7 +160,7 @@ __global__ void __launch_bounds__(128, kVjpCtas) k_vjp(DevMech m, int64_t n, con
       st.V = 1.0;
       st.P = 1e5;
       st.invT = 1e-3;
-      st.lnT = log(1000.0);
+      temperature_terms(m, st.T, st.invT, st.lnT, st.fx);
       st.lnP = log(1e5);
       st.Ctot = st.P / (RU * st.T);
       for (int k = 0; k < ns; k++) A.at(aC, k) = st.Ctot / ns;
@@ -187,7 +181,7 @@ __global__ void __launch_bounds__(128, kVjpCtas) k_vjp(DevMech m, int64_t n, con
       double cp, h, sr, cp2, dcp;
       nasa_eval(cb, T, invT, lnT, cp, h, sr);
       nasa_cp(cb, T, cp2, dcp);
-      A.at(aG, k) = h - sr;
+      A.at(aG, k) = fixed_gibbs(m, h - sr, st.fx.fast);
       A.at(aH, k) = h;
       A.at(aU, k) = ok ? u_wdot[(int64_t)k * ld + s] : 0.0;
       const double Ck = A.at(aC, k);
@@ -203,7 +197,6 @@ __global__ void __launch_bounds__(128, kVjpCtas) k_vjp(DevMech m, int64_t n, con
     const double dCb_S = MODE == PJ_CONP ? (Ctot - C_bath) * invV : Ctot / P;
     dden_T = RU * dden_T + Cx_bath * dCb_T;
     const double dden_S = MODE == PJ_CONP ? (Cx_bath * Ctot - den) * invV : Cx_bath * Ctot / P;
-    const double logPRT = m.log_pstd_over_r - lnT;
     const double mR_calT = -1.0 / (R_CAL * T);
 
     double gT = 0.0, gS = 0.0, gB = 0.0, w_bath = 0.0;
@@ -215,10 +208,9 @@ __global__ void __launch_bounds__(128, kVjpCtas) k_vjp(DevMech m, int64_t n, con
       const Rxn* __restrict__ r = m.rxn + i;
       const int kind = __ldg(&r->kind);
       const int nre = __ldg(&r->nreac), npr = __ldg(&r->nprod), rev = __ldg(&r->rev);
-      double lnkinf, dlnkf, dlnP, dlnkinf;
-      const double lnkf = ln_kf<true, GEN>(m, r, kind, lnT, invT, st.lnP, lnkinf, dlnkf, dlnP, dlnkinf);
-      double kf, kr;
-      rate_constants<GEN>(m, A, aG, r, rev, nre, npr, lnkf, logPRT, lnT, invT, kf, kr);
+      double dlnkf, dlnP, dlnkinf;
+      ln_kf_derivatives<GEN>(m, r, kind, lnT, invT, invT2, st.lnP, dlnkf, dlnP, dlnkinf);
+      const RateK rk = rate_constants<GEN>(m, A, aG, r, kind, rev, nre, npr, st.fx, T, lnT, invT, st.lnP);
       double dh = 0.0, du = 0.0;
 #pragma unroll
       for (int a = 0; a < PJ_MAX_SP; a++) {
@@ -236,10 +228,10 @@ __global__ void __launch_bounds__(128, kVjpCtas) k_vjp(DevMech m, int64_t n, con
         }
       }
       double dRf[PJ_MAX_SP], dRr[PJ_MAX_SP];
-      const double Rf = side_rate<true>(A, aC, r, 0, __ldg(&r->shape[0]), nre, kf, dRf);
+      const double Rf = side_rate<true>(A, aC, r, 0, __ldg(&r->shape[0]), nre, rk.kf, dRf);
       double Rr = 0.0, dlnkr = 0.0;
       if (rev) {
-        Rr = side_rate<true>(A, aC, r, PJ_MAX_SP, __ldg(&r->shape[1]), npr, kr, dRr);
+        Rr = side_rate<true>(A, aC, r, PJ_MAX_SP, __ldg(&r->shape[1]), npr, rk.kr, dRr);
         if (GEN && rev == 2)
           dlnkr = fma(__ldg(m.tab + __ldg(&r->tab_lo) + 2), invT2, __ldg(m.tab + __ldg(&r->tab_lo) + 1) * invT);
         else
@@ -261,15 +253,11 @@ __global__ void __launch_bounds__(128, kVjpCtas) k_vjp(DevMech m, int64_t n, con
           dcdT = dMdT;
           dcdS = dMdS;
         } else {
-          const double beta0 = __ldg(&r->beta0), theta0 = __ldg(&r->theta0);
-          const double lnk0 = fma(beta0, lnT, __ldg(&r->lnA0)) - theta0 * invT;
-          const double dlnk0 = fma(theta0, invT2, beta0 * invT);
-          const double rk = pj_exp(lnk0 - lnkinf);
-          const double Pr = rk * M;
-          double FxPr, FT;
-          const double F = falloff_F<true>(r, kind, T, invT, lnT, Pr, FxPr, FT);
+          const double dlnk0 = fma(__ldg(&r->theta0), invT2, __ldg(&r->beta0) * invT);
+          double F, FxPr, FT;
+          const double Pr = falloff_Pr_F<true>(m, r, kind, st.fx, T, invT, lnT, rk, M, F, FxPr, FT);
           const double i1p = 1.0 / (1.0 + Pr);
-          const double dPrdT = Pr * (dlnk0 - dlnkinf) + rk * dMdT;
+          const double dPrdT = Pr * (dlnk0 - dlnkinf) + rk.rk * dMdT;
           double cPr;
           if (GEN && __ldg(&r->chem)) {
             c = F * i1p;
@@ -281,7 +269,7 @@ __global__ void __launch_bounds__(128, kVjpCtas) k_vjp(DevMech m, int64_t n, con
             cPr = F * i1p * i1p + FxPr * i1p;
             dcdT = fr * FT + cPr * dPrdT;
           }
-          dcdM = cPr * rk;
+          dcdM = cPr * rk.rk;
           dcdS = dcdM * dMdS;
           Qpr = -Rn * cPr * Pr;  // k_inf divides Pr
         }

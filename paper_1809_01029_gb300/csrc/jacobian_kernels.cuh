@@ -111,13 +111,14 @@ constexpr int kCoopWarpsMax = 16;
 enum CoopSc {
   cT, cV, cP, cInvT, cInvV, cLnT, cLnP, cCtot, cCdum, cCxB, cDcpB, cDen, cDdenT, cDdenS, cDCbT, cDCbS,
   // the energy and state rows' per-state values (JacRowVars)
+  cL, cIT, cLP,  // FixedState (64-bit integers)
   cIden, cTdot, cRtvp, cCT, cJ00, cJ01, cX0, cX1, cAT_T, cAT_S, cAS_T, cAS_S, cATB, cASB, kCoopSc
 };
 // per-warp partial sums, [W][kCoopPart][32] doubles
 enum CoopPart { pAcc, pDen, pDden, pNum, pSum, pOm, pAT_T, pAT_S, pAS_T, pAS_S, pATB, pASB, pWb, kCoopPart };
 
-// per-state flags (int): valid T, V, P; valid state
-enum CoopFlag { fOk0, fOk, kCoopFlag };
+// per-state flags (int): valid T, V, P; valid state; fixed-point rate constants
+enum CoopFlag { fOk0, fOk, fFast, kCoopFlag };
 
 // per-state arrays C_k, g_k/RT then Cx_k, h_k/RT of a tile: [3][Ns][32] doubles
 __host__ __device__ constexpr size_t coop_arrays_bytes(int ns) {
@@ -237,9 +238,17 @@ __global__ void __launch_bounds__(MAXW * 32, 1)
       S(cT) = T;
       S(cV) = V;
       S(cP) = P;
-      S(cInvT) = 1.0 / T;
+      const double invT = 1.0 / T;
+      double lnT;
+      FixedState fx;
+      temperature_terms(m, T, invT, lnT, fx);
+      S(cInvT) = invT;
       S(cInvV) = 1.0 / V;
-      S(cLnT) = log(T);
+      S(cLnT) = lnT;
+      S(cL) = __longlong_as_double((long long)fx.L);
+      S(cIT) = __longlong_as_double((long long)fx.IT);
+      S(cLP) = __longlong_as_double((long long)fx.LP);
+      F(fFast) = fx.fast;
       S(cLnP) = m.has_pdep ? log(P) : 0.0;
       const double Ctot = P / (RU * T);
       S(cCtot) = Ctot;
@@ -263,12 +272,13 @@ __global__ void __launch_bounds__(MAXW * 32, 1)
       const double T = S(cT), V = S(cV), invT = S(cInvT), lnT = S(cLnT), cdum = S(cCdum);
       const bool ok0 = F(fOk0) != 0;
       double acc = 0.0, den = 0.0, dden = 0.0;
+      bool fast = true;
       for (int k = warp; k < ns; k += W) {
         const double* cb = nasa_block(m, k, T);
         double cp, h, sr, cp2, dcp;
         nasa_eval(cb, T, invT, lnT, cp, h, sr);
         nasa_cp(cb, T, cp2, dcp);
-        A.at(aG, k) = h - sr;
+        A.at(aG, k) = fixed_gibbs(m, h - sr, fast);
         A.at(aH, k) = h;
         const double cx = MODE == PJ_CONP ? cp : cp - 1.0;
         if (k < bath) {
@@ -282,6 +292,7 @@ __global__ void __launch_bounds__(MAXW * 32, 1)
           S(cDcpB) = dcp;
         }
       }
+      if (!fast) F(fFast) = 0;
       Pw(warp, pAcc) = acc;
       Pw(warp, pDen) = den;
       Pw(warp, pDden) = dden;
@@ -331,7 +342,10 @@ __global__ void __launch_bounds__(MAXW * 32, 1)
       v.Ctot = S(cCtot);
       v.invT2 = v.invT * v.invT;
       v.invV = S(cInvV);
-      v.logPRT = m.log_pstd_over_r - v.lnT;
+      v.fx.L = (uint64_t)__double_as_longlong(S(cL));
+      v.fx.IT = (uint64_t)__double_as_longlong(S(cIT));
+      v.fx.LP = __double_as_longlong(S(cLP));
+      v.fx.fast = F(fFast) != 0;
       v.dCb_T = S(cDCbT);
       v.dCb_S = S(cDCbS);
       v.AT_T = v.AT_S = v.AS_T = v.AS_S = v.ATB = v.ASB = DT(0);

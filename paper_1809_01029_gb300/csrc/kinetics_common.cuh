@@ -13,10 +13,69 @@
 
 namespace pj {
 
+// Per-state inputs of the fixed-point rate constants (fixed_math.cuh).  fast:
+// they may be used (128 K <= T < 65536 K and every |g_k/RT| in range, see
+// fixed_gibbs); other states take the FP64 path, out of line.
+struct FixedState {
+  uint64_t L, IT;  // log2(T) 2^59, 2^70 / T
+  int64_t LP;      // log2(P_std / (R T)) 2^51
+  bool fast;
+};
+
 struct StateScalars {
   double T, V, P, invT, lnT, Ctot;
   double lnP;  // ln P [Pa], formed only when some reaction depends on pressure
+  FixedState fx;
 };
+
+// ln T and the fixed-point inputs of temperature T > 0 (invT = 1/T rounded).
+// 1/T carries the residual of the rounding, ln T is log2(T) ln 2 from the
+// fixed point: both at least as exact as the FP64 operations.
+__device__ __forceinline__ void temperature_terms(const DevMech& m, double T, double invT, double& lnT,
+                                                  FixedState& f) {
+  f.fast = m.fx_ok && T >= 128.0 && T < 65536.0;
+  f.L = f.IT = 0;
+  f.LP = 0;
+  if (!f.fast) {
+    lnT = log(T);
+    return;
+  }
+  int e;
+  const uint64_t l = log2_fixed((uint64_t)__double_as_longlong(T), e, m.log_tab);
+  f.L = ((uint64_t)e << 59) + (l >> 3);
+  f.LP = m.log2_pstd_fx - (int64_t)(f.L >> 8);
+  lnT = __longlong_as_double((long long)fixed_to_double((int64_t)mulhi_approx(f.L, 0xb17217f7d1cf79acull), 59));
+  f.IT = __double2ull_rn(invT * 0x1p70) + (uint64_t)__double2ll_rn(fma(-T, invT, 1.0) * (invT * 0x1p70));
+}
+
+// g_k/RT as log2 units 2^51 (stored where the FP64 value would be); clears
+// fast when it is out of range
+__device__ __forceinline__ double fixed_gibbs(const DevMech& m, double g, bool& fast) {
+  fast = fast && ((uint32_t)__double2hiint(g) & 0x7fffffffu) < m.fx_g_hi;
+  return __longlong_as_double(__double2ll_rn(g * (1.4426950408889634074 * 0x1p51)));
+}
+
+// 2^(y 2^-51) as a double
+__device__ __noinline__ static double exp2_fixed_library(int64_t y) {
+  return exp2((double)y * 0x1p-51);
+}
+__device__ __forceinline__ double exp2_51(int64_t y) {
+  // |y| < 1016: a normal result
+  if ((uint32_t)(y >> 32) + (1016u << 19) >= (2032u << 19)) return exp2_fixed_library(y);
+  return __longlong_as_double((long long)exp2_fixed((int)(y >> 51), (uint64_t)y << 13, pj_exp_tab));
+}
+
+// log2 of a positive normal double, 2^51; ok = false for anything else
+__device__ __forceinline__ int64_t log2_51(const DevMech& m, double x, bool& ok) {
+  ok = ok && (uint32_t)__double2hiint(x) - 0x00100000u < 0x7fe00000u;
+  int e;
+  const uint64_t l = log2_fixed((uint64_t)__double_as_longlong(x), e, m.log_tab);
+  return ((int64_t)e << 51) + (int64_t)(l >> 11);
+}
+
+__device__ __forceinline__ double fixed51_to_double(int64_t y) {
+  return __longlong_as_double((long long)fixed_to_double(y, 51));
+}
 
 __device__ __forceinline__ bool has_third_body(int kind) { return kind >= PJ_THIRD_BODY && kind <= PJ_SRI; }
 
@@ -46,24 +105,83 @@ __device__ __forceinline__ bool load_state(const DevMech& m, const double* __res
   st.V = V;
   st.P = P;
   st.invT = 1.0 / T;
-  st.lnT = log(T);
+  temperature_terms(m, T, st.invT, st.lnT, st.fx);
   st.Ctot = Ctot;
   return ok;
 }
 
 // Troe / SRI broadening factor F(T, Pr) in FP64.  With derivatives also
-// returns FxPr = Pr dF/dPr (at fixed T) and FT = dF/dT (at fixed Pr),
-// evaluated in the derivative type DT (FP64, or FP32 for the Newton form).
-template <bool DERIV, typename DT = double>
-__device__ __forceinline__ double falloff_F(const Rxn* __restrict__ r, int kind, double T, double invT,
-                                            double lnT, double Pr, DT& FxPr, DT& FT) {
-  FxPr = DT(0);
-  FT = DT(0);
+// returns FxPr = Pr dF/dPr (at fixed T) and FT = dF/dT (at fixed Pr).  The
+// logarithms are fixed-point (l2Pr = log2(Pr) 2^51); ok = false, with nothing
+// returned, when an argument is not a positive normal number.
+//
+// Troe: with D = N - 0.14 xc and S = D^2 + xc^2, log10 F = L g, g = D^2 / S
+// (1 / (1 + (xc/D)^2)), so that F and its derivatives take one reciprocal:
+// dg/dx = -2 N xc D / S^2.  A log, an exp and a divide each were 9 to 30 FP64
+// operations; the fixed-point ones are none.
+template <bool DERIV>
+__device__ __forceinline__ double falloff_F(const DevMech& m, const Rxn* __restrict__ r, int kind, double T,
+                                            double invT, double lnT, int64_t l2Pr, bool& ok, double& FxPr,
+                                            double& FT) {
+  FxPr = 0.0;
+  FT = 0.0;
+  constexpr double LOG10_2 = 0.30102999566398119521;
   if (kind == PJ_TROE) {
     const double a = __ldg(&r->fp[0]), iT3 = __ldg(&r->fp[1]), iT1 = __ldg(&r->fp[2]);
     const double T2 = __ldg(&r->fp[3]), has2 = __ldg(&r->fp[4]);
     const double e3 = pj_exp(-T * iT3), e1 = pj_exp(-T * iT1);
     const double e2 = has2 != 0.0 ? pj_exp(-T2 * invT) : 0.0;
+    const double Fcent = (1.0 - a) * e3 + a * e1 + e2;
+    const double l2F = fixed51_to_double(log2_51(m, Fcent, ok));
+    if (!ok) return 1.0;
+    const double L = l2F * LOG10_2;
+    const double xc = fixed51_to_double(l2Pr) * LOG10_2 + (-0.4 - 0.67 * L);
+    const double NN = 0.75 - 1.27 * L;
+    const double D = NN - 0.14 * xc;
+    const double D2 = D * D;
+    const double iS = 1.0 / fma(xc, xc, D2);
+    const double g = D2 * iS;
+    const double F = pj_exp(LN10 * (L * g));
+    if (DERIV) {
+      const double t = -2.0 * (xc * D) * (L * iS) * iS;  // L dg/dx / N
+      const double dlg_dL = g + t * (1.1762 * xc - 0.67 * D);
+      const double dFcent = -(1.0 - a) * iT3 * e3 - a * iT1 * e1 + T2 * (invT * invT) * e2;
+      FxPr = F * (t * NN);
+      FT = F * dlg_dL * dFcent / Fcent;
+    }
+    return F;
+  }
+  if (kind == PJ_SRI) {
+    const double a = __ldg(&r->fp[0]), b = __ldg(&r->fp[1]), ic = __ldg(&r->fp[2]);
+    const double d = __ldg(&r->fp[3]), e = __ldg(&r->fp[4]);
+    const double x = fixed51_to_double(l2Pr) * LOG10_2;
+    const double X = 1.0 / (1.0 + x * x);
+    const double eb = pj_exp(-b * invT), ec = pj_exp(-T * ic);
+    const double Z = a * eb + ec;
+    const double lnZ = fixed51_to_double(log2_51(m, Z, ok)) * 0.69314718055994530942;
+    if (!ok) return 1.0;
+    const double F = d * pj_exp(X * lnZ + e * lnT);
+    if (DERIV) {
+      FxPr = F * (lnZ * (-2.0 * x * X * X)) * (1.0 / LN10);
+      const double dZ = (a * b) * invT * invT * eb - ic * ec;
+      FT = F * (X * dZ / Z + e * invT);
+    }
+    return F;
+  }
+  return 1.0;  // Lindemann
+}
+
+// The same with the library's logarithm, for any Pr and F_cent (zero, negative,
+// not finite, or a state outside the fixed point's range).  Out of line.
+__device__ __noinline__ static double falloff_F_library(const Rxn* __restrict__ r, int kind, double T, double invT,
+                                                        double lnT, double Pr, double& FxPr, double& FT) {
+  FxPr = 0.0;
+  FT = 0.0;
+  if (kind == PJ_TROE) {
+    const double a = __ldg(&r->fp[0]), iT3 = __ldg(&r->fp[1]), iT1 = __ldg(&r->fp[2]);
+    const double T2 = __ldg(&r->fp[3]), has2 = __ldg(&r->fp[4]);
+    const double e3 = exp(-T * iT3), e1 = exp(-T * iT1);
+    const double e2 = has2 != 0.0 ? exp(-T2 * invT) : 0.0;
     const double Fcent = (1.0 - a) * e3 + a * e1 + e2;
     const double L = log10(Fcent);
     const double x = log10(Pr);
@@ -73,18 +191,13 @@ __device__ __forceinline__ double falloff_F(const Rxn* __restrict__ r, int kind,
     const double D = NN - 0.14 * xc;
     const double f1 = xc / D;
     const double g = 1.0 / (1.0 + f1 * f1);
-    const double F = pj_exp(LN10 * (L * g));
-    if (DERIV) {
-      const DT Lt = DT(L), Dt = DT(D), f1t = DT(f1), gt = DT(g), Ft = DT(F), xct = DT(xc);
-      const DT iD = DT(1) / Dt;
-      const DT iD2 = iD * iD;
-      const DT m2fg2 = DT(-2) * f1t * gt * gt;
-      const DT dlg_dx = Lt * m2fg2 * DT(NN) * iD2;
-      const DT dlg_dL = gt + Lt * m2fg2 * (DT(-0.67) * Dt + DT(1.1762) * xct) * iD2;
-      const DT dFcent = DT(-(1.0 - a) * iT3) * DT(e3) - DT(a * iT1) * DT(e1) + DT(T2) * DT(invT * invT) * DT(e2);
-      FxPr = Ft * dlg_dx;
-      FT = Ft * dlg_dL * dFcent / DT(Fcent);
-    }
+    const double F = exp(LN10 * (L * g));
+    const double iD2 = 1.0 / (D * D);
+    const double m2fg2 = -2.0 * f1 * g * g;
+    const double dlg_dL = g + L * m2fg2 * (-0.67 * D + 1.1762 * xc) * iD2;
+    const double dFcent = -(1.0 - a) * iT3 * e3 - a * iT1 * e1 + T2 * (invT * invT) * e2;
+    FxPr = F * (L * m2fg2 * NN * iD2);
+    FT = F * dlg_dL * dFcent / Fcent;
     return F;
   }
   if (kind == PJ_SRI) {
@@ -92,19 +205,16 @@ __device__ __forceinline__ double falloff_F(const Rxn* __restrict__ r, int kind,
     const double d = __ldg(&r->fp[3]), e = __ldg(&r->fp[4]);
     const double x = log10(Pr);
     const double X = 1.0 / (1.0 + x * x);
-    const double eb = pj_exp(-b * invT), ec = pj_exp(-T * ic);
+    const double eb = exp(-b * invT), ec = exp(-T * ic);
     const double Z = a * eb + ec;
     const double lnZ = log(Z);
-    const double F = d * pj_exp(X * lnZ + e * lnT);
-    if (DERIV) {
-      const DT Xt = DT(X), Ft = DT(F), xt = DT(x), it = DT(invT);
-      FxPr = Ft * (DT(lnZ) * (DT(-2) * xt * Xt * Xt)) * DT(1.0 / LN10);
-      const DT dZ = DT(a * b) * it * it * DT(eb) - DT(ic) * DT(ec);
-      FT = Ft * (Xt * dZ / DT(Z) + DT(e) * it);
-    }
+    const double F = d * exp(X * lnZ + e * lnT);
+    FxPr = F * (lnZ * (-2.0 * x * X * X)) * (1.0 / LN10);
+    const double dZ = (a * b) * invT * invT * eb - ic * ec;
+    FT = F * (X * dZ / Z + e * invT);
     return F;
   }
-  return 1.0;  // Lindemann
+  return 1.0;
 }
 
 __device__ __forceinline__ double dneg(double x) {
@@ -276,65 +386,138 @@ __device__ __noinline__ double lnk_pdep(const DevMech& m, const Rxn* __restrict_
   return S;
 }
 
-// ln of reaction r's forward rate constant: the Arrhenius set for
-// elementary, third-body and falloff reactions, the low-pressure set for
-// chemically-activated ones, the P-log / Chebyshev forms otherwise.  lnkinf
-// is the Arrhenius set itself (the high-pressure limit in Pr).  With DER:
-// d_T, d_lnP of ln k_f and dinf_T of ln k_inf.
 template <bool B>
 struct BoolTag {
   static constexpr bool value = B;
 };
 
-template <bool DER, bool GEN = true>
-__device__ __forceinline__ double ln_kf(const DevMech& m, const Rxn* __restrict__ r, int kind, double lnT,
-                                        double invT, double lnP, double& lnkinf, double& d_T, double& d_lnP,
-                                        double& dinf_T) {
-  const double beta = __ldg(&r->beta), theta = __ldg(&r->theta);
-  lnkinf = fma(beta, lnT, __ldg(&r->lnA)) - theta * invT;
-  if (DER) {
-    dinf_T = fma(theta, invT * invT, beta * invT);
-    d_T = dinf_T;
-    d_lnP = 0.0;
-  }
-  if (!GEN) return lnkinf;  // plain reactions: the Arrhenius set
-  if (kind >= PJ_PLOG) return lnk_pdep<DER>(m, r, kind, lnT, invT, lnP, d_T, d_lnP);
-  if (__ldg(&r->chem)) {
-    const double beta0 = __ldg(&r->beta0), theta0 = __ldg(&r->theta0);
-    if (DER) d_T = fma(theta0, invT * invT, beta0 * invT);
-    return fma(beta0, lnT, __ldg(&r->lnA0)) - theta0 * invT;
-  }
-  return lnkinf;
+// Temperature and pressure derivatives of ln k: d_T, d_lnP of ln k_f (the
+// Arrhenius set for elementary, third-body and falloff reactions, the
+// low-pressure set for chemically-activated ones, the P-log / Chebyshev forms
+// otherwise) and dinf_T of ln k_inf (the Arrhenius set itself).
+template <bool GEN>
+__device__ __forceinline__ void ln_kf_derivatives(const DevMech& m, const Rxn* __restrict__ r, int kind, double lnT,
+                                                  double invT, double invT2, double lnP, double& d_T, double& d_lnP,
+                                                  double& dinf_T) {
+  dinf_T = fma(__ldg(&r->theta), invT2, __ldg(&r->beta) * invT);
+  d_T = dinf_T;
+  d_lnP = 0.0;
+  if (!GEN) return;
+  if (kind >= PJ_PLOG) lnk_pdep<true>(m, r, kind, lnT, invT, lnP, d_T, d_lnP);
+  else if (__ldg(&r->chem)) d_T = fma(__ldg(&r->theta0), invT2, __ldg(&r->beta0) * invT);
 }
 
-// Forward and reverse rate constants; the two exponentials sit in one basic
-// block so their dependency chains interleave.  rev == 2: explicit reverse
-// Arrhenius set instead of k_f / K_c.
-template <bool GEN = true, class SA>
-__device__ __forceinline__ void rate_constants(const DevMech& m, const SA& A, int aG, const Rxn* __restrict__ r,
-                                               int rev,
-                                               int nre, int npr, double lnkf, double logPRT, double lnT,
-                                               double invT, double& kf, double& kr) {
+// Rate constants of one reaction: k_f, k_r (0 when irreversible) and, for
+// falloff, rk = k_0 / k_inf and its log2 (2^51).
+struct RateK {
+  double kf, kr, rk;
+  int64_t l2rk;
+};
+
+// sum_k nu_k g_k/RT of a reaction, from the thermo polynomials (states
+// outside the fixed point's range)
+__device__ __noinline__ static double gibbs_sum(const double* __restrict__ nasa, const Rxn* __restrict__ r, double T,
+                                                double invT, double lnT) {
+  double dg = 0.0;
+  for (int a = 0; a < 2 * PJ_MAX_SP; a++) {
+    const bool react = a < PJ_MAX_SP;
+    if (react ? a >= __ldg(&r->nreac) : a - PJ_MAX_SP >= __ldg(&r->nprod)) continue;
+    const double* b = nasa + (size_t)__ldg(&r->sp[a]) * NASA_STRIDE;
+    if (!(T < __ldg(b + 14))) b += 16;
+    double cp, h, sr;
+    nasa_eval(b, T, invT, lnT, cp, h, sr);
+    dg = fma(react ? -__ldg(&r->nud[a]) : __ldg(&r->nud[a]), h - sr, dg);
+  }
+  return dg;
+}
+
+// The same in FP64 with the library's range: states outside the fixed
+// point's range.  Out of line.
+template <bool GEN>
+__device__ __noinline__ static void rate_constants_library(const DevMech& m, const Rxn* __restrict__ r, double T,
+                                                           double invT, double lnT, double lnP, RateK& k) {
+  const int kind = __ldg(&r->kind), rev = __ldg(&r->rev);
+  const double lninf = fma(__ldg(&r->beta), lnT, __ldg(&r->lnA)) - __ldg(&r->theta) * invT;
+  const double ln0 = fma(__ldg(&r->beta0), lnT, __ldg(&r->lnA0)) - __ldg(&r->theta0) * invT;
+  double lnkf = lninf, u0, u1;
+  if (GEN && kind >= PJ_PLOG) lnkf = lnk_pdep<false>(m, r, kind, lnT, invT, lnP, u0, u1);
+  else if (GEN && __ldg(&r->chem)) lnkf = ln0;
+  k.kf = exp(lnkf);
+  k.kr = 0.0;
   if (GEN && rev == 2) {
     const double* __restrict__ rt = m.tab + __ldg(&r->tab_lo);
-    const double larg = fma(__ldg(rt + 1), lnT, __ldg(rt)) - __ldg(rt + 2) * invT;
-    kf = pj_exp(lnkf);
-    kr = pj_exp(larg);
+    k.kr = exp(fma(__ldg(rt + 1), lnT, __ldg(rt)) - __ldg(rt + 2) * invT);
   } else if (rev) {
-    double dg = 0.0;
+    // kr = kf / Kc with Kc = exp(-dg) (P_std / R T)^dnu
+    k.kr = exp(lnkf + gibbs_sum(m.nasa, r, T, invT, lnT) - __ldg(&r->dnu) * (m.log_pstd_over_r - lnT));
+  }
+  k.rk = kind >= PJ_LINDEMANN && kind <= PJ_SRI ? exp(ln0 - lninf) : 0.0;
+  k.l2rk = 0;
+}
+
+// The exponents are sums of 64-bit fixed-point terms (the sum over the
+// species' Gibbs energies as integer adds), each within 2^-51 of exact, where
+// FP64 terms of size 32 to 64 round at 2^-48.
+template <bool GEN = true, class SA>
+__device__ __forceinline__ RateK rate_constants(const DevMech& m, const SA& A, int aG, const Rxn* __restrict__ r,
+                                                int kind, int rev, int nre, int npr, const FixedState& fx, double T,
+                                                double lnT, double invT, double lnP) {
+  RateK k;
+  if (!fx.fast) {
+    rate_constants_library<GEN>(m, r, T, invT, lnT, lnP, k);
+    return k;
+  }
+  int64_t y = arrhenius_fixed(__ldg(&r->fA), __ldg(&r->fB), __ldg(&r->fT), fx.L, fx.IT);
+  k.rk = 0.0;
+  k.l2rk = 0;
+  if (kind >= PJ_LINDEMANN && kind <= PJ_SRI) {
+    const int64_t y0 = arrhenius_fixed(__ldg(&r->fA0), __ldg(&r->fB0), __ldg(&r->fT0), fx.L, fx.IT);
+    k.l2rk = y0 - y;
+    k.rk = exp2_51(k.l2rk);
+    if (GEN && __ldg(&r->chem)) y = y0;
+  }
+  k.kr = 0.0;
+  if (GEN && rev == 2) {
+    const double* __restrict__ rt = m.tab + __ldg(&r->tab_lo);
+    k.kr = pj_exp(fma(__ldg(rt + 1), lnT, __ldg(rt)) - __ldg(rt + 2) * invT);
+    rev = 0;
+  }
+  int64_t dg = 0;  // log2(k_r / k_f): kr = kf / Kc, Kc = exp(-sum nu g) (P_std / R T)^dnu
+  if (rev) {
 #pragma unroll
     for (int a = 0; a < PJ_MAX_SP; a++) {
-      if (a < nre) dg = fma(-__ldg(&r->nud[a]), A.at(aG, __ldg(&r->sp[a])), dg);
-      if (a < npr) dg = fma(__ldg(&r->nud[PJ_MAX_SP + a]), A.at(aG, __ldg(&r->sp[PJ_MAX_SP + a])), dg);
+      if (a < nre) dg -= __ldg(&r->nu[a]) * __double_as_longlong(A.at(aG, __ldg(&r->sp[a])));
+      if (a < npr) dg += __ldg(&r->nu[PJ_MAX_SP + a]) * __double_as_longlong(A.at(aG, __ldg(&r->sp[PJ_MAX_SP + a])));
     }
-    // kr = kf / Kc with Kc = exp(-dg) (P_std / R T)^dnu
-    const double larg = lnkf + dg - __ldg(&r->dnu) * logPRT;
-    kf = pj_exp(lnkf);
-    kr = pj_exp(larg);
-  } else {
-    kf = pj_exp(lnkf);
-    kr = 0.0;
+    dg -= __ldg(&r->dnu_i) * fx.LP;
   }
+  if (GEN && kind >= PJ_PLOG) {
+    double u0, u1;
+    const double lnkf = lnk_pdep<false>(m, r, kind, lnT, invT, lnP, u0, u1);
+    k.kf = pj_exp(lnkf);
+    if (rev) k.kr = pj_exp(fma(fixed51_to_double(dg), 0.69314718055994530942, lnkf));
+    return k;
+  }
+  k.kf = exp2_51(y);
+  if (rev) k.kr = exp2_51(y + dg);
+  return k;
+}
+
+// Pressure modification of a falloff reaction: Pr and, in F, FxPr, FT, the
+// broadening factor and its derivatives (falloff_F).
+template <bool DERIV>
+__device__ __forceinline__ double falloff_Pr_F(const DevMech& m, const Rxn* __restrict__ r, int kind,
+                                               const FixedState& fx, double T, double invT, double lnT,
+                                               const RateK& k, double M, double& F, double& FxPr, double& FT) {
+  const double Pr = k.rk * M;
+  F = 1.0;
+  FxPr = FT = 0.0;
+  if (kind == PJ_LINDEMANN) return Pr;
+  bool ok = fx.fast;
+  const int64_t l2Pr = k.l2rk + log2_51(m, M, ok);
+  if (ok) F = falloff_F<DERIV>(m, r, kind, T, invT, lnT, l2Pr, ok, FxPr, FT);
+  if (!ok) F = falloff_F_library(r, kind, T, invT, lnT, Pr, FxPr, FT);
+  return Pr;
 }
 
 // Third-body concentration [M] = C_tot + sum_e (alpha_e - 1) C_e.

@@ -27,11 +27,10 @@ __device__ __forceinline__ void source_state(const DevMech& m, const SA& A, cons
   for (int k = 0; k < ns; k++) {
     double cp, h, sr;
     nasa_eval(nasa_block(m, k, T), T, invT, lnT, cp, h, sr);
-    A.at(aG, k) = h - sr;
+    A.at(aG, k) = fixed_gibbs(m, h - sr, st.fx.fast);
     den = fma(A.at(aC, k), MODE == PJ_CONP ? cp : cp - 1.0, den);
   }
   den *= RU;
-  const double logPRT = m.log_pstd_over_r - lnT;  // ln(P_std / (R T))
   double w_bath = 0.0;
 
   // Plain reactions (the first m.nr_plain in kernel order) run through a
@@ -44,23 +43,18 @@ __device__ __forceinline__ void source_state(const DevMech& m, const SA& A, cons
     const Rxn* __restrict__ r = m.rxn + i;
     const int kind = __ldg(&r->kind);
     const int nre = __ldg(&r->nreac), npr = __ldg(&r->nprod), rev = __ldg(&r->rev);
-    double lnkinf, u0, u1, u2;
-    const double lnkf = ln_kf<false, GEN>(m, r, kind, lnT, invT, st.lnP, lnkinf, u0, u1, u2);
-    double kf, kr;
-    rate_constants<GEN>(m, A, aG, r, rev, nre, npr, lnkf, logPRT, lnT, invT, kf, kr);
+    const RateK k = rate_constants<GEN>(m, A, aG, r, kind, rev, nre, npr, st.fx, T, lnT, invT, st.lnP);
     double dmy[PJ_MAX_SP];
-    const double Rf = side_rate<false>(A, aC, r, 0, __ldg(&r->shape[0]), nre, kf, dmy);
-    const double Rr = rev ? side_rate<false>(A, aC, r, PJ_MAX_SP, __ldg(&r->shape[1]), npr, kr, dmy) : 0.0;
+    const double Rf = side_rate<false>(A, aC, r, 0, __ldg(&r->shape[0]), nre, k.kf, dmy);
+    const double Rr = rev ? side_rate<false>(A, aC, r, PJ_MAX_SP, __ldg(&r->shape[1]), npr, k.kr, dmy) : 0.0;
     double c = 1.0;
     if (has_third_body(kind)) {
       const double M = third_body(m, A, aC, r, st.Ctot);
       if (kind == PJ_THIRD_BODY) {
         c = M;
       } else {
-        const double lnk0 = fma(__ldg(&r->beta0), lnT, __ldg(&r->lnA0)) - __ldg(&r->theta0) * invT;
-        const double Pr = pj_exp(lnk0 - lnkinf) * M;
-        double d1, d2;
-        const double F = falloff_F<false>(r, kind, T, invT, lnT, Pr, d1, d2);
+        double F, d1, d2;
+        const double Pr = falloff_Pr_F<false>(m, r, kind, st.fx, T, invT, lnT, k, M, F, d1, d2);
         // falloff: k_inf Pr/(1+Pr) F; chemically activated: k0 F/(1+Pr)
         c = ((GEN && __ldg(&r->chem)) ? 1.0 : Pr) / (1.0 + Pr) * F;
       }
@@ -148,7 +142,8 @@ __device__ __forceinline__ DT nu_times_t(int nu, double, DT x) {
 template <typename DT>
 struct JacVars {
   double T, V, P, invT, lnT, lnP, Ctot;
-  double invT2, invV, logPRT, dCb_T, dCb_S;  // dCb_*: derivatives of the bath-gas concentration
+  double invT2, invV, dCb_T, dCb_S;  // dCb_*: derivatives of the bath-gas concentration
+  FixedState fx;
   // energy-row (T) and state-row (S) weights for the T and S columns and for
   // the part common to every species column; bath-gas production rate
   DT AT_T, AT_S, AS_T, AS_S, ATB, ASB;
@@ -194,11 +189,11 @@ __device__ __forceinline__ void jac_reaction(const DevMech& m, const SA& A, JacV
   const int kind = __ldg(&r->kind);
   const int nre = __ldg(&r->nreac), npr = __ldg(&r->nprod);
   const int rev = __ldg(&r->rev);
-  double lnkinf, dlnkf_d, dlnP_d, dlnkinf_d;
-  const double lnkf = ln_kf<true, GEN>(m, r, kind, lnT, invT, v.lnP, lnkinf, dlnkf_d, dlnP_d, dlnkinf_d);
+  double dlnkf_d, dlnP_d, dlnkinf_d;
+  ln_kf_derivatives<GEN>(m, r, kind, lnT, invT, invT2, v.lnP, dlnkf_d, dlnP_d, dlnkinf_d);
   const DT dlnkf = DT(dlnkf_d);
-  double kf, kr;
-  rate_constants<GEN>(m, A, aG, r, rev, nre, npr, lnkf, v.logPRT, lnT, invT, kf, kr);
+  const RateK rk = rate_constants<GEN>(m, A, aG, r, kind, rev, nre, npr, v.fx, T, lnT, invT, v.lnP);
+  const double kf = rk.kf, kr = rk.kr;
   double dh = 0.0;
   if (TM) __syncwarp();
 #pragma unroll
@@ -234,20 +229,16 @@ __device__ __forceinline__ void jac_reaction(const DevMech& m, const SA& A, JacV
       dcdT = dMdT;
       dcdS = dMdS;
     } else {
-      const double beta0 = __ldg(&r->beta0), theta0 = __ldg(&r->theta0);
-      const double lnk0 = fma(beta0, lnT, __ldg(&r->lnA0)) - theta0 * invT;
-      const double dlnk0 = fma(theta0, invT2, beta0 * invT);
+      const double dlnk0 = fma(__ldg(&r->theta0), invT2, __ldg(&r->beta0) * invT);
       // per-reaction scalars of the blending function, in FP64 whatever DT
       // (its derivative can subtract terms of similar size)
-      const double rk = pj_exp(lnk0 - lnkinf);
-      const double Pr = rk * M;
-      double FxPr, FT;
-      const double F = falloff_F<true, double>(r, kind, T, invT, lnT, Pr, FxPr, FT);
+      double F, FxPr, FT;
+      const double Pr = falloff_Pr_F<true>(m, r, kind, v.fx, T, invT, lnT, rk, M, F, FxPr, FT);
       const double i1p = 1.0 / (1.0 + Pr);
       const double ab_d = __ldg(&r->alpha_bath);
       const double dMdT_d = ab_d * v.dCb_T;
       const double dMdS_d = MODE == PJ_CONP ? (ab_d * Ctot - M) * invV : ab_d * Ctot / P;
-      const double dPrdT = Pr * (dlnk0 - dlnkinf_d) + rk * dMdT_d;
+      const double dPrdT = Pr * (dlnk0 - dlnkinf_d) + rk.rk * dMdT_d;
       double cPr, dcdT_d;
       if (GEN && __ldg(&r->chem)) {
         // c = F / (1 + Pr): dc/dPr = (dF/dPr) / (1 + Pr) - F / (1 + Pr)^2
@@ -262,8 +253,8 @@ __device__ __forceinline__ void jac_reaction(const DevMech& m, const SA& A, JacV
         dcdT_d = fr * FT + cPr * dPrdT;
       }
       dcdT = DT(dcdT_d);
-      dcdM = DT(cPr * rk);
-      dcdS = DT(cPr * rk * dMdS_d);
+      dcdM = DT(cPr * rk.rk);
+      dcdS = DT(cPr * rk.rk * dMdS_d);
     }
   }
   const DT c_t = DT(c);
@@ -577,7 +568,7 @@ __device__ __forceinline__ void jacobian_state(const DevMech& m, const SA& A,
     st.V = 1.0;
     st.P = 1e5;
     st.invT = 1e-3;
-    st.lnT = log(1000.0);
+    temperature_terms(m, st.T, st.invT, st.lnT, st.fx);
     st.lnP = log(1e5);
     st.Ctot = st.P / (RU * st.T);
     for (int k = 0; k < ns; k++) A.at(aC, k) = st.Ctot / ns;
@@ -603,7 +594,7 @@ __device__ __forceinline__ void jacobian_state(const DevMech& m, const SA& A,
     double cp, h, sr, cp2, dcp;
     nasa_eval(cb, T, invT, lnT, cp, h, sr);
     nasa_cp(cb, T, cp2, dcp);
-    A.at(aG, k) = h - sr;
+    A.at(aG, k) = fixed_gibbs(m, h - sr, st.fx.fast);
     if (TM) tmem_st_f64(tm_row + 2u * (uint32_t)k, h);
     else A.at(aH, k) = h;
     const double Ck = A.at(aC, k);
@@ -625,7 +616,7 @@ __device__ __forceinline__ void jacobian_state(const DevMech& m, const SA& A,
   v.Ctot = Ctot;
   v.invT2 = invT2;
   v.invV = invV;
-  v.logPRT = m.log_pstd_over_r - lnT;
+  v.fx = st.fx;
   // derivatives of the bath-gas concentration
   v.dCb_T = -Ctot * invT;
   v.dCb_S = MODE == PJ_CONP ? (Ctot - C_bath) * invV : Ctot / P;

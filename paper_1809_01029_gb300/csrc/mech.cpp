@@ -324,6 +324,8 @@ int mech_build(pj_mech* m) {
   std::vector<char> dep;
   std::vector<double> tab;  // P-log entries and Chebyshev blocks
   bool has_pdep = false;
+  bool fx_ok = true;  // every rate constant fits the fixed-point path
+  int nu_max = 1;     // largest sum of the coefficients of both sides of a reversible reaction
   for (int q = 0; q < nr; q++) {
     const int i = m->perm[q];
     Rxn& r = rx[q];
@@ -410,7 +412,33 @@ int mech_build(pj_mech* m) {
       if (k < bath) dW += nu[k] * wfac[k];
     }
     r.dnu = dnu;
+    r.dnu_i = (int32_t)dnu;
     r.dW = dW;
+    // fixed-point Arrhenius sets; a set beyond their ranges (every sum of
+    // exponent terms must stay within the 2^12 of the fixed point) leaves the
+    // whole mechanism on the FP64 path
+    auto fixed_set = [&](double A, double beta, double Ea, int64_t& fA, int64_t& fB, int64_t& fT) {
+      const long double l2A = std::log2((long double)A);
+      const long double th = (long double)Ea / (long double)R_CAL * 1.442695040888963407359924681001892137L;
+      const long double l2p = std::fabs(std::log2((long double)P_STD / (long double)RU)) + 16.0L;
+      const long double worst = std::fabs(l2A) + 16.0L * std::fabs((long double)beta) + std::fabs(th) / 128.0L +
+                                std::fabs((long double)dnu) * l2p;
+      if (!(worst < 1900.0L) || !(std::fabs(beta) < 100.0) || !(std::fabs(th) < 0x1p17L)) {
+        fx_ok = false;
+        return;
+      }
+      fA = std::llrint(l2A * 0x1p51L + 1.5L);
+      fB = std::llrint((long double)beta * 0x1p56L);
+      fT = -std::llrint(th * 0x1p45L);
+    };
+    if (!pdep) fixed_set(m->A[i], m->beta[i], m->Ea[i], r.fA, r.fB, r.fT);
+    if (is_falloff(r.kind)) fixed_set(m->A0[i], m->beta0[i], m->Ea0[i], r.fA0, r.fB0, r.fT0);
+    if (r.rev) {
+      int side_sum = 0;
+      for (int a = 0; a < 2 * PJ_MAX_SP; a++)
+        side_sum += a < PJ_MAX_SP ? (a < r.nreac ? r.nu[a] : 0) : (a - PJ_MAX_SP < r.nprod ? r.nu[a] : 0);
+      nu_max = std::max(nu_max, side_sum);
+    }
     std::vector<double> al = alpha_of(m, i);
     r.alpha_bath = has_third_body(r.kind) ? al[bath] : 1.0;
     r.eff_lo = (int32_t)eff_sp.size();
@@ -508,7 +536,8 @@ int mech_build(pj_mech* m) {
   const size_t o_pcsc = align256(o_pcsr + (size_t)N * N * sizeof(int32_t));
   const size_t o_perm = align256(o_pcsc + (size_t)N * N * sizeof(int32_t));
   const size_t o_etab = align256(o_perm + (size_t)nr * sizeof(int32_t));
-  const size_t o_tab = align256(o_etab + 256 * sizeof(uint64_t));
+  const size_t o_ltab = align256(o_etab + 256 * sizeof(uint64_t));
+  const size_t o_tab = align256(o_ltab + 256 * sizeof(LogEntry));
   const size_t o_tcsr = align256(o_tab + tab.size() * sizeof(double));
   const size_t o_tcsc = align256(o_tcsr + tgt_csr.size() * sizeof(int32_t));
   const size_t o_dbg = align256(o_tcsc + tgt_csc.size() * sizeof(int32_t));
@@ -516,6 +545,17 @@ int mech_build(pj_mech* m) {
   // 2^63 2^(j/256) from extended precision
   uint64_t etab[256];
   for (int j = 0; j < 256; j++) etab[j] = (uint64_t)std::floor(std::exp2((long double)j / 256.0L) * 0x1p63L + 0.5L);
+
+  // r = ceil(2^15 / (1 + j/256)), t = log2(2^15 / r)
+  LogEntry ltab[256];
+  for (int j = 0; j < 256; j++) {
+    ltab[j].r = (uint64_t)((32768 * 256 + 255 + j) / (256 + j));
+    ltab[j].t = (uint64_t)std::floor(std::log2(32768.0L / (long double)ltab[j].r) * 0x1p62L + 0.5L);
+  }
+  // |g_k/RT| up to which sum nu g stays within half the fixed point's range
+  const double g_lim = std::min(1300.0, 2000.0 * 0.6931471805599453 / nu_max);
+  uint64_t g_bits;
+  std::memcpy(&g_bits, &g_lim, sizeof g_bits);
 
   std::vector<char> blob(total, 0);
   auto put = [&](size_t off, const void* src, size_t bytes) { if (bytes) std::memcpy(blob.data() + off, src, bytes); };
@@ -529,6 +569,7 @@ int mech_build(pj_mech* m) {
   put(o_pcsc, m->pos_csc.data(), m->pos_csc.size() * sizeof(int32_t));
   put(o_perm, m->perm.data(), m->perm.size() * sizeof(int32_t));
   put(o_etab, etab, sizeof etab);
+  put(o_ltab, ltab, sizeof ltab);
   put(o_tab, tab.data(), tab.size() * sizeof(double));
   put(o_tcsr, tgt_csr.data(), tgt_csr.size() * sizeof(int32_t));
   put(o_tcsc, tgt_csc.data(), tgt_csc.size() * sizeof(int32_t));
@@ -569,6 +610,10 @@ int mech_build(pj_mech* m) {
   dm.pos_csc = reinterpret_cast<const int32_t*>(b + o_pcsc);
   dm.perm = reinterpret_cast<const int32_t*>(b + o_perm);
   dm.exp_tab = reinterpret_cast<const uint64_t*>(b + o_etab);
+  dm.log_tab = reinterpret_cast<const LogEntry*>(b + o_ltab);
+  dm.log2_pstd_fx = std::llrint(std::log2((long double)P_STD / (long double)RU) * 0x1p51L);
+  dm.fx_ok = fx_ok ? 1 : 0;
+  dm.fx_g_hi = (uint32_t)(g_bits >> 32);
   dm.tab = reinterpret_cast<const double*>(b + o_tab);
   dm.tgt_csr = reinterpret_cast<const int32_t*>(b + o_tcsr);
   dm.tgt_csc = reinterpret_cast<const int32_t*>(b + o_tcsc);

@@ -6,6 +6,7 @@
 #include <string>
 #include <vector>
 
+#include "fixed_math.cuh"
 #include "pyjac_gb.h"
 
 namespace pj {
@@ -59,6 +60,11 @@ struct alignas(8) Rxn {
   int16_t tab_n, tab_m;           // P-log entries / Chebyshev N_T, N_P
   int32_t tgt_lo;                 // first of this reaction's Jacobian targets in tgt_csr / tgt_csc
   int32_t bath_in;                // the bath gas is one of its reactants or products
+  int32_t dnu_i, pad_;            // dnu as an integer
+  // the Arrhenius sets in fixed point (fixed_math.cuh: arrhenius_fixed):
+  // log2(A) 2^51, beta 2^56, -theta log2(e) 2^45
+  int64_t fA, fB, fT;             // (lnA, beta, theta)
+  int64_t fA0, fB0, fT0;          // (lnA0, beta0, theta0)
 };
 
 // One unit of a reaction's net stoichiometric coefficient for species k: a
@@ -73,6 +79,11 @@ struct RowNu {
 struct DevMech {
   int32_t ns, nr, N, nnz;
   double log_pstd_over_r;         // ln(P_std / R)
+  int64_t log2_pstd_fx;           // log2(P_std / R) 2^51
+  // fixed-point rate constants: usable for every reaction when fx_ok, at
+  // states with |g_k/RT| below the double whose high word is fx_g_hi
+  int32_t fx_ok;
+  uint32_t fx_g_hi;
   const double* nasa;             // [ns * NASA_STRIDE]
   const double* wfac;             // [ns] 1 - W_k / W_{Ns-1}
   const Rxn* rxn;                 // [nr]
@@ -85,6 +96,7 @@ struct DevMech {
   const int32_t* tgt_csc;         //   go to, in the order the Jacobian kernels make them
   const int32_t* perm;            // [nr] kernel order -> original reaction index
   const uint64_t* exp_tab;        // [256] 2^63 2^(j/256), rounded (pj_exp)
+  const LogEntry* log_tab;        // [256] table of log2_fixed
   const double* tab;              // P-log entries (ln P, ln A, beta, theta) and Chebyshev
                                   // blocks (cT1, cT0, cP1, cP0, ln10 * a_tp row-major)
   int32_t has_pdep;               // some reaction depends on P (P-log, Chebyshev)
