@@ -38,22 +38,33 @@ __host__ __device__ __forceinline__ uint32_t mulhi32(uint32_t a, uint32_t b) {
   return (uint32_t)(((uint64_t)a * b) >> 32);
 }
 
-// bits of the double 2^(n + frac 2^-64), -1022 <= n <= 1022, rounded to
-// nearest; tab[j] = round(2^63 2^(j/256)).  Error before the rounding below
-// 2^-59 relative.
-__host__ __device__ __forceinline__ uint64_t exp2_fixed(int n, uint64_t frac, const uint64_t* tab) {
+// 2^(frac 2^-64) 2^63; tab[j] = round(2^63 2^(j/256)).  Relative error below
+// 2^-59.
+__host__ __device__ __forceinline__ uint64_t exp2_significand(uint64_t frac, const uint64_t* tab) {
   const uint64_t T = tab[(uint32_t)(frac >> 56)];
   const uint64_t F = frac << 8;                                  // f 2^72
   const uint32_t F1 = (uint32_t)(F >> 32);                       // f 2^40
   uint32_t q = 0x5762u;                                          // c5 2^24
-  q = 0x00276557u + (mulhi32(F1, q) >> 4);                        // c4 2^28 (q 2^32 -> 2^28)
+  q = 0x00276557u + (mulhi32(F1, q) >> 4);                       // c4 2^28
   q = 0xe35846b8u + mulhi32(F1, q);                              // c3 2^36
   const uint32_t h = mulhi32(F1, q);                             // (c3 f + ..) 2^44
   const uint64_t s = 0x0f5fdeffc162c754ull + ((uint64_t)h << 18);  // c2 2^62
   const uint64_t P = 0xb17217f7d1cf79acull + (mulhi_approx(F, s) >> 6);  // c1 2^64
   const uint64_t v = mulhi_approx(F, P);                         // (2^f - 1) 2^72
-  const uint64_t M = T + (mulhi_approx(T, v) >> 8);              // 2^63 2^(j/256 + f)
+  return T + (mulhi_approx(T, v) >> 8);                          // 2^63 2^(j/256 + f)
+}
+
+// bits of the double M 2^(n - 63), -1022 <= n <= 1022, rounded to nearest
+__host__ __device__ __forceinline__ uint64_t pack_double(int n, uint64_t M) {
   return (((M >> 10) + 1u) >> 1) + ((uint64_t)(int64_t)(n + 1022) << 52);
+}
+
+// the same for any n: subnormals, zero and infinity
+__host__ __device__ __forceinline__ uint64_t pack_double_any(int n, uint64_t M) {
+  if ((uint32_t)(n + 1022) < 2045u) return pack_double(n, M);
+  if (n > 0) return 0x7ff0000000000000ull;
+  const int sh = -1022 - n;
+  return sh > 54 ? 0 : (((M >> 10) >> sh) + 1u) >> 1;
 }
 
 // bits of exp(x) for the double with bits b, |x| < 704: |x| and |x| log2(e)
@@ -80,7 +91,7 @@ __host__ __device__ __forceinline__ uint64_t exp_fixed_bits(uint64_t b, const ui
     Y = ~Y + (y == 0u);
   }
   n += (int)(Y >> 54);
-  return exp2_fixed(n, (Y << 10) | (y >> 22), tab);
+  return pack_double(n, exp2_significand((Y << 10) | (y >> 22), tab));
 }
 
 // One entry of the logarithm's table: r = ceil(2^15 / (1 + j/256)),

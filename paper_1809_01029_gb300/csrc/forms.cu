@@ -30,86 +30,6 @@ __device__ __forceinline__ double warp_sum(double v) {
 #define PJ_LANE0(lane) ((lane) == 0)
 #endif
 
-// Forward values y = (wdot_0 .. wdot_{Ns-1}, dT/dt): y[k*ld + s].
-template <int MODE, bool SPECIAL>
-__global__ void __launch_bounds__(128) k_eval_y(DevMech m, int64_t n, const double* __restrict__ param,
-                                                const double* __restrict__ phi, int64_t ld, double* __restrict__ y,
-                                                int* status, double* ws, int64_t ws_stride) {
-  PJ_DYN_SMEM;
-  load_exp_table(m.exp_tab);
-  const int ns = m.ns, bath = m.ns - 1;
-  const int64_t gtid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  StateArrays A;
-  A.ns = ns;
-  if (ws) {
-    A.base = ws + gtid;
-    A.stride = ws_stride;
-  } else {
-    A.base = smem + threadIdx.x;
-    A.stride = blockDim.x;
-  }
-  enum { aC = 0, aG = 1 };
-  for (int64_t s = gtid; s < n; s += (int64_t)gridDim.x * blockDim.x) {
-    StateScalars st;
-    if (!load_state<MODE>(m, phi, param, ld, s, A, aC, st)) {
-      write_nan_state(y, ld, s, ns + 1);
-      if (status) atomicAdd(status, 1);
-      continue;
-    }
-    const double T = st.T, invT = st.invT, lnT = st.lnT;
-    double* __restrict__ wrow = y + s;
-    for (int k = 0; k < ns - 1; k++) wrow[(int64_t)k * ld] = 0.0;
-    double den = 0.0;
-    for (int k = 0; k < ns; k++) {
-      double cp, h, sr;
-      nasa_eval(nasa_block(m, k, T), T, invT, lnT, cp, h, sr);
-      A.at(aG, k) = fixed_gibbs(m, h - sr, st.fx.fast);
-      den = fma(A.at(aC, k), MODE == PJ_CONP ? cp : cp - 1.0, den);
-    }
-    den *= RU;
-    double w_bath = 0.0;
-    // Plain reactions (the first m.nr_plain in kernel order) run through a
-    // body compiled without the special cases (chemically activated, explicit
-    // reverse, P-log, Chebyshev), the rest through the general one.
-    auto reaction = [&](int i, auto gen_tag) {
-      constexpr bool GEN = decltype(gen_tag)::value;
-      const Rxn* __restrict__ r = m.rxn + i;
-      const int kind = __ldg(&r->kind);
-      const int nre = __ldg(&r->nreac), npr = __ldg(&r->nprod), rev = __ldg(&r->rev);
-      const RateK k = rate_constants<GEN>(m, A, aG, r, kind, rev, nre, npr, st.fx, T, lnT, invT, st.lnP);
-      double dmy[PJ_MAX_SP];
-      const double Rf = side_rate<false>(A, aC, r, 0, __ldg(&r->shape[0]), nre, k.kf, dmy);
-      const double Rr = rev ? side_rate<false>(A, aC, r, PJ_MAX_SP, __ldg(&r->shape[1]), npr, k.kr, dmy) : 0.0;
-      double c = 1.0;
-      if (has_third_body(kind)) {
-        const double M = third_body(m, A, aC, r, st.Ctot);
-        if (kind == PJ_THIRD_BODY) {
-          c = M;
-        } else {
-          double F, d1, d2;
-          const double Pr = falloff_Pr_F<false>(m, r, kind, st.fx, T, invT, lnT, k, M, F, d1, d2);
-          c = ((GEN && __ldg(&r->chem)) ? 1.0 : Pr) / (1.0 + Pr) * F;
-        }
-      }
-      const double q = c * (Rf - Rr);
-      scatter_wdot(r, nre, npr, bath, q, wrow, ld, w_bath);
-    };
-    for (int i = 0; i < m.nr_plain; i++) reaction(i, BoolTag<false>{});
-    if (SPECIAL)
-      for (int i = m.nr_plain; i < m.nr; i++) reaction(i, BoolTag<true>{});
-
-    double num = 0.0;
-    for (int k = 0; k < ns; k++) {
-      double cp, h, sr;
-      nasa_eval(nasa_block(m, k, T), T, invT, lnT, cp, h, sr);
-      const double wk = k < bath ? __ldcg(wrow + (int64_t)k * ld) : w_bath;
-      num = fma(MODE == PJ_CONP ? h : h - 1.0, wk, num);
-    }
-    wrow[(int64_t)bath * ld] = w_bath;
-    y[(int64_t)ns * ld + s] = -(num * RU * T) / den;
-  }
-}
-
 // VJP.  Warps walk the batch 32 states at a time so that the per-reaction
 // parameter gradients can be summed over the warp with shuffles.  The
 // forward values y are produced on the way (needed for dT/dt's direct terms).
@@ -178,10 +98,11 @@ __global__ void __launch_bounds__(128, kVjpCtas) k_vjp(DevMech m, int64_t n, con
     double den = 0.0, dden_T = 0.0, Cx_bath = 0.0;
     for (int k = 0; k < ns; k++) {
       const double* cb = nasa_block(m, k, T);
-      double cp, h, sr, cp2, dcp;
-      nasa_eval(cb, T, invT, lnT, cp, h, sr);
+      double cp, g, cp2, dcp;
+      nasa_cp_g(cb, T, invT, lnT, cp, g);
       nasa_cp(cb, T, cp2, dcp);
-      A.at(aG, k) = fixed_gibbs(m, h - sr, st.fx.fast);
+      const double h = nasa_h(cb, T, invT);
+      A.at(aG, k) = fixed_gibbs(m, g, st.fx.fast);
       A.at(aH, k) = h;
       A.at(aU, k) = ok ? u_wdot[(int64_t)k * ld + s] : 0.0;
       const double Ck = A.at(aC, k);
@@ -454,25 +375,9 @@ size_t form_workspace_bytes(int op, const DevMech& m, int64_t n) {
     FormPlan p = form_plan(4, m, n, true);
     return align256(p.ws_bytes) + p.part_bytes;
   }
-  FormPlan p = form_plan(2, m, n, false);
-  return p.ws_bytes;
+  return source_plan(m.ns, n).arrays_bytes;
 }
 
-
-int launch_eval_y(const DevMech& m, int mode, int64_t n, const double* param, const double* phi, int64_t ld,
-                  double* y, int* status, void* work, size_t work_bytes, cudaStream_t st) {
-  FormPlan p = form_plan(2, m, n, false);
-  if (p.global_ws && (!work || work_bytes < p.ws_bytes))
-    return fail(PJ_ERR_NOMEM, "workspace too small for pj_eval_y (see pj_workspace_size)");
-  double* ws = p.global_ws ? static_cast<double*>(work) : nullptr;
-  const bool special = m.nr_plain < m.nr;
-  auto kern = mode == PJ_CONP ? (special ? k_eval_y<PJ_CONP, true> : k_eval_y<PJ_CONP, false>)
-                              : (special ? k_eval_y<PJ_CONV, true> : k_eval_y<PJ_CONV, false>);
-  int rc;
-  if ((rc = set_smem(kern, p.smem))) return rc;
-  kern<<<p.grid, p.tpb, p.smem, st>>>(m, n, param, phi, ld, y, status, ws, p.ws_stride);
-  return check_cuda(cudaGetLastError(), "k_eval_y launch");
-}
 
 int launch_vjp(const DevMech& m, int mode, int64_t n, const double* param, const double* phi, int64_t ld,
                const double* u_wdot, const double* u_T, double* y, double* g_phi, double* g_theta, int* status,

@@ -275,10 +275,11 @@ __global__ void __launch_bounds__(MAXW * 32, 1)
       bool fast = true;
       for (int k = warp; k < ns; k += W) {
         const double* cb = nasa_block(m, k, T);
-        double cp, h, sr, cp2, dcp;
-        nasa_eval(cb, T, invT, lnT, cp, h, sr);
+        double cp, g, cp2, dcp;
+        nasa_cp_g(cb, T, invT, lnT, cp, g);
         nasa_cp(cb, T, cp2, dcp);
-        A.at(aG, k) = fixed_gibbs(m, h - sr, fast);
+        const double h = nasa_h(cb, T, invT);
+        A.at(aG, k) = fixed_gibbs(m, g, fast);
         A.at(aH, k) = h;
         const double cx = MODE == PJ_CONP ? cp : cp - 1.0;
         if (k < bath) {

@@ -34,6 +34,7 @@
 
 #include "jacobian_kernels.cuh"  // k_jacobian_coop's tile and shared-memory size (the kernels: jacobian_inst.cu)
 #include "kinetics_state.cuh"
+#include "source_tile.cuh"
 #ifndef PJ_NO_LAUNCHERS
 #include "launch.h"
 #endif
@@ -43,28 +44,24 @@ namespace pj {
 // ---------------------------------------------------------------------------
 // source terms
 // ---------------------------------------------------------------------------
-// Shared memory holds C_k and g_k/RT per state; production rates are summed
-// by L2 reductions into the output rows (the bath gas in a register).
-template <int MODE, bool SPECIAL>
-__global__ void __launch_bounds__(128) k_source_terms(DevMech m, int64_t n, const double* __restrict__ param,
-                                                      const double* __restrict__ phi, int64_t ld,
-                                                      double* __restrict__ out, int* status, double* ws,
-                                                      int64_t ws_stride) {
+// A block of 16 warps per 32-state tile (source_tile.cuh), two blocks per SM,
+// tiles handed out block-cyclically.  Y: y = (wdot, dT/dt) instead of dPhi/dt.
+template <int MODE, bool SPECIAL, bool Y>
+__global__ void __launch_bounds__(kSrcWarps * 32, 2)
+    k_source_terms(const __grid_constant__ DevMech m, int64_t n, const double* __restrict__ param,
+                   const double* __restrict__ phi, int64_t ld, double* __restrict__ out, int* status, double* ws,
+                   double* arrays) {
   PJ_DYN_SMEM;
   load_exp_table(m.exp_tab);
-  const int ns = m.ns;
-  const int64_t gtid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  StateArrays A;
-  A.ns = ns;
-  if (ws) {
-    A.base = ws + gtid;
-    A.stride = ws_stride;
-  } else {
-    A.base = smem + threadIdx.x;
-    A.stride = blockDim.x;
+  const int lane = threadIdx.x & 31;
+  if (arrays) arrays += (size_t)blockIdx.x * source_arrays_ws_doubles(m.ns, false);
+  if (!Y) ws += (size_t)blockIdx.x * m.ns * kTile + lane;
+  for (int64_t tile = blockIdx.x; tile * kTile < n; tile += gridDim.x) {
+    const int64_t s = tile * kTile + lane;
+    const BatchIn in{param, phi, ld, s, s < n};
+    if constexpr (Y) source_tile<MODE, SPECIAL>(m, smem, arrays, in, YOut{out, ld, s, m.ns, status});
+    else source_tile<MODE, SPECIAL>(m, smem, arrays, in, SourceOut{out, ws, ld, s, m.ns, status});
   }
-  for (int64_t s = gtid; s < n; s += (int64_t)gridDim.x * blockDim.x)
-    source_state<MODE, SPECIAL>(m, A, param, phi, ld, s, out, status);
 }
 
 // pj_exp next to the library exp, for verification (pj_diag_exp).
@@ -105,17 +102,14 @@ int sm_count() {
 
 // Per-state arrays: in shared memory when 128 threads fit, else in a global
 // workspace with a grid-stride grid (trimmed to the resident blocks at
-// launch, see resident_grid).  The source terms always take the L1-cached
-// workspace, at up to eight blocks of 128 per SM: at 53 species shared
-// memory allowed two, and the workspace layout measured 1.18x faster.
+// launch, see resident_grid).
 LaunchPlan plan_for(int arrays, int ns, int64_t n) {
   LaunchPlan p{};
   const size_t per_thread = (size_t)arrays * ns * sizeof(double);
   // threads per SM that fit the per-state arrays in shared memory, as whole
   // warps; blocks of up to 128 threads so several can share an SM
   const int fit = (int)((kSmemCap / per_thread) / 32 * 32);
-  const bool source = arrays == source_arrays();
-  if (fit >= 128 && !source) {
+  if (fit >= 128) {
     p.global_ws = false;
     p.tpb = fit >= 256 ? 128 : (fit % 64 == 0 ? 64 : 32);
     p.smem = per_thread * p.tpb;
@@ -127,7 +121,7 @@ LaunchPlan plan_for(int arrays, int ns, int64_t n) {
     p.global_ws = true;
     p.tpb = 128;
     p.smem = 0;
-    const int64_t cap = (int64_t)sm_count() * (source ? 8 : 4);
+    const int64_t cap = (int64_t)sm_count() * 4;
     const int64_t blocks = (n + p.tpb - 1) / p.tpb;
     p.grid = (int)(blocks < cap ? (blocks < 1 ? 1 : blocks) : cap);
     p.ws_stride = (int64_t)p.grid * p.tpb;
@@ -139,20 +133,48 @@ LaunchPlan plan_for(int arrays, int ns, int64_t n) {
 int source_arrays() { return 2; }
 int jacobian_arrays() { return 3; }
 
+// The tile kernel's shape: arrays in shared memory while two blocks fit an
+// SM, then while one does, else in the workspace (two blocks).
+SourcePlan source_plan(int ns, int64_t n) {
+  SourcePlan p{};
+  const size_t in_smem = source_smem_bytes(ns, true);
+  p.arrays_smem = in_smem <= kSmemCap;
+  p.smem = source_smem_bytes(ns, p.arrays_smem);
+  p.ctas = p.smem + kBlockOverhead <= kSmemPerSm / 2 ? 2 : 1;
+  const int64_t tiles = (n + kTile - 1) / kTile;
+  p.grid = (int)std::max<int64_t>(1, std::min<int64_t>(tiles, (int64_t)sm_count() * p.ctas));
+  p.acc_bytes = (size_t)p.grid * ns * kTile * sizeof(double);
+  p.arrays_bytes = (size_t)p.grid * source_arrays_ws_doubles(ns, p.arrays_smem) * sizeof(double);
+  return p;
+}
+
+template <bool Y>
+static int launch_source_t(const DevMech& m, int mode, int64_t n, const double* param, const double* phi, int64_t ld,
+                           double* out, int* status, void* work, size_t work_bytes, cudaStream_t st) {
+  const SourcePlan p = source_plan(m.ns, n);
+  const size_t need = (Y ? 0 : p.acc_bytes) + p.arrays_bytes;
+  if (need && (!work || work_bytes < need))
+    return fail(PJ_ERR_NOMEM, Y ? "workspace too small for pj_eval_y (see pj_workspace_size)"
+                                : "workspace too small for the source-term kernel (see pj_workspace_size)");
+  double* arrays = p.arrays_bytes ? static_cast<double*>(work) : nullptr;
+  double* acc = Y ? nullptr : static_cast<double*>(work) + p.arrays_bytes / sizeof(double);
+  const bool special = m.nr_plain < m.nr;
+  auto kern = mode == PJ_CONP ? (special ? k_source_terms<PJ_CONP, true, Y> : k_source_terms<PJ_CONP, false, Y>)
+                              : (special ? k_source_terms<PJ_CONV, true, Y> : k_source_terms<PJ_CONV, false, Y>);
+  int rc;
+  if ((rc = set_smem(kern, p.smem))) return rc;
+  kern<<<p.grid, kSrcWarps * 32, p.smem, st>>>(m, n, param, phi, ld, out, status, acc, arrays);
+  return check_cuda(cudaGetLastError(), "k_source_terms launch");
+}
+
 int launch_source(const DevMech& m, int mode, int64_t n, const double* param, const double* phi, int64_t ld,
                   double* out, int* status, void* work, size_t work_bytes, cudaStream_t st) {
-  LaunchPlan p = plan_for(source_arrays(), m.ns, n);
-  if (p.global_ws && (!work || work_bytes < p.ws_bytes))
-    return fail(PJ_ERR_NOMEM, "workspace too small for the source-term kernel (see pj_workspace_size)");
-  double* ws = p.global_ws ? static_cast<double*>(work) : nullptr;
-  int rc;
-  const bool special = m.nr_plain < m.nr;
-  auto kern = mode == PJ_CONP ? (special ? k_source_terms<PJ_CONP, true> : k_source_terms<PJ_CONP, false>)
-                              : (special ? k_source_terms<PJ_CONV, true> : k_source_terms<PJ_CONV, false>);
-  if ((rc = set_smem(kern, p.smem))) return rc;
-  const LaunchPlan q = resident_grid(kern, p);
-  kern<<<q.grid, q.tpb, q.smem, st>>>(m, n, param, phi, ld, out, status, ws, q.ws_stride);
-  return check_cuda(cudaGetLastError(), "k_source_terms launch");
+  return launch_source_t<false>(m, mode, n, param, phi, ld, out, status, work, work_bytes, st);
+}
+
+int launch_eval_y(const DevMech& m, int mode, int64_t n, const double* param, const double* phi, int64_t ld,
+                  double* y, int* status, void* work, size_t work_bytes, cudaStream_t st) {
+  return launch_source_t<true>(m, mode, n, param, phi, ld, y, status, work, work_bytes, st);
 }
 
 // TMEM mode for the Jacobian.  Chosen when it keeps at least as many
@@ -305,7 +327,8 @@ size_t workspace_bytes(int arrays, int ns, int64_t n) {
     const size_t co = global ? coop_arrays_bytes(ns) * (size_t)tiles : 0;
     return std::max(pc, co);
   }
-  return plan_for(arrays, ns, n).ws_bytes;
+  const SourcePlan p = source_plan(ns, n);
+  return p.acc_bytes + p.arrays_bytes;
 }
 
 // Shared by the FP64 Jacobian and the FP32 Newton matrix: pick the layout,

@@ -56,20 +56,16 @@ __device__ __forceinline__ double fixed_gibbs(const DevMech& m, double g, bool& 
 }
 
 // 2^(y 2^-51) as a double
-__device__ __noinline__ static double exp2_fixed_library(int64_t y) {
-  return exp2((double)y * 0x1p-51);
-}
 __device__ __forceinline__ double exp2_51(int64_t y) {
-  // |y| < 1016: a normal result
-  if ((uint32_t)(y >> 32) + (1016u << 19) >= (2032u << 19)) return exp2_fixed_library(y);
-  return __longlong_as_double((long long)exp2_fixed((int)(y >> 51), (uint64_t)y << 13, pj_exp_tab));
+  return __longlong_as_double(
+      (long long)pack_double_any((int)(y >> 51), exp2_significand((uint64_t)y << 13, pj_exp_tab)));
 }
 
 // log2 of a positive normal double, 2^51; ok = false for anything else
-__device__ __forceinline__ int64_t log2_51(const DevMech& m, double x, bool& ok) {
+__device__ __forceinline__ int64_t log2_51(const LogEntry* __restrict__ log_tab, double x, bool& ok) {
   ok = ok && (uint32_t)__double2hiint(x) - 0x00100000u < 0x7fe00000u;
   int e;
-  const uint64_t l = log2_fixed((uint64_t)__double_as_longlong(x), e, m.log_tab);
+  const uint64_t l = log2_fixed((uint64_t)__double_as_longlong(x), e, log_tab);
   return ((int64_t)e << 51) + (int64_t)(l >> 11);
 }
 
@@ -120,7 +116,7 @@ __device__ __forceinline__ bool load_state(const DevMech& m, const double* __res
 // dg/dx = -2 N xc D / S^2.  A log, an exp and a divide each were 9 to 30 FP64
 // operations; the fixed-point ones are none.
 template <bool DERIV>
-__device__ __forceinline__ double falloff_F(const DevMech& m, const Rxn* __restrict__ r, int kind, double T,
+__device__ __forceinline__ double falloff_F(const LogEntry* __restrict__ log_tab, const Rxn* __restrict__ r, int kind, double T,
                                             double invT, double lnT, int64_t l2Pr, bool& ok, double& FxPr,
                                             double& FT) {
   FxPr = 0.0;
@@ -132,7 +128,7 @@ __device__ __forceinline__ double falloff_F(const DevMech& m, const Rxn* __restr
     const double e3 = pj_exp(-T * iT3), e1 = pj_exp(-T * iT1);
     const double e2 = has2 != 0.0 ? pj_exp(-T2 * invT) : 0.0;
     const double Fcent = (1.0 - a) * e3 + a * e1 + e2;
-    const double l2F = fixed51_to_double(log2_51(m, Fcent, ok));
+    const double l2F = fixed51_to_double(log2_51(log_tab, Fcent, ok));
     if (!ok) return 1.0;
     const double L = l2F * LOG10_2;
     const double xc = fixed51_to_double(l2Pr) * LOG10_2 + (-0.4 - 0.67 * L);
@@ -158,7 +154,7 @@ __device__ __forceinline__ double falloff_F(const DevMech& m, const Rxn* __restr
     const double X = 1.0 / (1.0 + x * x);
     const double eb = pj_exp(-b * invT), ec = pj_exp(-T * ic);
     const double Z = a * eb + ec;
-    const double lnZ = fixed51_to_double(log2_51(m, Z, ok)) * 0.69314718055994530942;
+    const double lnZ = fixed51_to_double(log2_51(log_tab, Z, ok)) * 0.69314718055994530942;
     if (!ok) return 1.0;
     const double F = d * pj_exp(X * lnZ + e * lnT);
     if (DERIV) {
@@ -423,7 +419,7 @@ __device__ __noinline__ static double gibbs_sum(const double* __restrict__ nasa,
     const bool react = a < PJ_MAX_SP;
     if (react ? a >= __ldg(&r->nreac) : a - PJ_MAX_SP >= __ldg(&r->nprod)) continue;
     const double* b = nasa + (size_t)__ldg(&r->sp[a]) * NASA_STRIDE;
-    if (!(T < __ldg(b + 14))) b += 16;
+    if (!(T < __ldg(b + 14))) b += NASA_RANGE;
     double cp, h, sr;
     nasa_eval(b, T, invT, lnT, cp, h, sr);
     dg = fma(react ? -__ldg(&r->nud[a]) : __ldg(&r->nud[a]), h - sr, dg);
@@ -467,7 +463,7 @@ __device__ __forceinline__ RateK rate_constants(const DevMech& m, const SA& A, i
     rate_constants_library<GEN>(m, r, T, invT, lnT, lnP, k);
     return k;
   }
-  int64_t y = arrhenius_fixed(__ldg(&r->fA), __ldg(&r->fB), __ldg(&r->fT), fx.L, fx.IT);
+  int64_t y = arrhenius_fixed(__ldg(&r->head.fA), __ldg(&r->head.fB), __ldg(&r->head.fT), fx.L, fx.IT);
   k.rk = 0.0;
   k.l2rk = 0;
   if (kind >= PJ_LINDEMANN && kind <= PJ_SRI) {
@@ -489,7 +485,7 @@ __device__ __forceinline__ RateK rate_constants(const DevMech& m, const SA& A, i
       if (a < nre) dg -= __ldg(&r->nu[a]) * __double_as_longlong(A.at(aG, __ldg(&r->sp[a])));
       if (a < npr) dg += __ldg(&r->nu[PJ_MAX_SP + a]) * __double_as_longlong(A.at(aG, __ldg(&r->sp[PJ_MAX_SP + a])));
     }
-    dg -= __ldg(&r->dnu_i) * fx.LP;
+    dg -= __ldg(&r->head.dnu_i) * fx.LP;
   }
   if (GEN && kind >= PJ_PLOG) {
     double u0, u1;
@@ -514,8 +510,8 @@ __device__ __forceinline__ double falloff_Pr_F(const DevMech& m, const Rxn* __re
   FxPr = FT = 0.0;
   if (kind == PJ_LINDEMANN) return Pr;
   bool ok = fx.fast;
-  const int64_t l2Pr = k.l2rk + log2_51(m, M, ok);
-  if (ok) F = falloff_F<DERIV>(m, r, kind, T, invT, lnT, l2Pr, ok, FxPr, FT);
+  const int64_t l2Pr = k.l2rk + log2_51(m.log_tab, M, ok);
+  if (ok) F = falloff_F<DERIV>(m.log_tab, r, kind, T, invT, lnT, l2Pr, ok, FxPr, FT);
   if (!ok) F = falloff_F_library(r, kind, T, invT, lnT, Pr, FxPr, FT);
   return Pr;
 }

@@ -52,7 +52,7 @@ using StateArrays = StateArraysT<8>;
 __device__ __forceinline__ const double* nasa_block(const DevMech& m, int k, double T) {
   const double* b = m.nasa + (size_t)k * NASA_STRIDE;
   const double tmid = __ldg(b + 14);
-  return T < tmid ? b : b + 16;
+  return T < tmid ? b : b + NASA_RANGE;
 }
 
 // cp/R, h/RT, s/R (NASA 7-coefficient polynomials).
@@ -62,6 +62,20 @@ __device__ __forceinline__ void nasa_eval(const double* __restrict__ c, double T
   cp = fma(fma(fma(fma(a4, T, a3), T, a2), T, a1), T, a0);
   h = fma(fma(fma(fma(__ldg(c + 10), T, __ldg(c + 9)), T, __ldg(c + 8)), T, __ldg(c + 7)), T, a0) + __ldg(c + 5) * invT;
   s = fma(a0, lnT, fma(fma(fma(fma(__ldg(c + 13), T, __ldg(c + 12)), T, __ldg(c + 11)), T, a1), T, __ldg(c + 6)));
+}
+
+// cp/R and g/RT = h/RT - s/R as one polynomial
+__device__ __forceinline__ void nasa_cp_g(const double* __restrict__ c, double T, double invT, double lnT, double& cp,
+                                          double& g) {
+  const double a0 = __ldg(c + 0), a1 = __ldg(c + 1), a2 = __ldg(c + 2), a3 = __ldg(c + 3), a4 = __ldg(c + 4);
+  cp = fma(fma(fma(fma(a4, T, a3), T, a2), T, a1), T, a0);
+  const double p = fma(fma(fma(__ldg(c + 17), T, __ldg(c + 16)), T, __ldg(c + 15)), T, __ldg(c + 7));
+  g = fma(__ldg(c + 5), invT, fma(-p, T, fma(-a0, lnT, a0 - __ldg(c + 6))));
+}
+
+// h/RT
+__device__ __forceinline__ double nasa_h(const double* __restrict__ c, double T, double invT) {
+  return fma(__ldg(c + 5), invT, fma(fma(fma(fma(__ldg(c + 10), T, __ldg(c + 9)), T, __ldg(c + 8)), T, __ldg(c + 7)), T, __ldg(c)));
 }
 
 // cp/R and d(cp/R)/dT

@@ -25,9 +25,9 @@ __device__ __forceinline__ void source_state(const DevMech& m, const SA& A, cons
   for (int k = 0; k < ns - 1; k++) wrow[(int64_t)k * ld] = 0.0;
   double den = 0.0;
   for (int k = 0; k < ns; k++) {
-    double cp, h, sr;
-    nasa_eval(nasa_block(m, k, T), T, invT, lnT, cp, h, sr);
-    A.at(aG, k) = fixed_gibbs(m, h - sr, st.fx.fast);
+    double cp, g;
+    nasa_cp_g(nasa_block(m, k, T), T, invT, lnT, cp, g);
+    A.at(aG, k) = fixed_gibbs(m, g, st.fx.fast);
     den = fma(A.at(aC, k), MODE == PJ_CONP ? cp : cp - 1.0, den);
   }
   den *= RU;
@@ -70,8 +70,7 @@ __device__ __forceinline__ void source_state(const DevMech& m, const SA& A, cons
   // energy equation and ideal-gas state equation
   double num = 0.0, Om = 0.0;
   for (int k = 0; k < ns; k++) {
-    double cp, h, sr;
-    nasa_eval(nasa_block(m, k, T), T, invT, lnT, cp, h, sr);
+    const double h = nasa_h(nasa_block(m, k, T), T, invT);
     const double wk = k < bath ? __ldcg(wrow + (int64_t)k * ld) : w_bath;
     num = fma(MODE == PJ_CONP ? h : h - 1.0, wk, num);
     if (k < bath) {
@@ -591,10 +590,11 @@ __device__ __forceinline__ void jacobian_state(const DevMech& m, const SA& A,
   double den = 0.0, dden_T = 0.0, Cx_bath = 0.0;
   for (int k = 0; k < ns; k++) {
     const double* cb = nasa_block(m, k, T);
-    double cp, h, sr, cp2, dcp;
-    nasa_eval(cb, T, invT, lnT, cp, h, sr);
+    double cp, g, cp2, dcp;
+    nasa_cp_g(cb, T, invT, lnT, cp, g);
     nasa_cp(cb, T, cp2, dcp);
-    A.at(aG, k) = fixed_gibbs(m, h - sr, st.fx.fast);
+    const double h = nasa_h(cb, T, invT);
+    A.at(aG, k) = fixed_gibbs(m, g, st.fx.fast);
     if (TM) tmem_st_f64(tm_row + 2u * (uint32_t)k, h);
     else A.at(aH, k) = h;
     const double Ck = A.at(aC, k);

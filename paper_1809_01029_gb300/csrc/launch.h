@@ -51,6 +51,16 @@ struct CoopPlan {
                     // doubles); 0: in shared memory
 };
 
+// Source-term tile kernel: accumulators (source terms; y accumulates in its
+// output) and, unless they fit in shared memory, the tile's arrays, per block.
+struct SourcePlan {
+  bool arrays_smem;
+  int ctas;             // blocks per SM
+  int grid;
+  size_t smem;
+  size_t acc_bytes, arrays_bytes;
+};
+
 // Tiles of several batches handed out by a block counter (the batched
 // plans), instead of consecutive tiles of the one batch a launch is given.
 struct CoopBatch {
@@ -84,6 +94,7 @@ int sm_count();
 int source_arrays();
 int jacobian_arrays();
 LaunchPlan plan_for(int arrays, int ns, int64_t n);
+SourcePlan source_plan(int ns, int64_t n);
 TmPlan tm_plan(int ns);
 CoopPlan coop_plan(const DevMech& m, int fmt, int dt_bytes, int64_t n);
 int jacobian_layout(const DevMech& m, int fmt, bool f32, int64_t n);   // PJ_LAYOUT_*

@@ -211,6 +211,24 @@ static void build_pattern(pj_mech* m) {
 
 static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
+// Tables of the fixed-point exponential and logarithm (fixed_math.cuh), from
+// extended precision; made once per process.
+struct MathTables {
+  uint64_t exp2[256];  // 2^63 2^(j/256)
+  LogEntry log2[256];  // r = ceil(2^15 / (1 + j/256)), t = 2^62 log2(2^15 / r)
+  MathTables() {
+    for (int j = 0; j < 256; j++) {
+      exp2[j] = (uint64_t)std::floor(std::exp2((long double)j / 256.0L) * 0x1p63L + 0.5L);
+      log2[j].r = (uint64_t)((32768 * 256 + 255 + j) / (256 + j));
+      log2[j].t = (uint64_t)std::floor(std::log2(32768.0L / (long double)log2[j].r) * 0x1p62L + 0.5L);
+    }
+  }
+};
+static const MathTables& math_tables() {
+  static const MathTables t;
+  return t;
+}
+
 int mech_build(pj_mech* m) {
   int rc = validate(m);
   if (rc) return rc;
@@ -308,11 +326,12 @@ int mech_build(pj_mech* m) {
   for (int k = 0; k < ns; k++) {
     for (int r = 0; r < 2; r++) {
       const double* a = r == 0 ? &m->nasa_low[k * 7] : &m->nasa_high[k * 7];
-      double* b = &nasa[(size_t)k * NASA_STRIDE + r * 16];
+      double* b = &nasa[(size_t)k * NASA_STRIDE + r * NASA_RANGE];
       for (int j = 0; j < 7; j++) b[j] = a[j];
       b[7] = a[1] / 2; b[8] = a[2] / 3; b[9] = a[3] / 4; b[10] = a[4] / 5;
       b[11] = a[2] / 2; b[12] = a[3] / 3; b[13] = a[4] / 4;
       b[14] = m->T_mid[k];
+      b[15] = a[2] / 6; b[16] = a[3] / 12; b[17] = a[4] / 20;
     }
     wfac[k] = 1.0 - m->W[k] / m->W[bath];
   }
@@ -412,7 +431,7 @@ int mech_build(pj_mech* m) {
       if (k < bath) dW += nu[k] * wfac[k];
     }
     r.dnu = dnu;
-    r.dnu_i = (int32_t)dnu;
+    r.head.dnu_i = (int32_t)dnu;
     r.dW = dW;
     // fixed-point Arrhenius sets; a set beyond their ranges (every sum of
     // exponent terms must stay within the 2^12 of the fixed point) leaves the
@@ -431,13 +450,38 @@ int mech_build(pj_mech* m) {
       fB = std::llrint((long double)beta * 0x1p56L);
       fT = -std::llrint(th * 0x1p45L);
     };
-    if (!pdep) fixed_set(m->A[i], m->beta[i], m->Ea[i], r.fA, r.fB, r.fT);
+    if (!pdep) fixed_set(m->A[i], m->beta[i], m->Ea[i], r.head.fA, r.head.fB, r.head.fT);
     if (is_falloff(r.kind)) fixed_set(m->A0[i], m->beta0[i], m->Ea0[i], r.fA0, r.fB0, r.fT0);
     if (r.rev) {
       int side_sum = 0;
       for (int a = 0; a < 2 * PJ_MAX_SP; a++)
         side_sum += a < PJ_MAX_SP ? (a < r.nreac ? r.nu[a] : 0) : (a - PJ_MAX_SP < r.nprod ? r.nu[a] : 0);
       nu_max = std::max(nu_max, side_sum);
+    }
+    // short-path head: the factors of each side, a coefficient of 2 as two
+    {
+      RxnHead& hd = r.head;
+      hd.kind = (uint8_t)r.kind;
+      hd.rev = (uint8_t)r.rev;
+      hd.lean = q < nr_plain ? 1 : 0;
+      for (int side = 0; side < 2; side++) {
+        int32_t* out = side ? hd.b : hd.f;
+        // in the order side_rate multiplies them: 2A + B as A B A, else last to first
+        const int32_t* sp = &r.sp[side * PJ_MAX_SP];
+        int cnt = 0;
+        if (r.shape[side] == SH_21) {
+          out[0] = out[2] = 32 * sp[0];
+          out[1] = 32 * sp[1];
+          cnt = 3;
+        } else {
+          for (int a = (side ? r.nprod : r.nreac) - 1; a >= 0; a--)
+            for (int u = 0; u < r.nu[side * PJ_MAX_SP + a]; u++, cnt++)
+              if (cnt < 3) out[cnt] = 32 * sp[a];
+        }
+        if (cnt < 1 || cnt > 3) hd.lean = 0;
+        for (int u = cnt; u >= 1 && u < 3; u++) out[u] = out[0];
+        (side ? hd.nb : hd.nf) = (uint8_t)std::min(cnt, 3);
+      }
     }
     std::vector<double> al = alpha_of(m, i);
     r.alpha_bath = has_third_body(r.kind) ? al[bath] : 1.0;
@@ -525,6 +569,24 @@ int mech_build(pj_mech* m) {
       for (int e = r.eff_lo; e < r.eff_hi; e++) slot(eff_sp[e]);
   }
 
+  // unit contributions to each species by chunk of reactions (net
+  // coefficients; the order within a species is the kernel order)
+  const int n_chunks = (nr + kGatherChunk - 1) / kGatherChunk;
+  std::vector<int32_t> gptr(1, 0);
+  std::vector<uint16_t> gather;
+  for (int c = 0; c < n_chunks; c++) {
+    const int q0 = c * kGatherChunk, q1 = std::min(nr, q0 + kGatherChunk);
+    std::vector<std::vector<int>> nus;
+    for (int q = q0; q < q1; q++) nus.push_back(net_nu(m, m->perm[q]));
+    for (int k = 0; k < ns; k++) {
+      for (int q = q0; q < q1; q++) {
+        const int v = nus[q - q0][k];
+        for (int u = 0; u < std::abs(v); u++) gather.push_back((uint16_t)((q - q0) | (v < 0 ? 0x8000 : 0)));
+      }
+      gptr.push_back((int32_t)gather.size());
+    }
+  }
+
   // one device allocation holding every constant array
   const size_t o_nasa = 0;
   const size_t o_wfac = align256(o_nasa + nasa.size() * sizeof(double));
@@ -541,17 +603,10 @@ int mech_build(pj_mech* m) {
   const size_t o_tcsr = align256(o_tab + tab.size() * sizeof(double));
   const size_t o_tcsc = align256(o_tcsr + tgt_csr.size() * sizeof(int32_t));
   const size_t o_dbg = align256(o_tcsc + tgt_csc.size() * sizeof(int32_t));
-  const size_t total = align256(o_dbg + sizeof(uint32_t));
-  // 2^63 2^(j/256) from extended precision
-  uint64_t etab[256];
-  for (int j = 0; j < 256; j++) etab[j] = (uint64_t)std::floor(std::exp2((long double)j / 256.0L) * 0x1p63L + 0.5L);
-
-  // r = ceil(2^15 / (1 + j/256)), t = log2(2^15 / r)
-  LogEntry ltab[256];
-  for (int j = 0; j < 256; j++) {
-    ltab[j].r = (uint64_t)((32768 * 256 + 255 + j) / (256 + j));
-    ltab[j].t = (uint64_t)std::floor(std::log2(32768.0L / (long double)ltab[j].r) * 0x1p62L + 0.5L);
-  }
+  const size_t o_gptr = align256(o_dbg + sizeof(uint32_t));
+  const size_t o_gath = align256(o_gptr + gptr.size() * sizeof(int32_t));
+  const size_t total = align256(o_gath + gather.size() * sizeof(uint16_t));
+  const MathTables& tables = math_tables();
   // |g_k/RT| up to which sum nu g stays within half the fixed point's range
   const double g_lim = std::min(1300.0, 2000.0 * 0.6931471805599453 / nu_max);
   uint64_t g_bits;
@@ -568,9 +623,11 @@ int mech_build(pj_mech* m) {
   put(o_pcsr, m->pos_csr.data(), m->pos_csr.size() * sizeof(int32_t));
   put(o_pcsc, m->pos_csc.data(), m->pos_csc.size() * sizeof(int32_t));
   put(o_perm, m->perm.data(), m->perm.size() * sizeof(int32_t));
-  put(o_etab, etab, sizeof etab);
-  put(o_ltab, ltab, sizeof ltab);
+  put(o_etab, tables.exp2, sizeof tables.exp2);
+  put(o_ltab, tables.log2, sizeof tables.log2);
   put(o_tab, tab.data(), tab.size() * sizeof(double));
+  put(o_gptr, gptr.data(), gptr.size() * sizeof(int32_t));
+  put(o_gath, gather.data(), gather.size() * sizeof(uint16_t));
   put(o_tcsr, tgt_csr.data(), tgt_csr.size() * sizeof(int32_t));
   put(o_tcsc, tgt_csc.data(), tgt_csc.size() * sizeof(int32_t));
 
@@ -617,6 +674,8 @@ int mech_build(pj_mech* m) {
   dm.tab = reinterpret_cast<const double*>(b + o_tab);
   dm.tgt_csr = reinterpret_cast<const int32_t*>(b + o_tcsr);
   dm.tgt_csc = reinterpret_cast<const int32_t*>(b + o_tcsc);
+  dm.gather_ptr = reinterpret_cast<const int32_t*>(b + o_gptr);
+  dm.gather = reinterpret_cast<const uint16_t*>(b + o_gath);
   dm.has_pdep = has_pdep ? 1 : 0;
   dm.nr_plain = nr_plain;
   dm.n_eff = (int32_t)eff_sp.size();

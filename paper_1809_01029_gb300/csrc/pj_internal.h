@@ -17,16 +17,21 @@ constexpr double R_CAL = 1.98720425864083;   // cal / (mol K)
 constexpr double P_STD = 101325.0;           // Pa
 constexpr double LN10 = 2.302585092994045684;
 
-// per-species NASA-7 block: two ranges of 16 doubles
+// per-species NASA-7 block: two ranges of 18 doubles
 //   [0..6]  a0..a6
 //   [7..10] a1/2, a2/3, a3/4, a4/5   (enthalpy polynomial)
 //   [11..13] a2/2, a3/3, a4/4        (entropy polynomial)
-//   [14]    T_mid (same in both ranges), [15] unused
-constexpr int NASA_STRIDE = 32;
+//   [14]    T_mid (same in both ranges)
+//   [15..17] a2/6, a3/12, a4/20      (g/RT polynomial, with a1/2)
+constexpr int NASA_RANGE = 18;
+constexpr int NASA_STRIDE = 2 * NASA_RANGE;
 
 // Stoichiometric pattern of one reaction side, chosen on the host so that the
 // kernels form C-products and their derivatives with exactly the multiplies
 // they need (species ordered to match the pattern).
+// Reactions per gather chunk of the source-term tile kernel.
+constexpr int kGatherChunk = 64;
+
 enum : int32_t {
   SH_1 = 0,    // A
   SH_2 = 1,    // 2A
@@ -36,9 +41,24 @@ enum : int32_t {
   SH_GEN = 5   // anything else (generic loop)
 };
 
+// The part of a reaction's record that the tile kernels' short path reads
+// (tile_rate): four 16-byte loads.  Reactions whose sides have more than
+// three factors (counting a coefficient of 2 as two), and the special types,
+// have lean = 0 and take the general path.
+struct alignas(16) RxnHead {
+  int64_t fA, fB, fT;             // the Arrhenius set in fixed point (arrhenius_fixed): log2(A) 2^51,
+                                  // beta 2^56, -theta log2(e) 2^45
+  int32_t dnu_i;                  // dnu as an integer
+  uint8_t lean, kind, rev, nf;    // nf, nb: factors of the forward and the reverse product (1 to 3)
+  uint8_t nb, pad0, pad1, pad2;
+  int32_t f[3], b[3];             // 32 x species index of each factor (unused ones repeat the first)
+  int32_t pad3;
+};
+
 // One reaction, packed for warp-uniform loads (every thread of a warp reads
 // the same record).  Reactions are stored in kernel order (see perm).
-struct alignas(8) Rxn {
+struct alignas(16) Rxn {
+  RxnHead head;
   double lnA, beta, theta;        // k = exp(lnA + beta lnT - theta/T), theta = Ea/R_cal [K]
   double lnA0, beta0, theta0;     // low-pressure limit (falloff)
   double dnu;                     // sum_k nu_k (equilibrium-constant pressure factor)
@@ -60,12 +80,9 @@ struct alignas(8) Rxn {
   int16_t tab_n, tab_m;           // P-log entries / Chebyshev N_T, N_P
   int32_t tgt_lo;                 // first of this reaction's Jacobian targets in tgt_csr / tgt_csc
   int32_t bath_in;                // the bath gas is one of its reactants or products
-  int32_t dnu_i, pad_;            // dnu as an integer
-  // the Arrhenius sets in fixed point (fixed_math.cuh: arrhenius_fixed):
-  // log2(A) 2^51, beta 2^56, -theta log2(e) 2^45
-  int64_t fA, fB, fT;             // (lnA, beta, theta)
-  int64_t fA0, fB0, fT0;          // (lnA0, beta0, theta0)
+  int64_t fA0, fB0, fT0;          // the low-pressure set in fixed point, as head.fA, fB, fT
 };
+static_assert(sizeof(RxnHead) == 64, "the head is four 16-byte loads");
 
 // One unit of a reaction's net stoichiometric coefficient for species k: a
 // species with |nu| = 2 has two such rows.
@@ -102,6 +119,12 @@ struct DevMech {
   int32_t has_pdep;               // some reaction depends on P (P-log, Chebyshev)
   int32_t nr_plain;               // plain reactions (kernel order): none chemically activated,
                                   // with explicit reverse parameters, P-log or Chebyshev
+  // production rates by species: the unit contributions of the reactions of
+  // chunk c (kGatherChunk reactions in kernel order) to species k are
+  // gather[gather_ptr[c * ns + k]] .. gather[gather_ptr[c * ns + k + 1]], each
+  // the reaction's index within the chunk, bit 15 set for a loss
+  const int32_t* gather_ptr;      // [chunks * ns + 1]
+  const uint16_t* gather;
   int32_t n_eff, n_rows, n_tgt;   // lengths of eff_sp / rows / each target list array
   uint32_t* dbg;                  // error word of the bounds-checked build (PJ_DEBUG_BOUNDS)
 };
