@@ -22,12 +22,18 @@ LIB_DBG = os.path.join(LIBDIR, "libpyjac_gb_dbg.so")
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 SOURCES = ["mech.cpp", "api.cpp", "kinetics.cu", "noalloc.cu", "forms.cu", "batch.cu", "fd.cu", "lu.cu", "lu_symbolic.cpp", "hostio.cpp"]
-# jacobian_inst.cu is compiled once per (layout, precision): object name,
-# then its defines (see the file's header)
+# jacobian_inst.cu is compiled once per (layout, precision), the cooperative
+# layout once per format too: object name, then its defines (see the file's
+# header)
 JAC_INSTANCES = [
     (f"jac_{lay}_{prec}", {"PJ_INST_TM": tm, "PJ_INST_F32": int(prec == "f32"),
                            "PJ_INST_NAME": f"launch_jac_{lay}_{prec}"})
-    for lay, tm in (("plain", -1), ("tm0", 0), ("tm1", 1), ("tm2", 2), ("coop", 3))
+    for lay, tm in (("plain", -1), ("tm0", 0), ("tm1", 1), ("tm2", 2))
+    for prec in ("f64", "f32")
+] + [
+    (f"jac_coop_{prec}_{fmt}", {"PJ_INST_TM": 3, "PJ_INST_F32": int(prec == "f32"), "PJ_INST_FMT": i,
+                                "PJ_INST_NAME": f"launch_jac_coop_{prec}_{fmt}"})
+    for i, fmt in enumerate(("csr", "csc", "dense"))
     for prec in ("f64", "f32")
 ]
 
@@ -75,6 +81,7 @@ def build(force: bool = False, verbose: bool = False, debug_bounds: bool = False
     extra = {"PJ_DEBUG_BOUNDS": 1} if debug_bounds else {}
     jobs = [(s, s, dict(extra), build_dir) for s in SOURCES if os.path.exists(os.path.join(CSRC, s))]
     jobs += [("jacobian_inst.cu", name, {**defs, **extra}, build_dir) for name, defs in JAC_INSTANCES]
+    jobs.reverse()  # the cooperative units, the longest, first
     t0 = time.time()
     with ThreadPoolExecutor(max_workers=min(len(jobs), max(2, os.cpu_count() or 2))) as ex:
         objs = list(ex.map(_compile, jobs))

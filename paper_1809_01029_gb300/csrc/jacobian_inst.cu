@@ -4,6 +4,8 @@
 //                0, 1, 2: k_jacobian_tm with that many of C_k, g_k/RT in
 //                shared memory; 3: k_jacobian_coop (32-state tiles);
 //   PJ_INST_F32  0: FP64 Jacobian; 1: FP32 Newton matrix M = I - h gamma J;
+//   PJ_INST_FMT  (k_jacobian_coop) the one format of this unit: PJ_CSR, PJ_CSC
+//                or PJ_DENSE;
 //   PJ_INST_NAME the launcher this unit defines (declared in launch.h),
 // so that the instantiations compile in parallel.
 #include "jacobian_kernels.cuh"
@@ -48,6 +50,13 @@ static int inst_launch(const DevMech& m, const InstPlan& p, int64_t n, const Jac
 }
 #endif
 
+#ifdef PJ_INST_FMT
+int PJ_INST_NAME(const DevMech& m, const InstPlan& p, int mode, int64_t n, const JacArgs& a, double* ws,
+                 cudaStream_t st) {
+  if (mode == PJ_CONP) return inst_launch<PJ_CONP, PJ_INST_FMT>(m, p, n, a, ws, st);
+  return inst_launch<PJ_CONV, PJ_INST_FMT>(m, p, n, a, ws, st);
+}
+#else
 int PJ_INST_NAME(const DevMech& m, const InstPlan& p, int mode, int fmt, int64_t n, const JacArgs& a, double* ws,
                  cudaStream_t st) {
   if (mode == PJ_CONP) {
@@ -59,5 +68,6 @@ int PJ_INST_NAME(const DevMech& m, const InstPlan& p, int mode, int fmt, int64_t
   if (fmt == PJ_CSC) return inst_launch<PJ_CONV, PJ_CSC>(m, p, n, a, ws, st);
   return inst_launch<PJ_CONV, PJ_DENSE>(m, p, n, a, ws, st);
 }
+#endif
 
 }  // namespace pj

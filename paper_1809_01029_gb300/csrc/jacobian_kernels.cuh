@@ -9,6 +9,7 @@
 #include <cuda_runtime.h>
 
 #include "kinetics_state.cuh"
+#include "lean_jacobian.cuh"
 #ifndef PJ_NO_LAUNCHERS
 #include "launch.h"
 #endif
@@ -153,7 +154,7 @@ __device__ __forceinline__ void st_zero_evict_last(float* a, uint64_t pol) {
 // of several batches from a counter, else the tiles of (n, param, phi, ...).
 template <int MODE, int FMT, typename DT, bool NEWTON, bool SPECIAL, int MAXW, bool BATCHED = false>
 __global__ void __launch_bounds__(MAXW * 32, 1)
-    k_jacobian_coop(DevMech m, int64_t n0, const double* __restrict__ param0, const double* __restrict__ phi0,
+    k_jacobian_coop(const __grid_constant__ DevMech m, int64_t n0, const double* __restrict__ param0, const double* __restrict__ phi0,
                     int64_t ld0, DT* __restrict__ J0, double* __restrict__ dphi0, int* status,
                     const double* __restrict__ hstep, double gamma, double* __restrict__ aws, CoopSrc src) {
   PJ_DYN_SMEM;
@@ -280,7 +281,7 @@ __global__ void __launch_bounds__(MAXW * 32, 1)
         nasa_cp(cb, T, cp2, dcp);
         const double h = nasa_h(cb, T, invT);
         A.at(aG, k) = fixed_gibbs(m, g, fast);
-        A.at(aH, k) = h;
+        A.at(aH, k) = fixed_enthalpy(m, h, fast);
         const double cx = MODE == PJ_CONP ? cp : cp - 1.0;
         if (k < bath) {
           const double c = ok0 ? phi[(int64_t)(k + 2) * ld + s] / V : cdum;
@@ -329,7 +330,16 @@ __global__ void __launch_bounds__(MAXW * 32, 1)
     }
     __syncthreads();
 
-    // D: the warp's reactions (i = warp, warp + W, ...)
+    // a tile with a state outside the fixed point's range takes the general
+    // path, with h_k/RT in FP64
+    const bool fast_tile = __all_sync(0xffffffffu, F(fFast) != 0);  // the same in every warp
+    if (!fast_tile) {
+      const double T = S(cT), invT = S(cInvT);
+      for (int k = warp; k < ns; k += W) A.at(aH, k) = nasa_h(nasa_block(m, k, T), T, invT);
+      __syncthreads();
+    }
+
+    // D: the warp's reactions
     const bool w = F(fOk) != 0;
     const JacOut<DT> o{J, wrow, ld, s, w, NEWTON && w ? DT(-hstep[s] * gamma) : DT(0)};
     {
@@ -354,8 +364,9 @@ __global__ void __launch_bounds__(MAXW * 32, 1)
       // reactions are handed out one at a time (a shared counter), so that
       // warps finish the phase within about one reaction of each other
       for (int i = warp; i < m.nr;) {
-        if (!SPECIAL || i < m.nr_plain) jac_reaction<MODE, FMT, DT, false, false, NEWTON>(m, A, v, o, i, 0u);
-        else jac_reaction<MODE, FMT, DT, true, false, NEWTON>(m, A, v, o, i, 0u);
+        const RxnHead h = load_head(m.rxn + i);
+        if (fast_tile && h.lean) lean_jacobian<MODE, FMT, DT, NEWTON>(m, m.rxn + i, h, A.base, v, o);
+        else v = general_jacobian<MODE, FMT, DT, NEWTON, SPECIAL>(m, A, v, o, i, fast_tile);
         int nx = 0;
         if (lane == 0) nx = atomicAdd(next_rxn, 1);
         i = __shfl_sync(0xffffffffu, nx, 0);
@@ -376,7 +387,8 @@ __global__ void __launch_bounds__(MAXW * 32, 1)
       double num = 0.0, sumCxW = 0.0, Om = 0.0;
       for (int k = warp; k < ns; k += W) {
         const double wb = k == bath ? sum_parts(pWb) : 0.0;
-        A.at(aG, k) = jac_species<MODE, FMT, DT, NEWTON>(m, k, T, V, A.at(aH, k), wb, o, num, sumCxW, Om);
+        const double hk = fast_tile ? fixed51_to_double(__double_as_longlong(A.at(aH, k))) : A.at(aH, k);
+        A.at(aG, k) = jac_species<MODE, FMT, DT, NEWTON>(m, k, T, V, hk, wb, o, num, sumCxW, Om);
       }
       Pw(warp, pNum) = num;
       Pw(warp, pSum) = sumCxW;
@@ -408,7 +420,7 @@ __global__ void __launch_bounds__(MAXW * 32, 1)
     for (int t = warp - 1; t >= 0 && t < 6; t += W - 1) {  // warps 1 .. W-1 (W >= 2)
       const int from[6] = {pAT_T, pAT_S, pAS_T, pAS_S, pATB, pASB};
       const int to[6] = {cAT_T, cAT_S, cAS_T, cAS_S, cATB, cASB};
-      S(to[t]) = sum_parts(from[t]);
+      S(to[t]) = t < 4 ? sum_parts(from[t]) * S(cInvV) : sum_parts(from[t]);
     }
     __syncthreads();
 

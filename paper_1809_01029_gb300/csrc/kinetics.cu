@@ -331,6 +331,18 @@ size_t workspace_bytes(int arrays, int ns, int64_t n) {
   return p.acc_bytes + p.arrays_bytes;
 }
 
+int launch_jac_coop_f64(const DevMech& m, const CoopPlan& p, int mode, int fmt, int64_t n, const JacArgs& a,
+                        double* ws, cudaStream_t st) {
+  return (fmt == PJ_CSR ? launch_jac_coop_f64_csr : fmt == PJ_CSC ? launch_jac_coop_f64_csc
+                                                                  : launch_jac_coop_f64_dense)(m, p, mode, n, a, ws, st);
+}
+
+int launch_jac_coop_f32(const DevMech& m, const CoopPlan& p, int mode, int fmt, int64_t n, const JacArgs& a,
+                        double* ws, cudaStream_t st) {
+  return (fmt == PJ_CSR ? launch_jac_coop_f32_csr : fmt == PJ_CSC ? launch_jac_coop_f32_csc
+                                                                  : launch_jac_coop_f32_dense)(m, p, mode, n, a, ws, st);
+}
+
 // Shared by the FP64 Jacobian and the FP32 Newton matrix: pick the layout,
 // check the workspace, call the launcher of that layout and precision.
 static int launch_jac_any(const DevMech& m, int mode, int fmt, int64_t n, const JacArgs& a, bool f32, void* work,

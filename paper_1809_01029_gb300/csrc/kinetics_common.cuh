@@ -55,6 +55,13 @@ __device__ __forceinline__ double fixed_gibbs(const DevMech& m, double g, bool& 
   return __longlong_as_double(__double2ll_rn(g * (1.4426950408889634074 * 0x1p51)));
 }
 
+// h_k/RT, 2^51 (stored where the FP64 value would be); clears fast when it is
+// out of range
+__device__ __forceinline__ double fixed_enthalpy(const DevMech& m, double h, bool& fast) {
+  fast = fast && ((uint32_t)__double2hiint(h) & 0x7fffffffu) < m.fx_h_hi;
+  return __longlong_as_double(__double2ll_rn(h * 0x1p51));
+}
+
 // 2^(y 2^-51) as a double
 __device__ __forceinline__ double exp2_51(int64_t y) {
   return __longlong_as_double(
@@ -69,6 +76,7 @@ __device__ __forceinline__ int64_t log2_51(const LogEntry* __restrict__ log_tab,
   return ((int64_t)e << 51) + (int64_t)(l >> 11);
 }
 
+// y 2^-51
 __device__ __forceinline__ double fixed51_to_double(int64_t y) {
   return __longlong_as_double((long long)fixed_to_double(y, 51));
 }

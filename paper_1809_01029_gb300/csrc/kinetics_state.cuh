@@ -143,8 +143,9 @@ struct JacVars {
   double T, V, P, invT, lnT, lnP, Ctot;
   double invT2, invV, dCb_T, dCb_S;  // dCb_*: derivatives of the bath-gas concentration
   FixedState fx;
-  // energy-row (T) and state-row (S) weights for the T and S columns and for
-  // the part common to every species column; bath-gas production rate
+  // energy-row (T) and state-row (S) weights for the T and S columns (times
+  // V) and for the part common to every species column; bath-gas production
+  // rate
   DT AT_T, AT_S, AS_T, AS_S, ATB, ASB;
   double w_bath;
 };
@@ -170,7 +171,7 @@ __device__ __forceinline__ DT nscale(const JacOut<DT>& o, DT x) {
 
 template <int MODE, int FMT, typename DT, bool GEN, bool TM, bool NEWTON, class SA>
 __device__ __forceinline__ void jac_reaction(const DevMech& m, const SA& A, JacVars<DT>& v, const JacOut<DT>& o,
-                                             int i, uint32_t tm_row) {
+                                             int i, uint32_t tm_row, bool hfix = false) {
   enum { aC = 0, aG = 1, aH = 2 };
   const int ns = m.ns, bath = m.ns - 1;
   DT* __restrict__ J = o.J;
@@ -178,7 +179,7 @@ __device__ __forceinline__ void jac_reaction(const DevMech& m, const SA& A, JacV
   const bool w = o.w;
   auto h_at = [&](int k) -> double {
     if (TM) return tmem_ld_f64(tm_row + 2u * (uint32_t)k);
-    return A.at(aH, k);
+    return hfix ? fixed51_to_double(__double_as_longlong(A.at(aH, k))) : A.at(aH, k);
   };
   const double T = v.T, P = v.P, invT = v.invT, lnT = v.lnT, Ctot = v.Ctot, invT2 = v.invT2, invV = v.invV;
   const DT invT_t = DT(invT), invV_t = DT(invV), V_t = DT(v.V);
@@ -312,14 +313,15 @@ __device__ __forceinline__ void jac_reaction(const DevMech& m, const SA& A, JacV
   // energy-row and state-row weights of this reaction
   const DT dE = DT(RU * T * (MODE == PJ_CONP ? dh : dh - __ldg(&r->dnu)));
   const DT dW = DT(__ldg(&r->dW));
-  v.AT_T = v.AT_T + dE * dqdT;
-  v.AT_S = v.AT_S + dE * dqdS;
-  v.AS_T = v.AS_T + dW * dqdT;
-  v.AS_S = v.AS_S + dW * dqdS;
+  const DT Vq_T = V_t * dqdT, Vq_S = V_t * dqdS;
+  v.AT_T = v.AT_T + dE * Vq_T;
+  v.AT_S = v.AT_S + dE * Vq_S;
+  v.AS_T = v.AS_T + dW * Vq_T;
+  v.AS_S = v.AS_S + dW * Vq_S;
 
   int row_lo = __ldg(&r->row_lo), row_hi = __ldg(&r->row_hi);
   if (!PJ_DBG_OK(m.dbg, row_lo >= 0 && row_lo <= row_hi && row_hi <= m.n_rows, PJ_DBG_ROWS)) row_hi = row_lo = 0;
-  const DT VdqdT = nscale<NEWTON>(o, V_t * dqdT), VdqdS = nscale<NEWTON>(o, V_t * dqdS);
+  const DT VdqdT = nscale<NEWTON>(o, Vq_T), VdqdS = nscale<NEWTON>(o, Vq_S);
   // sparse targets in the order of the reaction's target list (the host
   // builds it in exactly the order of the contributions below); dense
   // positions are plain arithmetic
@@ -459,10 +461,10 @@ __device__ __forceinline__ JacRowVars<DT> jac_row_vars(double T, double V, doubl
     x.x0 = DT(-P * Tdot * invT2 + RU * Om);
     x.x1 = DT(Tdot * invT);
   }
-  x.AT_T = AT_T;
-  x.AT_S = AT_S;
-  x.AS_T = AS_T;
-  x.AS_S = AS_S;
+  x.AT_T = AT_T * x.invV;
+  x.AT_S = AT_S * x.invV;
+  x.AS_T = AS_T * x.invV;
+  x.AS_S = AS_S * x.invV;
   x.ATB = ATB;
   x.ASB = ASB;
   return x;

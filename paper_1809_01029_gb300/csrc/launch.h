@@ -167,6 +167,16 @@ int launch_jac_coop_f64(const DevMech& m, const CoopPlan& p, int mode, int fmt, 
                         double* ws, cudaStream_t st);
 int launch_jac_coop_f32(const DevMech& m, const CoopPlan& p, int mode, int fmt, int64_t n, const JacArgs& a,
                         double* ws, cudaStream_t st);
+// one format of the cooperative layout each
+#define PJ_DECLARE_COOP(name)                                                                                     \
+  int name(const DevMech& m, const CoopPlan& p, int mode, int64_t n, const JacArgs& a, double* ws, cudaStream_t st);
+PJ_DECLARE_COOP(launch_jac_coop_f64_csr)
+PJ_DECLARE_COOP(launch_jac_coop_f64_csc)
+PJ_DECLARE_COOP(launch_jac_coop_f64_dense)
+PJ_DECLARE_COOP(launch_jac_coop_f32_csr)
+PJ_DECLARE_COOP(launch_jac_coop_f32_csc)
+PJ_DECLARE_COOP(launch_jac_coop_f32_dense)
+#undef PJ_DECLARE_COOP
 
 // Raise a kernel's dynamic shared-memory limit when it asks for more than
 // the default 48 KB.

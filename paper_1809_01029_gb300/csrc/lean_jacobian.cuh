@@ -1,0 +1,307 @@
+// The short path of the cooperative Jacobian kernel: one plain reaction with
+// at most three factors a side, at a tile of states within the fixed point's
+// range (all others: jac_reaction).
+//
+// What bounds it: the FP64 pipe at 16 cycles per warp instruction and SM, and
+// the L2 reductions at about the same (600 G reductions/s, 15.6 cycles per
+// warp instruction and SM), some 40 of which a reversible A + B = C + D
+// makes.  So everything that can leave the FP64 pipe has: the exponents, the
+// exponentials and the reaction enthalpy are integer fixed point, the
+// concentration derivative of R' = k prod C with respect to the volume is
+// -(number of factors) R', and an elementary reaction multiplies by no
+// pressure factor: 26 FP64 instructions (23 under constant volume, whose S
+// column such a reaction leaves alone) where the general path has 110.
+#pragma once
+
+#include "kinetics_state.cuh"
+#include "source_tile.cuh"
+
+namespace pj {
+
+// Any reaction at any state, out of line (by value: the caller's accumulators
+// stay in registers).
+template <int MODE, int FMT, typename DT, bool NEWTON, bool SPECIAL>
+__device__ __noinline__ static JacVars<DT> general_jacobian(const DevMech& m, const StateArrays A, JacVars<DT> v,
+                                                            const JacOut<DT> o, int i, bool hfix) {
+  if (!SPECIAL || i < m.nr_plain) jac_reaction<MODE, FMT, DT, false, false, NEWTON>(m, A, v, o, i, 0u, hfix);
+  else jac_reaction<MODE, FMT, DT, true, false, NEWTON>(m, A, v, o, i, 0u, hfix);
+  return v;
+}
+
+// Falloff blending c = Pr / (1 + Pr) F and its derivatives: cM = dc/dM at
+// fixed T, cT = dc/dT with M moving by dMdT.  Out of line, as falloff_factor.
+struct FalloffC {
+  double c, cM, cT;
+};
+__device__ __noinline__ static FalloffC falloff_derivatives(const Rxn* __restrict__ r,
+                                                            const LogEntry* __restrict__ log_tab, int kind, double T,
+                                                            double invT, double lnT, double rk, int64_t l2rk, double M,
+                                                            double dMdT) {
+  double F = 1.0, FxPr = 0.0, FT = 0.0;
+  const double Pr = rk * M;
+  if (kind != PJ_LINDEMANN) {
+    bool ok = true;
+    const int64_t l2Pr = l2rk + log2_51(log_tab, M, ok);
+    if (ok) F = falloff_F<true>(log_tab, r, kind, T, invT, lnT, l2Pr, ok, FxPr, FT);
+    if (!ok) F = falloff_F_library(r, kind, T, invT, lnT, Pr, FxPr, FT);
+  }
+  const double invT2 = invT * invT;
+  const double dlnrk = fma(__ldg(&r->theta0) - __ldg(&r->theta), invT2, (__ldg(&r->beta0) - __ldg(&r->beta)) * invT);
+  const double i1p = 1.0 / (1.0 + Pr);
+  const double fr = Pr * i1p;
+  const double cPr = F * i1p * i1p + FxPr * i1p;
+  return FalloffC{fr * F, cPr * rk, fr * FT + cPr * (Pr * dlnrk + rk * dMdT)};
+}
+
+// x in the derivative type.  To FP32 in integer instructions (the hardware
+// conversion takes an FP64-pipe slot): rounded to nearest, flushed to zero
+// below 2^-126, infinite beyond FP32's range.
+template <typename DT>
+__device__ __forceinline__ DT to_derivative(double x) {
+  if constexpr (sizeof(DT) == 8) {
+    return x;
+  } else {
+    const uint64_t b = (uint64_t)__double_as_longlong(x) + 0x10000000ull;
+    const uint32_t hi = (uint32_t)(b >> 32);
+    const int e = (int)((hi >> 20) & 0x7ffu) - 896;
+    uint32_t f = ((uint32_t)e << 23) | ((uint32_t)(b >> 29) & 0x7fffffu);
+    f = e < 1 ? 0u : f;
+    f = e > 254 ? 0x7f800000u : f;
+    return __uint_as_float(f | (hi & 0x80000000u));
+  }
+}
+
+// One side's product R = k prod C and dR/dC_a in species order (f: factors
+// as packed in the head).
+struct LeanSide {
+  double R, d0, d1, d2;
+};
+__device__ __forceinline__ LeanSide lean_side(const int32_t (&f)[3], int shape, const double* __restrict__ C, double k) {
+  LeanSide s;
+  const double c0 = C[f[0]];
+  s.d1 = s.d2 = 0.0;
+  if (shape == SH_1) {
+    s.R = k * c0;
+    s.d0 = k;
+    return s;
+  }
+  const double t = k * c0;
+  const double c1 = C[f[1]];
+  if (shape == SH_11) {
+    s.R = t * c1;
+    s.d0 = t;
+    s.d1 = k * c1;
+    return s;
+  }
+  if (shape == SH_2) {
+    s.R = t * c1;
+    s.d0 = t + t;
+    return s;
+  }
+  const double c2 = C[f[2]];
+  const double t1 = t * c1;
+  s.R = t1 * c2;
+  if (shape == SH_21) {  // A B A
+    s.d0 = t1 + t1;
+    s.d1 = t * c2;
+  } else {               // C B A
+    s.d0 = t1;
+    s.d1 = t * c2;
+    s.d2 = (k * c2) * c1;
+  }
+  return s;
+}
+
+__device__ __forceinline__ int shape_species(int shape) { return shape <= SH_2 ? 1 : shape <= SH_21 ? 2 : 3; }
+
+// negated when neg is not 0 (warp-uniform)
+__device__ __forceinline__ double flip(double x, uint32_t neg) {
+  return __hiloint2double(__double2hiint(x) ^ (int)(neg << 31), __double2loint(x));
+}
+__device__ __forceinline__ float flip(float x, uint32_t neg) { return __uint_as_float(__float_as_uint(x) ^ (neg << 31)); }
+
+// base: this lane's column of the tile's arrays C, g, h ([3][ns][32]).
+template <int MODE, int FMT, typename DT, bool NEWTON>
+__device__ __forceinline__ void lean_jacobian(const DevMech& m, const Rxn* __restrict__ r, const RxnHead& h,
+                                              const double* __restrict__ base, JacVars<DT>& v, const JacOut<DT>& o) {
+  const int ns = m.ns, bath = ns - 1;
+  const double* __restrict__ C = base;
+  const double* __restrict__ G = base + ns * kTile;
+  const double* __restrict__ H = base + 2 * ns * kTile;
+  RxnJac a;
+  {
+    const int4* __restrict__ p = reinterpret_cast<const int4*>(&r->jac);
+    int4* q = reinterpret_cast<int4*>(&a);
+#pragma unroll
+    for (int i = 0; i < 3; i++) q[i] = __ldg(p + i);
+  }
+  const bool rev = h.rev != 0;
+  const int64_t y = arrhenius_fixed(h.fA, h.fB, h.fT, v.fx.L, v.fx.IT);
+  const LeanSide sf = lean_side(h.f, a.shape[0], C, exp2_51(y));
+  LeanSide sb{0.0, 0.0, 0.0, 0.0};
+  if (rev) sb = lean_side(h.b, a.shape[1], C, exp2_51(y + lean_gibbs(h, G, v.fx.LP)));
+
+  // reaction enthalpy (internal energy) over RT, 2^51
+  int64_t dh;
+  {
+    auto hf = [&](int off) { return __double_as_longlong(H[off]); };
+    dh = hf(h.b[0]) - hf(h.f[0]);
+    if (h.nf > 1) dh -= hf(h.f[1]);
+    if (h.nb > 1) dh += hf(h.b[1]);
+    if (h.nf > 2) dh -= hf(h.f[2]);
+    if (h.nb > 2) dh += hf(h.b[2]);
+  }
+  const double de = fixed51_to_double(dh - ((int64_t)h.dnu_i << 51));  // sum nu h/RT - dnu
+  const double dhd = MODE == PJ_CONP && h.dnu_i != 0 ? de + (double)h.dnu_i : de;
+
+  // net rate and its T derivative: T d ln kf/dT = beta + theta/T, T d ln kr/dT
+  // = that - sum nu u/RT; times V.  V dR/dV at constant n: -(factors) R.
+  const double Ef = fma(a.theta, v.invT, a.beta);
+  const double Rn = sf.R - sb.R;
+  double VT = (sf.R * Ef - sb.R * (Ef - de)) * (v.V * v.invT);
+  double VS = 0.0;
+  if (MODE == PJ_CONP) {
+    if (rev && a.nfx != a.nbx) VS = (double)a.nbx * sb.R - (double)a.nfx * sf.R;
+    else VS = -(double)a.nfx * Rn;
+  }
+  double Gb = 0.0;  // dRn/dC of the bath gas itself
+  bool has_S = MODE == PJ_CONP;
+  if (a.bath) {
+    if (a.bath & 1) Gb += sf.d0;
+    if (a.bath & 2) Gb += sf.d1;
+    if (a.bath & 4) Gb += sf.d2;
+    if (a.bath & 8) Gb -= sb.d0;
+    if (a.bath & 16) Gb -= sb.d1;
+    if (a.bath & 32) Gb -= sb.d2;
+    VT = fma(Gb, v.V * v.dCb_T, VT);
+    VS = fma(Gb, v.V * v.dCb_S, VS);
+    has_S = true;
+  }
+
+  // pressure factor: scales the rate and every derivative
+  double c = 1.0, q = Rn;
+  double RcM = 0.0;  // Rn dc/dM
+  if (h.kind != PJ_ELEMENTARY) {
+    double M = v.Ctot;
+    for (int e = __ldg(&r->eff_lo), eh = __ldg(&r->eff_hi); e < eh; e++) {
+      if (!PJ_DBG_OK(m.dbg, e >= 0 && e < m.n_eff && __ldg(m.eff_sp + e) >= 0 && __ldg(m.eff_sp + e) < m.ns,
+                     PJ_DBG_EFF))
+        break;
+      M = fma(__ldg(m.eff_am1 + e), C[kTile * __ldg(m.eff_sp + e)], M);
+    }
+    const double ab = __ldg(&r->alpha_bath);
+    const double dMdT = ab * v.dCb_T;
+    const double dMdS = MODE == PJ_CONP ? (ab * v.Ctot - M) * v.invV : ab * (v.Ctot / v.P);
+    double cT = dMdT;
+    c = M;
+    RcM = Rn;
+    if (h.kind != PJ_THIRD_BODY) {
+      const int64_t l2rk = arrhenius_fixed(__ldg(&r->fA0), __ldg(&r->fB0), __ldg(&r->fT0), v.fx.L, v.fx.IT) - y;
+      const FalloffC fc =
+          falloff_derivatives(r, m.log_tab, h.kind, v.T, v.invT, v.lnT, exp2_51(l2rk), l2rk, M, dMdT);
+      c = fc.c;
+      cT = fc.cT;
+      RcM = Rn * fc.cM;
+    }
+    q = c * Rn;
+    VT = fma(c, VT, (Rn * cT) * v.V);
+    VS = fma(c, VS, (RcM * dMdS) * v.V);
+    has_S = true;
+  }
+
+  // energy- and state-row weights of this reaction
+  const DT dE = to_derivative<DT>((RU * v.T) * (MODE == PJ_CONP ? dhd : de));
+  const DT dW = DT(a.dW);
+  const DT VT_t = to_derivative<DT>(VT);
+  v.AT_T = v.AT_T + dE * VT_t;
+  v.AS_T = v.AS_T + dW * VT_t;
+  const DT jT = nscale<NEWTON>(o, VT_t);
+  DT jS = DT(0);
+  if (has_S) {
+    const DT VS_t = to_derivative<DT>(VS);
+    v.AT_S = v.AT_S + dE * VS_t;
+    v.AS_S = v.AS_S + dW * VS_t;
+    jS = nscale<NEWTON>(o, VS_t);
+  }
+
+  const int32_t* __restrict__ tg = (FMT == PJ_CSR ? m.tgt_csr : m.tgt_csc) + a.tgt_lo;
+  const RowNu* __restrict__ rows = m.rows + a.row_lo;
+  const int nrows = a.nrows;
+  DT* __restrict__ Js = o.J + o.s;
+  auto red = [&](int e, DT x) {
+    if (!PJ_DBG_OK(m.dbg, e >= 0 && e < (FMT == PJ_DENSE ? m.N * m.N : m.nnz), PJ_DBG_TARGET)) return;
+    if (o.w) red_add(Js + (uint64_t)(uint32_t)e * (uint64_t)o.ld, x);
+  };
+  auto entry = [&](int at, int row, int col) -> int { return FMT == PJ_DENSE ? row * m.N + col : __ldg(tg + at); };
+
+#pragma unroll 4
+  for (int p = 0; p < nrows; p++) {
+    const int k = __ldg(&rows[p].k);
+    const uint32_t neg = (a.neg >> p) & 1u;
+    red(entry(2 * p, k + 2, 0), flip(jT, neg));
+    if (has_S) red(entry(2 * p + 1, k + 2, 1), flip(jS, neg));
+    if (o.w) red_add(o.wrow + (int64_t)k * o.ld, flip(q, neg));
+  }
+  tg += 2 * nrows;
+
+  // species columns
+  auto slot = [&](int j, DT val) {
+    const DT vs = nscale<NEWTON>(o, val);
+#pragma unroll 4
+    for (int p = 0; p < nrows; p++)
+      red(entry(p, FMT == PJ_DENSE ? __ldg(&rows[p].k) + 2 : 0, j + 2), flip(vs, (a.neg >> p) & 1u));
+    red(entry(nrows, 0, j + 2), dE * vs);
+    red(entry(nrows + 1, 1, j + 2), dW * vs);
+    tg += nrows + 2;
+  };
+  const int nsf = shape_species(a.shape[0]), nsb = rev ? shape_species(a.shape[1]) : 0;
+  auto scaled = [&](double d) { return to_derivative<DT>(h.kind != PJ_ELEMENTARY ? c * d : d); };
+#pragma unroll
+  for (int s = 0; s < 3; s++) {
+    if (s < nsf && !(a.bath >> s & 1)) slot(FMT == PJ_DENSE ? __ldg(&r->sp[s]) : 0, scaled(s == 0 ? sf.d0 : s == 1 ? sf.d1 : sf.d2));
+    if (s < nsb && !(a.bath >> (3 + s) & 1))
+      slot(FMT == PJ_DENSE ? __ldg(&r->sp[PJ_MAX_SP + s]) : 0, dneg(scaled(s == 0 ? sb.d0 : s == 1 ? sb.d1 : sb.d2)));
+  }
+  double Bi = 0.0;  // minus the terms of the bath gas
+  if (h.kind != PJ_ELEMENTARY) {
+    for (int e = __ldg(&r->eff_lo), eh = __ldg(&r->eff_hi); e < eh; e++) {
+      if (!PJ_DBG_OK(m.dbg, e >= 0 && e < m.n_eff, PJ_DBG_EFF)) break;
+      const int j = __ldg(m.eff_sp + e);
+      const double val = RcM * __ldg(m.eff_am1 + e);
+      if (j == bath) Bi -= val;
+      else slot(j, to_derivative<DT>(val));
+    }
+  }
+  if (a.dense) {
+    Bi -= h.kind != PJ_ELEMENTARY ? c * Gb : Gb;
+    const DT B_t = to_derivative<DT>(Bi);
+    const DT Bs = nscale<NEWTON>(o, B_t);
+    for (int p = 0; p < nrows; p++) {
+      const int k = __ldg(&rows[p].k);
+      const DT val = flip(Bs, (a.neg >> p) & 1u);
+      if (FMT == PJ_CSR) {
+        // a dense row holds every species column, contiguous in CSR
+        const int64_t e2 = jpos<FMT>(m, k + 2, 2);
+        if (!PJ_DBG_OK(m.dbg, e2 >= 0 && e2 + ns - 1 <= m.nnz, PJ_DBG_POSMAP)) continue;
+        if (o.w)
+          for (int j = 0; j < ns - 1; j++) red_add(Js + (e2 + j) * o.ld, val);
+      } else {
+        if (o.w)
+          for (int j = 0; j < ns - 1; j++) jred(o.J, jpos<FMT>(m, k + 2, j + 2), o.ld, o.s, val);
+      }
+    }
+    v.ATB = v.ATB + dE * B_t;
+    v.ASB = v.ASB + dW * B_t;
+  }
+  if (a.bath) {  // the bath gas's own production rate: net coefficient times q
+    int nu = 0;
+#pragma unroll
+    for (int s = 0; s < 3; s++) {
+      if (s < h.nf && h.f[s] == kTile * bath) nu--;
+      if (s < h.nb && h.b[s] == kTile * bath) nu++;
+    }
+    v.w_bath = fma((double)nu, q, v.w_bath);
+  }
+}
+
+}  // namespace pj

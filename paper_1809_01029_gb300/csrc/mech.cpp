@@ -344,7 +344,7 @@ int mech_build(pj_mech* m) {
   std::vector<double> tab;  // P-log entries and Chebyshev blocks
   bool has_pdep = false;
   bool fx_ok = true;  // every rate constant fits the fixed-point path
-  int nu_max = 1;     // largest sum of the coefficients of both sides of a reversible reaction
+  int nu_max = 1;     // largest sum of the coefficients of both sides of a reaction
   for (int q = 0; q < nr; q++) {
     const int i = m->perm[q];
     Rxn& r = rx[q];
@@ -452,12 +452,10 @@ int mech_build(pj_mech* m) {
     };
     if (!pdep) fixed_set(m->A[i], m->beta[i], m->Ea[i], r.head.fA, r.head.fB, r.head.fT);
     if (is_falloff(r.kind)) fixed_set(m->A0[i], m->beta0[i], m->Ea0[i], r.fA0, r.fB0, r.fT0);
-    if (r.rev) {
-      int side_sum = 0;
-      for (int a = 0; a < 2 * PJ_MAX_SP; a++)
-        side_sum += a < PJ_MAX_SP ? (a < r.nreac ? r.nu[a] : 0) : (a - PJ_MAX_SP < r.nprod ? r.nu[a] : 0);
-      nu_max = std::max(nu_max, side_sum);
-    }
+    int nu_sum = 0;
+    for (int a = 0; a < 2 * PJ_MAX_SP; a++)
+      nu_sum += a < PJ_MAX_SP ? (a < r.nreac ? r.nu[a] : 0) : (a - PJ_MAX_SP < r.nprod ? r.nu[a] : 0);
+    nu_max = std::max(nu_max, nu_sum);
     // short-path head: the factors of each side, a coefficient of 2 as two
     {
       RxnHead& hd = r.head;
@@ -502,6 +500,26 @@ int mech_build(pj_mech* m) {
       for (int u = 0; u < std::abs(nu[k]); u++) rows.push_back(RowNu{k, nu[k] > 0 ? 1 : -1, nu[k] > 0 ? 1.0 : -1.0});
     r.row_hi = (int32_t)rows.size();
     r.dense = rate_dependence(m, i, dep) ? 1 : 0;
+    {
+      RxnJac& j = r.jac;
+      j.beta = r.beta;
+      j.theta = r.theta;
+      j.dW = r.dW;
+      j.row_lo = r.row_lo;
+      const int n_rows = r.row_hi - r.row_lo;
+      if (n_rows > 8) r.head.lean = 0;
+      j.nrows = (uint8_t)std::min(n_rows, 8);
+      for (int q2 = 0; q2 < j.nrows; q2++) j.neg |= (uint8_t)((rows[r.row_lo + q2].nu < 0) << q2);
+      j.dense = (uint8_t)r.dense;
+      for (int side = 0; side < 2; side++) {
+        j.shape[side] = (uint8_t)r.shape[side];
+        for (int a = 0; a < (side ? r.nprod : r.nreac); a++) {
+          const int at = side * PJ_MAX_SP + a;
+          if (r.sp[at] == bath) j.bath |= (uint8_t)(1 << (3 * side + std::min(a, 2)));
+          else (side ? j.nbx : j.nfx) += (uint8_t)r.nu[at];
+        }
+      }
+    }
     r.bath_in = 0;
     for (int a = 0; a < 2 * PJ_MAX_SP; a++) r.bath_in |= r.sp[a] == bath && (a % PJ_MAX_SP) < (a < PJ_MAX_SP ? r.nreac : r.nprod);
   }
@@ -546,7 +564,7 @@ int mech_build(pj_mech* m) {
   std::vector<int32_t> tgt_csr, tgt_csc;
   for (int q = 0; q < nr; q++) {
     Rxn& r = rx[q];
-    r.tgt_lo = (int32_t)tgt_csr.size();
+    r.tgt_lo = r.jac.tgt_lo = (int32_t)tgt_csr.size();
     auto push = [&](int i, int j) {
       tgt_csr.push_back(m->pos_csr[(size_t)i * N + j]);
       tgt_csc.push_back(m->pos_csc[(size_t)i * N + j]);
@@ -607,10 +625,13 @@ int mech_build(pj_mech* m) {
   const size_t o_gath = align256(o_gptr + gptr.size() * sizeof(int32_t));
   const size_t total = align256(o_gath + gather.size() * sizeof(uint16_t));
   const MathTables& tables = math_tables();
-  // |g_k/RT| up to which sum nu g stays within half the fixed point's range
+  // |g_k/RT| up to which sum nu g stays within half the fixed point's range,
+  // |h_k/RT| up to which sum nu h stays within it
   const double g_lim = std::min(1300.0, 2000.0 * 0.6931471805599453 / nu_max);
-  uint64_t g_bits;
+  const double h_lim = std::min(1300.0, 4000.0 / nu_max);
+  uint64_t g_bits, h_bits;
   std::memcpy(&g_bits, &g_lim, sizeof g_bits);
+  std::memcpy(&h_bits, &h_lim, sizeof h_bits);
 
   std::vector<char> blob(total, 0);
   auto put = [&](size_t off, const void* src, size_t bytes) { if (bytes) std::memcpy(blob.data() + off, src, bytes); };
@@ -671,6 +692,7 @@ int mech_build(pj_mech* m) {
   dm.log2_pstd_fx = std::llrint(std::log2((long double)P_STD / (long double)RU) * 0x1p51L);
   dm.fx_ok = fx_ok ? 1 : 0;
   dm.fx_g_hi = (uint32_t)(g_bits >> 32);
+  dm.fx_h_hi = (uint32_t)(h_bits >> 32);
   dm.tab = reinterpret_cast<const double*>(b + o_tab);
   dm.tgt_csr = reinterpret_cast<const int32_t*>(b + o_tcsr);
   dm.tgt_csc = reinterpret_cast<const int32_t*>(b + o_tcsc);

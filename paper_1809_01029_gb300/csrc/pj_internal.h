@@ -55,10 +55,21 @@ struct alignas(16) RxnHead {
   int32_t pad3;
 };
 
+// What the Jacobian's short path (lean_jacobian) reads besides the head.
+struct alignas(16) RxnJac {
+  double beta, theta, dW;         // as in Rxn
+  int32_t tgt_lo, row_lo;         // as in Rxn
+  uint8_t nrows, neg;             // rows; bit q set: row q's coefficient is -1
+  uint8_t shape[2];               // SH_* of the forward and the reverse side
+  uint8_t nfx, nbx;               // factors that are not the bath gas, by side
+  uint8_t bath, dense;            // bit a / 3 + a: reactant a / product a is the bath gas; Rxn::dense
+};
+
 // One reaction, packed for warp-uniform loads (every thread of a warp reads
 // the same record).  Reactions are stored in kernel order (see perm).
 struct alignas(16) Rxn {
   RxnHead head;
+  RxnJac jac;
   double lnA, beta, theta;        // k = exp(lnA + beta lnT - theta/T), theta = Ea/R_cal [K]
   double lnA0, beta0, theta0;     // low-pressure limit (falloff)
   double dnu;                     // sum_k nu_k (equilibrium-constant pressure factor)
@@ -82,7 +93,7 @@ struct alignas(16) Rxn {
   int32_t bath_in;                // the bath gas is one of its reactants or products
   int64_t fA0, fB0, fT0;          // the low-pressure set in fixed point, as head.fA, fB, fT
 };
-static_assert(sizeof(RxnHead) == 64, "the head is four 16-byte loads");
+static_assert(sizeof(RxnHead) == 64 && sizeof(RxnJac) == 48, "records are 16-byte loads");
 
 // One unit of a reaction's net stoichiometric coefficient for species k: a
 // species with |nu| = 2 has two such rows.
@@ -100,7 +111,7 @@ struct DevMech {
   // fixed-point rate constants: usable for every reaction when fx_ok, at
   // states with |g_k/RT| below the double whose high word is fx_g_hi
   int32_t fx_ok;
-  uint32_t fx_g_hi;
+  uint32_t fx_g_hi, fx_h_hi;      // and |h_k/RT| below fx_h_hi's
   const double* nasa;             // [ns * NASA_STRIDE]
   const double* wfac;             // [ns] 1 - W_k / W_{Ns-1}
   const Rxn* rxn;                 // [nr]
