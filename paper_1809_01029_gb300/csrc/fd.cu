@@ -75,7 +75,7 @@ __global__ void __launch_bounds__(kSrcWarps * 32, 2)
   for (int64_t tile = blockIdx.x; tile * kTile < n; tile += gridDim.x) {
     const int64_t s = tile * kTile + lane;
     const BatchIn in{param, phi, ld, s, s < n};
-    source_tile<MODE, SPECIAL>(m, smem, arrays, in, SourceOut{dphi, ws, ld, s, m.ns, status});
+    source_tile<MODE, SPECIAL, kEither>(m, smem, arrays, in, SourceOut{dphi, ws, ld, s, m.ns, status});
     __syncthreads();  // the source terms of every row before any warp reads them
     double lo = 0.0;
     if (in.active) {
@@ -89,7 +89,7 @@ __global__ void __launch_bounds__(kSrcWarps * 32, 2)
         const double x = phi[(int64_t)j * ld + s];
         h = (x + kFdScale * fmax(fabs(x), lo)) - x;
       }
-      source_tile<MODE, SPECIAL>(m, smem, arrays, FdIn<MODE>{in, j, lo}, FdOut<FMT>{m, J, dphi, ws, ld, s, j, h});
+      source_tile<MODE, SPECIAL, kEither>(m, smem, arrays, FdIn<MODE>{in, j, lo}, FdOut<FMT>{m, J, dphi, ws, ld, s, j, h});
     }
     __syncthreads();
   }

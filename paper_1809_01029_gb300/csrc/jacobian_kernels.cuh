@@ -146,14 +146,13 @@ __device__ __forceinline__ void st_zero_evict_last(float* a, uint64_t pol) {
   asm volatile("st.global.L2::cache_hint.b32 [%0], 0, %1;" ::"l"(a), "l"(pol) : "memory");
 }
 
-// MAXW: the most warps a block of this instance has (launch bound MAXW * 32
-// threads, one block per SM guaranteed): 16 caps registers at 128 per
-// thread, 8 allows 255.
-// aws: the per-state arrays of each block's tile in a global workspace
-// (mechanisms too large for shared memory), else null.  src.batches: tiles
+// Blocks of up to 16 warps: 128 registers a thread.
+// SHARED: the per-state arrays in shared memory (a compile-time choice, so
+// that they are addressed as shared memory), else in aws, a global workspace
+// (mechanisms too large for shared memory).  src.batches: tiles
 // of several batches from a counter, else the tiles of (n, param, phi, ...).
-template <int MODE, int FMT, typename DT, bool NEWTON, bool SPECIAL, int MAXW, bool BATCHED = false>
-__global__ void __launch_bounds__(MAXW * 32, 1)
+template <int MODE, int FMT, typename DT, bool NEWTON, bool SPECIAL, bool SHARED, bool BATCHED = false>
+__global__ void __launch_bounds__(kCoopWarpsMax * 32, 1)
     k_jacobian_coop(const __grid_constant__ DevMech m, int64_t n0, const double* __restrict__ param0, const double* __restrict__ phi0,
                     int64_t ld0, DT* __restrict__ J0, double* __restrict__ dphi0, int* status,
                     const double* __restrict__ hstep, double gamma, double* __restrict__ aws, CoopSrc src) {
@@ -168,7 +167,7 @@ __global__ void __launch_bounds__(MAXW * 32, 1)
   const int lane = threadIdx.x & 31, warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
   const int W = blockDim.x >> 5;
   const int64_t n_out = FMT == PJ_DENSE ? (int64_t)N * N : (int64_t)m.nnz;
-  double* const tsm = aws ? smem : smem + 3 * ns * kCoopTile;                     // the tile's scalars and sums
+  double* const tsm = SHARED ? smem + 3 * ns * kCoopTile : smem;                     // the tile's scalars and sums
   double* __restrict__ sc = tsm + lane;                                            // sc[v*32]
   double* __restrict__ part = tsm + kCoopSc * kCoopTile + lane;                    // part[(w*kCoopPart + v)*32]
   int* __restrict__ flags = reinterpret_cast<int*>(tsm + (kCoopSc + kCoopPart * W) * kCoopTile);
@@ -183,7 +182,7 @@ __global__ void __launch_bounds__(MAXW * 32, 1)
   };
   StateArrays A;
   A.ns = ns;
-  A.base = aws ? aws + (int64_t)blockIdx.x * 3 * ns * kCoopTile + lane : smem + lane;
+  A.base = SHARED ? smem + lane : aws + (int64_t)blockIdx.x * 3 * ns * kCoopTile + lane;
   A.stride = kCoopTile;
   enum { aC = 0, aG = 1, aH = 2 };
 
@@ -284,7 +283,7 @@ __global__ void __launch_bounds__(MAXW * 32, 1)
         A.at(aH, k) = fixed_enthalpy(m, h, fast);
         const double cx = MODE == PJ_CONP ? cp : cp - 1.0;
         if (k < bath) {
-          const double c = ok0 ? phi[(int64_t)(k + 2) * ld + s] / V : cdum;
+          const double c = ok0 ? concentration(phi[(int64_t)(k + 2) * ld + s], V, S(cInvV)) : cdum;
           A.at(aC, k) = c;
           acc += c;
           den = fma(c, cx, den);
@@ -332,7 +331,7 @@ __global__ void __launch_bounds__(MAXW * 32, 1)
 
     // a tile with a state outside the fixed point's range takes the general
     // path, with h_k/RT in FP64
-    const bool fast_tile = __all_sync(0xffffffffu, F(fFast) != 0);  // the same in every warp
+    const bool fast_tile = __all_sync(0xffffffffu, F(fFast) != 0) && ld < (1 << 28);  // the same in every warp
     if (!fast_tile) {
       const double T = S(cT), invT = S(cInvT);
       for (int k = warp; k < ns; k += W) A.at(aH, k) = nasa_h(nasa_block(m, k, T), T, invT);
@@ -514,11 +513,12 @@ template <int MODE, int FMT, typename DT, bool NEWTON, bool SPECIAL>
 static int launch_jac_coop_s(const DevMech& m, const CoopPlan& c, int64_t n, const JacArgs& a, double* ws,
                              cudaStream_t st) {
   // the batched plans' tile hand-out is an instance of its own (FP64
-  // Jacobian, up to 16 warps), so that the other instances carry none of its
-  // registers
-  auto kern = a.src.batches ? k_jacobian_coop<MODE, FMT, DT, NEWTON, SPECIAL, kCoopWarpsMax, !NEWTON>
-              : c.wide_regs ? k_jacobian_coop<MODE, FMT, DT, NEWTON, SPECIAL, 8>
-                            : k_jacobian_coop<MODE, FMT, DT, NEWTON, SPECIAL, kCoopWarpsMax>;
+  // Jacobian), so that the other instances carry none of its registers
+  const bool shared = c.ws_bytes == 0;
+  auto kern = a.src.batches ? (shared ? k_jacobian_coop<MODE, FMT, DT, NEWTON, SPECIAL, true, !NEWTON>
+                                      : k_jacobian_coop<MODE, FMT, DT, NEWTON, SPECIAL, false, !NEWTON>)
+                            : (shared ? k_jacobian_coop<MODE, FMT, DT, NEWTON, SPECIAL, true>
+                                      : k_jacobian_coop<MODE, FMT, DT, NEWTON, SPECIAL, false>);
   if (NEWTON && a.src.batches) return fail(PJ_ERR_UNSUPPORTED, "batched plans compute the FP64 Jacobian only");
   int rc;
   if ((rc = set_smem(kern, c.smem))) return rc;

@@ -46,7 +46,7 @@ namespace pj {
 // ---------------------------------------------------------------------------
 // A block of 16 warps per 32-state tile (source_tile.cuh), two blocks per SM,
 // tiles handed out block-cyclically.  Y: y = (wdot, dT/dt) instead of dPhi/dt.
-template <int MODE, bool SPECIAL, bool Y>
+template <int MODE, bool SPECIAL, bool Y, bool SHARED>
 __global__ void __launch_bounds__(kSrcWarps * 32, 2)
     k_source_terms(const __grid_constant__ DevMech m, int64_t n, const double* __restrict__ param,
                    const double* __restrict__ phi, int64_t ld, double* __restrict__ out, int* status, double* ws,
@@ -59,8 +59,8 @@ __global__ void __launch_bounds__(kSrcWarps * 32, 2)
   for (int64_t tile = blockIdx.x; tile * kTile < n; tile += gridDim.x) {
     const int64_t s = tile * kTile + lane;
     const BatchIn in{param, phi, ld, s, s < n};
-    if constexpr (Y) source_tile<MODE, SPECIAL>(m, smem, arrays, in, YOut{out, ld, s, m.ns, status});
-    else source_tile<MODE, SPECIAL>(m, smem, arrays, in, SourceOut{out, ws, ld, s, m.ns, status});
+    if constexpr (Y) source_tile<MODE, SPECIAL, SHARED ? kShared : kGlobal>(m, smem, arrays, in, YOut{out, ld, s, m.ns, status});
+    else source_tile<MODE, SPECIAL, SHARED ? kShared : kGlobal>(m, smem, arrays, in, SourceOut{out, ws, ld, s, m.ns, status});
   }
 }
 
@@ -159,8 +159,12 @@ static int launch_source_t(const DevMech& m, int mode, int64_t n, const double* 
   double* arrays = p.arrays_bytes ? static_cast<double*>(work) : nullptr;
   double* acc = Y ? nullptr : static_cast<double*>(work) + p.arrays_bytes / sizeof(double);
   const bool special = m.nr_plain < m.nr;
-  auto kern = mode == PJ_CONP ? (special ? k_source_terms<PJ_CONP, true, Y> : k_source_terms<PJ_CONP, false, Y>)
-                              : (special ? k_source_terms<PJ_CONV, true, Y> : k_source_terms<PJ_CONV, false, Y>);
+  auto pick = [&](auto shared) {
+    constexpr bool SH = decltype(shared)::value;
+    return mode == PJ_CONP ? (special ? k_source_terms<PJ_CONP, true, Y, SH> : k_source_terms<PJ_CONP, false, Y, SH>)
+                           : (special ? k_source_terms<PJ_CONV, true, Y, SH> : k_source_terms<PJ_CONV, false, Y, SH>);
+  };
+  auto kern = p.arrays_smem ? pick(BoolTag<true>{}) : pick(BoolTag<false>{});
   int rc;
   if ((rc = set_smem(kern, p.smem))) return rc;
   kern<<<p.grid, kSrcWarps * 32, p.smem, st>>>(m, n, param, phi, ld, out, status, acc, arrays);
@@ -251,16 +255,14 @@ TmPlan tm_plan(int ns) {
 // PYJAC_GB_JAC_LAYOUT=coop|percore forces one family (coop only where its
 // shared memory fits); PYJAC_GB_COOP_WARPS sets the warps per block (4, 8
 // or 16), PYJAC_GB_COOP_CTAS the blocks per SM (at most 16 / warps) and
-// PYJAC_GB_COOP_ARRAYS=global puts the arrays in the workspace; 8 warps in
-// one block per SM run the instance compiled for 255 registers.
+// PYJAC_GB_COOP_ARRAYS=global puts the arrays in the workspace.
 static int env_int(const char* name, int dflt) {
   const char* v = getenv(name);
   return v && *v ? atoi(v) : dflt;
 }
 
 bool coop_shape(const DevMech& m, int warps, int ctas, bool arrays_smem, int64_t tiles, CoopPlan& c) {
-  c = CoopPlan{false, warps, ctas, coop_smem_bytes(m.ns, warps, arrays_smem), sm_count() * ctas,
-               warps == 8 && ctas == 1, 0};
+  c = CoopPlan{false, warps, ctas, coop_smem_bytes(m.ns, warps, arrays_smem), sm_count() * ctas, 0};
   if (warps != 4 && warps != 8 && warps != 16) return false;
   if (ctas < 1 || ctas * warps > 16) return false;
   if (c.smem + kBlockOverhead > kSmemPerSm / (size_t)ctas || c.smem > kSmemCap) return false;
@@ -279,7 +281,7 @@ static bool coop_fit(const DevMech& m, int warps, int ctas, int64_t n, CoopPlan&
 }
 
 CoopPlan coop_plan(const DevMech& m, int fmt, int dt_bytes, int64_t n) {
-  CoopPlan c{false, 16, 1, 0, 0, false, 0};
+  CoopPlan c{false, 16, 1, 0, 0, 0};
   const char* lay = getenv("PYJAC_GB_JAC_LAYOUT");
   if (lay && strcmp(lay, "percore") == 0) return c;
   if (lay && strcmp(lay, "coop") == 0) {

@@ -81,6 +81,15 @@ __device__ __forceinline__ double fixed51_to_double(int64_t y) {
   return __longlong_as_double((long long)fixed_to_double(y, 51));
 }
 
+// n / V from iV = 1/V rounded: one correction of the quotient's residual, so
+// that it rounds as the division does but for rare halfway cases (three FP64
+// instructions for about nine).
+__device__ __forceinline__ double concentration(double n, double V, double iV) {
+  if ((uint32_t)__double2hiint(V) - 0x01800000u >= 0x7c000000u) return n / V;  // 1/V would leave the normal range
+  const double c = n * iV;
+  return fma(fma(-c, V, n), iV, c);
+}
+
 __device__ __forceinline__ bool has_third_body(int kind) { return kind >= PJ_THIRD_BODY && kind <= PJ_SRI; }
 
 // Load one state, fill C_k (k < Ns-1 as n_k/V; the bath gas as C_tot minus
@@ -95,8 +104,9 @@ __device__ __forceinline__ bool load_state(const DevMech& m, const double* __res
   const double P = MODE == PJ_CONP ? par : S;
   bool ok = (T > 0.0) && (V > 0.0) && (P > 0.0) && isfinite(T) && isfinite(V) && isfinite(P);
   double acc = 0.0;
+  const double iV = 1.0 / V;
   for (int k = 0; k < ns - 1; k++) {
-    const double c = phi[(int64_t)(k + 2) * ld + s] / V;
+    const double c = concentration(phi[(int64_t)(k + 2) * ld + s], V, iV);
     A.at(aC, k) = c;
     acc += c;
   }
@@ -114,44 +124,76 @@ __device__ __forceinline__ bool load_state(const DevMech& m, const double* __res
   return ok;
 }
 
-// Troe / SRI broadening factor F(T, Pr) in FP64.  With derivatives also
-// returns FxPr = Pr dF/dPr (at fixed T) and FT = dF/dT (at fixed Pr).  The
-// logarithms are fixed-point (l2Pr = log2(Pr) 2^51); ok = false, with nothing
-// returned, when an argument is not a positive normal number.
+// 1/x for x well within the normal range: the hardware's approximation and
+// two Newton steps (four FMAs; an IEEE division issues about nine FP64
+// instructions).
+__device__ __forceinline__ double reciprocal(double x) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  r = fma(r, fma(-x, r, 1.0), r);
+  return fma(r, fma(-x, r, 1.0), r);
+}
+
+// 1 / (1 + Pr); Pr beyond 2^1000 (or not finite, or negative) by division
+__device__ __forceinline__ double inverse_1p(double Pr) {
+  if ((uint32_t)__double2hiint(Pr) >= 0x7e700000u) return 1.0 / (1.0 + Pr);
+  return reciprocal(1.0 + Pr);
+}
+
+// Troe / SRI broadening factor F(T, Pr).  With derivatives also returns FxPr
+// = Pr dF/dPr (at fixed T) and FT = dF/dT (at fixed Pr).  For states within
+// the fixed point's range (128 <= T < 65536, IT = 2^70 / T); l2Pr = log2(Pr)
+// 2^51; ok = false, with nothing returned, when F_cent (or Z) is not a
+// positive normal number.
 //
 // Troe: with D = N - 0.14 xc and S = D^2 + xc^2, log10 F = L g, g = D^2 / S
 // (1 / (1 + (xc/D)^2)), so that F and its derivatives take one reciprocal:
-// dg/dx = -2 N xc D / S^2.  A log, an exp and a divide each were 9 to 30 FP64
-// operations; the fixed-point ones are none.
+// dg/dx = -2 N xc D / S^2.  Exponents, exponentials and logarithms are fixed
+// point: a falloff reaction's 126 FP64 instructions were 22 % of the
+// 53-species Jacobian's and 45 % of its source terms'.
 template <bool DERIV>
-__device__ __forceinline__ double falloff_F(const LogEntry* __restrict__ log_tab, const Rxn* __restrict__ r, int kind, double T,
-                                            double invT, double lnT, int64_t l2Pr, bool& ok, double& FxPr,
-                                            double& FT) {
+__device__ __forceinline__ double falloff_F(const LogEntry* __restrict__ log_tab, const Rxn* __restrict__ r, int kind,
+                                            double T, double invT, double lnT, uint64_t IT, int64_t l2Pr, bool& ok,
+                                            double& FxPr, double& FT) {
   FxPr = 0.0;
   FT = 0.0;
   constexpr double LOG10_2 = 0.30102999566398119521;
   if (kind == PJ_TROE) {
     const double a = __ldg(&r->fp[0]), iT3 = __ldg(&r->fp[1]), iT1 = __ldg(&r->fp[2]);
-    const double T2 = __ldg(&r->fp[3]), has2 = __ldg(&r->fp[4]);
-    const double e3 = pj_exp(-T * iT3), e1 = pj_exp(-T * iT1);
-    const double e2 = has2 != 0.0 ? pj_exp(-T2 * invT) : 0.0;
-    const double Fcent = (1.0 - a) * e3 + a * e1 + e2;
-    const double l2F = fixed51_to_double(log2_51(log_tab, Fcent, ok));
+    const double T2 = __ldg(&r->fp[3]);
+    const int fxr = __ldg(&r->troe_fx);
+    const uint64_t tb = (uint64_t)__double_as_longlong(T);
+    const uint64_t X = ((tb << 11) | 0x8000000000000000ull) >> (1039 - (int)(tb >> 52));  // T 2^47
+    const double e3 = fxr & 1 ? exp2_51(-(int64_t)mulhi_approx(__ldg(&r->tT3), X)) : pj_exp(-T * iT3);
+    const double e1 = fxr & 2 ? exp2_51(-(int64_t)mulhi_approx(__ldg(&r->tT1), X)) : pj_exp(-T * iT1);
+    double e2 = 0.0;
+    if (fxr & 4) e2 = exp2_51(-(int64_t)mulhi_approx(__ldg(&r->tT2), IT));
+    else if (__ldg(&r->fp[4]) != 0.0) e2 = pj_exp(-T2 * invT);
+    const double Fcent = fma(1.0 - a, e3, fma(a, e1, e2));
+    const int64_t l2F = log2_51(log_tab, Fcent, ok);
     if (!ok) return 1.0;
-    const double L = l2F * LOG10_2;
-    const double xc = fixed51_to_double(l2Pr) * LOG10_2 + (-0.4 - 0.67 * L);
-    const double NN = 0.75 - 1.27 * L;
-    const double D = NN - 0.14 * xc;
+    const double L = fixed51_to_double(l2F) * LOG10_2;
+    const double xc = fma(fixed51_to_double(l2Pr), LOG10_2, fma(-0.67, L, -0.4));
+    const double NN = fma(-1.27, L, 0.75);
+    const double D = fma(-0.14, xc, NN);
     const double D2 = D * D;
-    const double iS = 1.0 / fma(xc, xc, D2);
+    const double iS = reciprocal(fma(xc, xc, D2));
     const double g = D2 * iS;
-    const double F = pj_exp(LN10 * (L * g));
+    // F = 2^(l2F g): the product in fixed point while |log2 F_cent| < 16
+    const uint64_t gb = (uint64_t)__double_as_longlong(g);
+    const int gs = 1023 - (int)(gb >> 52);
+    double F;
+    if ((uint64_t)(l2F + (1ll << 55)) < (1ull << 56) && gs >= 0 && gs < 64)
+      F = exp2_51((mulhi_su(l2F << 8, ((gb << 11) | 0x8000000000000000ull) >> gs) + 64) >> 7);
+    else
+      F = pj_exp(LN10 * (L * g));
     if (DERIV) {
-      const double t = -2.0 * (xc * D) * (L * iS) * iS;  // L dg/dx / N
-      const double dlg_dL = g + t * (1.1762 * xc - 0.67 * D);
-      const double dFcent = -(1.0 - a) * iT3 * e3 - a * iT1 * e1 + T2 * (invT * invT) * e2;
+      const double Li = L * iS;
+      const double t = -2.0 * (xc * D) * (Li * iS);  // L dg/dx / N
+      const double dlg_dL = fma(t, fma(1.1762, xc, -0.67 * D), g);
+      const double dFcent = fma(T2 * (invT * invT), e2, -fma((1.0 - a) * iT3, e3, (a * iT1) * e1));
       FxPr = F * (t * NN);
-      FT = F * dlg_dL * dFcent / Fcent;
+      FT = F * dlg_dL * (dFcent * reciprocal(Fcent));
     }
     return F;
   }
@@ -159,7 +201,7 @@ __device__ __forceinline__ double falloff_F(const LogEntry* __restrict__ log_tab
     const double a = __ldg(&r->fp[0]), b = __ldg(&r->fp[1]), ic = __ldg(&r->fp[2]);
     const double d = __ldg(&r->fp[3]), e = __ldg(&r->fp[4]);
     const double x = fixed51_to_double(l2Pr) * LOG10_2;
-    const double X = 1.0 / (1.0 + x * x);
+    const double X = reciprocal(fma(x, x, 1.0));
     const double eb = pj_exp(-b * invT), ec = pj_exp(-T * ic);
     const double Z = a * eb + ec;
     const double lnZ = fixed51_to_double(log2_51(log_tab, Z, ok)) * 0.69314718055994530942;
@@ -519,7 +561,7 @@ __device__ __forceinline__ double falloff_Pr_F(const DevMech& m, const Rxn* __re
   if (kind == PJ_LINDEMANN) return Pr;
   bool ok = fx.fast;
   const int64_t l2Pr = k.l2rk + log2_51(m.log_tab, M, ok);
-  if (ok) F = falloff_F<DERIV>(m.log_tab, r, kind, T, invT, lnT, l2Pr, ok, FxPr, FT);
+  if (ok) F = falloff_F<DERIV>(m.log_tab, r, kind, T, invT, lnT, fx.IT, l2Pr, ok, FxPr, FT);
   if (!ok) F = falloff_F_library(r, kind, T, invT, lnT, Pr, FxPr, FT);
   return Pr;
 }

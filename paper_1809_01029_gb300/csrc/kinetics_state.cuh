@@ -351,14 +351,14 @@ __device__ __forceinline__ void jac_reaction(const DevMech& m, const SA& A, JacV
   auto slot = [&](int j, DT val) {
     if (j == bath) return;
     const DT vs = nscale<NEWTON>(o, val);
+    const int64_t eT = target(0, j + 2), eS = target(1, j + 2);
+    if (w) jred(J, eT, ld, s, dE * vs);
+    if (w) jred(J, eS, ld, s, dW * vs);
     for (int q2 = row_lo; q2 < row_hi; q2++) {
       const RowNu rn = m.rows[q2];
       const int64_t e = target(rn.k + 2, j + 2);
       if (w) jred(J, e, ld, s, nu_times_t<DT>(rn.nu, rn.nud, vs));
     }
-    const int64_t eT = target(0, j + 2), eS = target(1, j + 2);
-    if (w) jred(J, eT, ld, s, dE * vs);
-    if (w) jred(J, eS, ld, s, dW * vs);
   };
 #pragma unroll
   for (int a = 0; a < PJ_MAX_SP; a++) {

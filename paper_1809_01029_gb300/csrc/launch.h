@@ -46,7 +46,6 @@ struct CoopPlan {
   int ctas;
   size_t smem;
   int grid;
-  bool wide_regs;   // 8 warps, one block per SM, up to 255 registers a thread
   size_t ws_bytes;  // per-state arrays in a global workspace (grid x 3 Ns x 32
                     // doubles); 0: in shared memory
 };

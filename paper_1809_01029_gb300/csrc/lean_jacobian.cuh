@@ -35,19 +35,19 @@ struct FalloffC {
 };
 __device__ __noinline__ static FalloffC falloff_derivatives(const Rxn* __restrict__ r,
                                                             const LogEntry* __restrict__ log_tab, int kind, double T,
-                                                            double invT, double lnT, double rk, int64_t l2rk, double M,
-                                                            double dMdT) {
+                                                            double invT, double lnT, uint64_t IT, double rk,
+                                                            int64_t l2rk, double M, double dMdT) {
   double F = 1.0, FxPr = 0.0, FT = 0.0;
   const double Pr = rk * M;
   if (kind != PJ_LINDEMANN) {
     bool ok = true;
     const int64_t l2Pr = l2rk + log2_51(log_tab, M, ok);
-    if (ok) F = falloff_F<true>(log_tab, r, kind, T, invT, lnT, l2Pr, ok, FxPr, FT);
+    if (ok) F = falloff_F<true>(log_tab, r, kind, T, invT, lnT, IT, l2Pr, ok, FxPr, FT);
     if (!ok) F = falloff_F_library(r, kind, T, invT, lnT, Pr, FxPr, FT);
   }
   const double invT2 = invT * invT;
   const double dlnrk = fma(__ldg(&r->theta0) - __ldg(&r->theta), invT2, (__ldg(&r->beta0) - __ldg(&r->beta)) * invT);
-  const double i1p = 1.0 / (1.0 + Pr);
+  const double i1p = inverse_1p(Pr);
   const double fr = Pr * i1p;
   const double cPr = F * i1p * i1p + FxPr * i1p;
   return FalloffC{fr * F, cPr * rk, fr * FT + cPr * (Pr * dlnrk + rk * dMdT)};
@@ -114,11 +114,11 @@ __device__ __forceinline__ LeanSide lean_side(const int32_t (&f)[3], int shape, 
 
 __device__ __forceinline__ int shape_species(int shape) { return shape <= SH_2 ? 1 : shape <= SH_21 ? 2 : 3; }
 
-// negated when neg is not 0 (warp-uniform)
-__device__ __forceinline__ double flip(double x, uint32_t neg) {
-  return __hiloint2double(__double2hiint(x) ^ (int)(neg << 31), __double2loint(x));
+// x with its sign bit flipped by a mask (0 or 0x80000000)
+__device__ __forceinline__ double flip(double x, uint32_t sign) {
+  return __hiloint2double((int)((uint32_t)__double2hiint(x) ^ sign), __double2loint(x));
 }
-__device__ __forceinline__ float flip(float x, uint32_t neg) { return __uint_as_float(__float_as_uint(x) ^ (neg << 31)); }
+__device__ __forceinline__ float flip(float x, uint32_t sign) { return __uint_as_float(__float_as_uint(x) ^ sign); }
 
 // base: this lane's column of the tile's arrays C, g, h ([3][ns][32]).
 template <int MODE, int FMT, typename DT, bool NEWTON>
@@ -133,7 +133,7 @@ __device__ __forceinline__ void lean_jacobian(const DevMech& m, const Rxn* __res
     const int4* __restrict__ p = reinterpret_cast<const int4*>(&r->jac);
     int4* q = reinterpret_cast<int4*>(&a);
 #pragma unroll
-    for (int i = 0; i < 3; i++) q[i] = __ldg(p + i);
+    for (int i = 0; i < 4; i++) q[i] = __ldg(p + i);
   }
   const bool rev = h.rev != 0;
   const int64_t y = arrhenius_fixed(h.fA, h.fB, h.fT, v.fx.L, v.fx.IT);
@@ -161,8 +161,7 @@ __device__ __forceinline__ void lean_jacobian(const DevMech& m, const Rxn* __res
   double VT = (sf.R * Ef - sb.R * (Ef - de)) * (v.V * v.invT);
   double VS = 0.0;
   if (MODE == PJ_CONP) {
-    if (rev && a.nfx != a.nbx) VS = (double)a.nbx * sb.R - (double)a.nfx * sf.R;
-    else VS = -(double)a.nfx * Rn;
+    VS = rev && !a.same ? a.nbx * sb.R - a.nfx * sf.R : -a.nfx * Rn;
   }
   double Gb = 0.0;  // dRn/dC of the bath gas itself
   bool has_S = MODE == PJ_CONP;
@@ -198,7 +197,7 @@ __device__ __forceinline__ void lean_jacobian(const DevMech& m, const Rxn* __res
     if (h.kind != PJ_THIRD_BODY) {
       const int64_t l2rk = arrhenius_fixed(__ldg(&r->fA0), __ldg(&r->fB0), __ldg(&r->fT0), v.fx.L, v.fx.IT) - y;
       const FalloffC fc =
-          falloff_derivatives(r, m.log_tab, h.kind, v.T, v.invT, v.lnT, exp2_51(l2rk), l2rk, M, dMdT);
+          falloff_derivatives(r, m.log_tab, h.kind, v.T, v.invT, v.lnT, v.fx.IT, exp2_51(l2rk), l2rk, M, dMdT);
       c = fc.c;
       cT = fc.cT;
       RcM = Rn * fc.cM;
@@ -224,72 +223,87 @@ __device__ __forceinline__ void lean_jacobian(const DevMech& m, const Rxn* __res
     jS = nscale<NEWTON>(o, VS_t);
   }
 
-  const int32_t* __restrict__ tg = (FMT == PJ_CSR ? m.tgt_csr : m.tgt_csc) + a.tgt_lo;
-  const RowNu* __restrict__ rows = m.rows + a.row_lo;
-  const int nrows = a.nrows;
-  DT* __restrict__ Js = o.J + o.s;
-  auto red = [&](int e, DT x) {
-    if (!PJ_DBG_OK(m.dbg, e >= 0 && e < (FMT == PJ_DENSE ? m.N * m.N : m.nnz), PJ_DBG_TARGET)) return;
-    if (o.w) red_add(Js + (uint64_t)(uint32_t)e * (uint64_t)o.ld, x);
-  };
-  auto entry = [&](int at, int row, int col) -> int { return FMT == PJ_DENSE ? row * m.N + col : __ldg(tg + at); };
-
-#pragma unroll 4
-  for (int p = 0; p < nrows; p++) {
-    const int k = __ldg(&rows[p].k);
-    const uint32_t neg = (a.neg >> p) & 1u;
-    red(entry(2 * p, k + 2, 0), flip(jT, neg));
-    if (has_S) red(entry(2 * p + 1, k + 2, 1), flip(jS, neg));
-    if (o.w) red_add(o.wrow + (int64_t)k * o.ld, flip(q, neg));
-  }
-  tg += 2 * nrows;
-
-  // species columns
-  auto slot = [&](int j, DT val) {
-    const DT vs = nscale<NEWTON>(o, val);
-#pragma unroll 4
-    for (int p = 0; p < nrows; p++)
-      red(entry(p, FMT == PJ_DENSE ? __ldg(&rows[p].k) + 2 : 0, j + 2), flip(vs, (a.neg >> p) & 1u));
-    red(entry(nrows, 0, j + 2), dE * vs);
-    red(entry(nrows + 1, 1, j + 2), dW * vs);
-    tg += nrows + 2;
-  };
-  const int nsf = shape_species(a.shape[0]), nsb = rev ? shape_species(a.shape[1]) : 0;
-  auto scaled = [&](double d) { return to_derivative<DT>(h.kind != PJ_ELEMENTARY ? c * d : d); };
+  // Jacobian entries and production rates, by L2 reductions.  Addresses: an
+  // entry's row of ld values, 32 x 32 -> 64 bit (the caller checks that ld
+  // fits); up to four rows unrolled with their signs as masks.
+  const double Bbath = h.kind != PJ_ELEMENTARY ? c * Gb : Gb;
+  DT B_t = DT(0);
+  if (o.w) {
+    const int32_t* __restrict__ tg = (FMT == PJ_CSR ? m.tgt_csr : m.tgt_csc) + a.tgt_lo;
+    const RowNu* __restrict__ rows = m.rows + a.row_lo;
+    const int nrows = a.nrows;
+    const uint32_t ldJ = (uint32_t)o.ld * (uint32_t)sizeof(DT), ldw = (uint32_t)o.ld * 8u;
+    char* const Jb = reinterpret_cast<char*>(o.J + o.s);
+    char* const wb = reinterpret_cast<char*>(o.wrow);
+    uint32_t sg[4];
 #pragma unroll
-  for (int s = 0; s < 3; s++) {
-    if (s < nsf && !(a.bath >> s & 1)) slot(FMT == PJ_DENSE ? __ldg(&r->sp[s]) : 0, scaled(s == 0 ? sf.d0 : s == 1 ? sf.d1 : sf.d2));
-    if (s < nsb && !(a.bath >> (3 + s) & 1))
-      slot(FMT == PJ_DENSE ? __ldg(&r->sp[PJ_MAX_SP + s]) : 0, dneg(scaled(s == 0 ? sb.d0 : s == 1 ? sb.d1 : sb.d2)));
-  }
-  double Bi = 0.0;  // minus the terms of the bath gas
-  if (h.kind != PJ_ELEMENTARY) {
-    for (int e = __ldg(&r->eff_lo), eh = __ldg(&r->eff_hi); e < eh; e++) {
-      if (!PJ_DBG_OK(m.dbg, e >= 0 && e < m.n_eff, PJ_DBG_EFF)) break;
-      const int j = __ldg(m.eff_sp + e);
-      const double val = RcM * __ldg(m.eff_am1 + e);
-      if (j == bath) Bi -= val;
-      else slot(j, to_derivative<DT>(val));
+    for (int p = 0; p < 4; p++) sg[p] = (uint32_t)a.neg << (31 - p) & 0x80000000u;
+    auto red = [&](int e, DT x) {
+      if (!PJ_DBG_OK(m.dbg, e >= 0 && e < (FMT == PJ_DENSE ? m.N * m.N : m.nnz), PJ_DBG_TARGET)) return;
+      red_add(reinterpret_cast<DT*>(Jb + (uint64_t)(uint32_t)e * ldJ), x);
+    };
+    auto row = [&](int p, int k, uint32_t sign) {
+      red(FMT == PJ_DENSE ? (k + 2) * m.N : __ldg(tg + 2 * p), flip(jT, sign));
+      if (has_S) red(FMT == PJ_DENSE ? (k + 2) * m.N + 1 : __ldg(tg + 2 * p + 1), flip(jS, sign));
+      red_add(reinterpret_cast<double*>(wb + (uint64_t)(uint32_t)k * ldw), flip(q, sign));
+    };
+#pragma unroll
+    for (int p = 0; p < 4; p++)
+      if (p < nrows) row(p, a.k[p], sg[p]);
+    for (int p = 4; p < nrows; p++) row(p, __ldg(&rows[p].k), (uint32_t)a.neg << (31 - p) & 0x80000000u);
+    tg += 2 * nrows;
+
+    // species columns
+    auto slot = [&](int j, DT val) {
+      const DT vs = nscale<NEWTON>(o, val);
+      red(FMT == PJ_DENSE ? j + 2 : __ldg(tg), dE * vs);
+      red(FMT == PJ_DENSE ? m.N + j + 2 : __ldg(tg + 1), dW * vs);
+#pragma unroll
+      for (int p = 0; p < 4; p++)
+        if (p < nrows) red(FMT == PJ_DENSE ? (a.k[p] + 2) * m.N + j + 2 : __ldg(tg + 2 + p), flip(vs, sg[p]));
+      for (int p = 4; p < nrows; p++)
+        red(FMT == PJ_DENSE ? (__ldg(&rows[p].k) + 2) * m.N + j + 2 : __ldg(tg + 2 + p),
+            flip(vs, (uint32_t)a.neg << (31 - p) & 0x80000000u));
+      tg += nrows + 2;
+    };
+    const int nsf = shape_species(a.shape[0]), nsb = rev ? shape_species(a.shape[1]) : 0;
+    auto scaled = [&](double d) { return to_derivative<DT>(h.kind != PJ_ELEMENTARY ? c * d : d); };
+#pragma unroll
+    for (int s = 0; s < 3; s++) {
+      if (s < nsf && !(a.bath >> s & 1))
+        slot(FMT == PJ_DENSE ? __ldg(&r->sp[s]) : 0, scaled(s == 0 ? sf.d0 : s == 1 ? sf.d1 : sf.d2));
+      if (s < nsb && !(a.bath >> (3 + s) & 1))
+        slot(FMT == PJ_DENSE ? __ldg(&r->sp[PJ_MAX_SP + s]) : 0,
+             dneg(scaled(s == 0 ? sb.d0 : s == 1 ? sb.d1 : sb.d2)));
+    }
+    double Bi = -Bbath;  // minus the terms of the bath gas
+    if (h.kind != PJ_ELEMENTARY) {
+      for (int e = __ldg(&r->eff_lo), eh = __ldg(&r->eff_hi); e < eh; e++) {
+        if (!PJ_DBG_OK(m.dbg, e >= 0 && e < m.n_eff, PJ_DBG_EFF)) break;
+        const int j = __ldg(m.eff_sp + e);
+        const double val = RcM * __ldg(m.eff_am1 + e);
+        if (j == bath) Bi -= val;
+        else slot(j, to_derivative<DT>(val));
+      }
+    }
+    if (a.dense) {
+      B_t = to_derivative<DT>(Bi);
+      const DT Bs = nscale<NEWTON>(o, B_t);
+      for (int p = 0; p < nrows; p++) {
+        const int k = __ldg(&rows[p].k);
+        const DT val = flip(Bs, (uint32_t)a.neg << (31 - p) & 0x80000000u);
+        if (FMT == PJ_CSR) {
+          // a dense row holds every species column, contiguous in CSR
+          const int64_t e2 = jpos<FMT>(m, k + 2, 2);
+          if (!PJ_DBG_OK(m.dbg, e2 >= 0 && e2 + ns - 1 <= m.nnz, PJ_DBG_POSMAP)) continue;
+          for (int j = 0; j < ns - 1; j++) red((int)e2 + j, val);
+        } else {
+          for (int j = 0; j < ns - 1; j++) red((int)jpos<FMT>(m, k + 2, j + 2), val);
+        }
+      }
     }
   }
   if (a.dense) {
-    Bi -= h.kind != PJ_ELEMENTARY ? c * Gb : Gb;
-    const DT B_t = to_derivative<DT>(Bi);
-    const DT Bs = nscale<NEWTON>(o, B_t);
-    for (int p = 0; p < nrows; p++) {
-      const int k = __ldg(&rows[p].k);
-      const DT val = flip(Bs, (a.neg >> p) & 1u);
-      if (FMT == PJ_CSR) {
-        // a dense row holds every species column, contiguous in CSR
-        const int64_t e2 = jpos<FMT>(m, k + 2, 2);
-        if (!PJ_DBG_OK(m.dbg, e2 >= 0 && e2 + ns - 1 <= m.nnz, PJ_DBG_POSMAP)) continue;
-        if (o.w)
-          for (int j = 0; j < ns - 1; j++) red_add(Js + (e2 + j) * o.ld, val);
-      } else {
-        if (o.w)
-          for (int j = 0; j < ns - 1; j++) jred(o.J, jpos<FMT>(m, k + 2, j + 2), o.ld, o.s, val);
-      }
-    }
     v.ATB = v.ATB + dE * B_t;
     v.ASB = v.ASB + dW * B_t;
   }

@@ -451,6 +451,19 @@ int mech_build(pj_mech* m) {
       fT = -std::llrint(th * 0x1p45L);
     };
     if (!pdep) fixed_set(m->A[i], m->beta[i], m->Ea[i], r.head.fA, r.head.fB, r.head.fT);
+    if (r.kind == PJ_TROE) {
+      const long double l2e = 1.442695040888963407359924681001892137L;
+      const double* t = &m->troe[i * 4];
+      auto pack = [&](int bit, long double v, long double scale, long double most, uint64_t& out) {
+        if (v >= 0.0L && v < most) {
+          out = (uint64_t)std::floor(v * scale + 0.5L);
+          r.troe_fx |= 1 << bit;
+        }
+      };
+      pack(0, l2e / (long double)t[1], 0x1p68L, 0.058L, r.tT3);  // T < 65536 keeps T log2(e) / T3 below 2^12
+      pack(1, l2e / (long double)t[2], 0x1p68L, 0.058L, r.tT1);
+      if (m->troe_n[i] == 4) pack(2, (long double)t[3] * l2e, 0x1p45L, 0x1p17L, r.tT2);
+    }
     if (is_falloff(r.kind)) fixed_set(m->A0[i], m->beta0[i], m->Ea0[i], r.fA0, r.fB0, r.fT0);
     int nu_sum = 0;
     for (int a = 0; a < 2 * PJ_MAX_SP; a++)
@@ -507,18 +520,22 @@ int mech_build(pj_mech* m) {
       j.dW = r.dW;
       j.row_lo = r.row_lo;
       const int n_rows = r.row_hi - r.row_lo;
-      if (n_rows > 8) r.head.lean = 0;
+      if (n_rows > 8 || ns > 32767) r.head.lean = 0;
       j.nrows = (uint8_t)std::min(n_rows, 8);
-      for (int q2 = 0; q2 < j.nrows; q2++) j.neg |= (uint8_t)((rows[r.row_lo + q2].nu < 0) << q2);
+      for (int q2 = 0; q2 < j.nrows; q2++) {
+        j.neg |= (uint8_t)((rows[r.row_lo + q2].nu < 0) << q2);
+        if (q2 < 4) j.k[q2] = (uint16_t)rows[r.row_lo + q2].k;
+      }
       j.dense = (uint8_t)r.dense;
       for (int side = 0; side < 2; side++) {
         j.shape[side] = (uint8_t)r.shape[side];
         for (int a = 0; a < (side ? r.nprod : r.nreac); a++) {
           const int at = side * PJ_MAX_SP + a;
           if (r.sp[at] == bath) j.bath |= (uint8_t)(1 << (3 * side + std::min(a, 2)));
-          else (side ? j.nbx : j.nfx) += (uint8_t)r.nu[at];
+          else (side ? j.nbx : j.nfx) += r.nu[at];
         }
       }
+      j.same = j.nfx == j.nbx ? 1 : 0;
     }
     r.bath_in = 0;
     for (int a = 0; a < 2 * PJ_MAX_SP; a++) r.bath_in |= r.sp[a] == bath && (a % PJ_MAX_SP) < (a < PJ_MAX_SP ? r.nreac : r.nprod);
@@ -558,8 +575,8 @@ int mech_build(pj_mech* m) {
   // The sparse targets of each reaction's Jacobian contributions, in the
   // order jacobian_state makes them: per row it changes the T and S columns;
   // then per slot (reactant a, reversible product a, a = 0, 1, ..., then the
-  // non-unit efficiencies), skipping the bath gas, its column in each row and
-  // in rows T and S.  Read sequentially by the kernels instead of looking up
+  // non-unit efficiencies), skipping the bath gas, its column in rows T and
+  // S and in each row.  Read sequentially by the kernels instead of looking up
   // the N x N index map per contribution.
   std::vector<int32_t> tgt_csr, tgt_csc;
   for (int q = 0; q < nr; q++) {
@@ -575,9 +592,9 @@ int mech_build(pj_mech* m) {
     }
     auto slot = [&](int j) {
       if (j == bath) return;
-      for (int q2 = r.row_lo; q2 < r.row_hi; q2++) push(rows[q2].k + 2, j + 2);
       push(0, j + 2);
       push(1, j + 2);
+      for (int q2 = r.row_lo; q2 < r.row_hi; q2++) push(rows[q2].k + 2, j + 2);
     };
     for (int a = 0; a < PJ_MAX_SP; a++) {
       if (a < r.nreac) slot(r.sp[a]);

@@ -2,6 +2,7 @@
 // kernels of libpyjac_gb: packed mechanism constants and launch helpers.
 #pragma once
 
+#include <cstddef>
 #include <cstdint>
 #include <string>
 #include <vector>
@@ -61,8 +62,10 @@ struct alignas(16) RxnJac {
   int32_t tgt_lo, row_lo;         // as in Rxn
   uint8_t nrows, neg;             // rows; bit q set: row q's coefficient is -1
   uint8_t shape[2];               // SH_* of the forward and the reverse side
-  uint8_t nfx, nbx;               // factors that are not the bath gas, by side
   uint8_t bath, dense;            // bit a / 3 + a: reactant a / product a is the bath gas; Rxn::dense
+  uint8_t same, pad0;             // same: nfx == nbx
+  double nfx, nbx;                // factors that are not the bath gas, by side
+  uint16_t k[4];                  // species of the first four rows
 };
 
 // One reaction, packed for warp-uniform loads (every thread of a warp reads
@@ -92,8 +95,12 @@ struct alignas(16) Rxn {
   int32_t tgt_lo;                 // first of this reaction's Jacobian targets in tgt_csr / tgt_csc
   int32_t bath_in;                // the bath gas is one of its reactants or products
   int64_t fA0, fB0, fT0;          // the low-pressure set in fixed point, as head.fA, fB, fT
+  // Troe: log2(e)/T3 2^68, log2(e)/T1 2^68, T2 log2(e) 2^45; bit b of
+  // troe_fx: the b-th is within its range (else the FP64 argument is formed)
+  uint64_t tT3, tT1, tT2;
+  int32_t troe_fx, pad_;
 };
-static_assert(sizeof(RxnHead) == 64 && sizeof(RxnJac) == 48, "records are 16-byte loads");
+static_assert(sizeof(RxnHead) == 64 && sizeof(RxnJac) == 64 && offsetof(RxnJac, nfx) == 40, "records are 16-byte loads");
 
 // One unit of a reaction's net stoichiometric coefficient for species k: a
 // species with |nu| = 2 has two such rows.

@@ -25,7 +25,7 @@ namespace pj {
 constexpr int kTile = 32;
 constexpr int kSrcWarps = 16;  // warps per block
 
-enum SrcSc { zT, zV, zP, zInvT, zLnT, zLnP, zCtot, zL, zIT, zLP, zCdum, zDen, zCxB, kSrcSc };
+enum SrcSc { zT, zV, zP, zInvT, zInvV, zLnT, zLnP, zCtot, zL, zIT, zLP, zCdum, zDen, zCxB, kSrcSc };
 enum SrcPart { rAcc, rDen, rNum, rOm, kSrcPart };
 enum SrcFlag { gOk, gFast, kSrcFlag };
 
@@ -45,17 +45,18 @@ __host__ __device__ constexpr size_t source_arrays_ws_doubles(int ns, bool array
 // of line: it runs for about a fifth of the reactions, and its registers
 // would otherwise set every reaction's.
 __device__ __noinline__ static double falloff_factor(const Rxn* __restrict__ r, const LogEntry* __restrict__ log_tab,
-                                                     int kind, bool fast, double T, double invT, double lnT, double rk,
-                                                     int64_t l2rk, double M, bool chem) {
+                                                     int kind, bool fast, double T, double invT, double lnT, uint64_t IT,
+                                                     double rk, int64_t l2rk, double M, bool chem) {
   double F = 1.0, d1, d2;
   const double Pr = rk * M;
   if (kind != PJ_LINDEMANN) {
     bool ok = fast;
     const int64_t l2Pr = l2rk + log2_51(log_tab, M, ok);
-    if (ok) F = falloff_F<false>(log_tab, r, kind, T, invT, lnT, l2Pr, ok, d1, d2);
+    if (ok) F = falloff_F<false>(log_tab, r, kind, T, invT, lnT, IT, l2Pr, ok, d1, d2);
     if (!ok) F = falloff_F_library(r, kind, T, invT, lnT, Pr, d1, d2);
   }
-  return (chem ? 1.0 : Pr) / (1.0 + Pr) * F;
+  const double i1p = inverse_1p(Pr);
+  return (chem ? i1p : Pr * i1p) * F;
 }
 
 // Net rate of any reaction at any state.  Out of line (special types, sides
@@ -80,7 +81,7 @@ __device__ __noinline__ static double general_rate(const DevMech& m, double* bas
     const double M = third_body(m, A, aC, r, Ctot);
     c = kind == PJ_THIRD_BODY
             ? M
-            : falloff_factor(r, m.log_tab, kind, fx.fast, T, invT, lnT, k.rk, k.l2rk, M, SPECIAL && __ldg(&r->chem));
+            : falloff_factor(r, m.log_tab, kind, fx.fast, T, invT, lnT, fx.IT, k.rk, k.l2rk, M, SPECIAL && __ldg(&r->chem));
   }
   return c * (Rf - Rr);
 }
@@ -136,7 +137,7 @@ __device__ __forceinline__ double lean_rate(const DevMech& m, const Rxn* __restr
       q *= M;
     } else {
       const int64_t l2rk = arrhenius_fixed(__ldg(&r->fA0), __ldg(&r->fB0), __ldg(&r->fT0), fx.L, fx.IT) - y;
-      q *= falloff_factor(r, m.log_tab, h.kind, true, T, invT, lnT, exp2_51(l2rk), l2rk, M, false);
+      q *= falloff_factor(r, m.log_tab, h.kind, true, T, invT, lnT, fx.IT, exp2_51(l2rk), l2rk, M, false);
     }
   }
   return q;
@@ -146,18 +147,20 @@ __device__ __forceinline__ double lean_rate(const DevMech& m, const Rxn* __restr
 // acc(k) (this lane's production-rate accumulator of species k, not touched
 // where !act()), species(k, V, wk) for every k (the bath gas too), head(Tdot,
 // Sdot), invalid().  smem: source_smem_bytes; arrays: this block's
-// source_arrays_ws_doubles, or null with the arrays in shared memory.  Every
-// thread of the block calls it.
-template <int MODE, bool SPECIAL, class In, class Out>
+// source_arrays_ws_doubles, or null with the arrays in shared memory; AS: kShared
+// or kGlobal where that is known at compile time (shared-memory addressing in
+// place of generic loads), else kEither.  Every thread of the block calls it.
+enum ArraySpace { kShared, kGlobal, kEither };
+template <int MODE, bool SPECIAL, int AS, class In, class Out>
 __device__ __forceinline__ void source_tile(const DevMech& m, double* smem, double* arrays, const In& in,
                                             const Out& out) {
   const int ns = m.ns, bath = m.ns - 1, nr = m.nr;
   const int lane = threadIdx.x & 31, warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
   constexpr int W = kSrcWarps;
-  double* const base = (arrays ? arrays : smem) + lane;  // C then g, [2][ns][32]
+  double* const base = (AS == kShared ? smem : AS == kGlobal ? arrays : arrays ? arrays : smem) + lane;  // C then g, [2][ns][32]
   double* const C = base;
   double* const G = base + ns * kTile;
-  double* const qbuf = smem + (arrays ? 0 : 2 * ns * kTile) + lane;
+  double* const qbuf = smem + (AS == kGlobal || (AS == kEither && arrays) ? 0 : 2 * ns * kTile) + lane;
   double* const sc = qbuf + 2 * kGatherChunk * kTile;
   double* const part = sc + kSrcSc * kTile;
   int* const flags = reinterpret_cast<int*>(part - lane + kSrcPart * W * kTile) + lane;
@@ -194,6 +197,7 @@ __device__ __forceinline__ void source_tile(const DevMech& m, double* smem, doub
     S(zV) = V;
     S(zP) = P;
     S(zInvT) = invT;
+    S(zInvV) = 1.0 / V;
     S(zLnT) = lnT;
     S(zLnP) = m.has_pdep ? log(P) : 0.0;
     S(zCtot) = Ctot;
@@ -210,7 +214,7 @@ __device__ __forceinline__ void source_tile(const DevMech& m, double* smem, doub
 
   // B: concentrations and thermo of the warp's species
   {
-    const double T = S(zT), invT = S(zInvT), lnT = S(zLnT), cdum = S(zCdum), V = S(zV);
+    const double T = S(zT), invT = S(zInvT), lnT = S(zLnT), cdum = S(zCdum), V = S(zV), invV = S(zInvV);
     const bool ok0 = flags[gOk * kTile] != 0;
     double acc = 0.0, den = 0.0;
     bool fast = true;
@@ -220,7 +224,7 @@ __device__ __forceinline__ void source_tile(const DevMech& m, double* smem, doub
       G[k * kTile] = fixed_gibbs(m, g, fast);
       const double cx = MODE == PJ_CONP ? cp : cp - 1.0;
       if (k < bath) {
-        const double c = ok0 ? in.n(k) / V : cdum;
+        const double c = ok0 ? concentration(in.n(k), V, invV) : cdum;
         C[k * kTile] = c;
         acc += c;
         den = fma(c, cx, den);
