@@ -6,11 +6,11 @@
 // the L2 reductions at about the same (600 G reductions/s, 15.6 cycles per
 // warp instruction and SM), some 40 of which a reversible A + B = C + D
 // makes.  So everything that can leave the FP64 pipe has: the exponents, the
-// exponentials and the reaction enthalpy are integer fixed point, the
-// concentration derivative of R' = k prod C with respect to the volume is
-// -(number of factors) R', and an elementary reaction multiplies by no
-// pressure factor: 26 FP64 instructions (23 under constant volume, whose S
-// column such a reaction leaves alone) where the general path has 110.
+// exponentials and the reaction enthalpy are integer fixed point, the volume
+// derivative of R' = k prod C is -(number of factors) R', and an elementary
+// reaction multiplies by no pressure factor: 26 FP64 instructions (23 under
+// constant volume, whose S column such a reaction leaves alone) where the
+// general path has 110.
 #pragma once
 
 #include "kinetics_state.cuh"
@@ -71,47 +71,6 @@ __device__ __forceinline__ DT to_derivative(double x) {
   }
 }
 
-// One side's product R = k prod C and dR/dC_a in species order (f: factors
-// as packed in the head).
-struct LeanSide {
-  double R, d0, d1, d2;
-};
-__device__ __forceinline__ LeanSide lean_side(const int32_t (&f)[3], int shape, const double* __restrict__ C, double k) {
-  LeanSide s;
-  const double c0 = C[f[0]];
-  s.d1 = s.d2 = 0.0;
-  if (shape == SH_1) {
-    s.R = k * c0;
-    s.d0 = k;
-    return s;
-  }
-  const double t = k * c0;
-  const double c1 = C[f[1]];
-  if (shape == SH_11) {
-    s.R = t * c1;
-    s.d0 = t;
-    s.d1 = k * c1;
-    return s;
-  }
-  if (shape == SH_2) {
-    s.R = t * c1;
-    s.d0 = t + t;
-    return s;
-  }
-  const double c2 = C[f[2]];
-  const double t1 = t * c1;
-  s.R = t1 * c2;
-  if (shape == SH_21) {  // A B A
-    s.d0 = t1 + t1;
-    s.d1 = t * c2;
-  } else {               // C B A
-    s.d0 = t1;
-    s.d1 = t * c2;
-    s.d2 = (k * c2) * c1;
-  }
-  return s;
-}
-
 __device__ __forceinline__ int shape_species(int shape) { return shape <= SH_2 ? 1 : shape <= SH_21 ? 2 : 3; }
 
 // x with its sign bit flipped by a mask (0 or 0x80000000)
@@ -137,9 +96,25 @@ __device__ __forceinline__ void lean_jacobian(const DevMech& m, const Rxn* __res
   }
   const bool rev = h.rev != 0;
   const int64_t y = arrhenius_fixed(h.fA, h.fB, h.fT, v.fx.L, v.fx.IT);
-  const LeanSide sf = lean_side(h.f, a.shape[0], C, exp2_51(y));
-  LeanSide sb{0.0, 0.0, 0.0, 0.0};
-  if (rev) sb = lean_side(h.b, a.shape[1], C, exp2_51(y + lean_gibbs(h, G, v.fx.LP)));
+  const double kf = exp2_51(y);
+  double kr = 0.0;
+  if (rev) kr = exp2_51(y + lean_gibbs(h, G, v.fx.LP));
+  // both sides, the net rate and V dRn/dV at constant n, -(factors) R by side
+  LeanSide sf, sb;
+  double Rn, VS;
+  lean_shapes(h.code, [&](auto tf, auto tb) {
+    constexpr int SF = decltype(tf)::value, SB = decltype(tb)::value;
+    constexpr int nfac[5] = {1, 2, 2, 3, 3};
+    sf = lean_side<SF>(h.f, C, kf);
+    sb = lean_side<SB>(h.b, C, kr);
+    Rn = SB < 0 ? sf.R : sf.R - sb.R;
+    VS = 0.0;
+    if (MODE == PJ_CONP) {
+      constexpr int NF = nfac[SF], NB = SB < 0 ? NF : nfac[SB < 0 ? 0 : SB];
+      if (NF == NB) VS = NF == 1 ? dneg(Rn) : -(double)NF * Rn;
+      else VS = (NB == 1 ? sb.R : (double)NB * sb.R) - (NF == 1 ? sf.R : (double)NF * sf.R);
+    }
+  });
 
   // reaction enthalpy (internal energy) over RT, 2^51
   int64_t dh;
@@ -152,17 +127,13 @@ __device__ __forceinline__ void lean_jacobian(const DevMech& m, const Rxn* __res
     if (h.nb > 2) dh += hf(h.b[2]);
   }
   const double de = fixed51_to_double(dh - ((int64_t)h.dnu_i << 51));  // sum nu h/RT - dnu
-  const double dhd = MODE == PJ_CONP && h.dnu_i != 0 ? de + (double)h.dnu_i : de;
+  double dhd = de;
+  if (MODE == PJ_CONP && h.dnu_i != 0) dhd = fixed51_to_double(dh);
 
-  // net rate and its T derivative: T d ln kf/dT = beta + theta/T, T d ln kr/dT
-  // = that - sum nu u/RT; times V.  V dR/dV at constant n: -(factors) R.
+  // T derivative of the net rate: T d ln kf/dT = beta + theta/T, T d ln kr/dT
+  // = that - sum nu u/RT; times V
   const double Ef = fma(a.theta, v.invT, a.beta);
-  const double Rn = sf.R - sb.R;
   double VT = (sf.R * Ef - sb.R * (Ef - de)) * (v.V * v.invT);
-  double VS = 0.0;
-  if (MODE == PJ_CONP) {
-    VS = rev && !a.same ? a.nbx * sb.R - a.nfx * sf.R : -a.nfx * Rn;
-  }
   double Gb = 0.0;  // dRn/dC of the bath gas itself
   bool has_S = MODE == PJ_CONP;
   if (a.bath) {
@@ -173,12 +144,13 @@ __device__ __forceinline__ void lean_jacobian(const DevMech& m, const Rxn* __res
     if (a.bath & 16) Gb -= sb.d1;
     if (a.bath & 32) Gb -= sb.d2;
     VT = fma(Gb, v.V * v.dCb_T, VT);
+    if (MODE == PJ_CONP) VS = a.nbx * sb.R - a.nfx * sf.R;  // the bath gas's concentration is not n/V
     VS = fma(Gb, v.V * v.dCb_S, VS);
     has_S = true;
   }
 
   // pressure factor: scales the rate and every derivative
-  double c = 1.0, q = Rn;
+  double q = Rn;
   double RcM = 0.0;  // Rn dc/dM
   if (h.kind != PJ_ELEMENTARY) {
     double M = v.Ctot;
@@ -191,8 +163,7 @@ __device__ __forceinline__ void lean_jacobian(const DevMech& m, const Rxn* __res
     const double ab = __ldg(&r->alpha_bath);
     const double dMdT = ab * v.dCb_T;
     const double dMdS = MODE == PJ_CONP ? (ab * v.Ctot - M) * v.invV : ab * (v.Ctot / v.P);
-    double cT = dMdT;
-    c = M;
+    double cT = dMdT, c = M;
     RcM = Rn;
     if (h.kind != PJ_THIRD_BODY) {
       const int64_t l2rk = arrhenius_fixed(__ldg(&r->fA0), __ldg(&r->fB0), __ldg(&r->fT0), v.fx.L, v.fx.IT) - y;
@@ -206,6 +177,13 @@ __device__ __forceinline__ void lean_jacobian(const DevMech& m, const Rxn* __res
     VT = fma(c, VT, (Rn * cT) * v.V);
     VS = fma(c, VS, (RcM * dMdS) * v.V);
     has_S = true;
+    Gb *= c;
+    sf.d0 *= c;
+    sf.d1 *= c;
+    sf.d2 *= c;
+    sb.d0 *= c;
+    sb.d1 *= c;
+    sb.d2 *= c;
   }
 
   // energy- and state-row weights of this reaction
@@ -226,7 +204,6 @@ __device__ __forceinline__ void lean_jacobian(const DevMech& m, const Rxn* __res
   // Jacobian entries and production rates, by L2 reductions.  Addresses: an
   // entry's row of ld values, 32 x 32 -> 64 bit (the caller checks that ld
   // fits); up to four rows unrolled with their signs as masks.
-  const double Bbath = h.kind != PJ_ELEMENTARY ? c * Gb : Gb;
   DT B_t = DT(0);
   if (o.w) {
     const int32_t* __restrict__ tg = (FMT == PJ_CSR ? m.tgt_csr : m.tgt_csc) + a.tgt_lo;
@@ -267,16 +244,15 @@ __device__ __forceinline__ void lean_jacobian(const DevMech& m, const Rxn* __res
       tg += nrows + 2;
     };
     const int nsf = shape_species(a.shape[0]), nsb = rev ? shape_species(a.shape[1]) : 0;
-    auto scaled = [&](double d) { return to_derivative<DT>(h.kind != PJ_ELEMENTARY ? c * d : d); };
 #pragma unroll
     for (int s = 0; s < 3; s++) {
       if (s < nsf && !(a.bath >> s & 1))
-        slot(FMT == PJ_DENSE ? __ldg(&r->sp[s]) : 0, scaled(s == 0 ? sf.d0 : s == 1 ? sf.d1 : sf.d2));
+        slot(FMT == PJ_DENSE ? __ldg(&r->sp[s]) : 0, to_derivative<DT>(s == 0 ? sf.d0 : s == 1 ? sf.d1 : sf.d2));
       if (s < nsb && !(a.bath >> (3 + s) & 1))
         slot(FMT == PJ_DENSE ? __ldg(&r->sp[PJ_MAX_SP + s]) : 0,
-             dneg(scaled(s == 0 ? sb.d0 : s == 1 ? sb.d1 : sb.d2)));
+             dneg(to_derivative<DT>(s == 0 ? sb.d0 : s == 1 ? sb.d1 : sb.d2)));
     }
-    double Bi = -Bbath;  // minus the terms of the bath gas
+    double Bi = -Gb;  // minus the terms of the bath gas
     if (h.kind != PJ_ELEMENTARY) {
       for (int e = __ldg(&r->eff_lo), eh = __ldg(&r->eff_hi); e < eh; e++) {
         if (!PJ_DBG_OK(m.dbg, e >= 0 && e < m.n_eff, PJ_DBG_EFF)) break;

@@ -493,6 +493,7 @@ int mech_build(pj_mech* m) {
         for (int u = cnt; u >= 1 && u < 3; u++) out[u] = out[0];
         (side ? hd.nb : hd.nf) = (uint8_t)std::min(cnt, 3);
       }
+      if (hd.lean) hd.code = (uint8_t)(6 * r.shape[0] + (r.rev ? 1 + r.shape[1] : 0));
     }
     std::vector<double> al = alpha_of(m, i);
     r.alpha_bath = has_third_body(r.kind) ? al[bath] : 1.0;
@@ -535,7 +536,6 @@ int mech_build(pj_mech* m) {
           else (side ? j.nbx : j.nfx) += r.nu[at];
         }
       }
-      j.same = j.nfx == j.nbx ? 1 : 0;
     }
     r.bath_in = 0;
     for (int a = 0; a < 2 * PJ_MAX_SP; a++) r.bath_in |= r.sp[a] == bath && (a % PJ_MAX_SP) < (a < PJ_MAX_SP ? r.nreac : r.nprod);

@@ -51,7 +51,7 @@ struct alignas(16) RxnHead {
                                   // beta 2^56, -theta log2(e) 2^45
   int32_t dnu_i;                  // dnu as an integer
   uint8_t lean, kind, rev, nf;    // nf, nb: factors of the forward and the reverse product (1 to 3)
-  uint8_t nb, pad0, pad1, pad2;
+  uint8_t nb, code, pad1, pad2;   // code: 6 SH_* of the forward side + (rev ? 1 + SH_* of the reverse : 0)
   int32_t f[3], b[3];             // 32 x species index of each factor (unused ones repeat the first)
   int32_t pad3;
 };
@@ -63,7 +63,7 @@ struct alignas(16) RxnJac {
   uint8_t nrows, neg;             // rows; bit q set: row q's coefficient is -1
   uint8_t shape[2];               // SH_* of the forward and the reverse side
   uint8_t bath, dense;            // bit a / 3 + a: reactant a / product a is the bath gas; Rxn::dense
-  uint8_t same, pad0;             // same: nfx == nbx
+  uint8_t pad0, pad1;
   double nfx, nbx;                // factors that are not the bath gas, by side
   uint16_t k[4];                  // species of the first four rows
 };

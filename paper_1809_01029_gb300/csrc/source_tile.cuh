@@ -109,12 +109,59 @@ __device__ __forceinline__ int64_t lean_gibbs(const RxnHead& h, const double* __
   return s;
 }
 
-// k times the concentrations of a side
-__device__ __forceinline__ double lean_product(const int32_t (&f)[3], int n, const double* __restrict__ C, double k) {
-  double r = k * C[f[0]];
-  if (n > 1) r *= C[f[1]];
-  if (n > 2) r *= C[f[2]];
-  return r;
+// One side's product R = k prod C and dR/dC_a in species order (f: factors
+// as packed in the head; unused derivatives are left 0).
+struct LeanSide {
+  double R, d0, d1, d2;
+};
+template <int SHAPE>
+__device__ __forceinline__ LeanSide lean_side(const int32_t (&f)[3], const double* __restrict__ C, double k) {
+  LeanSide s{0.0, 0.0, 0.0, 0.0};
+  if constexpr (SHAPE < 0) return s;
+  const double c0 = C[f[0]];
+  if constexpr (SHAPE == SH_1) {
+    s.R = k * c0;
+    s.d0 = k;
+  } else if constexpr (SHAPE == SH_11 || SHAPE == SH_2) {
+    const double t = k * c0, c1 = C[f[1]];
+    s.R = t * c1;
+    s.d0 = SHAPE == SH_2 ? t + t : t;
+    if (SHAPE == SH_11) s.d1 = k * c1;
+  } else if constexpr (SHAPE >= 0) {
+    const double t = k * c0, c1 = C[f[1]], c2 = C[f[2]];
+    const double t1 = t * c1;
+    s.R = t1 * c2;
+    s.d0 = SHAPE == SH_21 ? t1 + t1 : t1;  // 2A + B as A B A, A + B + C as C B A
+    s.d1 = t * c2;
+    if (SHAPE == SH_111) s.d2 = (k * c2) * c1;
+  }
+  return s;
+}
+
+// f(forward shape, reverse shape or -1) with the shapes of a head's code as
+// compile-time constants.  A jump table: under conditions of its own each
+// shape's few FP64 instructions would be predicated, and the FP64 pipe
+// charges a predicated-off warp instruction like any other (20 of the 63 a
+// 53-species Jacobian reaction issued).
+template <int V>
+struct IntTag {
+  static constexpr int value = V;
+};
+template <class F>
+__device__ __forceinline__ void lean_shapes(int code, F&& f) {
+  switch (code) {
+#define PJ_SHAPE(sf, sb) \
+  case 6 * (sf) + 1 + (sb): f(IntTag<sf>{}, IntTag<sb>{}); break;
+#define PJ_SHAPES(sf) PJ_SHAPE(sf, -1) PJ_SHAPE(sf, 0) PJ_SHAPE(sf, 1) PJ_SHAPE(sf, 2) PJ_SHAPE(sf, 3) PJ_SHAPE(sf, 4)
+    PJ_SHAPES(0)
+    PJ_SHAPES(1)
+    PJ_SHAPES(2)
+    PJ_SHAPES(3)
+    PJ_SHAPES(4)
+#undef PJ_SHAPES
+#undef PJ_SHAPE
+    default: break;
+  }
 }
 
 // Net rate of reaction i at this lane's state, short path: every state of
@@ -123,8 +170,13 @@ __device__ __forceinline__ double lean_rate(const DevMech& m, const Rxn* __restr
                                             const double* __restrict__ C, const double* __restrict__ G,
                                             const FixedState& fx, double T, double invT, double lnT, double Ctot) {
   const int64_t y = arrhenius_fixed(h.fA, h.fB, h.fT, fx.L, fx.IT);
-  double q = lean_product(h.f, h.nf, C, exp2_51(y));
-  if (h.rev) q -= lean_product(h.b, h.nb, C, exp2_51(y + lean_gibbs(h, G, fx.LP)));
+  const double kf = exp2_51(y);
+  double kr = 0.0, q = 0.0;
+  if (h.rev) kr = exp2_51(y + lean_gibbs(h, G, fx.LP));
+  lean_shapes(h.code, [&](auto sf, auto sb) {
+    q = lean_side<decltype(sf)::value>(h.f, C, kf).R;
+    if (decltype(sb)::value >= 0) q -= lean_side<decltype(sb)::value>(h.b, C, kr).R;
+  });
   if (h.kind != PJ_ELEMENTARY) {
     double M = Ctot;
     for (int e = __ldg(&r->eff_lo), eh = __ldg(&r->eff_hi); e < eh; e++) {
