@@ -53,6 +53,18 @@ __device__ __noinline__ static FalloffC falloff_derivatives(const Rxn* __restric
   return FalloffC{fr * F, cPr * rk, fr * FT + cPr * (Pr * dlnrk + rk * dMdT)};
 }
 
+// sum nu h/RT - d over a short-path reaction's factors; H: this lane's h_k/RT
+// (fixed_enthalpy), 32 words per species
+__device__ __forceinline__ double lean_energy(const RxnHead& h, const double* __restrict__ H, int d) {
+  auto hf = [&](int off) { return __double_as_longlong(H[off]); };
+  int64_t s = hf(h.b[0]) - hf(h.f[0]) - ((int64_t)d << 51);
+  if (h.nf > 1) s -= hf(h.f[1]);
+  if (h.nb > 1) s += hf(h.b[1]);
+  if (h.nf > 2) s -= hf(h.f[2]);
+  if (h.nb > 2) s += hf(h.b[2]);
+  return fixed51_to_double(s);
+}
+
 // x in the derivative type.  To FP32 in integer instructions (the hardware
 // conversion takes an FP64-pipe slot): rounded to nearest, flushed to zero
 // below 2^-126, infinite beyond FP32's range.
@@ -116,24 +128,14 @@ __device__ __forceinline__ void lean_jacobian(const DevMech& m, const Rxn* __res
     }
   });
 
-  // reaction enthalpy (internal energy) over RT, 2^51
-  int64_t dh;
-  {
-    auto hf = [&](int off) { return __double_as_longlong(H[off]); };
-    dh = hf(h.b[0]) - hf(h.f[0]);
-    if (h.nf > 1) dh -= hf(h.f[1]);
-    if (h.nb > 1) dh += hf(h.b[1]);
-    if (h.nf > 2) dh -= hf(h.f[2]);
-    if (h.nb > 2) dh += hf(h.b[2]);
-  }
-  const double de = fixed51_to_double(dh - ((int64_t)h.dnu_i << 51));  // sum nu h/RT - dnu
+  const double de = lean_energy(h, H, h.dnu_i);  // sum nu h/RT - dnu
   double dhd = de;
-  if (MODE == PJ_CONP && h.dnu_i != 0) dhd = fixed51_to_double(dh);
+  if (MODE == PJ_CONP && h.dnu_i != 0) dhd = lean_energy(h, H, 0);
 
-  // T derivative of the net rate: T d ln kf/dT = beta + theta/T, T d ln kr/dT
-  // = that - sum nu u/RT; times V
+  // T derivative of the net rate: T d ln kf/dT = Ef = beta + theta/T, T d ln
+  // kr/dT = Ef - de, so T dRn/dT = Rn Ef + Rr de; times V
   const double Ef = fma(a.theta, v.invT, a.beta);
-  double VT = (sf.R * Ef - sb.R * (Ef - de)) * (v.V * v.invT);
+  double VT = fma(sb.R, de, Rn * Ef) * (v.V * v.invT);
   double Gb = 0.0;  // dRn/dC of the bath gas itself
   bool has_S = MODE == PJ_CONP;
   if (a.bath) {
