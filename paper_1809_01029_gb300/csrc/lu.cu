@@ -27,6 +27,7 @@
 #include <algorithm>
 #include <cstdlib>
 #include <cstring>
+#include <type_traits>
 
 #include "kinetics_device.cuh"
 #include "launch.h"
@@ -114,6 +115,15 @@ __device__ __forceinline__ float2 v_mul(float2 a, float2 b) {
 template <>
 __device__ __forceinline__ float4 v_mul(float4 a, float4 b) {
   return make_float4(a.x * b.x, a.y * b.y, a.z * b.z, a.w * b.w);
+}
+
+// bytes of a factorisation's lists in shared memory, and of the lists with
+// their row starts
+__host__ __device__ constexpr size_t lu_list_bytes(int n_ridx, int n_cidx) {
+  return ((size_t)n_ridx + (size_t)n_cidx + 1) & ~(size_t)1;
+}
+static size_t lu_lists_smem(const DevLu& L) {
+  return lu_list_bytes(L.n_ridx, L.n_cidx) + (size_t)2 * (L.N + 1) * sizeof(uint16_t);
 }
 
 // vals: CSR values of M (FROM_J = false) or of J (FROM_J: M = I - h gamma J
@@ -262,7 +272,12 @@ __global__ void __launch_bounds__(256) k_lu_factor(DevLu L, int64_t n, const T* 
 // pattern is closed under elimination, so rows(k+1) holds every row of
 // rows(k) but k+1 and no entry of the column changes after pivot k -- while
 // the other warps update the pairs of every other column.
-template <typename T, int S, bool FROM_J>
+//
+// LISTS: the per-pivot lists of column rows and row columns sit in shared
+// memory as bytes (N <= 255) behind the matrices.  From global memory they
+// come from L2 where the matrices leave L1 no room (111 species FP32: 26 of
+// 228 KB), in every pivot's serial chain.
+template <typename T, int S, bool FROM_J, bool LISTS>
 __global__ void __launch_bounds__(256) k_lu_factor_v(DevLu L, int64_t n, const T* __restrict__ vals, int64_t ld,
                                                      const double* __restrict__ hstep, double gamma,
                                                      T* __restrict__ lu, int* status) {
@@ -272,6 +287,20 @@ __global__ void __launch_bounds__(256) k_lu_factor_v(DevLu L, int64_t n, const T
   const int N = L.N, NP = L.NP, tid = threadIdx.x, nt = blockDim.x;
   const int lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
   const int NN = N * NP;
+  uint8_t* const s_list = reinterpret_cast<uint8_t*>(A + (size_t)NN);           // ridx then cidx
+  uint16_t* const s_ptr = reinterpret_cast<uint16_t*>(s_list + (LISTS ? lu_list_bytes(L.n_ridx, L.n_cidx) : 0));
+  if (LISTS) {
+    for (int t = tid; t < L.n_ridx; t += nt) s_list[t] = (uint8_t)__ldg(L.ridx + t);
+    for (int t = tid; t < L.n_cidx; t += nt) s_list[L.n_ridx + t] = (uint8_t)__ldg(L.cidx + t);
+    for (int t = tid; t <= N; t += nt) {
+      s_ptr[t] = (uint16_t)__ldg(L.rptr + t);
+      s_ptr[N + 1 + t] = (uint16_t)__ldg(L.cptr + t);
+    }
+  }
+  auto rptr = [&](int k) -> int { return LISTS ? s_ptr[k] : __ldg(L.rptr + k); };
+  auto cptr = [&](int k) -> int { return LISTS ? s_ptr[N + 1 + k] : __ldg(L.cptr + k); };
+  auto ridx = [&](int t) -> int { return LISTS ? s_list[t] : __ldg(L.ridx + t); };
+  auto cidx = [&](int t) -> int { return LISTS ? s_list[L.n_ridx + t] : __ldg(L.cidx + t); };
   __shared__ int bad[S];
   __shared__ V s_inv;
   __shared__ T s_hg[S];
@@ -289,9 +318,9 @@ __global__ void __launch_bounds__(256) k_lu_factor_v(DevLu L, int64_t n, const T
     }
     __syncwarp();
     const V inv = s_inv;
-    const int r0 = __ldg(L.rptr + c), nr = __ldg(L.rptr + c + 1) - r0;
+    const int r0 = rptr(c), nr = rptr(c + 1) - r0;
     for (int a = lane; a < nr; a += 32) {
-      const int i = __ldg(L.ridx + r0 + a);
+      const int i = ridx(r0 + a);
       A[i * NP + c] = v_mul(A[i * NP + c], inv);
     }
   };
@@ -323,15 +352,15 @@ __global__ void __launch_bounds__(256) k_lu_factor_v(DevLu L, int64_t n, const T
     if (warp == 0) finish_column(0);
     __syncthreads();
     for (int k = 0; k < N - 1; k++) {
-      const int r0 = __ldg(L.rptr + k), nr = __ldg(L.rptr + k + 1) - r0;
-      const int c0 = __ldg(L.cptr + k), nc = __ldg(L.cptr + k + 1) - c0;
+      const int r0 = rptr(k), nr = rptr(k + 1) - r0;
+      const int c0 = cptr(k), nc = cptr(k + 1) - c0;
       // column k+1 is cols(k)[0] when pivot k changes it (columns ascend)
-      const int j0 = nc > 0 && __ldg(L.cidx + c0) == k + 1 ? 1 : 0;
+      const int j0 = nc > 0 && cidx(c0) == k + 1 ? 1 : 0;
       if (warp == 0) {
         if (j0) {
           const V u = A[k * NP + k + 1];
           for (int a = lane; a < nr; a += 32) {
-            const int i = __ldg(L.ridx + r0 + a);
+            const int i = ridx(r0 + a);
             A[i * NP + k + 1] = v_fms(A[i * NP + k], u, A[i * NP + k + 1]);
           }
           __syncwarp();
@@ -354,15 +383,15 @@ __global__ void __launch_bounds__(256) k_lu_factor_v(DevLu L, int64_t n, const T
               ia++;
             }
           };
-          const int* __restrict__ ci = L.cidx + c0 + j0;
+          const int cb = c0 + j0;
           for (; p + 3 * ntw < tot; p += 4 * ntw) {
-            const int i0 = __ldg(L.ridx + r0 + ia), jj0 = __ldg(ci + jc);
+            const int i0 = ridx(r0 + ia), jj0 = cidx(cb + jc);
             step();
-            const int i1 = __ldg(L.ridx + r0 + ia), jj1 = __ldg(ci + jc);
+            const int i1 = ridx(r0 + ia), jj1 = cidx(cb + jc);
             step();
-            const int i2 = __ldg(L.ridx + r0 + ia), jj2 = __ldg(ci + jc);
+            const int i2 = ridx(r0 + ia), jj2 = cidx(cb + jc);
             step();
-            const int i3 = __ldg(L.ridx + r0 + ia), jj3 = __ldg(ci + jc);
+            const int i3 = ridx(r0 + ia), jj3 = cidx(cb + jc);
             step();
             const V l0 = A[i0 * NP + k], l1 = A[i1 * NP + k], l2 = A[i2 * NP + k], l3 = A[i3 * NP + k];
             const V u0 = A[k * NP + jj0], u1 = A[k * NP + jj1], u2 = A[k * NP + jj2], u3 = A[k * NP + jj3];
@@ -373,7 +402,7 @@ __global__ void __launch_bounds__(256) k_lu_factor_v(DevLu L, int64_t n, const T
             A[i3 * NP + jj3] = v_fms(l3, u3, v3);
           }
           for (; p < tot; p += ntw) {
-            const int i = __ldg(L.ridx + r0 + ia), j = __ldg(ci + jc);
+            const int i = ridx(r0 + ia), j = cidx(cb + jc);
             A[i * NP + j] = v_fms(A[i * NP + k], A[k * NP + j], A[i * NP + j]);
             step();
           }
@@ -518,18 +547,29 @@ static int launch_factor_t(const DevLu& L, int64_t n, const void* vals, int64_t 
   T* gws = p.smem ? nullptr : static_cast<T*>(work);
   int rc;
   if (p.smem) {
+    // the lists in shared memory where they leave the blocks per SM as they are
+    const size_t with_lists = p.dyn + lu_lists_smem(L);
+    const size_t per_sm = kSmemPerSm / (p.dyn + 1024 + 256), per_sm_l = kSmemPerSm / (with_lists + 1024 + 256);
+    const bool lists = L.N <= 255 && L.n_ridx <= 65535 && L.n_cidx <= 65535 && with_lists <= kSmemCap &&
+                       std::min<size_t>(16, per_sm) == std::min<size_t>(16, per_sm_l);
+    const size_t dyn = lists ? with_lists : p.dyn;
     auto pick = [&](auto kern) -> int {
       int r;
-      if ((r = set_smem(kern, p.dyn))) return r;
-      kern<<<p.grid, p.threads, p.dyn, st>>>(L, n, static_cast<const T*>(vals), ld, hstep, gamma,
+      if ((r = set_smem(kern, dyn))) return r;
+      kern<<<p.grid, p.threads, dyn, st>>>(L, n, static_cast<const T*>(vals), ld, hstep, gamma,
                                              static_cast<T*>(lu), status);
       return check_cuda(cudaGetLastError(), "k_lu_factor_v launch");
     };
+    auto pick_s = [&](auto tag) -> int {
+      constexpr int SS = decltype(tag)::value;
+      if (lists) return hstep ? pick(k_lu_factor_v<T, SS, true, true>) : pick(k_lu_factor_v<T, SS, false, true>);
+      return hstep ? pick(k_lu_factor_v<T, SS, true, false>) : pick(k_lu_factor_v<T, SS, false, false>);
+    };
     if constexpr (sizeof(T) == 4) {
-      if (p.S == 4) return hstep ? pick(k_lu_factor_v<T, 4, true>) : pick(k_lu_factor_v<T, 4, false>);
+      if (p.S == 4) return pick_s(std::integral_constant<int, 4>{});
     }
-    if (p.S == 2) return hstep ? pick(k_lu_factor_v<T, 2, true>) : pick(k_lu_factor_v<T, 2, false>);
-    return hstep ? pick(k_lu_factor_v<T, 1, true>) : pick(k_lu_factor_v<T, 1, false>);
+    if (p.S == 2) return pick_s(std::integral_constant<int, 2>{});
+    return pick_s(std::integral_constant<int, 1>{});
   }
   if (hstep) {
     auto kern = k_lu_factor<T, true>;

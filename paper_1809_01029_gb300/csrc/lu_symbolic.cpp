@@ -159,6 +159,8 @@ int lu_build(pj_mech* m) {
   L.nnz = m->nnz;
   L.lu_nnz = lu_nnz;
   L.nl = nl;
+  L.n_ridx = (int32_t)ridx.size();
+  L.n_cidx = (int32_t)cidx.size();
   if (m->device < 0) return PJ_OK;
 
   // one device allocation for the tables

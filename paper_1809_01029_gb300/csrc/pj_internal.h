@@ -151,6 +151,7 @@ struct DevMech {
 // order k, dense pivot-order positions r*N + c.
 struct DevLu {
   int32_t N, nnz, lu_nnz, nl;  // nnz: CSR entries of M; nl: strictly lower factor entries
+  int32_t n_ridx, n_cidx;      // lengths of ridx, cidx
   int32_t NP;                  // row stride of the dense pivot-order arrays (N rounded up to odd)
   const int32_t* perm;         // [N] state-vector index of pivot k
   const int32_t* rptr;         // [N+1] rows i > k of column k ...
