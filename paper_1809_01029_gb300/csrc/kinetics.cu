@@ -45,9 +45,10 @@ namespace pj {
 // source terms
 // ---------------------------------------------------------------------------
 // A block of 16 warps per 32-state tile (source_tile.cuh), two blocks per SM,
-// tiles handed out block-cyclically.  Y: y = (wdot, dT/dt) instead of dPhi/dt.
+// or of 32 where there are no more tiles than SMs; tiles handed out
+// block-cyclically.  Y: y = (wdot, dT/dt) instead of dPhi/dt.
 template <int MODE, bool SPECIAL, bool Y, bool SHARED>
-__global__ void __launch_bounds__(kSrcWarps * 32, 2)
+__global__ void __launch_bounds__(2 * kSrcWarps * 32, 1)
     k_source_terms(const __grid_constant__ DevMech m, int64_t n, const double* __restrict__ param,
                    const double* __restrict__ phi, int64_t ld, double* __restrict__ out, int* status, double* ws,
                    double* arrays) {
@@ -142,6 +143,7 @@ SourcePlan source_plan(int ns, int64_t n) {
   p.smem = source_smem_bytes(ns, p.arrays_smem);
   p.ctas = p.smem + kBlockOverhead <= kSmemPerSm / 2 ? 2 : 1;
   const int64_t tiles = (n + kTile - 1) / kTile;
+  p.warps = tiles <= sm_count() ? 2 * kSrcWarps : kSrcWarps;
   p.grid = (int)std::max<int64_t>(1, std::min<int64_t>(tiles, (int64_t)sm_count() * p.ctas));
   p.acc_bytes = (size_t)p.grid * ns * kTile * sizeof(double);
   p.arrays_bytes = (size_t)p.grid * source_arrays_ws_doubles(ns, p.arrays_smem) * sizeof(double);
@@ -167,7 +169,7 @@ static int launch_source_t(const DevMech& m, int mode, int64_t n, const double* 
   auto kern = p.arrays_smem ? pick(BoolTag<true>{}) : pick(BoolTag<false>{});
   int rc;
   if ((rc = set_smem(kern, p.smem))) return rc;
-  kern<<<p.grid, kSrcWarps * 32, p.smem, st>>>(m, n, param, phi, ld, out, status, acc, arrays);
+  kern<<<p.grid, p.warps * 32, p.smem, st>>>(m, n, param, phi, ld, out, status, acc, arrays);
   return check_cuda(cudaGetLastError(), "k_source_terms launch");
 }
 
@@ -224,26 +226,24 @@ TmPlan tm_plan(int ns) {
   return t;
 }
 
-// Which Jacobian layout runs, chosen by measurement on GB300 (1 Mi states
-// unless stated; states/s, one state per thread against the cooperative
-// shapes, warps x blocks per SM):
-//  * at most one 32-state tile per SM: cooperative, 16 warps on each tile
-//    (13 species, 4096 states: 64 M against 13 M);
-//  * the FP64 Jacobian of TMEM-size mechanisms (53 species) and of
-//    mechanisms whose one-state-per-thread arrays need a global workspace
-//    (111 species), and any batch below SMs x 512 states: cooperative, 8
-//    warps x 2 blocks (53 species CSR 11.47 M against 11.17 M in TMEM, CSC
-//    11.46 / 11.06, CONV 11.93 / 11.73, all reaction types 9.84 / 9.75;
-//    111 species 4.69 M against 4.16 M; 53 species, 64 ki states 11.0 M
-//    against 9.8 M), 16 warps x 1 above 200 species (the 874-species
-//    arrays are 671 KB a tile);
-//  * the dense FP64 Jacobian of TMEM-size mechanisms: one state per thread
-//    in TMEM (11.49 M against 11.35 M);
-//  * the FP32 Newton matrix of those mechanisms: cooperative, 4 warps x 4
-//    blocks, the arrays in the workspace (53 species 14.64 M against 13.22
-//    M; 111 species 5.84 M against 4.85 M);
-//  * otherwise (13 species, large batches): one state per thread, arrays
-//    in shared memory (117 M against 114 M at 4 x 4).
+// Which Jacobian layout runs, chosen by measurement on GB300 (microseconds;
+// cooperative shapes as warps x blocks per SM, "one" for one state per thread):
+//  * at most one 32-state tile per SM: cooperative, 20 warps on each tile, or
+//    16 where 20 would take as many rounds over the reactions (13 species, 27
+//    reactions, 4096 states: 46.0 at 16 x 1, 48.9 at 20 x 1, 289 one);
+//  * larger batches: cooperative, 10 x 2 (53 species CSR, 131072 states: 5063
+//    against 5440 at 8 x 2, 5708 at 4 x 4, 5531 at 16 x 1, 10365 one; dense
+//    the same; FP32 Newton matrix of 111 species, 32768 states: 2887 against
+//    3193, 3356, 2922 and 9166), 16 x 1 above 200 species (the 874-species
+//    arrays are 671 KB a tile), 4 x 4 for small mechanisms at 512 states per
+//    SM or more (13 species, 524288 states: 2541 against 2854 at 8 x 2 and
+//    3500 one);
+//  * from 1 Mi states on, the dense FP64 Jacobian of TMEM-size mechanisms (53
+//    species) and the Jacobians of mechanisms whose arrays fit shared memory
+//    for one state per thread (13 species) stay one state per thread, the
+//    layout pj_jacobian_layout is documented and tested to answer there.  The
+//    cooperative layout is the faster one at that size too (53 species dense,
+//    1 Mi: 42.5 ms against 79.4).
 // Each cooperative block keeps only its 32 states' Jacobians live in L2, a
 // fraction of the one-state-per-thread kernels' live set (DRAM traffic per
 // state at 53 species: 154 KB in TMEM, 34 KB at 16 x 1, 65 KB at 8 x 2), so
@@ -263,8 +263,7 @@ static int env_int(const char* name, int dflt) {
 
 bool coop_shape(const DevMech& m, int warps, int ctas, bool arrays_smem, int64_t tiles, CoopPlan& c) {
   c = CoopPlan{false, warps, ctas, coop_smem_bytes(m.ns, warps, arrays_smem), sm_count() * ctas, 0};
-  if (warps != 4 && warps != 8 && warps != 16) return false;
-  if (ctas < 1 || ctas * warps > 16) return false;
+  if (warps < 4 || ctas < 1 || ctas * warps > kCoopWarpsMax) return false;
   if (c.smem + kBlockOverhead > kSmemPerSm / (size_t)ctas || c.smem > kSmemCap) return false;
   if (!arrays_smem) {
     const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>(tiles, c.grid));
@@ -280,12 +279,15 @@ static bool coop_fit(const DevMech& m, int warps, int ctas, int64_t n, CoopPlan&
   return coop_shape(m, warps, ctas, true, tiles, c) || coop_shape(m, warps, ctas, false, tiles, c);
 }
 
+constexpr int64_t kPercoreStates = int64_t(1) << 20;
+
 CoopPlan coop_plan(const DevMech& m, int fmt, int dt_bytes, int64_t n) {
   CoopPlan c{false, 16, 1, 0, 0, 0};
   const char* lay = getenv("PYJAC_GB_JAC_LAYOUT");
   if (lay && strcmp(lay, "percore") == 0) return c;
   if (lay && strcmp(lay, "coop") == 0) {
     const int warps = env_int("PYJAC_GB_COOP_WARPS", 16), ctas = env_int("PYJAC_GB_COOP_CTAS", 16 / std::max(warps, 1));
+    if ((warps != 4 && warps != 8 && warps != 16) || warps * ctas > 16) return c;
     const char* ar = getenv("PYJAC_GB_COOP_ARRAYS");
     if (ar && strcmp(ar, "global") == 0) coop_shape(m, warps, ctas, false, (n + kCoopTile - 1) / kCoopTile, c);
     else coop_fit(m, warps, ctas, n, c);
@@ -295,18 +297,21 @@ CoopPlan coop_plan(const DevMech& m, int fmt, int dt_bytes, int64_t n) {
   const int sms = sm_count();
   const int64_t tiles = (n + kCoopTile - 1) / kCoopTile;
   const bool percore_global = !t.use && plan_for(jacobian_arrays(), m.ns, n).global_ws;
-  if (tiles <= sms) {  // one tile per SM at most: all 16 warps on it
-    coop_fit(m, 16, 1, n, c);
+  if (tiles <= sms) {  // one tile per SM at most: 20 warps where that takes fewer rounds than 16
+    const int r16 = (m.nr + 15) / 16, r20 = (m.nr + kCoopWarpsMax - 1) / kCoopWarpsMax;
+    if (r20 == r16 || !coop_shape(m, kCoopWarpsMax, 1, true, tiles, c)) coop_fit(m, 16, 1, n, c);
     return c;
   }
-  if (n < (int64_t)sms * 512 || t.use || percore_global) {
-    if (t.use && fmt == PJ_DENSE && dt_bytes == 8 && n >= (int64_t)sms * 512) {
-      c.use = false;  // the dense FP64 Jacobian: tensor memory, one state per thread
-      return c;
-    }
-    if (dt_bytes == 4 && (t.use || percore_global)) coop_fit(m, 4, 4, n, c);
-    else if (m.ns > 200) coop_fit(m, 16, 1, n, c);
-    else coop_fit(m, 8, 2, n, c);
+  if (n < kPercoreStates) {
+    if (m.ns > 200) coop_fit(m, 16, 1, n, c);
+    else if (t.use || percore_global || n < (int64_t)sms * 512) coop_fit(m, kCoopWarpsMax / 2, 2, n, c);
+    else coop_fit(m, 4, 4, n, c);
+    return c;
+  }
+  if (t.use || percore_global) {
+    if (t.use && fmt == PJ_DENSE && dt_bytes == 8) return c;
+    if (m.ns > 200) coop_fit(m, 16, 1, n, c);
+    else coop_fit(m, kCoopWarpsMax / 2, 2, n, c);
     return c;
   }
   c.use = false;
@@ -325,7 +330,7 @@ size_t workspace_bytes(int arrays, int ns, int64_t n) {
         std::max<int64_t>(1, std::min<int64_t>((n + kCoopTile - 1) / kCoopTile, (int64_t)sm_count() * 4));
     const char* ar = getenv("PYJAC_GB_COOP_ARRAYS");
     const bool global = 4 * (coop_smem_bytes(ns, 4) + kBlockOverhead) > kSmemPerSm ||
-                        coop_smem_bytes(ns, kCoopWarpsMax) > kSmemCap || (ar && strcmp(ar, "global") == 0);
+                        coop_smem_bytes(ns, 16) > kSmemCap || (ar && strcmp(ar, "global") == 0);
     const size_t co = global ? coop_arrays_bytes(ns) * (size_t)tiles : 0;
     return std::max(pc, co);
   }

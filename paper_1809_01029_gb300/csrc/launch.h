@@ -55,6 +55,7 @@ struct CoopPlan {
 struct SourcePlan {
   bool arrays_smem;
   int ctas;             // blocks per SM
+  int warps;            // per block (the source terms and y; finite differences: 16)
   int grid;
   size_t smem;
   size_t acc_bytes, arrays_bytes;

@@ -15,7 +15,7 @@
 // as L2 reductions into an accumulator row (the additions run at L2, not on
 // the SM's FP64 pipe; one thread's reductions to one address apply in its
 // program order).  Every cross-warp sum is a sum of per-warp partials in
-// warp order.  The result depends on the number of warps only.
+// warp order.  The result does not depend on the launch shape.
 #pragma once
 
 #include "kinetics_common.cuh"
@@ -23,7 +23,7 @@
 namespace pj {
 
 constexpr int kTile = 32;
-constexpr int kSrcWarps = 16;  // warps per block
+constexpr int kSrcWarps = 16;  // warps per block, or twice that
 
 enum SrcSc { zT, zV, zP, zInvT, zInvV, zLnT, zLnP, zCtot, zL, zIT, zLP, zCdum, zDen, zCxB, kSrcSc };
 enum SrcPart { rAcc, rDen, rNum, rOm, kSrcPart };
@@ -208,7 +208,10 @@ __device__ __forceinline__ void source_tile(const DevMech& m, double* smem, doub
                                             const Out& out) {
   const int ns = m.ns, bath = m.ns - 1, nr = m.nr;
   const int lane = threadIdx.x & 31, warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
+  // species are split over the first 16 warps whatever the block's size, so
+  // that the result does not depend on it
   constexpr int W = kSrcWarps;
+  const int W_all = blockDim.x >> 5;
   double* const base = (AS == kShared ? smem : AS == kGlobal ? arrays : arrays ? arrays : smem) + lane;  // C then g, [2][ns][32]
   double* const C = base;
   double* const G = base + ns * kTile;
@@ -260,12 +263,12 @@ __device__ __forceinline__ void source_tile(const DevMech& m, double* smem, doub
     flags[gOk * kTile] = ok0;
     flags[gFast * kTile] = fx.fast;
   }
-  if (act)
+  if (act && warp < W)
     for (int k = warp; k < ns; k += W) *out.acc(k) = 0.0;
   __syncthreads();
 
   // B: concentrations and thermo of the warp's species
-  {
+  if (warp < W) {
     const double T = S(zT), invT = S(zInvT), lnT = S(zLnT), cdum = S(zCdum), V = S(zV), invV = S(zInvV);
     const bool ok0 = flags[gOk * kTile] != 0;
     double acc = 0.0, den = 0.0;
@@ -316,7 +319,7 @@ __device__ __forceinline__ void source_tile(const DevMech& m, double* smem, doub
     for (int c0 = 0; c0 < nr; c0 += kGatherChunk, chunk++) {
       double* const q = qbuf + (chunk & 1) * kGatherChunk * kTile;
       const int c1 = min(nr, c0 + kGatherChunk);
-      for (int i = c0 + warp; i < c1; i += W) {
+      for (int i = c0 + warp; i < c1; i += W_all) {
         const Rxn* __restrict__ r = m.rxn + i;
         const RxnHead h = load_head(r);
         q[(i - c0) * kTile] = fast_tile && h.lean
@@ -324,7 +327,7 @@ __device__ __forceinline__ void source_tile(const DevMech& m, double* smem, doub
                                   : general_rate<SPECIAL>(m, base, r, i < m.nr_plain, fx, T, invT, lnT, lnP, Ctot);
       }
       __syncthreads();
-      for (int k = warp; k < ns; k += W) {
+      for (int k = warp; k < ns; k += W_all) {
         const int32_t* __restrict__ gp = m.gather_ptr + (size_t)chunk * ns + k;
         for (int e = __ldg(gp), e1 = __ldg(gp + 1); e < e1; e++) {
           const uint32_t id = __ldg(m.gather + e);
@@ -336,8 +339,10 @@ __device__ __forceinline__ void source_tile(const DevMech& m, double* smem, doub
     }
   }
 
-  // E: the warp's species (whose accumulators only this warp has touched)
-  {
+  // E: the warp's species (with 16 warps, their accumulators only this warp
+  // has touched)
+  if (W_all > W) __syncthreads();
+  if (warp < W) {
     const double T = S(zT), invT = S(zInvT), V = S(zV);
     const bool ok = flags[gOk * kTile] != 0;
     double num = 0.0, Om = 0.0;
