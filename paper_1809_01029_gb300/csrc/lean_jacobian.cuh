@@ -67,19 +67,20 @@ __device__ __forceinline__ double lean_energy(const RxnHead& h, const double* __
 
 // x in the derivative type.  To FP32 in integer instructions (the hardware
 // conversion takes an FP64-pipe slot): rounded to nearest, flushed to zero
-// below 2^-126, infinite beyond FP32's range.
+// below 2^-126, infinite beyond FP32's range, NaN for NaN.
 template <typename DT>
 __device__ __forceinline__ DT to_derivative(double x) {
   if constexpr (sizeof(DT) == 8) {
     return x;
   } else {
     const uint64_t b = (uint64_t)__double_as_longlong(x) + 0x10000000ull;
-    const uint32_t hi = (uint32_t)(b >> 32);
-    const int e = (int)((hi >> 20) & 0x7ffu) - 896;
+    const int e = (int)((uint32_t)(b >> 52) & 0x7ffu) - 896;
     uint32_t f = ((uint32_t)e << 23) | ((uint32_t)(b >> 29) & 0x7fffffu);
     f = e < 1 ? 0u : f;
     f = e > 254 ? 0x7f800000u : f;
-    return __uint_as_float(f | (hi & 0x80000000u));
+    const uint64_t a = (uint64_t)__double_as_longlong(x) & 0x7fffffffffffffffull;
+    f = a > 0x7ff0000000000000ull ? 0x7fc00000u : f;
+    return __uint_as_float(f | ((uint32_t)__double2hiint(x) & 0x80000000u));
   }
 }
 
