@@ -917,7 +917,8 @@ def main():
                 "work_per_state": fp64_work,
                 "work_source": "oracle operation count (oracle/work_counts.json, oracle/opcount.py): add, mul, "
                                "fma 1, exp 9, log 30.2, div 5.7 DFMA-equivalents; entry accumulations (L2 "
-                               "reductions) not counted",
+                               "reductions) not counted; the kernels evaluate exponents, exponentials and "
+                               "logarithms in integer fixed point, so that frac can exceed 1",
                 "counts": counts, "class_shares": class_shares(counts, weights),
                 "peak_source": "derived: 2 FP64 FMA/clk/SM x SMs x max SM clock"}
     roofline["t_roof"] = t_roof(fp64_work, algorithmic_bytes(args.op, m.n_species, h), n, ms, peak, weights)

@@ -363,12 +363,11 @@ int pj_debug_set_target(const pj_mech* mech, int fmt, int32_t index, int32_t val
 /* The kernel layout the Jacobian entries (pj_eval_jacobian_sparse / dense,
  * fmt PJ_CSR, PJ_CSC or PJ_DENSE) and the FP32 Newton matrix (prec PJ_F32)
  * use for n states of this mechanism on the current device: *layout =
- * PJ_LAYOUT_*.  The choice was measured on GB300: the cooperative layout
- * for batches of at most one 32-state tile per SM, for batches below one
- * round of the one-state-per-thread kernels, and for the sparse Jacobians
- * and FP32 Newton matrices of mechanisms too large for per-thread shared
- * memory; tensor memory for the dense Jacobian of such mechanisms; shared
- * memory, one state per thread, for small mechanisms on large batches.  The
+ * PJ_LAYOUT_*.  The cooperative layout for all batches below 1 Mi states,
+ * and for the sparse Jacobians and FP32 Newton matrices of mechanisms too
+ * large for per-thread shared memory; from 1 Mi states on, tensor memory for
+ * the dense Jacobian of such mechanisms and shared memory, one state per
+ * thread, for small mechanisms.  The
  * cooperative layout keeps few Jacobians live in L2 (a third to a half of
  * the DRAM traffic at 53 species) and is not bit-reproducible (see
  * pj_eval_jacobian_sparse).  Errors: PJ_ERR_ARG, PJ_ERR_CUDA (no device
@@ -422,8 +421,8 @@ int pj_vjp(const pj_mech* mech, int mode, int64_t n, const double* d_param, cons
            const double* d_u_wdot, const double* d_u_T, double* d_y, double* d_g_phi, double* d_g_theta,
            int* d_status, void* d_work, size_t work_bytes, void* stream);
 
-/* Diagnostic: the library's FP64 exponential (Tang's table-driven method,
- * used by every kernel for rate constants and falloff factors) and CUDA's
+/* Diagnostic: the library's FP64 exponential (Tang's table-driven method in
+ * integer fixed point, used for rate constants and falloff factors) and CUDA's
  * exp for the same n device inputs, so that its error can be verified. */
 int pj_diag_exp(const pj_mech* mech, int64_t n, const double* d_x, double* d_y_ours, double* d_y_lib,
                 void* stream);

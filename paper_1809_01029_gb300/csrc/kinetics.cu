@@ -1,18 +1,16 @@
 // Source terms and the analytical Jacobian of the molar, explicitly
-// mass-conserving formulation (Sec. 2.2), one thermochemical state per
-// thread ("shallow" vectorisation, Sec. 2.1) over a structure-of-arrays
-// batch.
+// mass-conserving formulation (Sec. 2.2) over a structure-of-arrays batch,
+// lane = state.
 //
 // GB300 design notes:
 //  * The path is bound by the FP64 pipe (2 FP64 FMA per clock per SM on this
 //    part, a 64th of the FP32 rate), not by HBM, so the kernels minimise
-//    FP64 instructions: one exp per forward rate, one per reverse rate (from
-//    ln kf - ln Kc), the T-only pieces once per reaction, ln T and 1/T once
-//    per state.
-//  * One warp per SM sub-partition already saturates that pipe when it has
-//    independent work, so blocks of 128 threads keep each state's
-//    concentrations, Gibbs energies and enthalpies on chip (shared memory and
-//    TMEM) or, for large mechanisms, in a global workspace.
+//    FP64 instructions: exponents, exponentials and logarithms are integer
+//    fixed point (fixed_math.cuh), one exponential per forward rate and one
+//    per reverse rate (from ln kf - ln Kc).
+//  * The warps of a block share 32 states: concentrations, Gibbs energies and
+//    enthalpies sit once in shared memory or, for large mechanisms, in a
+//    global workspace.
 //  * Reaction constants are read warp-uniformly (every thread of a warp works
 //    on the same reaction), so there is no divergence except the NASA range.
 //  * Jacobian entries are accumulated with fire-and-forget FP64 reductions
@@ -20,7 +18,8 @@
 //    the SM and no FP64 add on the SM).  One state per thread, each entry is
 //    owned by one thread, whose reductions apply in program order, so results
 //    are deterministic; the cooperative layout sums one entry from several
-//    warps, in an order that can change between runs.
+//    warps, in an order that can change between runs.  The source terms'
+//    sums are in a fixed order (source_tile.cuh).
 //    Targets come from a static full -> sparse index map built at mechanism
 //    load (the mapping Sec. 3.4 proposes instead of a per-entry search).
 //  * This file holds the source-term kernel and the launch planning; the

@@ -78,8 +78,7 @@ __device__ __forceinline__ DT to_derivative(double x) {
     uint32_t f = ((uint32_t)e << 23) | ((uint32_t)(b >> 29) & 0x7fffffu);
     f = e < 1 ? 0u : f;
     f = e > 254 ? 0x7f800000u : f;
-    const uint64_t a = (uint64_t)__double_as_longlong(x) & 0x7fffffffffffffffull;
-    f = a > 0x7ff0000000000000ull ? 0x7fc00000u : f;
+    if (e == 1151) f |= (uint32_t)(b >> 29) & 0x7fffffu;  // infinity, or NaN (quiet: a high fraction bit is set)
     return __uint_as_float(f | ((uint32_t)__double2hiint(x) & 0x80000000u));
   }
 }

@@ -278,7 +278,7 @@ __global__ void __launch_bounds__(256) k_lu_factor(DevLu L, int64_t n, const T* 
 // come from L2 where the matrices leave L1 no room (111 species FP32: 26 of
 // 228 KB), in every pivot's serial chain.
 template <typename T, int S, bool FROM_J, bool LISTS>
-__global__ void __launch_bounds__(256) k_lu_factor_v(DevLu L, int64_t n, const T* __restrict__ vals, int64_t ld,
+__global__ void __launch_bounds__(256, sizeof(T) == 4 && S == 2 ? 3 : 4) k_lu_factor_v(DevLu L, int64_t n, const T* __restrict__ vals, int64_t ld,
                                                      const double* __restrict__ hstep, double gamma,
                                                      T* __restrict__ lu, int* status) {
   using V = typename LuVec<T, S>::V;
@@ -366,10 +366,49 @@ __global__ void __launch_bounds__(256) k_lu_factor_v(DevLu L, int64_t n, const T
           __syncwarp();
         }
         finish_column(k + 1);
+      } else if (sizeof(T) == 4 && S <= 2) {
+        // FP32 of larger matrices (bound by instructions and latency, idle lanes are free): lanes
+        // over up to 128 columns, whose index and U entry stay in registers,
+        // the other warps over rows, four rows' loads in flight; seven
+        // instructions a pair of states where the flattened form has eighteen
+        const int ncw = nc - j0, cb = c0 + j0, nw = (nt >> 5) - 1;
+        for (int cc = 0; cc < ncw; cc += 128) {
+          int jj[4];
+          V u[4];
+#pragma unroll
+          for (int q = 0; q < 4; q++) {
+            const int c = cc + 32 * q + lane;
+            jj[q] = c < ncw ? cidx(cb + c) : -1;
+            u[q] = A[k * NP + (c < ncw ? jj[q] : k)];
+          }
+          for (int a = warp - 1; a < nr; a += 4 * nw) {
+            V* row[4];
+            V l[4];
+#pragma unroll
+            for (int t = 0; t < 4; t++) {
+              const int at = a + t * nw;
+              row[t] = A + (at < nr ? ridx(r0 + at) : k) * NP;
+              l[t] = row[t][k];
+            }
+#pragma unroll
+            for (int q = 0; q < 4; q++) {
+              if (cc + 32 * q >= ncw) break;
+              if (jj[q] >= 0) {
+                V v[4];
+#pragma unroll
+                for (int t = 0; t < 4; t++) v[t] = row[t][jj[q]];
+#pragma unroll
+                for (int t = 0; t < 4; t++)
+                  if (a + t * nw < nr) row[t][jj[q]] = v_fms(l[t], u[q], v[t]);
+              }
+            }
+          }
+        }
       } else {
-        // the nr x (nc - j0) update of the other columns, flattened over the
-        // other warps: pair p = a * ncw + c, four pairs at a time (distinct
-        // pairs touch distinct entries, so their loads go out first)
+        // FP64, and four FP32 states a block: the nr x (nc - j0) update of the
+        // other columns, flattened over the other warps so that they stay full (the FP64 pipe charges idle
+        // lanes): pair p = a * ncw + c, four pairs at a time (distinct pairs
+        // touch distinct entries, so their loads go out first)
         const int ncw = nc - j0, tot = nr * ncw, ntw = nt - 32;
         int p = tid - 32;
         if (p < tot) {
