@@ -19,9 +19,10 @@
 //    index work and the loop are shared by the S states, whose fused
 //    multiply-adds are independent).  The factors are gathered into the
 //    storage order.
-//  * Solve: one state per thread, streaming the factors in storage order
+//  * Solve: four warps per 32 states, streaming the factors in storage order
 //    (coalesced across the warp), forward substitution then backward; the
-//    solution sits in shared memory when N values per thread fit.
+//    solution sits in shared memory (matrices too large for that: one state
+//    per thread, the solution in x).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -464,66 +465,96 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 && S == 2 ? 3 : 4) k_lu_fa
   }
 }
 
-// x may alias b.  X: the solution of this thread's state, in shared memory
-// (stride blockDim.x) or in x itself (stride ld).
-template <typename T, bool SMEM_X>
+// Solve of 32 states (lane = state) by the four warps of a block.  A row's sum
+// has four chains of fused multiply-adds (entries e, e + 4, e + 8, .. of
+// chain e mod 4, the last entries mod 4 on chain 0): warp i runs chain i, the
+// chains' sums meet in shared memory (double-buffered: one barrier a row) and
+// every warp forms the row's value, so that no second barrier is needed.  One
+// thread per state and row kept eight loads in flight; what bounds the solve
+// is the latency of streaming the factors, so a batch of 8191 states of 111
+// species left most of the chip idle.  x may alias b (read before the last
+// barrier, written after it).
+template <typename T>
 __global__ void __launch_bounds__(128) k_lu_solve(DevLu L, int64_t n, const T* __restrict__ lu, int64_t ld,
                                                   const T* b, T* x) {
   extern __shared__ __align__(16) unsigned char lu_smem[];
-  const int N = L.N;
-  for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < n; s += (int64_t)gridDim.x * blockDim.x) {
-    T* X = SMEM_X ? reinterpret_cast<T*>(lu_smem) + threadIdx.x : x + s;
-    const int64_t xs = SMEM_X ? blockDim.x : ld;
-    // sum over storage entries [e, e1) of value * X[column], four independent
-    // partial sums so that the factor loads stream; FP32 takes eight entries
-    // a step (eight loads in flight: 17 % faster at 111 species; FP64 was
-    // slower that way)
-    auto dot = [&](int e, int e1) -> T {
-      T p0 = T(0), p1 = T(0), p2 = T(0), p3 = T(0);
-      for (; sizeof(T) == 4 && e + 7 < e1; e += 8) {
-        const int c0 = __ldg(L.xcol + e), c1 = __ldg(L.xcol + e + 1);
-        const int c2 = __ldg(L.xcol + e + 2), c3 = __ldg(L.xcol + e + 3);
-        const int c4 = __ldg(L.xcol + e + 4), c5 = __ldg(L.xcol + e + 5);
-        const int c6 = __ldg(L.xcol + e + 6), c7 = __ldg(L.xcol + e + 7);
-        const T v0 = lu[(int64_t)e * ld + s], v1 = lu[(int64_t)(e + 1) * ld + s];
-        const T v2 = lu[(int64_t)(e + 2) * ld + s], v3 = lu[(int64_t)(e + 3) * ld + s];
-        const T v4 = lu[(int64_t)(e + 4) * ld + s], v5 = lu[(int64_t)(e + 5) * ld + s];
-        const T v6 = lu[(int64_t)(e + 6) * ld + s], v7 = lu[(int64_t)(e + 7) * ld + s];
-        p0 = fma_t(v0, X[(int64_t)c0 * xs], p0);
-        p1 = fma_t(v1, X[(int64_t)c1 * xs], p1);
-        p2 = fma_t(v2, X[(int64_t)c2 * xs], p2);
-        p3 = fma_t(v3, X[(int64_t)c3 * xs], p3);
-        p0 = fma_t(v4, X[(int64_t)c4 * xs], p0);
-        p1 = fma_t(v5, X[(int64_t)c5 * xs], p1);
-        p2 = fma_t(v6, X[(int64_t)c6 * xs], p2);
-        p3 = fma_t(v7, X[(int64_t)c7 * xs], p3);
+  const int N = L.N, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  T* const X = reinterpret_cast<T*>(lu_smem) + lane;   // [N][32]
+  T* const part = X + N * 32;                          // [2][4][32]
+  for (int64_t tile = blockIdx.x; tile * 32 < n; tile += gridDim.x) {
+    const int64_t s = tile * 32 + lane;
+    const bool act = s < n;
+    const T* __restrict__ f = lu + (act ? s : n - 1);  // a lane past the batch repeats the last state
+    const T* const bs = b + (act ? s : n - 1);
+    // the sum over storage entries [e, e1) of value * X[column]; the value it
+    // is subtracted from is read before the barrier
+    auto row_sum = [&](int e, int e1, int buf) -> T {
+      T p = T(0);
+      const int n4 = (e1 - e) >> 2;
+#pragma unroll 8
+      for (int t = 0; t < n4; t++) {
+        const int q = e + 4 * t + warp;
+        p = fma_t(f[(int64_t)q * ld], X[__ldg(L.xcol + q) * 32], p);
       }
-      for (; e + 3 < e1; e += 4) {
-        const int c0 = __ldg(L.xcol + e), c1 = __ldg(L.xcol + e + 1);
-        const int c2 = __ldg(L.xcol + e + 2), c3 = __ldg(L.xcol + e + 3);
-        p0 = fma_t(lu[(int64_t)e * ld + s], X[(int64_t)c0 * xs], p0);
-        p1 = fma_t(lu[(int64_t)(e + 1) * ld + s], X[(int64_t)c1 * xs], p1);
-        p2 = fma_t(lu[(int64_t)(e + 2) * ld + s], X[(int64_t)c2 * xs], p2);
-        p3 = fma_t(lu[(int64_t)(e + 3) * ld + s], X[(int64_t)c3 * xs], p3);
-      }
-      for (; e < e1; e++) p0 = fma_t(lu[(int64_t)e * ld + s], X[(int64_t)__ldg(L.xcol + e) * xs], p0);
-      return (p0 + p1) + (p2 + p3);
+      if (warp == 0)
+        for (int q = e + 4 * n4; q < e1; q++) p = fma_t(f[(int64_t)q * ld], X[__ldg(L.xcol + q) * 32], p);
+      part[(4 * buf + warp) * 32] = p;
+      __syncthreads();
+      const T* w = part + 4 * buf * 32;
+      return (w[0] + w[32]) + (w[64] + w[96]);
     };
     // forward: y_k = b_perm[k] - sum_{j<k} L_kj y_j, y kept at X[perm[k]]
     for (int k = 0; k < N; k++) {
       const int pk = __ldg(L.perm + k);
-      const T bk = b[(int64_t)pk * ld + s];
-      X[(int64_t)pk * xs] = bk - dot(__ldg(L.lptr + k), __ldg(L.lptr + k + 1));
+      const T bk = bs[(int64_t)pk * ld];
+      X[pk * 32] = bk - row_sum(__ldg(L.lptr + k), __ldg(L.lptr + k + 1), k & 1);
     }
     // backward: z_k = (y_k - sum_{j>k} U_kj z_j) / U_kk
     for (int q = 0; q < N; q++) {
       const int e0 = __ldg(L.uptr + q), e1 = __ldg(L.uptr + q + 1);
       const int pk = __ldg(L.perm + (N - 1 - q));
-      const T yk = X[(int64_t)pk * xs];
-      X[(int64_t)pk * xs] = (yk - dot(e0 + 1, e1)) * lu[(int64_t)e0 * ld + s];
+      const T d = f[(int64_t)e0 * ld];
+      const T yk = X[pk * 32];
+      X[pk * 32] = (yk - row_sum(e0 + 1, e1, (N + q) & 1)) * d;
     }
-    if (SMEM_X)
-      for (int v = 0; v < N; v++) x[(int64_t)v * ld + s] = X[(int64_t)v * xs];
+    if (act)
+      for (int v = warp; v < N; v += 4) x[(int64_t)v * ld + s] = X[v * 32];
+    __syncthreads();
+  }
+}
+
+// The same with one state per thread and the solution in x itself, for
+// matrices whose solutions do not fit in shared memory (the same sums).
+template <typename T>
+__global__ void __launch_bounds__(128) k_lu_solve_global(DevLu L, int64_t n, const T* __restrict__ lu, int64_t ld,
+                                                         const T* b, T* x) {
+  const int N = L.N;
+  for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < n; s += (int64_t)gridDim.x * blockDim.x) {
+    T* X = x + s;
+    auto dot = [&](int e, int e1) -> T {
+      T p0 = T(0), p1 = T(0), p2 = T(0), p3 = T(0);
+      for (; e + 3 < e1; e += 4) {
+        const int c0 = __ldg(L.xcol + e), c1 = __ldg(L.xcol + e + 1);
+        const int c2 = __ldg(L.xcol + e + 2), c3 = __ldg(L.xcol + e + 3);
+        p0 = fma_t(lu[(int64_t)e * ld + s], X[(int64_t)c0 * ld], p0);
+        p1 = fma_t(lu[(int64_t)(e + 1) * ld + s], X[(int64_t)c1 * ld], p1);
+        p2 = fma_t(lu[(int64_t)(e + 2) * ld + s], X[(int64_t)c2 * ld], p2);
+        p3 = fma_t(lu[(int64_t)(e + 3) * ld + s], X[(int64_t)c3 * ld], p3);
+      }
+      for (; e < e1; e++) p0 = fma_t(lu[(int64_t)e * ld + s], X[(int64_t)__ldg(L.xcol + e) * ld], p0);
+      return (p0 + p1) + (p2 + p3);
+    };
+    for (int k = 0; k < N; k++) {
+      const int pk = __ldg(L.perm + k);
+      const T bk = b[(int64_t)pk * ld + s];
+      X[(int64_t)pk * ld] = bk - dot(__ldg(L.lptr + k), __ldg(L.lptr + k + 1));
+    }
+    for (int q = 0; q < N; q++) {
+      const int e0 = __ldg(L.uptr + q), e1 = __ldg(L.uptr + q + 1);
+      const int pk = __ldg(L.perm + (N - 1 - q));
+      const T yk = X[(int64_t)pk * ld];
+      X[(int64_t)pk * ld] = (yk - dot(e0 + 1, e1)) * lu[(int64_t)e0 * ld + s];
+    }
   }
 }
 
@@ -633,21 +664,19 @@ int launch_lu_factor(const DevLu& L, int prec, int64_t n, const void* vals, int6
 template <typename T>
 static int launch_solve_t(const DevLu& L, int64_t n, const void* lu, int64_t ld, const void* b, void* x,
                           cudaStream_t st) {
-  const size_t xs_bytes = (size_t)L.N * sizeof(T) * 128;
-  const bool smem_x = xs_bytes <= 200 * 1024;
-  const int64_t blocks = (n + 127) / 128;
+  const size_t smem = (size_t)(L.N + 8) * 32 * sizeof(T);
   int rc;
-  if (smem_x) {
-    auto kern = k_lu_solve<T, true>;
-    if ((rc = set_smem(kern, xs_bytes))) return rc;
+  if (smem <= kSmemCap) {
+    auto kern = k_lu_solve<T>;
+    if ((rc = set_smem(kern, smem))) return rc;
     int occ = 1;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, 128, xs_bytes) != cudaSuccess || occ < 1) occ = 1;
-    const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(blocks, (int64_t)sm_count() * occ));
-    kern<<<(unsigned)grid, 128, xs_bytes, st>>>(L, n, static_cast<const T*>(lu), ld, static_cast<const T*>(b),
-                                                static_cast<T*>(x));
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, 128, smem) != cudaSuccess || occ < 1) occ = 1;
+    const int64_t grid = std::max<int64_t>(1, std::min<int64_t>((n + 31) / 32, (int64_t)sm_count() * occ));
+    kern<<<(unsigned)grid, 128, smem, st>>>(L, n, static_cast<const T*>(lu), ld, static_cast<const T*>(b),
+                                            static_cast<T*>(x));
   } else {
-    auto kern = k_lu_solve<T, false>;
-    const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(blocks, (int64_t)sm_count() * 16));
+    auto kern = k_lu_solve_global<T>;
+    const int64_t grid = std::max<int64_t>(1, std::min<int64_t>((n + 127) / 128, (int64_t)sm_count() * 16));
     kern<<<(unsigned)grid, 128, 0, st>>>(L, n, static_cast<const T*>(lu), ld, static_cast<const T*>(b),
                                          static_cast<T*>(x));
   }
