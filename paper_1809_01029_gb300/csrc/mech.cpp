@@ -14,6 +14,7 @@
 #include <string>
 
 #include "pj_internal.h"
+#include "rxn_pack.h"
 
 namespace pj {
 
@@ -410,19 +411,13 @@ int mech_build(pj_mech* m) {
         if (ssp[a] >= 0) mem.push_back({snu[a], ssp[a]});
       // larger coefficients first, so 2A + B maps onto SH_21
       std::stable_sort(mem.begin(), mem.end(), [](auto x, auto y) { return x.first > y.first; });
-      int32_t shape = SH_GEN;
-      if (mem.size() == 1 && mem[0].first == 1) shape = SH_1;
-      else if (mem.size() == 1 && mem[0].first == 2) shape = SH_2;
-      else if (mem.size() == 2 && mem[0].first == 1 && mem[1].first == 1) shape = SH_11;
-      else if (mem.size() == 2 && mem[0].first == 2 && mem[1].first == 1) shape = SH_21;
-      else if (mem.size() == 3 && mem[0].first == 1 && mem[1].first == 1 && mem[2].first == 1) shape = SH_111;
-      r.shape[side] = shape;
       for (size_t a = 0; a < mem.size(); a++) {
         r.sp[side * PJ_MAX_SP + a] = mem[a].second;
         r.nu[side * PJ_MAX_SP + a] = mem[a].first;
         r.nud[side * PJ_MAX_SP + a] = (double)mem[a].first;
       }
       (side ? r.nprod : r.nreac) = (int32_t)mem.size();
+      r.shape[side] = side_shape(&r.nu[side * PJ_MAX_SP], (int)mem.size());
     }
     std::vector<int> nu = net_nu(m, i);
     double dnu = 0, dW = 0;
@@ -469,32 +464,7 @@ int mech_build(pj_mech* m) {
     for (int a = 0; a < 2 * PJ_MAX_SP; a++)
       nu_sum += a < PJ_MAX_SP ? (a < r.nreac ? r.nu[a] : 0) : (a - PJ_MAX_SP < r.nprod ? r.nu[a] : 0);
     nu_max = std::max(nu_max, nu_sum);
-    // short-path head: the factors of each side, a coefficient of 2 as two
-    {
-      RxnHead& hd = r.head;
-      hd.kind = (uint8_t)r.kind;
-      hd.rev = (uint8_t)r.rev;
-      hd.lean = q < nr_plain ? 1 : 0;
-      for (int side = 0; side < 2; side++) {
-        int32_t* out = side ? hd.b : hd.f;
-        // in the order side_rate multiplies them: 2A + B as A B A, else last to first
-        const int32_t* sp = &r.sp[side * PJ_MAX_SP];
-        int cnt = 0;
-        if (r.shape[side] == SH_21) {
-          out[0] = out[2] = 32 * sp[0];
-          out[1] = 32 * sp[1];
-          cnt = 3;
-        } else {
-          for (int a = (side ? r.nprod : r.nreac) - 1; a >= 0; a--)
-            for (int u = 0; u < r.nu[side * PJ_MAX_SP + a]; u++, cnt++)
-              if (cnt < 3) out[cnt] = 32 * sp[a];
-        }
-        if (cnt < 1 || cnt > 3) hd.lean = 0;
-        for (int u = cnt; u >= 1 && u < 3; u++) out[u] = out[0];
-        (side ? hd.nb : hd.nf) = (uint8_t)std::min(cnt, 3);
-      }
-      if (hd.lean) hd.code = (uint8_t)(6 * r.shape[0] + (r.rev ? 1 + r.shape[1] : 0));
-    }
+    pack_head(r, q < nr_plain);
     std::vector<double> al = alpha_of(m, i);
     r.alpha_bath = has_third_body(r.kind) ? al[bath] : 1.0;
     r.eff_lo = (int32_t)eff_sp.size();

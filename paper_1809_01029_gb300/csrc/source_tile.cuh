@@ -142,7 +142,8 @@ __device__ __forceinline__ LeanSide lean_side(const int32_t (&f)[3], const doubl
 // compile-time constants.  A jump table: under conditions of its own each
 // shape's few FP64 instructions would be predicated, and the FP64 pipe
 // charges a predicated-off warp instruction like any other (20 of the 63 a
-// 53-species Jacobian reaction issued).
+// 53-species Jacobian reaction issued).  Short-path reactions only: pack_head
+// gives no other the flag, and theirs no code beyond the table.
 template <int V>
 struct IntTag {
   static constexpr int value = V;
