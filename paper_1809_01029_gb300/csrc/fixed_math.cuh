@@ -55,14 +55,15 @@ __host__ __device__ __forceinline__ uint64_t exp2_significand(uint64_t frac, con
   return T + (mulhi_approx(T, v) >> 8);                          // 2^63 2^(j/256 + f)
 }
 
-// bits of the double M 2^(n - 63), -1022 <= n <= 1022, rounded to nearest
+// bits of the double M 2^(n - 63), 2^63 <= M, -1022 <= n <= 1023, rounded to
+// nearest (at n = 1023 up to infinity)
 __host__ __device__ __forceinline__ uint64_t pack_double(int n, uint64_t M) {
   return (((M >> 10) + 1u) >> 1) + ((uint64_t)(int64_t)(n + 1022) << 52);
 }
 
 // the same for any n: subnormals, zero and infinity
 __host__ __device__ __forceinline__ uint64_t pack_double_any(int n, uint64_t M) {
-  if ((uint32_t)(n + 1022) < 2045u) return pack_double(n, M);
+  if ((uint32_t)(n + 1022) < 2046u) return pack_double(n, M);
   if (n > 0) return 0x7ff0000000000000ull;
   const int sh = -1022 - n;
   return sh > 54 ? 0 : (((M >> 10) >> sh) + 1u) >> 1;

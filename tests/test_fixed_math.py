@@ -49,13 +49,14 @@ int main() {
   }
   std::mt19937_64 rng(5);
 
-  // 2^(n + frac 2^-64) normal, subnormal and zero
-  for (int n = -1100; n <= 1022; n++)
+  // 2^(n + frac 2^-64) of any n: normal, both edges, subnormal, zero, infinity
+  for (int n = -1100; n <= 1030; n++)
     for (int t = 0; t < 300; t++) {
       const uint64_t frac = t == 0 ? 0 : t == 1 ? ~0ull : t == 2 ? 1ull << 63 : rng();
       const long double want = std::ldexp(std::exp2((long double)frac * 0x1p-64L), n);
       const double got = d(pack_double_any(n, exp2_significand(frac, tab)));
-      check(std::isfinite(got) && std::fabs(got - want) <= 0.54L * ulp(want), "exp2", n + frac * 0x1p-64L);
+      if (want >= 0x1.fffffffffffff8p1023L) check(std::isinf(got), "exp2 overflow", n + frac * 0x1p-64L);
+      else check(std::isfinite(got) && std::fabs(got - want) <= 0.54L * ulp(want), "exp2", n + frac * 0x1p-64L);
     }
 
   // exp(x), |x| < 704
