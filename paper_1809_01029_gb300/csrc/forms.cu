@@ -40,7 +40,7 @@ enum VjpSc {
   vUT, vMRT, vGB, vTv, kVjpSc
 };
 enum VjpPart { wAcc, wDen, wDden, wNum, wSum, wGT, wGS, wGB, kVjpPart };
-enum VjpFlag { xOk, xFast, kVjpFlag };
+enum VjpFlag { xOk, xFast, kVjpFlag };  // xFast: 1 in the fixed point's range; 0: T out of it; 2: some g_k or h_k
 
 __host__ __device__ constexpr size_t vjp_arrays_bytes(int ns) { return (size_t)4 * ns * kTile * sizeof(double); }
 __host__ __device__ constexpr size_t vjp_smem_bytes(int ns, bool arrays_smem) {
@@ -56,19 +56,200 @@ struct VjpVars {
   double gT, gS, gB;
 };
 
-// Any reaction at any state, out of line.  base: this lane's column of C, g, h,
-// u ([4][ns][32]); wrow, grow: the warp's rows of wdot and of d/dn; returns
-// the adjoint part of the parameter gradient.
-template <int MODE, bool SPECIAL>
-struct VjpGeneral {
+// A plain reaction with at most three factors a side (as lean_jacobian);
+// returns ubar Q.
+template <int MODE, bool MIXED>
+__device__ __forceinline__ double lean_vjp(const DevMech& m, const Rxn* __restrict__ r, const RxnHead& h,
+                                           const double* __restrict__ base, VjpVars& v, double* __restrict__ wrow,
+                                           double* __restrict__ grow) {
+  const int ns = m.ns, bath = ns - 1;
+  const double* __restrict__ C = base;
+  const double* __restrict__ G = base + ns * kTile;
+  const double* __restrict__ H = base + 2 * ns * kTile;
+  const double* __restrict__ U = base + 3 * ns * kTile;
+  RxnJac a;
+  {
+    const int4* __restrict__ p = reinterpret_cast<const int4*>(&r->jac);
+    int4* q = reinterpret_cast<int4*>(&a);
+#pragma unroll
+    for (int i = 0; i < 4; i++) q[i] = __ldg(p + i);
+  }
+  const bool rev = h.rev != 0;
+  const LeanK k = lean_constants<MIXED>(m, r, h, G, v.fx, v.lnT, v.invT);
+  LeanSide sf, sb;
+  double Rn, SV, du;  // SV: V dRn/dV at constant n; du = sum nu u
+  lean_shapes(h.code, [&](auto tf, auto tb) {
+    constexpr int SF = decltype(tf)::value, SB = decltype(tb)::value;
+    constexpr int nfac[5] = {1, 2, 2, 3, 3};
+    sf = lean_side<SF>(h.f, C, k.kf);
+    sb = lean_side<SB>(h.b, C, k.kr);
+    Rn = SB < 0 ? sf.R : sf.R - sb.R;
+    constexpr int NF = nfac[SF], NB = SB < 0 ? 0 : nfac[SB < 0 ? 0 : SB];
+    SV = 0.0;
+    if (MODE == PJ_CONP) {
+      if (NF == NB || SB < 0) SV = NF == 1 ? dneg(Rn) : -(double)NF * Rn;
+      else SV = (NB == 1 ? sb.R : (double)NB * sb.R) - (NF == 1 ? sf.R : (double)NF * sf.R);
+    }
+    du = dneg(U[h.f[0]]);
+    if (NF > 1) du -= U[h.f[1]];
+    if (NF > 2) du -= U[h.f[2]];
+    if (SB >= 0) {
+      du += U[h.b[0]];
+      if (NB > 1) du += U[h.b[1]];
+      if (NB > 2) du += U[h.b[2]];
+    }
+  });
+  if (!rev) {
+    du += U[h.b[0]];
+    if (h.nb > 1) du += U[h.b[1]];
+    if (h.nb > 2) du += U[h.b[2]];
+  }
+  const double de = lean_energy<MIXED>(h, H, h.dnu_i, v.fx.fast);  // sum nu h/RT - dnu
+  double dhd = de;
+  if (MODE == PJ_CONP && h.dnu_i != 0) dhd = lean_energy<MIXED>(h, H, 0, v.fx.fast);
+  const double ub = fma(-v.uTE, dhd, du);
+  const double ubV = ub * v.invV;
+
+  // derivatives of the net rate (lean_jacobian)
+  const double Ef = fma(a.theta, v.invT, a.beta);
+  double qT = fma(sb.R, de, Rn * Ef) * v.invT;
+  double qS = MODE == PJ_CONP ? SV * v.invV : 0.0;
+  double Gb = 0.0;
+  bool has_S = MODE == PJ_CONP;
+  if (a.bath) {
+    if (a.bath & 1) Gb += sf.d0;
+    if (a.bath & 2) Gb += sf.d1;
+    if (a.bath & 4) Gb += sf.d2;
+    if (a.bath & 8) Gb -= sb.d0;
+    if (a.bath & 16) Gb -= sb.d1;
+    if (a.bath & 32) Gb -= sb.d2;
+    qT = fma(Gb, v.dCb_T, qT);
+    if (MODE == PJ_CONP) qS = (a.nbx * sb.R - a.nfx * sf.R) * v.invV;
+    qS = fma(Gb, v.dCb_S, qS);
+    has_S = true;
+  }
+  double q = Rn, Q = Rn, ubVc = ubV;
+  if (h.kind != PJ_ELEMENTARY) {
+    double M = v.Ctot;
+    for (int e = __ldg(&r->eff_lo), eh = __ldg(&r->eff_hi); e < eh; e++) {
+      if (!PJ_DBG_OK(m.dbg, e >= 0 && e < m.n_eff && __ldg(m.eff_sp + e) >= 0 && __ldg(m.eff_sp + e) < m.ns,
+                     PJ_DBG_EFF))
+        break;
+      M = fma(__ldg(m.eff_am1 + e), C[kTile * __ldg(m.eff_sp + e)], M);
+    }
+    const double ab = __ldg(&r->alpha_bath);
+    const double dMdT = ab * v.dCb_T;
+    const double dMdS = MODE == PJ_CONP ? (ab * v.Ctot - M) * v.invV : ab * (v.Ctot / v.P);
+    double cT = dMdT, c = M, RcM = Rn;
+    if (h.kind != PJ_THIRD_BODY) {
+      int64_t l2rk;
+      const double rk = lean_falloff<MIXED>(r, k, v.fx, v.lnT, v.invT, l2rk);
+      const FalloffC fc =
+          falloff_derivatives<MIXED>(r, m.log_tab, h.kind, v.T, v.invT, v.lnT, v.fx.IT, rk, l2rk, M, dMdT);
+      c = fc.c;
+      cT = fc.cT;
+      RcM = Rn * fc.cM;
+    }
+    q = c * Rn;
+    Q = h.kind != PJ_THIRD_BODY ? fma(-RcM, M, q) : q;  // k_inf divides Pr: - Rn Pr dc/dPr
+    qT = fma(c, qT, Rn * cT);
+    qS = fma(c, qS, RcM * dMdS);
+    has_S = true;
+    ubVc = ubV * c;
+    double Bi = 0.0;
+    for (int e = __ldg(&r->eff_lo), eh = __ldg(&r->eff_hi); e < eh; e++) {
+      if (!PJ_DBG_OK(m.dbg, e >= 0 && e < m.n_eff, PJ_DBG_EFF)) break;
+      const int j = __ldg(m.eff_sp + e);
+      const double val = RcM * __ldg(m.eff_am1 + e);
+      if (j == bath) Bi -= val;
+      else red_add(grow + j * kTile, ubV * val);
+    }
+    v.gB = fma(ubV, Bi, v.gB);
+  }
+  if (a.bath) v.gB = fma(-ubVc, Gb, v.gB);
+  v.gT = fma(ub, qT, v.gT);
+  if (has_S) v.gS = fma(ub, qS, v.gS);
+
+  // production rates and amount gradients into the warp's rows
+  const double nq = dneg(q);
+#pragma unroll
+  for (int s = 0; s < 3; s++) {
+    if (s < h.nf) red_add(wrow + h.f[s], nq);
+    if (s < h.nb) red_add(wrow + h.b[s], q);
+  }
+  // slots in species order: the factors last to first (2A + B: A, B)
+  auto slot = [&](int sp, double d) { red_add(grow + kTile * sp, ubVc * d); };
+  const int nsf = shape_species(a.shape[0]), nsb = rev ? shape_species(a.shape[1]) : 0;
+#pragma unroll
+  for (int s = 0; s < 3; s++) {
+    if (s < nsf && !(a.bath >> s & 1)) slot(__ldg(&r->sp[s]), s == 0 ? sf.d0 : s == 1 ? sf.d1 : sf.d2);
+    if (s < nsb && !(a.bath >> (3 + s) & 1))
+      slot(__ldg(&r->sp[PJ_MAX_SP + s]), dneg(s == 0 ? sb.d0 : s == 1 ? sb.d1 : sb.d2));
+  }
+  return ub * Q;
+}
+
+// What a reaction needs of its state (sc: this lane's scalars of the tile; ok: a
+// valid state), and the sums over a warp's reactions.
+__device__ __forceinline__ VjpVars vjp_vars(const double* __restrict__ sc, bool fast, bool ok) {
+  auto S = [&](int v) { return sc[v * kTile]; };
   VjpVars v;
-  double wq;
-};
+  v.T = S(vT);
+  v.V = S(vV);
+  v.P = S(vP);
+  v.invT = S(vInvT);
+  v.invV = S(vInvV);
+  v.lnT = S(vLnT);
+  v.lnP = S(vLnP);
+  v.Ctot = S(vCtot);
+  v.dCb_T = S(vDCbT);
+  v.dCb_S = S(vDCbS);
+  v.uTE = ok ? S(vUT) * S(vIden) * (RU * v.T) : 0.0;
+  v.fx.L = (uint64_t)__double_as_longlong(S(vL));
+  v.fx.IT = (uint64_t)__double_as_longlong(S(vIT));
+  v.fx.LP = __double_as_longlong(S(vLP));
+  v.fx.fast = fast;
+  return v;
+}
+template <class F>
+__device__ __forceinline__ void vjp_sums(VjpVars& v, F&& f) {
+  f(0, v.gT);
+  f(1, v.gS);
+  f(2, v.gB);
+}
+
+// Two out-of-line bodies beside the inlined short path.  Both take the state
+// from and leave their sums in shared memory (part: this lane's of the warp;
+// as general_jacobian), short-path reactions from wGT on and the others from
+// wAcc on (free between phases C and E), so that the sums of a state come in the
+// same order whichever body its tile needs.
+//
+// A short-path reaction in a tile with a state outside the fixed point's range,
+// each lane by its own state: what a state gives does not depend on its tile
+// mates.
+template <int MODE>
+__device__ __noinline__ static double mixed_vjp(const DevMech& m, double* base, const double* sc, double* part,
+                                                const Rxn* __restrict__ r, bool fast, bool ok, double* wrow,
+                                                double* grow) {
+  part += wGT * kTile;
+  VjpVars v = vjp_vars(sc, fast, ok);
+  vjp_sums(v, [&](int p, double& x) { x = part[p * kTile]; });
+  const double w = lean_vjp<MODE, true>(m, r, load_head(r), base, v, wrow, grow);
+  vjp_sums(v, [&](int p, double& x) { part[p * kTile] = x; });
+  return w;
+}
+
+// Any other reaction at any state.  base: this lane's column of C, g, h, u
+// ([4][ns][32]); wrow, grow: the warp's rows of wdot and of d/dn; returns the
+// adjoint part of the parameter gradient.
 template <int MODE, bool SPECIAL>
-__device__ __noinline__ static VjpGeneral<MODE, SPECIAL> general_vjp(const DevMech& m, double* base,
-                                                                     const Rxn* __restrict__ r, bool plain, VjpVars v,
-                                                                     bool hfix, double* wrow, double* grow) {
+__device__ __noinline__ static double general_vjp(const DevMech& m, double* base, const double* sc, double* part,
+                                                  const Rxn* __restrict__ r, bool plain, bool fast, bool ok, double* wrow,
+                                                  double* grow) {
   enum { aC = 0, aG = 1, aH = 2, aU = 3 };
+  part += wAcc * kTile;
+  VjpVars v = vjp_vars(sc, fast, ok);
+  vjp_sums(v, [&](int p, double& x) { x = part[p * kTile]; });
   StateArrays A;
   A.ns = m.ns;
   A.base = base;
@@ -79,7 +260,7 @@ __device__ __noinline__ static VjpGeneral<MODE, SPECIAL> general_vjp(const DevMe
   const int nre = __ldg(&r->nreac), npr = __ldg(&r->nprod), rev = __ldg(&r->rev);
   double dlnkf, dlnP, dlnkinf;
   ln_kf_derivatives<SPECIAL>(m, r, kind, lnT, invT, invT2, v.lnP, dlnkf, dlnP, dlnkinf);
-  const RateK rk = rate_constants<SPECIAL>(m, A, aG, r, kind, rev, nre, npr, v.fx, T, lnT, invT, v.lnP);
+  const RateK rk = rate_constants<SPECIAL>(m, A, aG, r, kind, rev, nre, npr, v.fx, lnT, invT, v.lnP);
   double dh = 0.0, du = 0.0;
   for (int a = 0; a < 2 * PJ_MAX_SP; a++) {
     const bool react = a < PJ_MAX_SP;
@@ -87,7 +268,7 @@ __device__ __noinline__ static VjpGeneral<MODE, SPECIAL> general_vjp(const DevMe
     const int k = __ldg(&r->sp[a]);
     const double nu = react ? -__ldg(&r->nud[a]) : __ldg(&r->nud[a]);
     const double hk = A.at(aH, k);
-    dh = fma(nu, hfix ? fixed51_to_double(__double_as_longlong(hk)) : hk, dh);
+    dh = fma(nu, fast ? fixed51_to_double(__double_as_longlong(hk)) : hk, dh);
     du = fma(nu, A.at(aU, k), du);
   }
   double dRf[PJ_MAX_SP], dRr[PJ_MAX_SP];
@@ -183,141 +364,7 @@ __device__ __noinline__ static VjpGeneral<MODE, SPECIAL> general_vjp(const DevMe
     }
   }
   v.gB = fma(ubV, Bi, v.gB);
-  return VjpGeneral<MODE, SPECIAL>{v, ub * Q};
-}
-
-// A plain reaction with at most three factors a side, at a tile of states
-// within the fixed point's range (as lean_jacobian); returns ubar Q.
-template <int MODE>
-__device__ __forceinline__ double lean_vjp(const DevMech& m, const Rxn* __restrict__ r, const RxnHead& h,
-                                           const double* __restrict__ base, VjpVars& v, double* __restrict__ wrow,
-                                           double* __restrict__ grow) {
-  const int ns = m.ns, bath = ns - 1;
-  const double* __restrict__ C = base;
-  const double* __restrict__ G = base + ns * kTile;
-  const double* __restrict__ H = base + 2 * ns * kTile;
-  const double* __restrict__ U = base + 3 * ns * kTile;
-  RxnJac a;
-  {
-    const int4* __restrict__ p = reinterpret_cast<const int4*>(&r->jac);
-    int4* q = reinterpret_cast<int4*>(&a);
-#pragma unroll
-    for (int i = 0; i < 4; i++) q[i] = __ldg(p + i);
-  }
-  const bool rev = h.rev != 0;
-  const int64_t y = arrhenius_fixed(h.fA, h.fB, h.fT, v.fx.L, v.fx.IT);
-  const double kf = exp2_51(y);
-  double kr = 0.0;
-  if (rev) kr = exp2_51(y + lean_gibbs(h, G, v.fx.LP));
-  LeanSide sf, sb;
-  double Rn, SV, du;  // SV: V dRn/dV at constant n; du = sum nu u
-  lean_shapes(h.code, [&](auto tf, auto tb) {
-    constexpr int SF = decltype(tf)::value, SB = decltype(tb)::value;
-    constexpr int nfac[5] = {1, 2, 2, 3, 3};
-    sf = lean_side<SF>(h.f, C, kf);
-    sb = lean_side<SB>(h.b, C, kr);
-    Rn = SB < 0 ? sf.R : sf.R - sb.R;
-    constexpr int NF = nfac[SF], NB = SB < 0 ? 0 : nfac[SB < 0 ? 0 : SB];
-    SV = 0.0;
-    if (MODE == PJ_CONP) {
-      if (NF == NB || SB < 0) SV = NF == 1 ? dneg(Rn) : -(double)NF * Rn;
-      else SV = (NB == 1 ? sb.R : (double)NB * sb.R) - (NF == 1 ? sf.R : (double)NF * sf.R);
-    }
-    du = dneg(U[h.f[0]]);
-    if (NF > 1) du -= U[h.f[1]];
-    if (NF > 2) du -= U[h.f[2]];
-    if (SB >= 0) {
-      du += U[h.b[0]];
-      if (NB > 1) du += U[h.b[1]];
-      if (NB > 2) du += U[h.b[2]];
-    }
-  });
-  if (!rev) {
-    du += U[h.b[0]];
-    if (h.nb > 1) du += U[h.b[1]];
-    if (h.nb > 2) du += U[h.b[2]];
-  }
-  const double de = lean_energy(h, H, h.dnu_i);  // sum nu h/RT - dnu
-  double dhd = de;
-  if (MODE == PJ_CONP && h.dnu_i != 0) dhd = lean_energy(h, H, 0);
-  const double ub = fma(-v.uTE, dhd, du);
-  const double ubV = ub * v.invV;
-
-  // derivatives of the net rate (lean_jacobian)
-  const double Ef = fma(a.theta, v.invT, a.beta);
-  double qT = fma(sb.R, de, Rn * Ef) * v.invT;
-  double qS = MODE == PJ_CONP ? SV * v.invV : 0.0;
-  double Gb = 0.0;
-  bool has_S = MODE == PJ_CONP;
-  if (a.bath) {
-    if (a.bath & 1) Gb += sf.d0;
-    if (a.bath & 2) Gb += sf.d1;
-    if (a.bath & 4) Gb += sf.d2;
-    if (a.bath & 8) Gb -= sb.d0;
-    if (a.bath & 16) Gb -= sb.d1;
-    if (a.bath & 32) Gb -= sb.d2;
-    qT = fma(Gb, v.dCb_T, qT);
-    if (MODE == PJ_CONP) qS = (a.nbx * sb.R - a.nfx * sf.R) * v.invV;
-    qS = fma(Gb, v.dCb_S, qS);
-    has_S = true;
-  }
-  double q = Rn, Q = Rn, ubVc = ubV;
-  if (h.kind != PJ_ELEMENTARY) {
-    double M = v.Ctot;
-    for (int e = __ldg(&r->eff_lo), eh = __ldg(&r->eff_hi); e < eh; e++) {
-      if (!PJ_DBG_OK(m.dbg, e >= 0 && e < m.n_eff && __ldg(m.eff_sp + e) >= 0 && __ldg(m.eff_sp + e) < m.ns,
-                     PJ_DBG_EFF))
-        break;
-      M = fma(__ldg(m.eff_am1 + e), C[kTile * __ldg(m.eff_sp + e)], M);
-    }
-    const double ab = __ldg(&r->alpha_bath);
-    const double dMdT = ab * v.dCb_T;
-    const double dMdS = MODE == PJ_CONP ? (ab * v.Ctot - M) * v.invV : ab * (v.Ctot / v.P);
-    double cT = dMdT, c = M, RcM = Rn;
-    if (h.kind != PJ_THIRD_BODY) {
-      const int64_t l2rk = arrhenius_fixed(__ldg(&r->fA0), __ldg(&r->fB0), __ldg(&r->fT0), v.fx.L, v.fx.IT) - y;
-      const FalloffC fc =
-          falloff_derivatives(r, m.log_tab, h.kind, v.T, v.invT, v.lnT, v.fx.IT, exp2_51(l2rk), l2rk, M, dMdT);
-      c = fc.c;
-      cT = fc.cT;
-      RcM = Rn * fc.cM;
-    }
-    q = c * Rn;
-    Q = h.kind != PJ_THIRD_BODY ? fma(-RcM, M, q) : q;  // k_inf divides Pr: - Rn Pr dc/dPr
-    qT = fma(c, qT, Rn * cT);
-    qS = fma(c, qS, RcM * dMdS);
-    has_S = true;
-    ubVc = ubV * c;
-    double Bi = 0.0;
-    for (int e = __ldg(&r->eff_lo), eh = __ldg(&r->eff_hi); e < eh; e++) {
-      if (!PJ_DBG_OK(m.dbg, e >= 0 && e < m.n_eff, PJ_DBG_EFF)) break;
-      const int j = __ldg(m.eff_sp + e);
-      const double val = RcM * __ldg(m.eff_am1 + e);
-      if (j == bath) Bi -= val;
-      else red_add(grow + j * kTile, ubV * val);
-    }
-    v.gB = fma(ubV, Bi, v.gB);
-  }
-  if (a.bath) v.gB = fma(-ubVc, Gb, v.gB);
-  v.gT = fma(ub, qT, v.gT);
-  if (has_S) v.gS = fma(ub, qS, v.gS);
-
-  // production rates and amount gradients into the warp's rows
-  const double nq = dneg(q);
-#pragma unroll
-  for (int s = 0; s < 3; s++) {
-    if (s < h.nf) red_add(wrow + h.f[s], nq);
-    if (s < h.nb) red_add(wrow + h.b[s], q);
-  }
-  // slots in species order: the factors last to first (2A + B: A, B)
-  auto slot = [&](int sp, double d) { red_add(grow + kTile * sp, ubVc * d); };
-  const int nsf = shape_species(a.shape[0]), nsb = rev ? shape_species(a.shape[1]) : 0;
-#pragma unroll
-  for (int s = 0; s < 3; s++) {
-    if (s < nsf && !(a.bath >> s & 1)) slot(__ldg(&r->sp[s]), s == 0 ? sf.d0 : s == 1 ? sf.d1 : sf.d2);
-    if (s < nsb && !(a.bath >> (3 + s) & 1))
-      slot(__ldg(&r->sp[PJ_MAX_SP + s]), dneg(s == 0 ? sb.d0 : s == 1 ? sb.d1 : sb.d2));
-  }
+  vjp_sums(v, [&](int p, double& x) { part[p * kTile] = x; });
   return ub * Q;
 }
 
@@ -417,14 +464,15 @@ __global__ void __launch_bounds__(kVjpWarps * 32, kVjpCtas)
       const double T = S(vT), V = S(vV), invT = S(vInvT), invV = S(vInvV), lnT = S(vLnT), cdum = S(vCdum);
       const bool ok0 = flags[xOk * kTile] != 0;
       double acc = 0.0, den = 0.0, dden = 0.0;
-      bool fast = true;
+      const bool fast0 = flags[xFast * kTile] != 0;
+      bool fast = fast0;
       for (int k = warp; k < ns; k += W) {
         const double* cb = nasa_block(m, k, T);
         double cp, g, cp2, dcp;
         nasa_cp_g(cb, T, invT, lnT, cp, g);
         nasa_cp(cb, T, cp2, dcp);
-        G[k * kTile] = fixed_gibbs(m, g, fast);
-        H[k * kTile] = fixed_enthalpy(m, nasa_h(cb, T, invT), fast);
+        G[k * kTile] = gibbs_entry(m, g, fast);
+        H[k * kTile] = enthalpy_entry(m, nasa_h(cb, T, invT), fast);
         U[k * kTile] = ok0 ? u_wdot[(int64_t)k * ld + s] : 0.0;
         const double cx = MODE == PJ_CONP ? cp : cp - 1.0;
         if (k < bath) {
@@ -438,7 +486,7 @@ __global__ void __launch_bounds__(kVjpWarps * 32, kVjpCtas)
           S(vDcpB) = dcp;
         }
       }
-      if (!fast) flags[xFast * kTile] = 0;
+      if (fast0 && !fast) flags[xFast * kTile] = 2;  // found out of range part of the way
       Pw(warp, wAcc) = acc;
       Pw(warp, wDen) = den;
       Pw(warp, wDden) = dden;
@@ -446,7 +494,18 @@ __global__ void __launch_bounds__(kVjpWarps * 32, kVjpCtas)
     __syncthreads();
 
     // C: bath gas by subtraction, validity (an invalid state's cotangents
-    // become zero), the energy equation's denominator and its derivatives
+    // become zero), the energy equation's denominator and its derivatives; the
+    // entries of a state found out of range, again
+    if (flags[xFast * kTile] == 2) {
+      const double T = S(vT), invT = S(vInvT), lnT = S(vLnT);
+      for (int k = warp; k < ns; k += W) {
+        const double* cb = nasa_block(m, k, T);
+        double cp, g;
+        nasa_cp_g(cb, T, invT, lnT, cp, g);
+        G[k * kTile] = g;
+        H[k * kTile] = nasa_h(cb, T, invT);
+      }
+    }
     if (warp == 0) {
       const double Ctot = S(vCtot), P = S(vP), invT = S(vInvT), invV = S(vInvV);
       const double acc = sum_parts(wAcc);
@@ -471,48 +530,26 @@ __global__ void __launch_bounds__(kVjpWarps * 32, kVjpCtas)
     }
     __syncthreads();
     const bool ok = flags[xOk * kTile] != 0;
-    const bool fast_tile = __all_sync(0xffffffffu, flags[xFast * kTile] != 0);  // the same in every warp
-    if (!fast_tile) {
-      const double T = S(vT), invT = S(vInvT);
-      for (int k = warp; k < ns; k += W) H[k * kTile] = nasa_h(nasa_block(m, k, T), T, invT);
-      __syncthreads();
-    }
+    const bool fast = flags[xFast * kTile] == 1;
+    const bool fast_tile = __all_sync(0xffffffffu, fast);  // the same in every warp
 
     // D: the warp's reactions, in a fixed order
     {
-      VjpVars v;
-      v.T = S(vT);
-      v.V = S(vV);
-      v.P = S(vP);
-      v.invT = S(vInvT);
-      v.invV = S(vInvV);
-      v.lnT = S(vLnT);
-      v.lnP = S(vLnP);
-      v.Ctot = S(vCtot);
-      v.dCb_T = S(vDCbT);
-      v.dCb_S = S(vDCbS);
-      v.uTE = ok ? S(vUT) * S(vIden) * (RU * v.T) : 0.0;
-      v.fx.L = (uint64_t)__double_as_longlong(S(vL));
-      v.fx.IT = (uint64_t)__double_as_longlong(S(vIT));
-      v.fx.LP = __double_as_longlong(S(vLP));
-      v.fx.fast = flags[xFast * kTile] != 0;
-      v.gT = v.gS = v.gB = 0.0;
+      double* const my_sums = part + warp * kVjpPart * kTile;
+      VjpVars v = vjp_vars(sc, true, ok);
+      vjp_sums(v, [&](int p, double& x) { x = my_sums[(wAcc + p) * kTile] = my_sums[(wGT + p) * kTile] = 0.0; });
       for (int i = warp; i < nr; i += W) {
         const Rxn* __restrict__ r = m.rxn + i;
         const RxnHead h = load_head(r);
         double w;
-        if (fast_tile && h.lean) {
-          w = lean_vjp<MODE>(m, r, h, base, v, wrow, grow);
-        } else {
-          const auto g = general_vjp<MODE, SPECIAL>(m, base, r, i < m.nr_plain, v, fast_tile, wrow, grow);
-          v = g.v;
-          w = g.wq;
-        }
+        if (fast_tile && h.lean) w = lean_vjp<MODE, false>(m, r, h, base, v, wrow, grow);
+        else if (h.lean) w = mixed_vjp<MODE>(m, base, sc, my_sums, r, fast, ok, wrow, grow);
+        else w = general_vjp<MODE, SPECIAL>(m, base, sc, my_sums, r, i < m.nr_plain, fast, ok, wrow, grow);
         wq[(size_t)i * kTile + lane] = ok ? w : 0.0;
       }
-      Pw(warp, wGT) = v.gT;
-      Pw(warp, wGS) = v.gS;
-      Pw(warp, wGB) = v.gB;
+      vjp_sums(v, [&](int p, double& x) {
+        my_sums[(wGT + p) * kTile] = (my_sums[(wGT + p) * kTile] + x) + my_sums[(wAcc + p) * kTile];
+      });
     }
     __syncthreads();
 
@@ -525,7 +562,7 @@ __global__ void __launch_bounds__(kVjpWarps * 32, kVjpCtas)
         double cp, dcp;
         nasa_cp(nasa_block(m, k, T), T, cp, dcp);
         const double cx = RU * (MODE == PJ_CONP ? cp : cp - 1.0);
-        const double hk = fast_tile ? fixed51_to_double(__double_as_longlong(H[k * kTile])) : H[k * kTile];
+        const double hk = fast ? fixed51_to_double(__double_as_longlong(H[k * kTile])) : H[k * kTile];
         const double wk = sum_rows(0, k);
         G[k * kTile] = cx;
         num = fma(MODE == PJ_CONP ? hk : hk - 1.0, wk, num);

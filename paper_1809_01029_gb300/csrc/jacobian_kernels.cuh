@@ -119,6 +119,7 @@ enum CoopSc {
 enum CoopPart { pAcc, pDen, pDden, pNum, pSum, pOm, pAT_T, pAT_S, pAS_T, pAS_S, pATB, pASB, pWb, kCoopPart };
 
 // per-state flags (int): valid T, V, P; valid state; fixed-point rate constants
+// (1; 0: T out of range; 2: some g_k or h_k)
 enum CoopFlag { fOk0, fOk, fFast, kCoopFlag };
 
 // per-state arrays C_k, g_k/RT then Cx_k, h_k/RT of a tile: [3][Ns][32] doubles
@@ -144,6 +145,59 @@ __device__ __forceinline__ void st_zero_evict_last(double* a, uint64_t pol) {
 }
 __device__ __forceinline__ void st_zero_evict_last(float* a, uint64_t pol) {
   asm volatile("st.global.L2::cache_hint.b32 [%0], 0, %1;" ::"l"(a), "l"(pol) : "memory");
+}
+
+// What a reaction needs of its state (sc: this lane's scalars of the tile), and
+// the warp's sums over its reactions.
+template <typename DT>
+__device__ __forceinline__ void coop_load(JacVars<DT>& v, const double* __restrict__ sc, bool fast) {
+  auto S = [&](int i) { return sc[i * kCoopTile]; };
+  v.T = S(cT);
+  v.V = S(cV);
+  v.P = S(cP);
+  v.invT = S(cInvT);
+  v.lnT = S(cLnT);
+  v.lnP = S(cLnP);
+  v.Ctot = S(cCtot);
+  v.invT2 = v.invT * v.invT;
+  v.invV = S(cInvV);
+  v.fx.L = (uint64_t)__double_as_longlong(S(cL));
+  v.fx.IT = (uint64_t)__double_as_longlong(S(cIT));
+  v.fx.LP = __double_as_longlong(S(cLP));
+  v.fx.fast = fast;
+  v.dCb_T = S(cDCbT);
+  v.dCb_S = S(cDCbS);
+}
+template <typename DT, class F>
+__device__ __forceinline__ void coop_sums(JacVars<DT>& v, F&& f) {
+  f(pAT_T, v.AT_T);
+  f(pAT_S, v.AT_S);
+  f(pAS_T, v.AS_T);
+  f(pAS_S, v.AS_S);
+  f(pATB, v.ATB);
+  f(pASB, v.ASB);
+}
+
+// Any reaction at any state, out of line; h_k/RT as enthalpy_entry stored it.
+// It takes the state from and leaves its sums (as DT, in part: this lane's of
+// the warp) in shared memory: with both passed by value a call cost as much as
+// the reaction (every reaction type, 16411 states: 1172 us by value, 1104; CSR at
+// 53 species with every tile on this path, 131072 states: 16.9 ms, 12.9).
+template <int MODE, int FMT, typename DT, bool NEWTON, bool SPECIAL>
+__device__ __noinline__ static void general_jacobian(const DevMech& m, double* base, const double* sc, double* part,
+                                                     const JacOut<DT> o, int i, bool fast) {
+  StateArrays A;
+  A.ns = m.ns;
+  A.base = base;
+  A.stride = kCoopTile;
+  JacVars<DT> v;
+  coop_load(v, sc, fast);
+  coop_sums(v, [&](int p, DT& x) { x = *reinterpret_cast<DT*>(part + p * kCoopTile); });
+  v.w_bath = part[pWb * kCoopTile];
+  if (!SPECIAL || i < m.nr_plain) jac_reaction<MODE, FMT, DT, false, false, NEWTON>(m, A, v, o, i, 0u, fast);
+  else jac_reaction<MODE, FMT, DT, true, false, NEWTON>(m, A, v, o, i, 0u, fast);
+  coop_sums(v, [&](int p, DT& x) { *reinterpret_cast<DT*>(part + p * kCoopTile) = x; });
+  part[pWb * kCoopTile] = v.w_bath;
 }
 
 // Blocks of up to 20 warps: 96 registers a thread (10 warps in each of two blocks
@@ -274,15 +328,16 @@ __global__ void __launch_bounds__(kCoopWarpsMax * 32, 1)
       const double T = S(cT), V = S(cV), invT = S(cInvT), lnT = S(cLnT), cdum = S(cCdum);
       const bool ok0 = F(fOk0) != 0;
       double acc = 0.0, den = 0.0, dden = 0.0;
-      bool fast = true;
+      const bool fast0 = F(fFast) != 0;
+      bool fast = fast0;
       for (int k = warp; k < ns; k += W) {
         const double* cb = nasa_block(m, k, T);
         double cp, g, cp2, dcp;
         nasa_cp_g(cb, T, invT, lnT, cp, g);
         nasa_cp(cb, T, cp2, dcp);
         const double h = nasa_h(cb, T, invT);
-        A.at(aG, k) = fixed_gibbs(m, g, fast);
-        A.at(aH, k) = fixed_enthalpy(m, h, fast);
+        A.at(aG, k) = gibbs_entry(m, g, fast);
+        A.at(aH, k) = enthalpy_entry(m, h, fast);
         const double cx = MODE == PJ_CONP ? cp : cp - 1.0;
         if (k < bath) {
           const double c = ok0 ? concentration(phi[(int64_t)(k + 2) * ld + s], V, S(cInvV)) : cdum;
@@ -295,7 +350,7 @@ __global__ void __launch_bounds__(kCoopWarpsMax * 32, 1)
           S(cDcpB) = dcp;
         }
       }
-      if (!fast) F(fFast) = 0;
+      if (fast0 && !fast) F(fFast) = 2;  // found out of range part of the way
       Pw(warp, pAcc) = acc;
       Pw(warp, pDen) = den;
       Pw(warp, pDden) = dden;
@@ -303,7 +358,18 @@ __global__ void __launch_bounds__(kCoopWarpsMax * 32, 1)
     __syncthreads();
 
     // C: bath gas by subtraction, validity, denominator of the energy
-    // equation and the bath-gas derivatives (warp 0)
+    // equation and the bath-gas derivatives (warp 0); the entries of a state
+    // found out of range, again
+    if (F(fFast) == 2) {
+      const double T = S(cT), invT = S(cInvT), lnT = S(cLnT);
+      for (int k = warp; k < ns; k += W) {
+        const double* cb = nasa_block(m, k, T);
+        double cp, g;
+        nasa_cp_g(cb, T, invT, lnT, cp, g);
+        A.at(aG, k) = g;
+        A.at(aH, k) = nasa_h(cb, T, invT);
+      }
+    }
     if (warp == 0) {
       const double Ctot = S(cCtot), P = S(cP), invT = S(cInvT), invV = S(cInvV);
       const double acc = sum_parts(pAcc);
@@ -331,54 +397,41 @@ __global__ void __launch_bounds__(kCoopWarpsMax * 32, 1)
     }
     __syncthreads();
 
-    // a tile with a state outside the fixed point's range takes the general
-    // path, with h_k/RT in FP64
-    const bool fast_tile = __all_sync(0xffffffffu, F(fFast) != 0) && ld < (1 << 28);  // the same in every warp
-    if (!fast_tile) {
-      const double T = S(cT), invT = S(cInvT);
-      for (int k = warp; k < ns; k += W) A.at(aH, k) = nasa_h(nasa_block(m, k, T), T, invT);
-      __syncthreads();
-    }
+    // a tile with a state outside the fixed point's range takes the general path
+    const bool fast = F(fFast) == 1;
+    const bool fast_tile = __all_sync(0xffffffffu, fast) && ld < (1 << 28);  // the same in every warp
 
     // D: the warp's reactions
     const bool w = F(fOk) != 0;
     const JacOut<DT> o{J, wrow, ld, s, w, NEWTON && w ? DT(-hstep[s] * gamma) : DT(0)};
     {
+      double* const my_part = part + warp * kCoopPart * kCoopTile;
       JacVars<DT> v;
-      v.T = S(cT);
-      v.V = S(cV);
-      v.P = S(cP);
-      v.invT = S(cInvT);
-      v.lnT = S(cLnT);
-      v.lnP = S(cLnP);
-      v.Ctot = S(cCtot);
-      v.invT2 = v.invT * v.invT;
-      v.invV = S(cInvV);
-      v.fx.L = (uint64_t)__double_as_longlong(S(cL));
-      v.fx.IT = (uint64_t)__double_as_longlong(S(cIT));
-      v.fx.LP = __double_as_longlong(S(cLP));
-      v.fx.fast = F(fFast) != 0;
-      v.dCb_T = S(cDCbT);
-      v.dCb_S = S(cDCbS);
-      v.AT_T = v.AT_S = v.AS_T = v.AS_S = v.ATB = v.ASB = DT(0);
-      v.w_bath = 0.0;
+      coop_load(v, sc, true);
+      coop_sums(v, [&](int p, DT& x) { x = *reinterpret_cast<DT*>(my_part + p * kCoopTile) = DT(0); });
+      v.w_bath = my_part[pWb * kCoopTile] = 0.0;
       // reactions are handed out one at a time (a shared counter), so that
       // warps finish the phase within about one reaction of each other
+      int again = 0;
       for (int i = warp; i < m.nr;) {
         const RxnHead h = load_head(m.rxn + i);
+        if constexpr (!NEWTON) {
+          // the state's values loaded for each reaction: kept in registers over
+          // the loop they cost the short path spills (CSR at 53 species, 262144
+          // states: 10.36 ms, 9.98; the FP32 Newton matrix is better without)
+          asm volatile("" : "+r"(again));
+          coop_load(v, sc + again, true);
+        }
         if (fast_tile && h.lean) lean_jacobian<MODE, FMT, DT, NEWTON>(m, m.rxn + i, h, A.base, v, o);
-        else v = general_jacobian<MODE, FMT, DT, NEWTON, SPECIAL>(m, A, v, o, i, fast_tile);
+        else general_jacobian<MODE, FMT, DT, NEWTON, SPECIAL>(m, A.base, sc, my_part, o, i, fast);
         int nx = 0;
         if (lane == 0) nx = atomicAdd(next_rxn, 1);
         i = __shfl_sync(0xffffffffu, nx, 0);
       }
-      Pw(warp, pAT_T) = double(v.AT_T);
-      Pw(warp, pAT_S) = double(v.AT_S);
-      Pw(warp, pAS_T) = double(v.AS_T);
-      Pw(warp, pAS_S) = double(v.AS_S);
-      Pw(warp, pATB) = double(v.ATB);
-      Pw(warp, pASB) = double(v.ASB);
-      Pw(warp, pWb) = v.w_bath;
+      coop_sums(v, [&](int p, DT& x) {
+        my_part[p * kCoopTile] = double(x + *reinterpret_cast<DT*>(my_part + p * kCoopTile));
+      });
+      my_part[pWb * kCoopTile] += v.w_bath;
     }
     __syncthreads();
 
@@ -388,7 +441,7 @@ __global__ void __launch_bounds__(kCoopWarpsMax * 32, 1)
       double num = 0.0, sumCxW = 0.0, Om = 0.0;
       for (int k = warp; k < ns; k += W) {
         const double wb = k == bath ? sum_parts(pWb) : 0.0;
-        const double hk = fast_tile ? fixed51_to_double(__double_as_longlong(A.at(aH, k))) : A.at(aH, k);
+        const double hk = fast ? fixed51_to_double(__double_as_longlong(A.at(aH, k))) : A.at(aH, k);
         A.at(aG, k) = jac_species<MODE, FMT, DT, NEWTON>(m, k, T, V, hk, wb, o, num, sumCxW, Om);
       }
       Pw(warp, pNum) = num;

@@ -15,7 +15,8 @@ namespace pj {
 
 // Per-state inputs of the fixed-point rate constants (fixed_math.cuh).  fast:
 // they may be used (128 K <= T < 65536 K and every |g_k/RT| in range, see
-// fixed_gibbs); other states take the FP64 path, out of line.
+// gibbs_entry); other states take the FP64 path (rate_constants_fp64), out of
+// line.
 struct FixedState {
   uint64_t L, IT;  // log2(T) 2^59, 2^70 / T
   int64_t LP;      // log2(P_std / (R T)) 2^51
@@ -48,18 +49,30 @@ __device__ __forceinline__ void temperature_terms(const DevMech& m, double T, do
   f.IT = __double2ull_rn(invT * 0x1p70) + (uint64_t)__double2ll_rn(fma(-T, invT, 1.0) * (invT * 0x1p70));
 }
 
-// g_k/RT as log2 units 2^51 (stored where the FP64 value would be); clears
-// fast when it is out of range
-__device__ __forceinline__ double fixed_gibbs(const DevMech& m, double g, bool& fast) {
+// What the reactions read of g_k/RT: log2 units 2^51 at a state within the
+// fixed point's range, else the value itself.  Clears fast when g is out of
+// range; entries made before that have to be made again.
+__device__ __forceinline__ double gibbs_entry(const DevMech& m, double g, bool& fast) {
   fast = fast && ((uint32_t)__double2hiint(g) & 0x7fffffffu) < m.fx_g_hi;
-  return __longlong_as_double(__double2ll_rn(g * (1.4426950408889634074 * 0x1p51)));
+  return fast ? __longlong_as_double(__double2ll_rn(g * (1.4426950408889634074 * 0x1p51))) : g;
 }
 
-// h_k/RT, 2^51 (stored where the FP64 value would be); clears fast when it is
-// out of range
-__device__ __forceinline__ double fixed_enthalpy(const DevMech& m, double h, bool& fast) {
+// The same of h_k/RT: units 2^51.
+__device__ __forceinline__ double enthalpy_entry(const DevMech& m, double h, bool& fast) {
   fast = fast && ((uint32_t)__double2hiint(h) & 0x7fffffffu) < m.fx_h_hi;
-  return __longlong_as_double(__double2ll_rn(h * 0x1p51));
+  return fast ? __longlong_as_double(__double2ll_rn(h * 0x1p51)) : h;
+}
+
+// g_k/RT of every species as it is: a state that was found out of range part
+// of the way.  Out of line.
+template <class SA>
+__device__ __noinline__ static void gibbs_entries_again(const DevMech& m, const SA A, int aG, double T, double invT,
+                                                        double lnT) {
+  for (int k = 0; k < m.ns; k++) {
+    double cp, g;
+    nasa_cp_g(nasa_block(m, k, T), T, invT, lnT, cp, g);
+    A.at(aG, k) = g;
+  }
 }
 
 // 2^(y 2^-51) as a double
@@ -141,10 +154,10 @@ __device__ __forceinline__ double inverse_1p(double Pr) {
 }
 
 // Troe / SRI broadening factor F(T, Pr).  With derivatives also returns FxPr
-// = Pr dF/dPr (at fixed T) and FT = dF/dT (at fixed Pr).  For states within
-// the fixed point's range (128 <= T < 65536, IT = 2^70 / T); l2Pr = log2(Pr)
-// 2^51; ok = false, with nothing returned, when F_cent (or Z) is not a
-// positive normal number.
+// = Pr dF/dPr (at fixed T) and FT = dF/dT (at fixed Pr).  fxr: which of Troe's
+// exponents fit the fixed point (Rxn::troe_fx; the third also needs 128 <= T,
+// IT = 2^70 / T); l2Pr = log2(Pr) 2^51; ok = false, with nothing returned, when
+// F_cent (or Z) is not a positive normal number.
 //
 // Troe: with D = N - 0.14 xc and S = D^2 + xc^2, log10 F = L g, g = D^2 / S
 // (1 / (1 + (xc/D)^2)), so that F and its derivatives take one reciprocal:
@@ -153,7 +166,8 @@ __device__ __forceinline__ double inverse_1p(double Pr) {
 // 53-species Jacobian's and 45 % of its source terms'.
 template <bool DERIV>
 __device__ __forceinline__ double falloff_F(const LogEntry* __restrict__ log_tab, const Rxn* __restrict__ r, int kind,
-                                            double T, double invT, double lnT, uint64_t IT, int64_t l2Pr, bool& ok,
+                                            double T, double invT, double lnT, uint64_t IT, int fxr, int64_t l2Pr,
+                                            bool& ok,
                                             double& FxPr, double& FT) {
   FxPr = 0.0;
   FT = 0.0;
@@ -161,7 +175,6 @@ __device__ __forceinline__ double falloff_F(const LogEntry* __restrict__ log_tab
   if (kind == PJ_TROE) {
     const double a = __ldg(&r->fp[0]), iT3 = __ldg(&r->fp[1]), iT1 = __ldg(&r->fp[2]);
     const double T2 = __ldg(&r->fp[3]);
-    const int fxr = __ldg(&r->troe_fx);
     const uint64_t tb = (uint64_t)__double_as_longlong(T);
     const uint64_t X = ((tb << 11) | 0x8000000000000000ull) >> (1039 - (int)(tb >> 52));  // T 2^47
     const double e3 = fxr & 1 ? exp2_51(-(int64_t)mulhi_approx(__ldg(&r->tT3), X)) : pj_exp(-T * iT3);
@@ -217,8 +230,8 @@ __device__ __forceinline__ double falloff_F(const LogEntry* __restrict__ log_tab
   return 1.0;  // Lindemann
 }
 
-// The same with the library's logarithm, for any Pr and F_cent (zero, negative,
-// not finite, or a state outside the fixed point's range).  Out of line.
+// The same with the library's logarithm, for any Pr and F_cent (zero, subnormal,
+// negative or not finite).  Out of line.
 __device__ __noinline__ static double falloff_F_library(const Rxn* __restrict__ r, int kind, double T, double invT,
                                                         double lnT, double Pr, double& FxPr, double& FT) {
   FxPr = 0.0;
@@ -460,45 +473,44 @@ struct RateK {
   int64_t l2rk;
 };
 
-// sum_k nu_k g_k/RT of a reaction, from the thermo polynomials (states
-// outside the fixed point's range)
-__device__ __noinline__ static double gibbs_sum(const double* __restrict__ nasa, const Rxn* __restrict__ r, double T,
-                                                double invT, double lnT) {
-  double dg = 0.0;
-  for (int a = 0; a < 2 * PJ_MAX_SP; a++) {
-    const bool react = a < PJ_MAX_SP;
-    if (react ? a >= __ldg(&r->nreac) : a - PJ_MAX_SP >= __ldg(&r->nprod)) continue;
-    const double* b = nasa + (size_t)__ldg(&r->sp[a]) * NASA_STRIDE;
-    if (!(T < __ldg(b + 14))) b += NASA_RANGE;
-    double cp, h, sr;
-    nasa_eval(b, T, invT, lnT, cp, h, sr);
-    dg = fma(react ? -__ldg(&r->nud[a]) : __ldg(&r->nud[a]), h - sr, dg);
-  }
-  return dg;
-}
+// l2rk where log2(rk) is not known in fixed point
+constexpr int64_t kNoLog2 = INT64_MIN;
 
-// The same in FP64 with the library's range: states outside the fixed
-// point's range.  Out of line.
-template <bool GEN>
-__device__ __noinline__ static void rate_constants_library(const DevMech& m, const Rxn* __restrict__ r, double T,
-                                                           double invT, double lnT, double lnP, RateK& k) {
-  const int kind = __ldg(&r->kind), rev = __ldg(&r->rev);
+// The rate constants in FP64, from the stored g_k/RT: states outside the
+// fixed point's range (A by value: its address taken would put it in memory).
+template <bool GEN, class SA>
+__device__ __noinline__ static RateK rate_constants_fp64(const DevMech& m, const SA A, int aG, const Rxn* __restrict__ r,
+                                                         int kind, int rev, double lnT, double invT, double lnP) {
+  RateK k;
   const double lninf = fma(__ldg(&r->beta), lnT, __ldg(&r->lnA)) - __ldg(&r->theta) * invT;
-  const double ln0 = fma(__ldg(&r->beta0), lnT, __ldg(&r->lnA0)) - __ldg(&r->theta0) * invT;
-  double lnkf = lninf, u0, u1;
+  double lnkf = lninf;
+  k.rk = 0.0;
+  k.l2rk = kNoLog2;
+  if (kind >= PJ_LINDEMANN && kind <= PJ_SRI) {
+    const double ln0 = fma(__ldg(&r->beta0), lnT, __ldg(&r->lnA0)) - __ldg(&r->theta0) * invT;
+    k.rk = pj_exp(ln0 - lninf);
+    if (GEN && __ldg(&r->chem)) lnkf = ln0;
+  }
+  double u0, u1;
   if (GEN && kind >= PJ_PLOG) lnkf = lnk_pdep<false>(m, r, kind, lnT, invT, lnP, u0, u1);
-  else if (GEN && __ldg(&r->chem)) lnkf = ln0;
-  k.kf = exp(lnkf);
+  k.kf = pj_exp(lnkf);
   k.kr = 0.0;
   if (GEN && rev == 2) {
     const double* __restrict__ rt = m.tab + __ldg(&r->tab_lo);
-    k.kr = exp(fma(__ldg(rt + 1), lnT, __ldg(rt)) - __ldg(rt + 2) * invT);
+    k.kr = pj_exp(fma(__ldg(rt + 1), lnT, __ldg(rt)) - __ldg(rt + 2) * invT);
   } else if (rev) {
-    // kr = kf / Kc with Kc = exp(-dg) (P_std / R T)^dnu
-    k.kr = exp(lnkf + gibbs_sum(m.nasa, r, T, invT, lnT) - __ldg(&r->dnu) * (m.log_pstd_over_r - lnT));
+    // kr = kf / Kc with Kc = exp(-sum nu g) (P_std / R T)^dnu
+    const int nre = __ldg(&r->nreac), npr = __ldg(&r->nprod);
+    double dg = 0.0;
+#pragma unroll
+    for (int a = 0; a < PJ_MAX_SP; a++) {
+      if (a < nre) dg = fma(-__ldg(&r->nud[a]), A.at(aG, __ldg(&r->sp[a])), dg);
+      if (a < npr) dg = fma(__ldg(&r->nud[PJ_MAX_SP + a]), A.at(aG, __ldg(&r->sp[PJ_MAX_SP + a])), dg);
+    }
+    if (__ldg(&r->head.dnu_i) != 0) dg = fma(-__ldg(&r->dnu), m.log_pstd_over_r - lnT, dg);
+    k.kr = pj_exp(lnkf + dg);
   }
-  k.rk = kind >= PJ_LINDEMANN && kind <= PJ_SRI ? exp(ln0 - lninf) : 0.0;
-  k.l2rk = 0;
+  return k;
 }
 
 // The exponents are sums of 64-bit fixed-point terms (the sum over the
@@ -506,13 +518,10 @@ __device__ __noinline__ static void rate_constants_library(const DevMech& m, con
 // FP64 terms of size 32 to 64 round at 2^-48.
 template <bool GEN = true, class SA>
 __device__ __forceinline__ RateK rate_constants(const DevMech& m, const SA& A, int aG, const Rxn* __restrict__ r,
-                                                int kind, int rev, int nre, int npr, const FixedState& fx, double T,
+                                                int kind, int rev, int nre, int npr, const FixedState& fx,
                                                 double lnT, double invT, double lnP) {
+  if (!fx.fast) return rate_constants_fp64<GEN>(m, A, aG, r, kind, rev, lnT, invT, lnP);
   RateK k;
-  if (!fx.fast) {
-    rate_constants_library<GEN>(m, r, T, invT, lnT, lnP, k);
-    return k;
-  }
   int64_t y = arrhenius_fixed(__ldg(&r->head.fA), __ldg(&r->head.fB), __ldg(&r->head.fT), fx.L, fx.IT);
   k.rk = 0.0;
   k.l2rk = 0;
@@ -549,20 +558,33 @@ __device__ __forceinline__ RateK rate_constants(const DevMech& m, const SA& A, i
   return k;
 }
 
+// The broadening factor of Pr = rk M and its derivatives (falloff_F); l2rk:
+// log2(rk) 2^51.  MIXED: or kNoLog2, at any temperature.
+template <bool DERIV, bool MIXED>
+__device__ __forceinline__ void falloff_broadening(const Rxn* __restrict__ r, const LogEntry* __restrict__ log_tab,
+                                                   int kind, uint64_t IT, double T, double invT, double lnT,
+                                                   int64_t l2rk, double M, double Pr, double& F, double& FxPr,
+                                                   double& FT) {
+  F = 1.0;
+  FxPr = FT = 0.0;
+  if (kind == PJ_LINDEMANN) return;
+  bool ok = true;
+  const bool known = !MIXED || l2rk != kNoLog2;
+  int64_t l2Pr = log2_51(log_tab, known ? M : Pr, ok);
+  if (known) l2Pr += l2rk;
+  const int fits = !MIXED || IT != 0 ? 7 : T < 65536.0 && T >= 1.0 ? 3 : 0;
+  if (ok) F = falloff_F<DERIV>(log_tab, r, kind, T, invT, lnT, IT, __ldg(&r->troe_fx) & fits, l2Pr, ok, FxPr, FT);
+  if (!ok) F = falloff_F_library(r, kind, T, invT, lnT, Pr, FxPr, FT);
+}
+
 // Pressure modification of a falloff reaction: Pr and, in F, FxPr, FT, the
-// broadening factor and its derivatives (falloff_F).
+// broadening factor and its derivatives.
 template <bool DERIV>
 __device__ __forceinline__ double falloff_Pr_F(const DevMech& m, const Rxn* __restrict__ r, int kind,
                                                const FixedState& fx, double T, double invT, double lnT,
                                                const RateK& k, double M, double& F, double& FxPr, double& FT) {
   const double Pr = k.rk * M;
-  F = 1.0;
-  FxPr = FT = 0.0;
-  if (kind == PJ_LINDEMANN) return Pr;
-  bool ok = fx.fast;
-  const int64_t l2Pr = k.l2rk + log2_51(m.log_tab, M, ok);
-  if (ok) F = falloff_F<DERIV>(m.log_tab, r, kind, T, invT, lnT, fx.IT, l2Pr, ok, FxPr, FT);
-  if (!ok) F = falloff_F_library(r, kind, T, invT, lnT, Pr, FxPr, FT);
+  falloff_broadening<DERIV, true>(r, m.log_tab, kind, fx.IT, T, invT, lnT, k.l2rk, M, Pr, F, FxPr, FT);
   return Pr;
 }
 

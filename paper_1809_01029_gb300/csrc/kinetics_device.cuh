@@ -55,16 +55,7 @@ __device__ __forceinline__ const double* nasa_block(const DevMech& m, int k, dou
   return T < tmid ? b : b + NASA_RANGE;
 }
 
-// cp/R, h/RT, s/R (NASA 7-coefficient polynomials).
-__device__ __forceinline__ void nasa_eval(const double* __restrict__ c, double T, double invT, double lnT,
-                                          double& cp, double& h, double& s) {
-  const double a0 = __ldg(c + 0), a1 = __ldg(c + 1), a2 = __ldg(c + 2), a3 = __ldg(c + 3), a4 = __ldg(c + 4);
-  cp = fma(fma(fma(fma(a4, T, a3), T, a2), T, a1), T, a0);
-  h = fma(fma(fma(fma(__ldg(c + 10), T, __ldg(c + 9)), T, __ldg(c + 8)), T, __ldg(c + 7)), T, a0) + __ldg(c + 5) * invT;
-  s = fma(a0, lnT, fma(fma(fma(fma(__ldg(c + 13), T, __ldg(c + 12)), T, __ldg(c + 11)), T, a1), T, __ldg(c + 6)));
-}
-
-// cp/R and g/RT = h/RT - s/R as one polynomial
+// cp/R and g/RT = h/RT - s/R as one polynomial (NASA 7-coefficient form)
 __device__ __forceinline__ void nasa_cp_g(const double* __restrict__ c, double T, double invT, double lnT, double& cp,
                                           double& g) {
   const double a0 = __ldg(c + 0), a1 = __ldg(c + 1), a2 = __ldg(c + 2), a3 = __ldg(c + 3), a4 = __ldg(c + 4);

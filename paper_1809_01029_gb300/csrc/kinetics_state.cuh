@@ -24,12 +24,14 @@ __device__ __forceinline__ void source_state(const DevMech& m, const SA& A, cons
   double* __restrict__ wrow = out + 2 * ld + s;   // wdot_k accumulates at wrow[k*ld]
   for (int k = 0; k < ns - 1; k++) wrow[(int64_t)k * ld] = 0.0;
   double den = 0.0;
+  const bool fast0 = st.fx.fast;
   for (int k = 0; k < ns; k++) {
     double cp, g;
     nasa_cp_g(nasa_block(m, k, T), T, invT, lnT, cp, g);
-    A.at(aG, k) = fixed_gibbs(m, g, st.fx.fast);
+    A.at(aG, k) = gibbs_entry(m, g, st.fx.fast);
     den = fma(A.at(aC, k), MODE == PJ_CONP ? cp : cp - 1.0, den);
   }
+  if (fast0 && !st.fx.fast) gibbs_entries_again(m, A, aG, T, invT, lnT);
   den *= RU;
   double w_bath = 0.0;
 
@@ -43,7 +45,7 @@ __device__ __forceinline__ void source_state(const DevMech& m, const SA& A, cons
     const Rxn* __restrict__ r = m.rxn + i;
     const int kind = __ldg(&r->kind);
     const int nre = __ldg(&r->nreac), npr = __ldg(&r->nprod), rev = __ldg(&r->rev);
-    const RateK k = rate_constants<GEN>(m, A, aG, r, kind, rev, nre, npr, st.fx, T, lnT, invT, st.lnP);
+    const RateK k = rate_constants<GEN>(m, A, aG, r, kind, rev, nre, npr, st.fx, lnT, invT, st.lnP);
     double dmy[PJ_MAX_SP];
     const double Rf = side_rate<false>(A, aC, r, 0, __ldg(&r->shape[0]), nre, k.kf, dmy);
     const double Rr = rev ? side_rate<false>(A, aC, r, PJ_MAX_SP, __ldg(&r->shape[1]), npr, k.kr, dmy) : 0.0;
@@ -192,7 +194,7 @@ __device__ __forceinline__ void jac_reaction(const DevMech& m, const SA& A, JacV
   double dlnkf_d, dlnP_d, dlnkinf_d;
   ln_kf_derivatives<GEN>(m, r, kind, lnT, invT, invT2, v.lnP, dlnkf_d, dlnP_d, dlnkinf_d);
   const DT dlnkf = DT(dlnkf_d);
-  const RateK rk = rate_constants<GEN>(m, A, aG, r, kind, rev, nre, npr, v.fx, T, lnT, invT, v.lnP);
+  const RateK rk = rate_constants<GEN>(m, A, aG, r, kind, rev, nre, npr, v.fx, lnT, invT, v.lnP);
   const double kf = rk.kf, kr = rk.kr;
   double dh = 0.0;
   if (TM) __syncwarp();
@@ -590,13 +592,14 @@ __device__ __forceinline__ void jacobian_state(const DevMech& m, const SA& A,
 
   // thermo, energy-equation denominator D = sum_k C_k Cx_k and dD/dT
   double den = 0.0, dden_T = 0.0, Cx_bath = 0.0;
+  const bool fast0 = st.fx.fast;
   for (int k = 0; k < ns; k++) {
     const double* cb = nasa_block(m, k, T);
     double cp, g, cp2, dcp;
     nasa_cp_g(cb, T, invT, lnT, cp, g);
     nasa_cp(cb, T, cp2, dcp);
     const double h = nasa_h(cb, T, invT);
-    A.at(aG, k) = fixed_gibbs(m, g, st.fx.fast);
+    A.at(aG, k) = gibbs_entry(m, g, st.fx.fast);
     if (TM) tmem_st_f64(tm_row + 2u * (uint32_t)k, h);
     else A.at(aH, k) = h;
     const double Ck = A.at(aC, k);
@@ -605,6 +608,8 @@ __device__ __forceinline__ void jacobian_state(const DevMech& m, const SA& A,
     dden_T = fma(Ck, dcp, dden_T);
     if (k == bath) Cx_bath = RU * cx;
   }
+  if (fast0 && !st.fx.fast) gibbs_entries_again(m, A, aG, T, invT, lnT);
+  if (TM) __syncwarp();
   if (TM) tmem_wait_st();
   den *= RU;
   const double C_bath = A.at(aC, bath);

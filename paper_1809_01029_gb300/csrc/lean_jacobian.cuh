@@ -18,33 +18,19 @@
 
 namespace pj {
 
-// Any reaction at any state, out of line (by value: the caller's accumulators
-// stay in registers).
-template <int MODE, int FMT, typename DT, bool NEWTON, bool SPECIAL>
-__device__ __noinline__ static JacVars<DT> general_jacobian(const DevMech& m, const StateArrays A, JacVars<DT> v,
-                                                            const JacOut<DT> o, int i, bool hfix) {
-  if (!SPECIAL || i < m.nr_plain) jac_reaction<MODE, FMT, DT, false, false, NEWTON>(m, A, v, o, i, 0u, hfix);
-  else jac_reaction<MODE, FMT, DT, true, false, NEWTON>(m, A, v, o, i, 0u, hfix);
-  return v;
-}
-
 // Falloff blending c = Pr / (1 + Pr) F and its derivatives: cM = dc/dM at
 // fixed T, cT = dc/dT with M moving by dMdT.  Out of line, as falloff_factor.
 struct FalloffC {
   double c, cM, cT;
 };
+template <bool MIXED>
 __device__ __noinline__ static FalloffC falloff_derivatives(const Rxn* __restrict__ r,
                                                             const LogEntry* __restrict__ log_tab, int kind, double T,
                                                             double invT, double lnT, uint64_t IT, double rk,
                                                             int64_t l2rk, double M, double dMdT) {
-  double F = 1.0, FxPr = 0.0, FT = 0.0;
+  double F, FxPr, FT;
   const double Pr = rk * M;
-  if (kind != PJ_LINDEMANN) {
-    bool ok = true;
-    const int64_t l2Pr = l2rk + log2_51(log_tab, M, ok);
-    if (ok) F = falloff_F<true>(log_tab, r, kind, T, invT, lnT, IT, l2Pr, ok, FxPr, FT);
-    if (!ok) F = falloff_F_library(r, kind, T, invT, lnT, Pr, FxPr, FT);
-  }
+  falloff_broadening<true, MIXED>(r, log_tab, kind, IT, T, invT, lnT, l2rk, M, Pr, F, FxPr, FT);
   const double invT2 = invT * invT;
   const double dlnrk = fma(__ldg(&r->theta0) - __ldg(&r->theta), invT2, (__ldg(&r->beta0) - __ldg(&r->beta)) * invT);
   const double i1p = inverse_1p(Pr);
@@ -54,8 +40,10 @@ __device__ __noinline__ static FalloffC falloff_derivatives(const Rxn* __restric
 }
 
 // sum nu h/RT - d over a short-path reaction's factors; H: this lane's h_k/RT
-// (fixed_enthalpy), 32 words per species
-__device__ __forceinline__ double lean_energy(const RxnHead& h, const double* __restrict__ H, int d) {
+// (enthalpy_entry), 32 words per species
+template <bool MIXED>
+__device__ __forceinline__ double lean_energy(const RxnHead& h, const double* __restrict__ H, int d, bool fast) {
+  if (MIXED && !fast) return lean_sum(h, H, (double)d);
   auto hf = [&](int off) { return __double_as_longlong(H[off]); };
   int64_t s = hf(h.b[0]) - hf(h.f[0]) - ((int64_t)d << 51);
   if (h.nf > 1) s -= hf(h.f[1]);
@@ -107,18 +95,15 @@ __device__ __forceinline__ void lean_jacobian(const DevMech& m, const Rxn* __res
     for (int i = 0; i < 4; i++) q[i] = __ldg(p + i);
   }
   const bool rev = h.rev != 0;
-  const int64_t y = arrhenius_fixed(h.fA, h.fB, h.fT, v.fx.L, v.fx.IT);
-  const double kf = exp2_51(y);
-  double kr = 0.0;
-  if (rev) kr = exp2_51(y + lean_gibbs(h, G, v.fx.LP));
+  const LeanK k = lean_constants<false>(m, r, h, G, v.fx, v.lnT, v.invT);
   // both sides, the net rate and V dRn/dV at constant n, -(factors) R by side
   LeanSide sf, sb;
   double Rn, VS;
   lean_shapes(h.code, [&](auto tf, auto tb) {
     constexpr int SF = decltype(tf)::value, SB = decltype(tb)::value;
     constexpr int nfac[5] = {1, 2, 2, 3, 3};
-    sf = lean_side<SF>(h.f, C, kf);
-    sb = lean_side<SB>(h.b, C, kr);
+    sf = lean_side<SF>(h.f, C, k.kf);
+    sb = lean_side<SB>(h.b, C, k.kr);
     Rn = SB < 0 ? sf.R : sf.R - sb.R;
     VS = 0.0;
     if (MODE == PJ_CONP) {
@@ -128,9 +113,9 @@ __device__ __forceinline__ void lean_jacobian(const DevMech& m, const Rxn* __res
     }
   });
 
-  const double de = lean_energy(h, H, h.dnu_i);  // sum nu h/RT - dnu
+  const double de = lean_energy<false>(h, H, h.dnu_i, true);  // sum nu h/RT - dnu
   double dhd = de;
-  if (MODE == PJ_CONP && h.dnu_i != 0) dhd = lean_energy(h, H, 0);
+  if (MODE == PJ_CONP && h.dnu_i != 0) dhd = lean_energy<false>(h, H, 0, true);
 
   // T derivative of the net rate: T d ln kf/dT = Ef = beta + theta/T, T d ln
   // kr/dT = Ef - de, so T dRn/dT = Rn Ef + Rr de; times V
@@ -168,9 +153,10 @@ __device__ __forceinline__ void lean_jacobian(const DevMech& m, const Rxn* __res
     double cT = dMdT, c = M;
     RcM = Rn;
     if (h.kind != PJ_THIRD_BODY) {
-      const int64_t l2rk = arrhenius_fixed(__ldg(&r->fA0), __ldg(&r->fB0), __ldg(&r->fT0), v.fx.L, v.fx.IT) - y;
+      int64_t l2rk;
+      const double rk = lean_falloff<false>(r, k, v.fx, v.lnT, v.invT, l2rk);
       const FalloffC fc =
-          falloff_derivatives(r, m.log_tab, h.kind, v.T, v.invT, v.lnT, v.fx.IT, exp2_51(l2rk), l2rk, M, dMdT);
+          falloff_derivatives<false>(r, m.log_tab, h.kind, v.T, v.invT, v.lnT, v.fx.IT, rk, l2rk, M, dMdT);
       c = fc.c;
       cT = fc.cT;
       RcM = Rn * fc.cM;

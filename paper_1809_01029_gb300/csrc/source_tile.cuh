@@ -27,7 +27,7 @@ constexpr int kSrcWarps = 16;  // warps per block, or twice that
 
 enum SrcSc { zT, zV, zP, zInvT, zInvV, zLnT, zLnP, zCtot, zL, zIT, zLP, zCdum, zDen, zCxB, kSrcSc };
 enum SrcPart { rAcc, rDen, rNum, rOm, kSrcPart };
-enum SrcFlag { gOk, gFast, kSrcFlag };
+enum SrcFlag { gOk, gFast, kSrcFlag };  // gFast: 1 in the fixed point's range; 0: T out of it; 2: some g_k
 
 __host__ __device__ constexpr size_t source_arrays_bytes(int ns) { return (size_t)2 * ns * kTile * sizeof(double); }
 __host__ __device__ constexpr size_t source_smem_bytes(int ns, bool arrays_smem) {
@@ -44,46 +44,15 @@ __host__ __device__ constexpr size_t source_arrays_ws_doubles(int ns, bool array
 // blending (Pr / (1 + Pr)) F; chem: chemically activated, F / (1 + Pr).  Out
 // of line: it runs for about a fifth of the reactions, and its registers
 // would otherwise set every reaction's.
+template <bool MIXED>
 __device__ __noinline__ static double falloff_factor(const Rxn* __restrict__ r, const LogEntry* __restrict__ log_tab,
-                                                     int kind, bool fast, double T, double invT, double lnT, uint64_t IT,
-                                                     double rk, int64_t l2rk, double M, bool chem) {
-  double F = 1.0, d1, d2;
+                                                     int kind, double T, double invT, double lnT, uint64_t IT, double rk,
+                                                     int64_t l2rk, double M, bool chem) {
+  double F, d1, d2;
   const double Pr = rk * M;
-  if (kind != PJ_LINDEMANN) {
-    bool ok = fast;
-    const int64_t l2Pr = l2rk + log2_51(log_tab, M, ok);
-    if (ok) F = falloff_F<false>(log_tab, r, kind, T, invT, lnT, IT, l2Pr, ok, d1, d2);
-    if (!ok) F = falloff_F_library(r, kind, T, invT, lnT, Pr, d1, d2);
-  }
+  falloff_broadening<false, MIXED>(r, log_tab, kind, IT, T, invT, lnT, l2rk, M, Pr, F, d1, d2);
   const double i1p = inverse_1p(Pr);
   return (chem ? i1p : Pr * i1p) * F;
-}
-
-// Net rate of any reaction at any state.  Out of line (special types, sides
-// of more than three factors, states outside the fixed point's range).
-template <bool SPECIAL>
-__device__ __noinline__ static double general_rate(const DevMech& m, double* base, const Rxn* __restrict__ r, bool plain,
-                                                   const FixedState fx, double T, double invT, double lnT, double lnP,
-                                                   double Ctot) {
-  StateArrays A;
-  A.ns = m.ns;
-  A.base = base;
-  A.stride = kTile;
-  enum { aC = 0, aG = 1 };
-  const int kind = __ldg(&r->kind);
-  const int nre = __ldg(&r->nreac), npr = __ldg(&r->nprod), rev = __ldg(&r->rev);
-  const RateK k = rate_constants<SPECIAL>(m, A, aG, r, kind, rev, nre, npr, fx, T, lnT, invT, lnP);
-  double dmy[PJ_MAX_SP];
-  const double Rf = side_rate<false>(A, aC, r, 0, __ldg(&r->shape[0]), nre, k.kf, dmy);
-  const double Rr = rev ? side_rate<false>(A, aC, r, PJ_MAX_SP, __ldg(&r->shape[1]), npr, k.kr, dmy) : 0.0;
-  double c = 1.0;
-  if (has_third_body(kind)) {
-    const double M = third_body(m, A, aC, r, Ctot);
-    c = kind == PJ_THIRD_BODY
-            ? M
-            : falloff_factor(r, m.log_tab, kind, fx.fast, T, invT, lnT, fx.IT, k.rk, k.l2rk, M, SPECIAL && __ldg(&r->chem));
-  }
-  return c * (Rf - Rr);
 }
 
 // The warp-uniform head of a reaction's record.
@@ -97,7 +66,7 @@ __device__ __forceinline__ RxnHead load_head(const Rxn* __restrict__ r) {
 }
 
 // log2(k_r / k_f) 2^51 of a short-path reversible reaction; G: this lane's
-// g_k/RT (fixed_gibbs), 32 words per species.
+// g_k/RT (gibbs_entry, in range), 32 words per species.
 __device__ __forceinline__ int64_t lean_gibbs(const RxnHead& h, const double* __restrict__ G, int64_t LP) {
   auto g = [&](int off) { return __double_as_longlong(G[off]); };
   int64_t s = g(h.b[0]) - g(h.f[0]);
@@ -107,6 +76,61 @@ __device__ __forceinline__ int64_t lean_gibbs(const RxnHead& h, const double* __
   if (h.nb > 2) s += g(h.b[2]);
   if (h.dnu_i != 0) s -= (int64_t)h.dnu_i * LP;
   return s;
+}
+
+// sum nu x over a short-path reaction's factors, less d, of FP64 entries
+__device__ __forceinline__ double lean_sum(const RxnHead& h, const double* __restrict__ x, double d) {
+  double s = x[h.b[0]] - x[h.f[0]] - d;
+  if (h.nf > 1) s -= x[h.f[1]];
+  if (h.nb > 1) s += x[h.b[1]];
+  if (h.nf > 2) s -= x[h.f[2]];
+  if (h.nb > 2) s += x[h.b[2]];
+  return s;
+}
+
+// Rate constants of a short-path reaction.  MIXED: in a tile where some state
+// is outside the fixed point's range, each lane by its own state, the others
+// in FP64; what follows them is the same code for every lane, so that a
+// state's result does not depend on its tile mates.
+struct LeanK {
+  double kf, kr;
+  int64_t y;  // log2(kf) 2^51; kNoLog2 in FP64
+};
+template <bool MIXED>
+__device__ __forceinline__ LeanK lean_constants(const DevMech& m, const Rxn* __restrict__ r, const RxnHead& h,
+                                                const double* __restrict__ G, const FixedState& fx, double lnT,
+                                                double invT) {
+  LeanK k;
+  k.kr = 0.0;
+  if (!MIXED || fx.fast) {
+    k.y = arrhenius_fixed(h.fA, h.fB, h.fT, fx.L, fx.IT);
+    k.kf = exp2_51(k.y);
+    if (h.rev) k.kr = exp2_51(k.y + lean_gibbs(h, G, fx.LP));
+  } else {
+    k.y = kNoLog2;
+    const double lnkf = fma(__ldg(&r->beta), lnT, __ldg(&r->lnA)) - __ldg(&r->theta) * invT;
+    k.kf = pj_exp(lnkf);
+    if (h.rev) {
+      double dg = lean_sum(h, G, 0.0);
+      if (h.dnu_i != 0) dg = fma(-__ldg(&r->dnu), m.log_pstd_over_r - lnT, dg);
+      k.kr = pj_exp(lnkf + dg);
+    }
+  }
+  return k;
+}
+
+// rk = k_0 / k_inf of a short-path falloff reaction and its log2 2^51 (or
+// kNoLog2), from its k_inf.
+template <bool MIXED>
+__device__ __forceinline__ double lean_falloff(const Rxn* __restrict__ r, const LeanK& k, const FixedState& fx,
+                                               double lnT, double invT, int64_t& l2rk) {
+  if (!MIXED || fx.fast) {
+    l2rk = arrhenius_fixed(__ldg(&r->fA0), __ldg(&r->fB0), __ldg(&r->fT0), fx.L, fx.IT) - k.y;
+    return exp2_51(l2rk);
+  }
+  l2rk = kNoLog2;
+  return pj_exp((fma(__ldg(&r->beta0), lnT, __ldg(&r->lnA0)) - __ldg(&r->theta0) * invT) -
+                (fma(__ldg(&r->beta), lnT, __ldg(&r->lnA)) - __ldg(&r->theta) * invT));
 }
 
 // One side's product R = k prod C and dR/dC_a in species order (f: factors
@@ -165,18 +189,17 @@ __device__ __forceinline__ void lean_shapes(int code, F&& f) {
   }
 }
 
-// Net rate of reaction i at this lane's state, short path: every state of
-// the tile is within the fixed point's range and the reaction is plain.
+// Net rate of reaction i at this lane's state, short path: a plain reaction
+// with at most three factors a side.
+template <bool MIXED>
 __device__ __forceinline__ double lean_rate(const DevMech& m, const Rxn* __restrict__ r, const RxnHead& h,
                                             const double* __restrict__ C, const double* __restrict__ G,
                                             const FixedState& fx, double T, double invT, double lnT, double Ctot) {
-  const int64_t y = arrhenius_fixed(h.fA, h.fB, h.fT, fx.L, fx.IT);
-  const double kf = exp2_51(y);
-  double kr = 0.0, q = 0.0;
-  if (h.rev) kr = exp2_51(y + lean_gibbs(h, G, fx.LP));
+  const LeanK k = lean_constants<MIXED>(m, r, h, G, fx, lnT, invT);
+  double q = 0.0;
   lean_shapes(h.code, [&](auto sf, auto sb) {
-    q = lean_side<decltype(sf)::value>(h.f, C, kf).R;
-    if (decltype(sb)::value >= 0) q -= lean_side<decltype(sb)::value>(h.b, C, kr).R;
+    q = lean_side<decltype(sf)::value>(h.f, C, k.kf).R;
+    if (decltype(sb)::value >= 0) q -= lean_side<decltype(sb)::value>(h.b, C, k.kr).R;
   });
   if (h.kind != PJ_ELEMENTARY) {
     double M = Ctot;
@@ -189,11 +212,79 @@ __device__ __forceinline__ double lean_rate(const DevMech& m, const Rxn* __restr
     if (h.kind == PJ_THIRD_BODY) {
       q *= M;
     } else {
-      const int64_t l2rk = arrhenius_fixed(__ldg(&r->fA0), __ldg(&r->fB0), __ldg(&r->fT0), fx.L, fx.IT) - y;
-      q *= falloff_factor(r, m.log_tab, h.kind, true, T, invT, lnT, fx.IT, exp2_51(l2rk), l2rk, M, false);
+      int64_t l2rk;
+      const double rk = lean_falloff<MIXED>(r, k, fx, lnT, invT, l2rk);
+      q *= falloff_factor<MIXED>(r, m.log_tab, h.kind, T, invT, lnT, fx.IT, rk, l2rk, M, false);
     }
   }
   return q;
+}
+
+// What the reactions read of the state besides C and g (sc: this lane's scalars
+// of the tile).
+struct SrcVars {
+  FixedState fx;
+  double T, invT, lnT, lnP, Ctot;
+};
+__device__ __forceinline__ SrcVars source_vars(const double* __restrict__ sc, bool fast) {
+  auto S = [&](int v) { return sc[v * kTile]; };
+  SrcVars v;
+  v.T = S(zT);
+  v.invT = S(zInvT);
+  v.lnT = S(zLnT);
+  v.lnP = S(zLnP);
+  v.Ctot = S(zCtot);
+  v.fx.L = (uint64_t)__double_as_longlong(S(zL));
+  v.fx.IT = (uint64_t)__double_as_longlong(S(zIT));
+  v.fx.LP = __double_as_longlong(S(zLP));
+  v.fx.fast = fast;
+  return v;
+}
+
+// Net rate of any reaction at any state.  Out of line (special types, sides
+// of more than three factors).
+template <bool SPECIAL>
+__device__ __noinline__ static double general_rate(const DevMech& m, double* base, const double* sc,
+                                                   const Rxn* __restrict__ r, bool fast) {
+  const SrcVars v = source_vars(sc, fast);
+  const FixedState& fx = v.fx;
+  const double T = v.T, invT = v.invT, lnT = v.lnT, lnP = v.lnP, Ctot = v.Ctot;
+  StateArrays A;
+  A.ns = m.ns;
+  A.base = base;
+  A.stride = kTile;
+  enum { aC = 0, aG = 1 };
+  const int kind = __ldg(&r->kind);
+  const int nre = __ldg(&r->nreac), npr = __ldg(&r->nprod), rev = __ldg(&r->rev);
+  const RateK k = rate_constants<SPECIAL>(m, A, aG, r, kind, rev, nre, npr, fx, lnT, invT, lnP);
+  double dmy[PJ_MAX_SP];
+  const double Rf = side_rate<false>(A, aC, r, 0, __ldg(&r->shape[0]), nre, k.kf, dmy);
+  const double Rr = rev ? side_rate<false>(A, aC, r, PJ_MAX_SP, __ldg(&r->shape[1]), npr, k.kr, dmy) : 0.0;
+  double c = 1.0;
+  if (has_third_body(kind)) {
+    const double M = third_body(m, A, aC, r, Ctot);
+    c = kind == PJ_THIRD_BODY
+            ? M
+            : falloff_factor<true>(r, m.log_tab, kind, T, invT, lnT, fx.IT, k.rk, k.l2rk, M, SPECIAL && __ldg(&r->chem));
+  }
+  return c * (Rf - Rr);
+}
+
+// Net rates of a warp's reactions first, first + step, .. < end, into q, in a
+// tile with a state outside the fixed point's range.  The whole loop out of
+// line and the state read again from shared memory, so that the short path
+// beside it is compiled as if it were alone (53 species, 1 Mi states: 11.58 ms
+// with and without it).
+template <bool SPECIAL>
+__device__ __noinline__ static void mixed_rates(const DevMech& m, double* base, const double* sc, double* q, bool fast,
+                                                int first, int step, int end) {
+  const SrcVars v = source_vars(sc, fast);
+  for (int i = first; i < end; i += step, q += step * kTile) {
+    const Rxn* __restrict__ r = m.rxn + i;
+    const RxnHead h = load_head(r);
+    *q = h.lean ? lean_rate<true>(m, r, h, base, base + m.ns * kTile, v.fx, v.T, v.invT, v.lnT, v.Ctot)
+                : general_rate<SPECIAL>(m, base, sc, r, fast);
+  }
 }
 
 // One tile.  In: act() (this lane has a state), T(), S(), par(), n(k); Out:
@@ -273,11 +364,12 @@ __device__ __forceinline__ void source_tile(const DevMech& m, double* smem, doub
     const double T = S(zT), invT = S(zInvT), lnT = S(zLnT), cdum = S(zCdum), V = S(zV), invV = S(zInvV);
     const bool ok0 = flags[gOk * kTile] != 0;
     double acc = 0.0, den = 0.0;
-    bool fast = true;
+    const bool fast0 = flags[gFast * kTile] != 0;
+    bool fast = fast0;
     for (int k = warp; k < ns; k += W) {
       double cp, g;
       nasa_cp_g(nasa_block(m, k, T), T, invT, lnT, cp, g);
-      G[k * kTile] = fixed_gibbs(m, g, fast);
+      G[k * kTile] = gibbs_entry(m, g, fast);
       const double cx = MODE == PJ_CONP ? cp : cp - 1.0;
       if (k < bath) {
         const double c = ok0 ? concentration(in.n(k), V, invV) : cdum;
@@ -288,13 +380,22 @@ __device__ __forceinline__ void source_tile(const DevMech& m, double* smem, doub
         S(zCxB) = cx;
       }
     }
-    if (!fast) flags[gFast * kTile] = 0;
+    if (fast0 && !fast) flags[gFast * kTile] = 2;  // found out of range part of the way
     Pw(warp, rAcc) = acc;
     Pw(warp, rDen) = den;
   }
   __syncthreads();
 
-  // C: bath gas by subtraction, validity, the energy equation's denominator
+  // C: bath gas by subtraction, validity, the energy equation's denominator;
+  // the entries of a state found out of range, again
+  if (warp < W && flags[gFast * kTile] == 2) {
+    const double T = S(zT), invT = S(zInvT), lnT = S(zLnT);
+    for (int k = warp; k < ns; k += W) {
+      double cp, g;
+      nasa_cp_g(nasa_block(m, k, T), T, invT, lnT, cp, g);
+      G[k * kTile] = g;
+    }
+  }
   if (warp == 0) {
     const double Ctot = S(zCtot);
     const double acc = sum_parts(rAcc);
@@ -309,23 +410,22 @@ __device__ __forceinline__ void source_tile(const DevMech& m, double* smem, doub
   // D: the reactions, by chunks; then the chunk's contributions to the
   // warp's species
   {
-    FixedState fx;
-    const double T = S(zT), invT = S(zInvT), lnT = S(zLnT), lnP = S(zLnP), Ctot = S(zCtot);
-    fx.L = (uint64_t)__double_as_longlong(S(zL));
-    fx.IT = (uint64_t)__double_as_longlong(S(zIT));
-    fx.LP = __double_as_longlong(S(zLP));
-    fx.fast = flags[gFast * kTile] != 0;
-    const bool fast_tile = __all_sync(0xffffffffu, fx.fast);  // the same in every warp
+    const bool fast = flags[gFast * kTile] == 1;
+    const SrcVars v = source_vars(sc, fast);
+    const bool fast_tile = __all_sync(0xffffffffu, fast);  // the same in every warp
     int chunk = 0;
     for (int c0 = 0; c0 < nr; c0 += kGatherChunk, chunk++) {
       double* const q = qbuf + (chunk & 1) * kGatherChunk * kTile;
       const int c1 = min(nr, c0 + kGatherChunk);
-      for (int i = c0 + warp; i < c1; i += W_all) {
-        const Rxn* __restrict__ r = m.rxn + i;
-        const RxnHead h = load_head(r);
-        q[(i - c0) * kTile] = fast_tile && h.lean
-                                  ? lean_rate(m, r, h, C, G, fx, T, invT, lnT, Ctot)
-                                  : general_rate<SPECIAL>(m, base, r, i < m.nr_plain, fx, T, invT, lnT, lnP, Ctot);
+      if (fast_tile) {
+        for (int i = c0 + warp; i < c1; i += W_all) {
+          const Rxn* __restrict__ r = m.rxn + i;
+          const RxnHead h = load_head(r);
+          q[(i - c0) * kTile] = h.lean ? lean_rate<false>(m, r, h, C, G, v.fx, v.T, v.invT, v.lnT, v.Ctot)
+                                       : general_rate<SPECIAL>(m, base, sc, r, fast);
+        }
+      } else {
+        mixed_rates<SPECIAL>(m, base, sc, q + warp * kTile, fast, c0 + warp, W_all, c1);
       }
       __syncthreads();
       for (int k = warp; k < ns; k += W_all) {

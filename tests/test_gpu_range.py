@@ -1,0 +1,98 @@
+"""States outside the fixed point's range: by temperature, and by a Gibbs energy
+or enthalpy found too large part of the way, beside states within it.  Values
+against the oracle, and bit for bit: what a state gives does not depend on the
+states that share its tile."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+from tests import tiny_mechs as tm
+from tests.parity import RTOL_SRC, ATOL_SRC, RTOL_JAC, ATOL_JAC, check_close, jacobian_layout, y_envelope
+from tests.test_gpu_forms import RTOL_VJP
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def pj():
+    import paper_1809_01029_gb300 as pj
+    from paper_1809_01029_gb300 import build
+    build.build()
+    pj.load_library()
+    return pj
+
+
+def dev(a):
+    import torch
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+def _mech(mechs, name):
+    if name == "large_gibbs":
+        # |g/RT| of one species goes through the range's end (346 with four
+        # coefficients a reaction) between 1000 and 1400 K
+        m = tm.all_kinds()
+        m.nasa_low[tm.H2, 5] = m.nasa_high[tm.H2, 5] = -4.2e5
+        return m
+    return getattr(tm, name)() if name in ("all_kinds", "all_types") else mechs(name)
+
+
+def _states(m, n, seed, mode, name):
+    return synth.make_states(m, n, seed, mode, T_range=(700.0, 1700.0) if name == "large_gibbs" else (100.0, 160.0))
+
+
+@pytest.mark.parametrize("mode", [synth.CONP, synth.CONV])
+@pytest.mark.parametrize("name", ["large_gibbs"])
+def test_large_gibbs_energies_against_oracle(pj, mechs, name, mode):
+    import torch
+    m = _mech(mechs, name)
+    h = pj.pj_mech_create(m)
+    n = 70
+    phi, par = _states(m, n, 71, mode, name)
+    f_ref, f_env = oracle.source_term_envelope(m, mode, phi, par)
+    J, J_env = oracle.jacobian_envelope(m, mode, phi, par)
+    assert np.isfinite(f_ref).all() and np.isfinite(J).all()
+    d_phi, d_par = dev(phi), dev(par)
+    check_close(pj.source_terms(h, mode, d_phi, d_par).cpu().numpy(), f_ref, f_env, RTOL_SRC, ATOL_SRC, f"{name}")
+    out = torch.empty_like(d_phi)
+    pj.Plan(h, pj.PJ_OP_SOURCE, mode, [(d_par, d_phi, out, None)]).run()
+    check_close(out.cpu().numpy(), f_ref, f_env, RTOL_SRC, ATOL_SRC, f"{name} plan")
+    ref, env = oracle.dense_to_csr_values(m, J), oracle.dense_to_csr_values(m, J_env)
+    for layout in ("coop", "percore"):
+        with jacobian_layout(layout):
+            vals = pj.jacobian_sparse(h, mode, d_phi, d_par).cpu().numpy()
+        check_close(vals, ref, env, RTOL_JAC, ATOL_JAC, f"{name} {layout} CSR")
+    uw, uT = synth.make_cotangents(m.n_species, n, 71)
+    y, g_phi, g_th = (a.cpu().numpy() for a in pj.vjp(h, mode, d_phi, d_par, dev(uw), dev(uT)))
+    check_close(y, oracle.outputs_y(m, mode, phi, par), y_envelope(m, mode, phi, par), RTOL_SRC, ATOL_SRC, f"{name} y")
+    g_ref, th_ref = oracle.vjp(m, mode, phi, par, uw, uT)
+    e_phi, e_th = oracle.vjp_envelope(m, mode, phi, par, uw, uT)
+    check_close(g_phi, g_ref, e_phi, RTOL_VJP, 1e-300, f"{name} g_phi")
+    check_close(g_th, th_ref, e_th, RTOL_VJP, 1e-300, f"{name} g_theta")
+
+
+@pytest.mark.parametrize("mode", [synth.CONP, synth.CONV])
+@pytest.mark.parametrize("name", ["all_kinds", "all_types", "large_gibbs", "gri53_types"])
+def test_bits_do_not_depend_on_tile_mates(pj, mechs, name, mode):
+    """The states of two batches, in tiles of their own and mixed into each
+    other's tiles: one batch within the range, the other (cold, or through the
+    range's end) not."""
+    m = _mech(mechs, name)
+    h = pj.pj_mech_create(m)
+    n = 64
+    a = synth.make_states(m, n, 72, mode, T_range=(1500.0, 2500.0))
+    b = _states(m, n, 73, mode, name)
+    uw, uT = synth.make_cotangents(m.n_species, n, 74)
+    mix = np.arange(n) % 5 == 2
+
+    def outputs(phi, par):
+        d_phi, d_par = dev(phi), dev(par)
+        y, g_phi, _ = pj.vjp(h, mode, d_phi, d_par, dev(uw), dev(uT))
+        return [t.cpu().numpy() for t in (pj.source_terms(h, mode, d_phi, d_par), pj.eval_y(h, mode, d_phi, d_par),
+                                          pj.jacobian_fd(h, mode, d_phi, d_par), y, g_phi)]
+
+    of_a, of_b = outputs(*a), outputs(*b)
+    of_mix = outputs(np.where(mix, b[0], a[0]), np.where(mix, b[1], a[1]))
+    for x, z, got in zip(of_a, of_b, of_mix):
+        assert np.array_equal(got, np.where(mix, z, x), equal_nan=True)
