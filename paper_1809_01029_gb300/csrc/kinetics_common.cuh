@@ -34,7 +34,7 @@ struct StateScalars {
 // fixed point: both at least as exact as the FP64 operations.
 __device__ __forceinline__ void temperature_terms(const DevMech& m, double T, double invT, double& lnT,
                                                   FixedState& f) {
-  f.fast = m.fx_ok && T >= 128.0 && T < 65536.0;
+  f.fast = T >= 128.0 && T < 65536.0;
   f.L = f.IT = 0;
   f.LP = 0;
   if (!f.fast) {
@@ -476,11 +476,13 @@ struct RateK {
 // l2rk where log2(rk) is not known in fixed point
 constexpr int64_t kNoLog2 = INT64_MIN;
 
-// The rate constants in FP64, from the stored g_k/RT: states outside the
-// fixed point's range (A by value: its address taken would put it in memory).
+// The rate constants in FP64, from the stored g_k/RT (gfix: in fixed point):
+// states and reactions outside the fixed point's range (A by value: its address
+// taken would put it in memory).
 template <bool GEN, class SA>
 __device__ __noinline__ static RateK rate_constants_fp64(const DevMech& m, const SA A, int aG, const Rxn* __restrict__ r,
-                                                         int kind, int rev, double lnT, double invT, double lnP) {
+                                                         int kind, int rev, double lnT, double invT, double lnP,
+                                                         bool gfix) {
   RateK k;
   const double lninf = fma(__ldg(&r->beta), lnT, __ldg(&r->lnA)) - __ldg(&r->theta) * invT;
   double lnkf = lninf;
@@ -501,11 +503,15 @@ __device__ __noinline__ static RateK rate_constants_fp64(const DevMech& m, const
   } else if (rev) {
     // kr = kf / Kc with Kc = exp(-sum nu g) (P_std / R T)^dnu
     const int nre = __ldg(&r->nreac), npr = __ldg(&r->nprod);
+    auto g = [&](int k) {
+      const double x = A.at(aG, k);
+      return gfix ? fixed51_to_double(__double_as_longlong(x)) * 0.69314718055994530942 : x;
+    };
     double dg = 0.0;
 #pragma unroll
     for (int a = 0; a < PJ_MAX_SP; a++) {
-      if (a < nre) dg = fma(-__ldg(&r->nud[a]), A.at(aG, __ldg(&r->sp[a])), dg);
-      if (a < npr) dg = fma(__ldg(&r->nud[PJ_MAX_SP + a]), A.at(aG, __ldg(&r->sp[PJ_MAX_SP + a])), dg);
+      if (a < nre) dg = fma(-__ldg(&r->nud[a]), g(__ldg(&r->sp[a])), dg);
+      if (a < npr) dg = fma(__ldg(&r->nud[PJ_MAX_SP + a]), g(__ldg(&r->sp[PJ_MAX_SP + a])), dg);
     }
     if (__ldg(&r->head.dnu_i) != 0) dg = fma(-__ldg(&r->dnu), m.log_pstd_over_r - lnT, dg);
     k.kr = pj_exp(lnkf + dg);
@@ -520,7 +526,7 @@ template <bool GEN = true, class SA>
 __device__ __forceinline__ RateK rate_constants(const DevMech& m, const SA& A, int aG, const Rxn* __restrict__ r,
                                                 int kind, int rev, int nre, int npr, const FixedState& fx,
                                                 double lnT, double invT, double lnP) {
-  if (!fx.fast) return rate_constants_fp64<GEN>(m, A, aG, r, kind, rev, lnT, invT, lnP);
+  if (!fx.fast || !__ldg(&r->fx)) return rate_constants_fp64<GEN>(m, A, aG, r, kind, rev, lnT, invT, lnP, fx.fast);
   RateK k;
   int64_t y = arrhenius_fixed(__ldg(&r->head.fA), __ldg(&r->head.fB), __ldg(&r->head.fT), fx.L, fx.IT);
   k.rk = 0.0;

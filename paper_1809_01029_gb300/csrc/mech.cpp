@@ -344,7 +344,6 @@ int mech_build(pj_mech* m) {
   std::vector<char> dep;
   std::vector<double> tab;  // P-log entries and Chebyshev blocks
   bool has_pdep = false;
-  bool fx_ok = true;  // every rate constant fits the fixed-point path
   int nu_max = 1;     // largest sum of the coefficients of both sides of a reaction
   for (int q = 0; q < nr; q++) {
     const int i = m->perm[q];
@@ -430,7 +429,8 @@ int mech_build(pj_mech* m) {
     r.dW = dW;
     // fixed-point Arrhenius sets; a set beyond their ranges (every sum of
     // exponent terms must stay within the 2^12 of the fixed point) leaves the
-    // whole mechanism on the FP64 path
+    // reaction on the FP64 path
+    r.fx = 1;
     auto fixed_set = [&](double A, double beta, double Ea, int64_t& fA, int64_t& fB, int64_t& fT) {
       const long double l2A = std::log2((long double)A);
       const long double th = (long double)Ea / (long double)R_CAL * 1.442695040888963407359924681001892137L;
@@ -438,7 +438,7 @@ int mech_build(pj_mech* m) {
       const long double worst = std::fabs(l2A) + 16.0L * std::fabs((long double)beta) + std::fabs(th) / 128.0L +
                                 std::fabs((long double)dnu) * l2p;
       if (!(worst < 1900.0L) || !(std::fabs(beta) < 100.0) || !(std::fabs(th) < 0x1p17L)) {
-        fx_ok = false;
+        r.fx = 0;
         return;
       }
       fA = std::llrint(l2A * 0x1p51L + 1.5L);
@@ -464,7 +464,7 @@ int mech_build(pj_mech* m) {
     for (int a = 0; a < 2 * PJ_MAX_SP; a++)
       nu_sum += a < PJ_MAX_SP ? (a < r.nreac ? r.nu[a] : 0) : (a - PJ_MAX_SP < r.nprod ? r.nu[a] : 0);
     nu_max = std::max(nu_max, nu_sum);
-    pack_head(r, q < nr_plain);
+    pack_head(r, q < nr_plain && r.fx);
     std::vector<double> al = alpha_of(m, i);
     r.alpha_bath = has_third_body(r.kind) ? al[bath] : 1.0;
     r.eff_lo = (int32_t)eff_sp.size();
@@ -677,7 +677,6 @@ int mech_build(pj_mech* m) {
   dm.exp_tab = reinterpret_cast<const uint64_t*>(b + o_etab);
   dm.log_tab = reinterpret_cast<const LogEntry*>(b + o_ltab);
   dm.log2_pstd_fx = std::llrint(std::log2((long double)P_STD / (long double)RU) * 0x1p51L);
-  dm.fx_ok = fx_ok ? 1 : 0;
   dm.fx_g_hi = (uint32_t)(g_bits >> 32);
   dm.fx_h_hi = (uint32_t)(h_bits >> 32);
   dm.tab = reinterpret_cast<const double*>(b + o_tab);

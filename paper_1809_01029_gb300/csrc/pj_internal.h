@@ -43,9 +43,10 @@ enum : int32_t {
 };
 
 // The part of a reaction's record that the tile kernels' short path reads
-// (tile_rate): four 16-byte loads.  Reactions whose sides have more than
-// three factors (counting a coefficient of 2 as two), and the special types,
-// have lean = 0 and take the general path.
+// (lean_rate, lean_jacobian, lean_vjp): four 16-byte loads.  Reactions whose
+// sides have more than three factors (counting a coefficient of 2 as two) or a
+// coefficient of 3, whose constants do not fit the fixed point, and the special
+// types have lean = 0 and take the general path.
 struct alignas(16) RxnHead {
   int64_t fA, fB, fT;             // the Arrhenius set in fixed point (arrhenius_fixed): log2(A) 2^51,
                                   // beta 2^56, -theta log2(e) 2^45
@@ -98,7 +99,8 @@ struct alignas(16) Rxn {
   // Troe: log2(e)/T3 2^68, log2(e)/T1 2^68, T2 log2(e) 2^45; bit b of
   // troe_fx: the b-th is within its range (else the FP64 argument is formed)
   uint64_t tT3, tT1, tT2;
-  int32_t troe_fx, pad_;
+  int32_t troe_fx;
+  int32_t fx;                     // its Arrhenius sets fit the fixed point (else it is evaluated in FP64)
 };
 static_assert(sizeof(RxnHead) == 64 && sizeof(RxnJac) == 64 && offsetof(RxnJac, nfx) == 40, "records are 16-byte loads");
 
@@ -115,10 +117,9 @@ struct DevMech {
   int32_t ns, nr, N, nnz;
   double log_pstd_over_r;         // ln(P_std / R)
   int64_t log2_pstd_fx;           // log2(P_std / R) 2^51
-  // fixed-point rate constants: usable for every reaction when fx_ok, at
-  // states with |g_k/RT| below the double whose high word is fx_g_hi
-  int32_t fx_ok;
-  uint32_t fx_g_hi, fx_h_hi;      // and |h_k/RT| below fx_h_hi's
+  // fixed-point rate constants: usable at states with |g_k/RT| below the double
+  // whose high word is fx_g_hi and |h_k/RT| below fx_h_hi's
+  uint32_t fx_g_hi, fx_h_hi;
   const double* nasa;             // [ns * NASA_STRIDE]
   const double* wfac;             // [ns] 1 - W_k / W_{Ns-1}
   const Rxn* rxn;                 // [nr]

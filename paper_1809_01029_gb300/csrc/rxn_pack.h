@@ -20,7 +20,8 @@ inline int32_t side_shape(const int32_t* nu, int n) {
 
 // The factors of each side (a coefficient of 2 as two factors), the jump
 // table's code and whether the reaction may take the short path; r holds the
-// reaction's sides, shapes, kind and rev.  plain: none of the special types.
+// reaction's sides, shapes, kind and rev.  plain: none of the special types
+// and constants within the fixed point.
 //
 // The short path's jump table (lean_shapes) has the shapes SH_1 .. SH_111
 // only, and code has room for no other: a side of shape SH_GEN takes the

@@ -96,3 +96,38 @@ def test_bits_do_not_depend_on_tile_mates(pj, mechs, name, mode):
     of_mix = outputs(np.where(mix, b[0], a[0]), np.where(mix, b[1], a[1]))
     for x, z, got in zip(of_a, of_b, of_mix):
         assert np.array_equal(got, np.where(mix, z, x), equal_nan=True)
+
+
+def test_a_reaction_outside_leaves_the_others_inside(pj):
+    """A reaction whose constants the fixed point cannot hold: the species it
+    does not touch keep their production rates bit for bit, and its own agree
+    with the oracle (an elementary, a falloff and a third-body reaction)."""
+    import torch
+    n = 70
+    extra = [dict(reac=[(tm.N, 1), (tm.O2, 1)], prod=[(tm.NO, 1), (tm.O, 1)], A=1.0e9, Ea=2.0e5),
+             dict(reac=[(tm.NO, 1)], prod=[(tm.N, 1), (tm.O, 1)], A=1.0e9, Ea=1.0e3, kind=synth.TROE, A0=1.0e10, Ea0=-1.9e5,
+                  troe=(0.6, 100.0, 1500.0)),
+             dict(reac=[(tm.N, 2)], prod=[(tm.N2, 1)], A=1.0e3, beta=101.0, kind=synth.THIRD_BODY, eff={tm.H2: 2.0})]
+    base = [dict(reac=[(tm.H, 1), (tm.O2, 1)], prod=[(tm.OH, 1), (tm.O, 1)], A=2.0e11, beta=-0.3, Ea=15000.0),
+            dict(reac=[(tm.OH, 2)], prod=[(tm.H2, 1), (tm.HO2, 1)], A=7.0e10, beta=-0.4, kind=synth.TROE, A0=2.0e12,
+                 beta0=-0.8, Ea0=-1500.0, troe=(0.7, 90.0, 1800.0, 5000.0), eff={tm.H2O: 6.0}),
+            dict(reac=[(tm.H, 1), (tm.OH, 1)], prod=[(tm.H2O, 1)], A=2.0e16, beta=-1.9, kind=synth.THIRD_BODY)]
+    for e in extra:  # finite at the batch's temperatures
+        e["A"] *= 1500.0 ** -e.get("beta", 0.0) * np.exp(e.get("Ea", 0.0) / (1.98720425864083 * 1500.0))
+        if "A0" in e:
+            e["A0"] *= np.exp(e["Ea0"] / (1.98720425864083 * 1500.0))
+    few, all_ = (synth.build_mechanism("m", tm.SP, rx, seed=21) for rx in (base, base + extra))
+    phi, par = synth.make_states(all_, n, 75, synth.CONP, T_range=(1300.0, 1700.0))
+    f_ref, f_env = oracle.source_term_envelope(all_, synth.CONP, phi, par)
+    J, J_env = oracle.jacobian_envelope(all_, synth.CONP, phi, par)
+    assert np.isfinite(f_ref).all() and np.isfinite(J).all()
+    y_few, y_all = (pj.eval_y(pj.pj_mech_create(m), synth.CONP, dev(phi), dev(par)) for m in (few, all_))
+    untouched = [tm.H, tm.H2, tm.OH, tm.H2O, tm.HO2]
+    assert torch.equal(y_few[untouched], y_all[untouched])
+    h = pj.pj_mech_create(all_)
+    check_close(pj.source_terms(h, synth.CONP, dev(phi), dev(par)).cpu().numpy(), f_ref, f_env, RTOL_SRC, ATOL_SRC, "extra")
+    for layout in ("coop", "percore"):
+        with jacobian_layout(layout):
+            vals = pj.jacobian_sparse(h, synth.CONP, dev(phi), dev(par)).cpu().numpy()
+        check_close(vals, oracle.dense_to_csr_values(all_, J), oracle.dense_to_csr_values(all_, J_env), RTOL_JAC, ATOL_JAC,
+                    f"extra {layout} CSR")
