@@ -522,6 +522,7 @@ __global__ void __launch_bounds__(kVjpWarps * 32, kVjpCtas)
       S(vDdenT) = RU * (sum_parts(wDden) + Cns * S(vDcpB)) + Cx_bath * dCb_T;
       S(vDdenS) = MODE == PJ_CONP ? (Cx_bath * Ctot - den) * invV : Cx_bath * Ctot / P;
       flags[xOk * kTile] = ok;
+      if (!ok) S(vMRT) = 0.0;  // -1/T may be infinite; the state takes no part in the parameters' sums
       if (act && !ok) {
         write_nan_state(g_phi, ld, s, ns + 1);
         write_nan_state(y, ld, s, ns + 1);

@@ -131,3 +131,21 @@ def test_a_reaction_outside_leaves_the_others_inside(pj):
             vals = pj.jacobian_sparse(h, synth.CONP, dev(phi), dev(par)).cpu().numpy()
         check_close(vals, oracle.dense_to_csr_values(all_, J), oracle.dense_to_csr_values(all_, J_env), RTOL_JAC, ATOL_JAC,
                     f"extra {layout} CSR")
+
+
+def test_invalid_state_of_subnormal_temperature(pj):
+    """1/T is infinite; the state is invalid and leaves the parameter gradients
+    as if it were not there."""
+    m = tm.all_kinds()
+    h = pj.pj_mech_create(m)
+    n = 40
+    phi, par = synth.make_states(m, n, 76, synth.CONP)
+    uw, uT = synth.make_cotangents(m.n_species, n, 76)
+    bad = phi.copy()
+    bad[0, 7] = 1e-310
+    good = np.arange(n) != 7
+    y, g_phi, g_th = (a.cpu().numpy() for a in pj.vjp(h, synth.CONP, dev(bad), dev(par), dev(uw), dev(uT)))
+    assert np.isnan(y[:, 7]).all() and np.isnan(g_phi[:, 7]).all()
+    _, th_ref = oracle.vjp(m, synth.CONP, phi[:, good], par[good], uw[:, good], uT[good])
+    _, e_th = oracle.vjp_envelope(m, synth.CONP, phi[:, good], par[good], uw[:, good], uT[good])
+    check_close(g_th, th_ref, e_th, RTOL_VJP, 1e-300, "g_theta beside a state of subnormal temperature")
