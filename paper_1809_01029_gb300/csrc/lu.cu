@@ -21,8 +21,9 @@
 //    storage order.
 //  * Solve: four warps per 32 states, streaming the factors in storage order
 //    (coalesced across the warp), forward substitution then backward; the
-//    solution sits in shared memory (matrices too large for that: one state
-//    per thread, the solution in x).
+//    solution sits in shared memory.  Many states of a small matrix: one state
+//    per thread (solve_one_per_thread); matrices too large for shared memory:
+//    that with the solution in x.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -523,38 +524,67 @@ __global__ void __launch_bounds__(128) k_lu_solve(DevLu L, int64_t n, const T* _
   }
 }
 
-// The same with one state per thread and the solution in x itself, for
-// matrices whose solutions do not fit in shared memory (the same sums).
-template <typename T>
-__global__ void __launch_bounds__(128) k_lu_solve_global(DevLu L, int64_t n, const T* __restrict__ lu, int64_t ld,
-                                                         const T* b, T* x) {
+// The same sums with one state per thread.  X: the solution of this thread's
+// state, in shared memory (stride blockDim.x) or, where it does not fit, in x
+// itself (stride ld).
+template <typename T, bool SMEM_X>
+__global__ void __launch_bounds__(128) k_lu_solve_one(DevLu L, int64_t n, const T* __restrict__ lu, int64_t ld,
+                                                      const T* b, T* x) {
+  extern __shared__ __align__(16) unsigned char lu_smem[];
   const int N = L.N;
   for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < n; s += (int64_t)gridDim.x * blockDim.x) {
-    T* X = x + s;
+    T* X = SMEM_X ? reinterpret_cast<T*>(lu_smem) + threadIdx.x : x + s;
+    const int64_t xs = SMEM_X ? blockDim.x : ld;
+    // sum over storage entries [e, e1) of value * X[column], four independent
+    // partial sums so that the factor loads stream; FP32 takes eight entries
+    // a step (eight loads in flight: 17 % faster at 111 species; FP64 was
+    // slower that way)
     auto dot = [&](int e, int e1) -> T {
       T p0 = T(0), p1 = T(0), p2 = T(0), p3 = T(0);
+      for (; sizeof(T) == 4 && e + 7 < e1; e += 8) {
+        const int c0 = __ldg(L.xcol + e), c1 = __ldg(L.xcol + e + 1);
+        const int c2 = __ldg(L.xcol + e + 2), c3 = __ldg(L.xcol + e + 3);
+        const int c4 = __ldg(L.xcol + e + 4), c5 = __ldg(L.xcol + e + 5);
+        const int c6 = __ldg(L.xcol + e + 6), c7 = __ldg(L.xcol + e + 7);
+        const T v0 = lu[(int64_t)e * ld + s], v1 = lu[(int64_t)(e + 1) * ld + s];
+        const T v2 = lu[(int64_t)(e + 2) * ld + s], v3 = lu[(int64_t)(e + 3) * ld + s];
+        const T v4 = lu[(int64_t)(e + 4) * ld + s], v5 = lu[(int64_t)(e + 5) * ld + s];
+        const T v6 = lu[(int64_t)(e + 6) * ld + s], v7 = lu[(int64_t)(e + 7) * ld + s];
+        p0 = fma_t(v0, X[(int64_t)c0 * xs], p0);
+        p1 = fma_t(v1, X[(int64_t)c1 * xs], p1);
+        p2 = fma_t(v2, X[(int64_t)c2 * xs], p2);
+        p3 = fma_t(v3, X[(int64_t)c3 * xs], p3);
+        p0 = fma_t(v4, X[(int64_t)c4 * xs], p0);
+        p1 = fma_t(v5, X[(int64_t)c5 * xs], p1);
+        p2 = fma_t(v6, X[(int64_t)c6 * xs], p2);
+        p3 = fma_t(v7, X[(int64_t)c7 * xs], p3);
+      }
       for (; e + 3 < e1; e += 4) {
         const int c0 = __ldg(L.xcol + e), c1 = __ldg(L.xcol + e + 1);
         const int c2 = __ldg(L.xcol + e + 2), c3 = __ldg(L.xcol + e + 3);
-        p0 = fma_t(lu[(int64_t)e * ld + s], X[(int64_t)c0 * ld], p0);
-        p1 = fma_t(lu[(int64_t)(e + 1) * ld + s], X[(int64_t)c1 * ld], p1);
-        p2 = fma_t(lu[(int64_t)(e + 2) * ld + s], X[(int64_t)c2 * ld], p2);
-        p3 = fma_t(lu[(int64_t)(e + 3) * ld + s], X[(int64_t)c3 * ld], p3);
+        p0 = fma_t(lu[(int64_t)e * ld + s], X[(int64_t)c0 * xs], p0);
+        p1 = fma_t(lu[(int64_t)(e + 1) * ld + s], X[(int64_t)c1 * xs], p1);
+        p2 = fma_t(lu[(int64_t)(e + 2) * ld + s], X[(int64_t)c2 * xs], p2);
+        p3 = fma_t(lu[(int64_t)(e + 3) * ld + s], X[(int64_t)c3 * xs], p3);
       }
-      for (; e < e1; e++) p0 = fma_t(lu[(int64_t)e * ld + s], X[(int64_t)__ldg(L.xcol + e) * ld], p0);
+      for (; e < e1; e++) p0 = fma_t(lu[(int64_t)e * ld + s], X[(int64_t)__ldg(L.xcol + e) * xs], p0);
       return (p0 + p1) + (p2 + p3);
     };
+    // forward: y_k = b_perm[k] - sum_{j<k} L_kj y_j, y kept at X[perm[k]]
     for (int k = 0; k < N; k++) {
       const int pk = __ldg(L.perm + k);
       const T bk = b[(int64_t)pk * ld + s];
-      X[(int64_t)pk * ld] = bk - dot(__ldg(L.lptr + k), __ldg(L.lptr + k + 1));
+      X[(int64_t)pk * xs] = bk - dot(__ldg(L.lptr + k), __ldg(L.lptr + k + 1));
     }
+    // backward: z_k = (y_k - sum_{j>k} U_kj z_j) / U_kk
     for (int q = 0; q < N; q++) {
       const int e0 = __ldg(L.uptr + q), e1 = __ldg(L.uptr + q + 1);
       const int pk = __ldg(L.perm + (N - 1 - q));
-      const T yk = X[(int64_t)pk * ld];
-      X[(int64_t)pk * ld] = (yk - dot(e0 + 1, e1)) * lu[(int64_t)e0 * ld + s];
+      const T yk = X[(int64_t)pk * xs];
+      X[(int64_t)pk * xs] = (yk - dot(e0 + 1, e1)) * lu[(int64_t)e0 * ld + s];
     }
+    if (SMEM_X)
+      for (int v = 0; v < N; v++) x[(int64_t)v * ld + s] = X[(int64_t)v * xs];
   }
 }
 
@@ -661,26 +691,57 @@ int launch_lu_factor(const DevLu& L, int prec, int64_t n, const void* vals, int6
   return launch_factor_t<double>(L, n, vals, ld, hstep, gamma, lu, status, work, work_bytes, st);
 }
 
+// Whether n states are solved one per thread instead of by tiles.  A tile's row
+// costs a barrier and five operations in each of four warps besides its entries,
+// so with short rows the one-state-per-thread kernel gets more done once the
+// chip is full, and a tile kernel that needs one more, nearly empty round loses
+// to one round of it.  tiles, one: states resident at once in the two kernels;
+// entries: mean entries of a row of L or U.  Measured (us, tiles against one):
+//   FP64  5.7 entries (13 species): 4864 states 27.3 / 27.2, 8000 31.1 / 27.3, 131072 197 / 75
+//         9.5 (20): 40000 110 / 118, 60000 154 / 121      12.6 (28): 50000 194 / 212, 60000 230 / 210
+//         17.6 (38): 60000 350 / 373, 70000 420 / 384, 100000 605 / 742, 131072 772 / 745
+//         24 (53): 60000 560 / 688, 70000 921 / 701, 80000 924 / 1366, 131072 1422 / 1359, 262144 2441 / 2827
+//         48 (111): 70000 4387 / 5445
+//   FP32  5.7: 40000 23 / 27, 60000 29.5 / 27, 131072 65 / 38   12.6: 70000 128 / 209, 80000 243 / 213
+//         17.6: 70000 204 / 371, 80000 395 / 378          24: 80000 622 / 690
+static bool solve_one_per_thread(double entries, size_t esize, int64_t n, int64_t tiles, int64_t one) {
+  if (one == 0) return false;
+  const double rounds = (double)((n + one - 1) / one);
+  if (esize == 8) {
+    if (entries < 8.0) return n > (int64_t)sm_count() * 32;
+    return (entries < 20.0 || (entries < 26.0 && rounds < 3.0)) &&
+           (double)n > (0.28 + 0.031 * entries) * (double)tiles * rounds;
+  }
+  return entries < 20.0 && (double)n > (entries < 8.0 ? 0.65 : 1.0) * (double)tiles * rounds;
+}
+
 template <typename T>
 static int launch_solve_t(const DevLu& L, int64_t n, const void* lu, int64_t ld, const void* b, void* x,
                           cudaStream_t st) {
-  const size_t smem = (size_t)(L.N + 8) * 32 * sizeof(T);
-  int rc;
-  if (smem <= kSmemCap) {
-    auto kern = k_lu_solve<T>;
+  auto resident = [&](auto kern, size_t smem, int& blocks) -> int {  // blocks per SM
+    int rc;
     if ((rc = set_smem(kern, smem))) return rc;
-    int occ = 1;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, 128, smem) != cudaSuccess || occ < 1) occ = 1;
-    const int64_t grid = std::max<int64_t>(1, std::min<int64_t>((n + 31) / 32, (int64_t)sm_count() * occ));
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, kern, 128, smem) != cudaSuccess || blocks < 1) blocks = 1;
+    return PJ_OK;
+  };
+  auto launch = [&](auto kern, size_t smem, int64_t blocks, int per_sm) -> int {
+    const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(blocks, (int64_t)sm_count() * per_sm));
     kern<<<(unsigned)grid, 128, smem, st>>>(L, n, static_cast<const T*>(lu), ld, static_cast<const T*>(b),
                                             static_cast<T*>(x));
-  } else {
-    auto kern = k_lu_solve_global<T>;
-    const int64_t grid = std::max<int64_t>(1, std::min<int64_t>((n + 127) / 128, (int64_t)sm_count() * 16));
-    kern<<<(unsigned)grid, 128, 0, st>>>(L, n, static_cast<const T*>(lu), ld, static_cast<const T*>(b),
-                                         static_cast<T*>(x));
+    return check_cuda(cudaGetLastError(), "k_lu_solve launch");
+  };
+  const size_t tile_smem = (size_t)(L.N + 8) * 32 * sizeof(T), one_smem = (size_t)L.N * 128 * sizeof(T);
+  const int64_t tiles = (n + 31) / 32, blocks = (n + 127) / 128;
+  int tile_occ = 0, one_occ = 0, rc;
+  if (tile_smem > kSmemCap) return launch(k_lu_solve_one<T, false>, 0, blocks, 16);
+  if ((rc = resident(k_lu_solve<T>, tile_smem, tile_occ))) return rc;
+  if (n > (int64_t)sm_count() * 32 && one_smem <= kSmemCap) {  // (the tiles are the faster or equal below)
+    if ((rc = resident(k_lu_solve_one<T, true>, one_smem, one_occ))) return rc;
+    if (solve_one_per_thread(0.5 * L.lu_nnz / L.N, sizeof(T), n, (int64_t)sm_count() * tile_occ * 32,
+                             (int64_t)sm_count() * one_occ * 128))
+      return launch(k_lu_solve_one<T, true>, one_smem, blocks, one_occ);
   }
-  return check_cuda(cudaGetLastError(), "k_lu_solve launch");
+  return launch(k_lu_solve<T>, tile_smem, tiles, tile_occ);
 }
 
 int launch_lu_solve(const DevLu& L, int prec, int64_t n, const void* lu, int64_t ld, const void* b, void* x,
