@@ -236,7 +236,7 @@ int pj_sparsity(const pj_mech* mech, int fmt, int32_t* h_ptr, int32_t* h_idx);
  * with wdot_k = sum_i nu_ki R_i c_i; dT/dt from species enthalpies (CONP) or
  * internal energies (CONV); dV/dt or dP/dt from the ideal-gas law with the
  * bath gas closing the mass balance) for n states.  d_work / work_bytes: device
- * scratch of at least pj_workspace_size(PJ_OP_SOURCE) bytes (NULL when 0);
+ * scratch of at least pj_workspace_size(PJ_OP_SOURCE) bytes (never 0);
  * PJ_ERR_NOMEM if it is too small. */
 int pj_eval_source_terms(const pj_mech* mech, int mode, int64_t n, const double* d_param,
                          const double* d_phi, int64_t ld, double* d_dphi, int* d_status,
@@ -383,9 +383,11 @@ int pj_jacobian_layout(const pj_mech* mech, int fmt, int prec, int64_t n, int32_
 #define PJ_OP_FD 5
 #define PJ_OP_LU 6
 
-/* Device scratch (bytes) an operation needs for a batch of n states; 0 when
- * the per-state working arrays fit in shared memory (PJ_OP_VJP always needs
- * room for its per-warp parameter-gradient partial sums). */
+/* Device scratch (bytes) an operation needs for a batch of n states.
+ * PJ_OP_SOURCE (production-rate accumulators), PJ_OP_FD (the same) and
+ * PJ_OP_VJP (a block's rows of production rates and gradients, the adjoint of
+ * each reaction, the blocks' parameter-gradient sums) always need some; the
+ * others 0 where the per-state working arrays fit in shared memory. */
 int pj_workspace_size(const pj_mech* mech, int op, int64_t n, size_t* bytes);
 
 /* First-order forward finite-difference Jacobian, the comparator of

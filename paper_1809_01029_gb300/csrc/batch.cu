@@ -195,7 +195,7 @@ static int plan_configure(pj_plan* p, int tpb, int bps, int use_smem) {
     if (p->op != 1) return fail(PJ_ERR_UNSUPPORTED, "plan: the cooperative layout computes Jacobians only");
     CoopPlan c{};
     if (!coop_shape(p->mech->dm, tpb / 32, bps, use_smem != 0, plan_max_tiles(p), c))
-      return fail(PJ_ERR_UNSUPPORTED, "plan: cooperative shape does not fit (blocks x warps <= 16 per SM, "
+      return fail(PJ_ERR_UNSUPPORTED, "plan: cooperative shape does not fit (blocks x warps <= 20 per SM, "
                                       "shared memory)");
     drop_graph(p);
     int rc = plan_workspace(p, c.ws_bytes);

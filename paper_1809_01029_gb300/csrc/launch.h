@@ -77,8 +77,8 @@ struct CoopSrc {
   unsigned long long* counter;  // zeroed before the launch
 };
 
-// Shape the cooperative layout: `warps` (4, 8, 16) warps per block, `ctas`
-// blocks per SM, per-state arrays in shared memory (arrays_smem) or in a
+// Shape the cooperative layout: `warps` (4 to 20) warps per block, `ctas`
+// blocks per SM (at most 20 warps in all), per-state arrays in shared memory (arrays_smem) or in a
 // global workspace; false when it does not fit.  tiles bounds the grid.
 bool coop_shape(const DevMech& m, int warps, int ctas, bool arrays_smem, int64_t tiles, CoopPlan& c);
 
